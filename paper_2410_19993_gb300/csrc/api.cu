@@ -216,6 +216,10 @@ static int cr_sweep_launches(const xbar_s* h, int B, bool initial) {
   return 3 + L + (initial ? 0 : L + 1);
 }
 
+// kernel launches of one CUDA-core block-Thomas substitution (sweep.cu): the inward part, unless an
+// input vector (V) meets no left chain or the system has one column, and the outward part
+static int sweep_launches(int meet, int N, bool V) { return 1 + (meet > 0 || (!V && meet < N - 1) ? 1 : 0); }
+
 // BF16 terms of the tensor-core sweep for refinement correction `it` (0-based).  A correction
 // only needs accuracy relative to its own size, so the first two are solved with two terms
 // (~2^-17 per product); one term (2^-9 per product, accumulated over the 2N - 1 dependent steps)
@@ -357,6 +361,8 @@ static xbar_status solve_rows(xbar_s* h, int B, const double* dV, double* dI, do
       sp.src = m2.src_pl;
       sp.V = nullptr;
       sp.rhs = rhs;
+      sp.meet = g->meet;
+      sp.first_only = !dvWL && !dvBL;  // the currents are read from the first block
       sp.z = (double*)g->z.p;
       sp.w = w2;
       sp.I = (double*)g->sI.p;
@@ -450,6 +456,8 @@ static xbar_status solve_rows_mixed(xbar_s* h, int B, const double* dV, double* 
   sp.src = m2.src32;
   sp.V = nullptr;
   sp.rhs = (const float*)g->rhat.p;
+  sp.meet = g->meet;
+  sp.first_only = false;
   sp.z = (float*)g->z.p;
   sp.w = (float*)g->dhat.p;
   sp.I = (double*)g->sI.p;
@@ -550,25 +558,48 @@ static xbar_status do_factor_cr(xbar_t h, bool equilibrate) {
   return XBAR_OK;
 }
 
-template <typename T>
-static xbar_status do_factor(xbar_t h, bool equilibrate, bool upload) {
+// FP64 block Thomas, eliminated from both ends (factor64.cu)
+static xbar_status do_factor64(xbar_t h) {
+  MapDev& m = h->m;
+  XB_CUDA(ensure(h->A, h->X, (size_t)m.N * m.Mp * m.Mp * sizeof(double)));
+  XB_CUDA(ensure(h->A, h->fpbuf, factor64_buf_bytes(m.Mp)));
+  XB_CUDA(ensure(h->A, h->fbar, factor64_flag_bytes()));
+  h->meet = factor64_meet(m.Mp, m.N);
+  Factor64Params fp;
+  fp.M = m.M;
+  fp.Mp = m.Mp;
+  fp.N = m.N;
+  fp.meet = h->meet;
+  fp.gsrc = m.gs;
+  fp.gw = m.gw;
+  fp.Coff = m.Coff;
+  fp.h = m.h;
+  fp.X = (double*)h->X.p;
+  fp.buf = (double*)h->fpbuf.p;
+  fp.flags = (unsigned*)h->fbar.p;
+  fp.status = h->status;
+  PhaseScope ps(h, XBAR_PHASE_FACTOR, 1);
+  XB_CUDA(launch_factor64(fp, h->st));
+  h->tc_ready = 0;
+  return XBAR_OK;
+}
+
+static xbar_status do_factor32(xbar_t h, bool upload) {
   MapDev& m = h->m;
   const int Mp = m.Mp, N = m.N;
-  const int PB = factor_panel_width<T>();
-  int bpm;
-  // FP64 needs many SMs (the FP64 pipe is 1/64 of FP32); FP32 is latency-bound, so fewer blocks
-  // (cheaper cross-block barriers) with 16 rows each
-  if (Mp <= 32) bpm = 1;
-  else bpm = std::min(h->nsm, Mp / (sizeof(T) == 8 ? 2 : 16));
+  const int PB = factor_panel_width();
+  // latency-bound: few blocks (cheap cross-block barriers) with 16 rows each
+  int bpm = Mp <= 32 ? 1 : std::min(h->nsm, Mp / 16);
   if (bpm < 1) bpm = 1;
-  XB_CUDA(ensure(h->A, h->X, (size_t)N * Mp * Mp * sizeof(T)));
-  XB_CUDA(ensure(h->A, h->fsig, 2 * (size_t)Mp * sizeof(T)));
+  XB_CUDA(ensure(h->A, h->X, (size_t)N * Mp * Mp * sizeof(float)));
+  XB_CUDA(ensure(h->A, h->fsig, 2 * (size_t)Mp * sizeof(float)));
   size_t pbuf_n = 2 * (size_t)PB * Mp;
-  if (sizeof(T) == 4 && factor_cluster_supported(Mp)) pbuf_n = std::max(pbuf_n, factor_cluster_pbuf_floats(Mp));
-  XB_CUDA(ensure(h->A, h->fpbuf, pbuf_n * sizeof(T)));
+  if (factor_cluster_supported(Mp)) pbuf_n = std::max(pbuf_n, factor_cluster_pbuf_floats(Mp));
+  XB_CUDA(ensure(h->A, h->fpbuf, pbuf_n * sizeof(float)));
   XB_CUDA(ensure(h->A, h->fbar, 2 * sizeof(unsigned)));
-  XB_CUDA(ensure(h->A, h->fparams, sizeof(FactorParams<T>)));
-  FactorParams<T> fp;
+  XB_CUDA(ensure(h->A, h->fparams, sizeof(FactorParams)));
+  h->meet = N - 1;  // one chain, column 0 to N - 1
+  FactorParams fp;
   memset(&fp, 0, sizeof(fp));  // padding too: the block is compared byte for byte below
   fp.M = m.M;
   fp.Mp = Mp;
@@ -577,11 +608,11 @@ static xbar_status do_factor(xbar_t h, bool equilibrate, bool upload) {
   fp.gw = m.gw;
   fp.Coff = m.Coff;
   fp.h = m.h;
-  fp.s = equilibrate ? m.s_eq : nullptr;
-  fp.e = equilibrate ? m.e_eq : m.e_pl;
-  fp.X = (T*)h->X.p;
-  fp.sig = (T*)h->fsig.p;
-  fp.pbuf = (T*)h->fpbuf.p;
+  fp.s = m.s_eq;
+  fp.e = m.e_eq;
+  fp.X = (float*)h->X.p;
+  fp.sig = (float*)h->fsig.p;
+  fp.pbuf = (float*)h->fpbuf.p;
   fp.bar = (unsigned*)h->fbar.p;
   XB_CUDA(cudaMemsetAsync(h->fbar.p, 0, 2 * sizeof(unsigned), h->st));
   if (upload) {
@@ -599,13 +630,13 @@ static xbar_status do_factor(xbar_t h, bool equilibrate, bool upload) {
       h->fparams_dev = h->fparams.p;
     }
   }
-  PhaseScope ps(h, XBAR_PHASE_FACTOR, sizeof(T) == 4 && use_tc_sweep(h) ? 2 : 1);
-  if (sizeof(T) == 4 && use_cluster_factor(h))
-    XB_CUDA(launch_factor_cluster((const FactorParams<float>*)h->fparams.p, 1, Mp, h->status, h->st));
+  PhaseScope ps(h, XBAR_PHASE_FACTOR, use_tc_sweep(h) ? 2 : 1);
+  if (use_cluster_factor(h))
+    XB_CUDA(launch_factor_cluster((const FactorParams*)h->fparams.p, 1, Mp, h->status, h->st));
   else
-    XB_CUDA(launch_factor<T>((const FactorParams<T>*)h->fparams.p, 1, Mp, bpm, h->status, h->st));
+    XB_CUDA(launch_factor((const FactorParams*)h->fparams.p, 1, Mp, bpm, h->status, h->st));
   h->tc_ready = 0;
-  if (sizeof(T) == 4 && use_tc_sweep(h)) {
+  if (use_tc_sweep(h)) {
     XB_CUDA(ensure(h->A, h->Xt, sweep_tc_tile_bytes(Mp, N)));
     XB_CUDA(launch_sweep_tc_tile((const float*)h->X.p, h->Xt.p, Mp, N, h->st));
     h->tc_ready = 1;
@@ -641,7 +672,7 @@ xbar_status xbar::factor_handle(xbar_s* h, xbar_precision p, bool upload_params)
   h->tc_ready = 0;
   xbar_status s;
   if (cr) s = (p == XBAR_FP64) ? do_factor_cr<double>(h, false) : do_factor_cr<float>(h, true);
-  else s = (p == XBAR_FP64) ? do_factor<double>(h, false, upload_params) : do_factor<float>(h, true, upload_params);
+  else s = (p == XBAR_FP64) ? do_factor64(h) : do_factor32(h, upload_params);
   if (s != XBAR_OK) return s;
   h->cr_active = cr ? 1 : 0;
   h->prec = p;
@@ -808,6 +839,8 @@ extern "C" xbar_status xbar_solve(xbar_t h, int B, const double* V, double* I, d
     sp.src = m.src_pl;
     sp.V = dV;
     sp.rhs = nullptr;
+    sp.meet = h->meet;
+    sp.first_only = false;
     sp.z = (double*)h->z.p;
     sp.w = want_v ? (double*)h->w64.p : nullptr;
     sp.I = dI;
@@ -829,7 +862,7 @@ extern "C" xbar_status xbar_solve(xbar_t h, int B, const double* V, double* I, d
       ca.I = dI;
       XB_CUDA(cr_sweep<double>(h, h->cr64, ca));
     } else {
-      PhaseScope ps(h, XBAR_PHASE_SWEEP);
+      PhaseScope ps(h, XBAR_PHASE_SWEEP, sweep_launches(h->meet, N, true));
       XB_CUDA(launch_sweep<double>(sp, st));
     }
     rp.w = (double*)h->w64.p;
@@ -866,6 +899,8 @@ extern "C" xbar_status xbar_solve(xbar_t h, int B, const double* V, double* I, d
     sp.src = m.src32;
     sp.V = dV;
     sp.rhs = nullptr;
+    sp.meet = h->meet;
+    sp.first_only = false;
     sp.z = (float*)h->z.p;
     sp.w = (float*)h->dhat.p;
     sp.I = dI;
@@ -1028,7 +1063,7 @@ xbar_status xbar::solve_device_driven(xbar_s* h, int B, const double* dV, double
     SweepParams<double> sp;
     sp.M = M; sp.Mp = Mp; sp.N = N; sp.B = B; sp.Bp = Bp; sp.Bpad = Bpad;
     sp.X = (const double*)h->X.p; sp.e = m.e_pl; sp.hs = m.h; sp.src = m.src_pl;
-    sp.V = dV; sp.rhs = nullptr; sp.z = (double*)h->z.p; sp.w = nullptr; sp.I = dI;
+    sp.V = dV; sp.rhs = nullptr; sp.meet = h->meet; sp.first_only = false; sp.z = (double*)h->z.p; sp.w = nullptr; sp.I = dI;
     sp.accumulate = 0; sp.max_rel = nullptr; sp.status = h->status;
     XB_CUDA(launch_ir_init(state, st));
     XB_CUDA(launch_sweep<double>(sp, st));
@@ -1049,7 +1084,7 @@ xbar_status xbar::solve_device_driven(xbar_s* h, int B, const double* dV, double
   SweepParams<float> sp;
   sp.M = M; sp.Mp = Mp; sp.N = N; sp.B = B; sp.Bp = Bp; sp.Bpad = Bpad;
   sp.X = (const float*)h->X.p; sp.e = m.e32; sp.hs = m.hs32; sp.src = m.src32;
-  sp.V = dV; sp.rhs = nullptr; sp.z = (float*)h->z.p; sp.w = (float*)h->dhat.p; sp.I = dI;
+  sp.V = dV; sp.rhs = nullptr; sp.meet = h->meet; sp.first_only = false; sp.z = (float*)h->z.p; sp.w = (float*)h->dhat.p; sp.I = dI;
   sp.accumulate = 0; sp.max_rel = nullptr; sp.status = h->status;
   auto sweep = [&](int terms) -> cudaError_t {
     return tc ? launch_sweep_tc(sp, h->Xt.p, terms, st) : launch_sweep<float>(sp, st);
@@ -1306,6 +1341,8 @@ extern "C" xbar_status xbar_solve_noalloc(xbar_t h, int B, const double* V, doub
   sp.src = m.src_pl;
   sp.V = V;
   sp.rhs = nullptr;
+  sp.meet = h->meet;
+  sp.first_only = false;
   sp.z = (double*)scratch;
   sp.w = nullptr;
   sp.I = I;

@@ -1,5 +1,5 @@
-// factor.cu -- block Thomas factorization of the word-line system (Sec. II-C: one decomposition
-// per conductance map).
+// factor.cu -- FP32 block Thomas factorization of the word-line system (Sec. II-C: one decomposition
+// per conductance map); FP64 factors are in factor64.cu, cluster-sized FP32 ones in factor_cluster.cu.
 //
 // After the bit lines are eliminated inside each column (assemble.cu) the word-line unknowns form
 // a block-tridiagonal system with dense M x M diagonal blocks C_j and couplings -g_w I between
@@ -32,35 +32,26 @@ namespace xbar {
 
 constexpr int kFactorThreads = 256;
 
-template <typename T>
-struct FacPB;
-template <>
-struct FacPB<double> { static constexpr int value = 16; };
-template <>
-struct FacPB<float> { static constexpr int value = 16; };
+constexpr int kFactorPB = 16;
 
-template <typename T>
-int factor_panel_width() { return FacPB<T>::value; }
+int factor_panel_width() { return kFactorPB; }
 
-template <typename T>
-size_t factor_smem_bytes(int Mp, int R) {
-  constexpr int PB = FacPB<T>::value;
+static size_t factor_smem_bytes(int Mp, int R) {
+  constexpr int PB = kFactorPB;
   size_t n = (size_t)R * Mp + (size_t)PB * Mp + PB * PB + (size_t)R * PB + Mp + R;
-  return n * sizeof(T) + 16;
+  return n * sizeof(float) + 16;
 }
 
-template <typename T>
-__device__ __forceinline__ T warp_sum(T v) {
+__device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
 
-template <typename T>
 __global__ void __launch_bounds__(kFactorThreads)
-    factor_kernel(const FactorParams<T>* __restrict__ maps, int blocks_per_map, unsigned* status) {
-  constexpr int PB = FacPB<T>::value;
-  const FactorParams<T> p = maps[blockIdx.x / blocks_per_map];
+    factor_kernel(const FactorParams* __restrict__ maps, int blocks_per_map, unsigned* status) {
+  constexpr int PB = kFactorPB;
+  const FactorParams p = maps[blockIdx.x / blocks_per_map];
   const int g = blockIdx.x % blocks_per_map;
   const int M = p.M, Mp = p.Mp, N = p.N;
   const int R = (Mp + blocks_per_map - 1) / blocks_per_map;  // rows per block
@@ -70,17 +61,17 @@ __global__ void __launch_bounds__(kFactorThreads)
   constexpr int nwarps = kFactorThreads / 32;
 
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* rows = reinterpret_cast<T*>(smem_raw);   // [R][Mp]
-  T* pn = rows + (size_t)R * Mp;              // [PB][Mp]
-  T* D = pn + (size_t)PB * Mp;                // [PB][PB]
-  T* W = D + PB * PB;                         // [R][PB]
-  T* sigv = W + R * PB;                       // [Mp]
-  T* sgm = sigv + Mp;                         // [R] sigma_j of own rows
+  float* rows = reinterpret_cast<float*>(smem_raw);   // [R][Mp]
+  float* pn = rows + (size_t)R * Mp;              // [PB][Mp]
+  float* D = pn + (size_t)PB * Mp;                // [PB][PB]
+  float* W = D + PB * PB;                         // [R][PB]
+  float* sigv = W + R * PB;                       // [Mp]
+  float* sgm = sigv + Mp;                         // [R] sigma_j of own rows
   __shared__ unsigned flag;
-  __shared__ T rinv_s;
+  __shared__ float rinv_s;
 
   const uint64_t limit = wait_limit(status);
-  const T gw = (T)p.gw;
+  const float gw = (float)p.gw;
   const int npanel = Mp / PB;
 
   for (int j = 0; j < N; ++j) {
@@ -92,22 +83,22 @@ __global__ void __launch_bounds__(kFactorThreads)
 
     // (1) sigma_j of own rows (needs X^_{j-1} own rows, still in `rows`, and all of sigma_{j-1})
     if (j > 0) {
-      const T* sp = p.sig + (size_t)((j - 1) & 1) * Mp;
+      const float* sp = p.sig + (size_t)((j - 1) & 1) * Mp;
       for (int k = tid; k < Mp; k += kFactorThreads)
-        sigv[k] = ld_cg(sp + k) * (sjm ? (T)sjm[k] : (T)1);
+        sigv[k] = ld_cg(sp + k) * (sjm ? (float)sjm[k] : 1.0f);
       __syncthreads();
       for (int r = warp; r < nr; r += nwarps) {
         const int i = r0 + r;
-        T acc = 0;
+        float acc = 0;
         for (int k = lane; k < Mp; k += 32) acc += rows[(size_t)r * Mp + k] * sigv[k];
         acc = warp_sum(acc);
         if (lane == 0)
-          sgm[r] = (i < M) ? (T)hj[i] + gw * (sjm ? (T)sjm[i] : (T)1) * acc : (T)0;
+          sgm[r] = (i < M) ? (float)hj[i] + gw * (sjm ? (float)sjm[i] : 1.0f) * acc : 0.0f;
       }
     } else {
       for (int r = tid; r < nr; r += kFactorThreads) {
         const int i = r0 + r;
-        sgm[r] = (i < M) ? (T)(hj[i] + p.gsrc) : (T)0;
+        sgm[r] = (i < M) ? (float)(hj[i] + p.gsrc) : 0.0f;
       }
     }
     __syncthreads();
@@ -115,7 +106,7 @@ __global__ void __launch_bounds__(kFactorThreads)
 
     // (2) X^_{j-1} own rows to the output
     if (j > 0) {
-      T* Xo = p.X + (size_t)(j - 1) * Mp * Mp + (size_t)r0 * Mp;
+      float* Xo = p.X + (size_t)(j - 1) * Mp * Mp + (size_t)r0 * Mp;
       for (int t = tid; t < nr * Mp; t += kFactorThreads) Xo[t] = rows[t];
     }
     __syncthreads();
@@ -123,28 +114,28 @@ __global__ void __launch_bounds__(kFactorThreads)
     // (3) Z^_j own rows: off-diagonal, then the subtraction-free diagonal
     for (int t = tid; t < nr * Mp; t += kFactorThreads) {
       const int r = t / Mp, k = t - r * Mp, i = r0 + r;
-      T v = 0;
+      float v = 0;
       if (i < M && k < M && k != i) {
-        const T si = sj ? (T)sj[i] : (T)1, sk = sj ? (T)sj[k] : (T)1;
-        v = si * sk * (T)Cj[(size_t)i * Mp + k];
-        if (j > 0) v -= (T)ejm[i] * (T)ejm[k] * rows[t];
+        const float si = sj ? (float)sj[i] : 1.0f, sk = sj ? (float)sj[k] : 1.0f;
+        v = si * sk * (float)Cj[(size_t)i * Mp + k];
+        if (j > 0) v -= (float)ejm[i] * (float)ejm[k] * rows[t];
       }
       rows[t] = v;
     }
     __syncthreads();
     for (int r = warp; r < nr; r += nwarps) {
       const int i = r0 + r;
-      T acc = 0;
+      float acc = 0;
       for (int k = lane; k < Mp; k += 32) {
-        const T sk = sj ? (T)sj[k] : (T)1;
+        const float sk = sj ? (float)sj[k] : 1.0f;
         if (k < M) acc += fabs(rows[(size_t)r * Mp + k]) / sk;
       }
       acc = warp_sum(acc);
       if (lane == 0) {
-        T d = 1;
+        float d = 1;
         if (i < M) {
-          const T si = sj ? (T)sj[i] : (T)1;
-          d = si * si * (sgm[r] + (j < N - 1 ? gw : (T)0)) + si * acc;
+          const float si = sj ? (float)sj[i] : 1.0f;
+          d = si * si * (sgm[r] + (j < N - 1 ? gw : 0.0f)) + si * acc;
         }
         rows[(size_t)r * Mp + i] = d;
       }
@@ -154,7 +145,7 @@ __global__ void __launch_bounds__(kFactorThreads)
     for (int pp = 0; pp < npanel; ++pp) {
       const int P0 = pp * PB;
       const unsigned pc = (unsigned)(j * npanel + pp);
-      T* pb = p.pbuf + (size_t)(pc & 1) * PB * Mp;
+      float* pb = p.pbuf + (size_t)(pc & 1) * PB * Mp;
       __syncthreads();
       for (int t = tid; t < nr * Mp; t += kFactorThreads) {
         const int r = t / Mp, i = r0 + r;
@@ -166,18 +157,18 @@ __global__ void __launch_bounds__(kFactorThreads)
       for (int t = tid; t < PB * PB; t += kFactorThreads) D[t] = pn[(size_t)(t / PB) * Mp + P0 + t % PB];
       // invert the pivot block in place (scalar sweep operator, no pivoting).  The reciprocal of
       // each pivot is formed once, by the thread that owns that diagonal entry.
-      if (tid == 0) rinv_s = (T)1 / D[0];
+      if (tid == 0) rinv_s = 1.0f / D[0];
       for (int q = 0; q < PB; ++q) {
         __syncthreads();
         constexpr int PER = (PB * PB + kFactorThreads - 1) / kFactorThreads;
-        T nv[PER];
-        const T ri = rinv_s;
+        float nv[PER];
+        const float ri = rinv_s;
 #pragma unroll
         for (int u = 0; u < PER; ++u) {
           const int t = tid + u * kFactorThreads;
           if (t < PB * PB) {
             const int a = t / PB, b = t % PB;
-            const T aq = D[a * PB + q], qb = D[q * PB + b], v = D[t];
+            const float aq = D[a * PB + q], qb = D[q * PB + b], v = D[t];
             if (a == q && b == q) nv[u] = ri;
             else if (a == q) nv[u] = qb * ri;
             else if (b == q) nv[u] = -aq * ri;
@@ -190,7 +181,7 @@ __global__ void __launch_bounds__(kFactorThreads)
           const int t = tid + u * kFactorThreads;
           if (t < PB * PB) {
             D[t] = nv[u];
-            if (q + 1 < PB && t == (q + 1) * (PB + 1)) rinv_s = (T)1 / nv[u];
+            if (q + 1 < PB && t == (q + 1) * (PB + 1)) rinv_s = 1.0f / nv[u];
           }
         }
       }
@@ -199,7 +190,7 @@ __global__ void __launch_bounds__(kFactorThreads)
       for (int t = tid; t < nr * PB; t += kFactorThreads) {
         const int r = t / PB, m = t % PB, i = r0 + r;
         if (i >= P0 && i < P0 + PB) continue;
-        T acc = 0;
+        float acc = 0;
 #pragma unroll
         for (int q = 0; q < PB; ++q) acc += rows[(size_t)r * Mp + P0 + q] * D[q * PB + m];
         W[t] = acc;
@@ -208,13 +199,13 @@ __global__ void __launch_bounds__(kFactorThreads)
       for (int t = tid; t < nr * Mp; t += kFactorThreads) {
         const int r = t / Mp, k = t - r * Mp, i = r0 + r;
         const bool kin = (k >= P0 && k < P0 + PB);
-        T v;
+        float v;
         if (i >= P0 && i < P0 + PB) {  // panel row: D * (old panel rows)
           const int q = i - P0;
           if (kin) {
             v = D[q * PB + (k - P0)];
           } else {
-            T acc = 0;
+            float acc = 0;
 #pragma unroll
             for (int m = 0; m < PB; ++m) acc += D[q * PB + m] * pn[(size_t)m * Mp + k];
             v = acc;
@@ -222,7 +213,7 @@ __global__ void __launch_bounds__(kFactorThreads)
         } else if (kin) {
           v = -W[r * PB + (k - P0)];
         } else {
-          T acc = rows[t];
+          float acc = rows[t];
 #pragma unroll
           for (int m = 0; m < PB; ++m) acc -= W[r * PB + m] * pn[(size_t)m * Mp + k];
           v = acc;
@@ -232,16 +223,15 @@ __global__ void __launch_bounds__(kFactorThreads)
     }
     __syncthreads();
   }
-  T* Xo = p.X + (size_t)(N - 1) * Mp * Mp + (size_t)r0 * Mp;
+  float* Xo = p.X + (size_t)(N - 1) * Mp * Mp + (size_t)r0 * Mp;
   for (int t = tid; t < nr * Mp; t += kFactorThreads) Xo[t] = rows[t];
 }
 
-template <typename T>
-cudaError_t launch_factor(const FactorParams<T>* maps_dev, int nmaps, int Mp_max, int blocks_per_map,
+cudaError_t launch_factor(const FactorParams* maps_dev, int nmaps, int Mp_max, int blocks_per_map,
                           unsigned* status, cudaStream_t st) {
   const int R = (Mp_max + blocks_per_map - 1) / blocks_per_map;
-  const size_t smem = factor_smem_bytes<T>(Mp_max, R);
-  cudaError_t err = cudaFuncSetAttribute(factor_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  const size_t smem = factor_smem_bytes(Mp_max, R);
+  cudaError_t err = cudaFuncSetAttribute(factor_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
   if (err != cudaSuccess) return err;
   cudaLaunchConfig_t cfg = {};
@@ -254,14 +244,7 @@ cudaError_t launch_factor(const FactorParams<T>* maps_dev, int nmaps, int Mp_max
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = (nmaps * blocks_per_map > 1) ? 1 : 0;  // one block needs no co-residency guarantee
-  return cudaLaunchKernelEx(&cfg, factor_kernel<T>, maps_dev, blocks_per_map, status);
+  return cudaLaunchKernelEx(&cfg, factor_kernel, maps_dev, blocks_per_map, status);
 }
-
-template int factor_panel_width<double>();
-template int factor_panel_width<float>();
-template size_t factor_smem_bytes<double>(int, int);
-template size_t factor_smem_bytes<float>(int, int);
-template cudaError_t launch_factor<double>(const FactorParams<double>*, int, int, int, unsigned*, cudaStream_t);
-template cudaError_t launch_factor<float>(const FactorParams<float>*, int, int, int, unsigned*, cudaStream_t);
 
 }  // namespace xbar

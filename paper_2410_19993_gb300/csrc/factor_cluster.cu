@@ -113,9 +113,9 @@ __device__ __forceinline__ void rank16_update(float (&acc)[16], const float* __r
 }
 
 __global__ void __launch_bounds__(kThreads, 1)
-    factor_cluster_kernel(const FactorParams<float>* __restrict__ maps, int C, unsigned* status) {
+    factor_cluster_kernel(const FactorParams* __restrict__ maps, int C, unsigned* status) {
   constexpr int R = kRows;  // rows per block = panel width
-  const FactorParams<float> p = maps[blockIdx.x / C];
+  const FactorParams p = maps[blockIdx.x / C];
   const uint32_t g = cluster_rank();
   const int M = p.M, Mp = p.Mp, N = p.N;
   const int r0 = (int)g * R;
@@ -404,7 +404,7 @@ bool factor_cluster_supported(int Mp) { return Mp >= 2 * kRows && Mp <= 16 * kRo
 
 int factor_cluster_size(int Mp) { return Mp / kRows; }
 
-cudaError_t launch_factor_cluster(const FactorParams<float>* maps_dev, int nmaps, int Mp, unsigned* status,
+cudaError_t launch_factor_cluster(const FactorParams* maps_dev, int nmaps, int Mp, unsigned* status,
                                   cudaStream_t st) {
   const int C = factor_cluster_size(Mp);
   const size_t smem = factor_cluster_smem_bytes(Mp, kRows);

@@ -115,11 +115,12 @@ struct xbar_s {
   // factor
   xbar::Buf X, fsig, fpbuf, fbar, fparams;
   // host copy of the parameter block last uploaded to `fparams` (skip identical uploads)
-  unsigned char fparams_host[sizeof(xbar::FactorParams<double>)] = {};
+  unsigned char fparams_host[sizeof(xbar::FactorParams)] = {};
   size_t fparams_bytes = 0;
   const void* fparams_dev = nullptr;
   xbar::Buf Xt;    // tensor-core tiled TF32 hi/lo copy of the FP32 factor
   int tc_ready = 0;
+  int meet = 0;    // block Thomas: column in which the factor's elimination chains meet
   // solve workspace
   xbar::Buf z, dhat, rhat, w64, phi, maxrel, rmax, irstate;
   xbar::Buf w1;  // FP32 refinement state written by the initial tensor-core sweep

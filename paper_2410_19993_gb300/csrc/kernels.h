@@ -49,34 +49,47 @@ cudaError_t launch_store_g(const MapDev& m, const double* G_dev, unsigned* statu
 cudaError_t launch_assemble(const MapDev& m, cudaStream_t st);
 
 // ---- factor -----------------------------------------------------------------------------------
-template <typename T>
-struct FactorParams {
+struct FactorParams {  // FP32 factors
   int M, Mp, N;
   double gsrc, gw;
   const double* Coff;
   const double* h;
   const double* s;    // nullptr = no equilibration
   const double* e;
-  T* X;               // [N][Mp][Mp] output
-  T* sig;             // [2][Mp] scratch
-  T* pbuf;            // scratch: [2][PB][Mp] (factor.cu), factor_cluster_pbuf_floats (factor_cluster.cu)
+  float* X;           // [N][Mp][Mp] output
+  float* sig;         // [2][Mp] scratch
+  float* pbuf;           // scratch: [2][PB][Mp] (factor.cu), factor_cluster_pbuf_floats (factor_cluster.cu)
   unsigned* bar;      // 2 words, zeroed
 };
 
-// One group of `blocks_per_map` co-resident blocks factors each map; `maps` is a device array.
-template <typename T>
-cudaError_t launch_factor(const FactorParams<T>* maps_dev, int nmaps, int Mp_max, int blocks_per_map,
+// FP32 factor (factor.cu): one group of `blocks_per_map` co-resident blocks factors each map; `maps`
+// is a device array.
+cudaError_t launch_factor(const FactorParams* maps_dev, int nmaps, int Mp_max, int blocks_per_map,
                           unsigned* status, cudaStream_t st);
-template <typename T>
 int factor_panel_width();
-template <typename T>
-size_t factor_smem_bytes(int Mp, int rows_per_block);
+
+// FP64 factor (factor64.cu): two chains that meet in column `meet` (left 0 .. meet - 1, right N - 1 ..
+// meet + 1); Mp <= 1024.  One cooperative launch; `flags` is cleared by it.
+struct Factor64Params {
+  int M, Mp, N, meet;
+  double gsrc, gw;
+  const double* Coff;
+  const double* h;
+  double* X;          // [N][Mp][Mp] output
+  double* buf;        // factor64_buf_bytes scratch
+  unsigned* flags;    // factor64_flag_bytes
+  unsigned* status;
+};
+int factor64_meet(int Mp, int N);  // the meeting column
+size_t factor64_buf_bytes(int Mp);
+size_t factor64_flag_bytes();
+cudaError_t launch_factor64(const Factor64Params& p, cudaStream_t st);
 
 // FP32 factor on a thread-block cluster (factor_cluster.cu): 32 <= Mp <= 256
 bool factor_cluster_supported(int Mp);
 int factor_cluster_size(int Mp);
 size_t factor_cluster_pbuf_floats(int Mp);  // panel-slot scratch (FactorParams::pbuf) of one map
-cudaError_t launch_factor_cluster(const FactorParams<float>* maps_dev, int nmaps, int Mp, unsigned* status,
+cudaError_t launch_factor_cluster(const FactorParams* maps_dev, int nmaps, int Mp, unsigned* status,
                                   cudaStream_t st);
 
 // ---- sweeps (forward + back substitution, current extraction) ---------------------------------
@@ -88,7 +101,10 @@ struct SweepParams {
   const T* hs;         // [N][Mp]
   const T* src;        // [Mp]   initial mode: rhs_0 = src * V_b
   const double* V;     // [B][M] initial mode, else nullptr
-  const T* rhs;        // [N][Mp][Bpad] correction mode, else nullptr
+  const T* rhs;        // [N][Mp][Bpad] full right-hand side, else nullptr
+  int meet;            // column in which the factor's two elimination chains meet (N - 1: one chain)
+  bool first_only;     // full right-hand side: only column 0 of the solution is wanted (w and I of the
+                       // other columns may be left unwritten)
   T* z;                // N * Mp * Bpad scratch, layout private to each sweep kernel
   T* w;                // [N][Mp][Bpad] solution, or nullptr
   double* I;           // [B][N]

@@ -2,14 +2,22 @@
 // U V = y for every right-hand side; Sec. III-A: one decomposition serves the whole batch),
 // followed by extraction of the bit-line currents.
 //
-// With the block Thomas factor X_j of the word-line system (factor.cu), the substitutions are
-//     forward   z_0 = X_0 r_0,      z_j = X_j (r_j + e_{j-1} o z_{j-1})     j = 1 .. N-1
-//     back      w_{N-1} = z_{N-1},  w_j = z_j + X_j (e_j o w_{j+1})          j = N-2 .. 0
-//     currents  I_j = hs_j . w_j
+// With the block Thomas factor X_j of the word-line system, whose two elimination chains (columns
+// 0 .. m-1 and N-1 .. m+1) meet in column m (factor64.cu; m = N-1: one chain, factor.cu), the
+// substitutions are
+//     inward   z_j = X_j (r_j + e_{j-1} o z_{j-1})   j = 0 .. m-1    (left chain)
+//              z_j = X_j (r_j + e_j o z_{j+1})       j = N-1 .. m+1  (right chain)
+//     meet     w_m = X_m (r_m + e_{m-1} o z_{m-1} + e_m o z_{m+1})
+//     outward  w_j = z_j + X_j (e_j o w_{j+1})       j = m-1 .. 0
+//              w_j = z_j + X_j (e_{j-1} o w_{j-1})   j = m+1 .. N-1
+//     currents I_j = hs_j . w_j
 // where e_j is the (equilibrated) coupling between columns j and j+1 and r the right-hand side
-// (for an input vector V only r_0 = src o V is nonzero; refinement passes give a full r).  Every
-// step is a dense (Mp x Mp) x (Mp x Bp) product over a panel of Bp input vectors, so one block
-// owns one panel and walks all 2N-1 steps; z_j goes to global memory between the two sweeps.
+// (for an input vector V only r_0 = src o V is nonzero, so z is zero on the right and the right chain
+// has no inward part; refinement passes give a full r).  Every step is a dense (Mp x Mp) x (Mp x Bp)
+// product over a panel of Bp input vectors.  The inward and the outward parts are two launches; in each
+// a block owns one panel and one chain, so the chains of a panel run side by side and a solve is N
+// dependent steps deep instead of 2N - 1, with 1.5 N products for an input vector instead of 2N - 1.
+// (Both blocks of a panel form w_m, one product of N.)  z_j goes to global memory in between.
 //
 // Data movement: X_j is streamed through shared memory in chunks of KC rows by the bulk-copy
 // (TMA) engine, double-buffered and completed on mbarriers with bounded waits; the running
@@ -101,8 +109,9 @@ __device__ __forceinline__ void load_vec(T (&r)[n], const T* p) {
   }
 }
 
-template <typename T, int TR, int TC>
-__global__ void __launch_bounds__(sweep_max_threads<TR, TC>()) sweep_kernel(SweepParams<T> p, int KC) {
+// chain of a block: blockIdx.y + chain0.  kOut: the meeting column and the outward part.
+template <typename T, int TR, int TC, bool kOut>
+__global__ void __launch_bounds__(sweep_max_threads<TR, TC>()) sweep_kernel(SweepParams<T> p, int KC, int chain0) {
   const int Mp = p.Mp, N = p.N, Bp = p.Bp, Bpad = p.Bpad;
   const int nrg = Mp / TR, ncg = Bp / TC;
   const int tid = threadIdx.x;
@@ -124,13 +133,18 @@ __global__ void __launch_bounds__(sweep_max_threads<TR, TC>()) sweep_kernel(Swee
   }
 
   const int chunks_per_step = Mp / KC;
-  const int nsteps = 2 * N - 1;
+  const int m = p.meet, chain = (int)blockIdx.y + chain0;
+  const int len = chain == 0 ? m : N - 1 - m;  // columns of the chain
+  const int nsteps = len + (kOut ? 1 : 0);
+  // column of step s: inward 0, 1, .. (left) or N-1, N-2, .. (right); outward m, then away from it
+  const int jdir = (chain == 0) == kOut ? -1 : 1, jstart = kOut ? m : (chain == 0 ? 0 : N - 1);
+  auto col_of = [&](int s) { return jstart + jdir * s; };
   const long long nchunks = (long long)nsteps * chunks_per_step;
   const unsigned chunk_bytes = (unsigned)(KC * Mp * sizeof(T));
   auto chunk_src = [&](long long c) -> const T* {
     const int s = (int)(c / chunks_per_step);
     const int k0 = (int)(c - (long long)s * chunks_per_step) * KC;
-    const int j = s < N ? s : 2 * N - 2 - s;
+    const int j = col_of(s);
     return p.X + ((size_t)j * Mp + k0) * Mp;
   };
 
@@ -145,8 +159,8 @@ __global__ void __launch_bounds__(sweep_max_threads<TR, TC>()) sweep_kernel(Swee
     bulk_g2s(xs, chunk_src(0), chunk_bytes, &mbar[0]);
   }
 
-  // input of step 0
-  const T* r0 = p.rhs;
+  // input of step 0: the right-hand side of its column and, in the meeting column, both chains' z
+  const bool from_left = kOut && m > 0, from_right = kOut && !p.V && m + 1 < N;
 #pragma unroll
   for (int a = 0; a < TR; ++a) {
     const int i = i0 + a;
@@ -154,8 +168,10 @@ __global__ void __launch_bounds__(sweep_max_threads<TR, TC>()) sweep_kernel(Swee
     for (int c = 0; c < TC; ++c) {
       const int b = b0 + c0 + c;
       T v;
-      if (p.V) v = (i < p.M && b < p.B) ? p.src[i] * (T)p.V[(size_t)b * p.M + i] : (T)0;
-      else v = r0[(size_t)i * Bpad + b];
+      if (p.V) v = (jstart == 0 && i < p.M && b < p.B) ? p.src[i] * (T)p.V[(size_t)b * p.M + i] : (T)0;
+      else v = p.rhs[((size_t)jstart * Mp + i) * Bpad + b];
+      if (from_left) v = fma(p.e[(size_t)(m - 1) * Mp + i], p.z[((size_t)(m - 1) * Mp + i) * Bpad + b], v);
+      if (from_right) v = fma(p.e[(size_t)m * Mp + i], p.z[((size_t)(m + 1) * Mp + i) * Bpad + b], v);
       vin[(size_t)i * Bp + c0 + c] = v;
     }
   }
@@ -165,8 +181,7 @@ __global__ void __launch_bounds__(sweep_max_threads<TR, TC>()) sweep_kernel(Swee
   long long c = 0;
   float local_max = 0.0f;
   for (int s = 0; s < nsteps; ++s) {
-    const bool fwd = s < N;
-    const int j = fwd ? s : 2 * N - 2 - s;
+    const int j = col_of(s);
 #pragma unroll
     for (int a = 0; a < TR; ++a)
 #pragma unroll
@@ -199,19 +214,18 @@ __global__ void __launch_bounds__(sweep_max_threads<TR, TC>()) sweep_kernel(Swee
 
     // ---- epilogue of step s ------------------------------------------------------------------
     const size_t rowbase = (size_t)j * Mp;
-    if (fwd) {
+    if (!kOut) {
 #pragma unroll
       for (int a = 0; a < TR; ++a)
 #pragma unroll
         for (int b = 0; b < TC; ++b) p.z[(rowbase + i0 + a) * Bpad + b0 + c0 + b] = acc[a][b];
-    } else {
+    } else if (s > 0 && (chain == 0 || !p.V)) {
 #pragma unroll
       for (int a = 0; a < TR; ++a)
 #pragma unroll
         for (int b = 0; b < TC; ++b) acc[a][b] += p.z[(rowbase + i0 + a) * Bpad + b0 + c0 + b];
     }
-    const bool have_w = !fwd || s == N - 1;  // w_{N-1} = z_{N-1}
-    if (have_w) {
+    if (kOut && (s > 0 || chain == 0)) {  // w_m is reported by the left block
       if (p.w) {
 #pragma unroll
         for (int a = 0; a < TR; ++a)
@@ -268,11 +282,9 @@ __global__ void __launch_bounds__(sweep_max_threads<TR, TC>()) sweep_kernel(Swee
     }
     // input of step s+1
     if (s + 1 < nsteps) {
-      const bool nfwd = s + 1 < N;
-      const int jn = nfwd ? s + 1 : 2 * N - 3 - s;  // column of the next step
-      const int jc = nfwd ? j : jn;                 // coupling index: e_{j} (fwd) or e_{jn} (bwd)
-      const T* ev = p.e + (size_t)jc * Mp;
-      const T* rn = (nfwd && p.rhs) ? p.rhs + (size_t)jn * Mp * Bpad : nullptr;
+      const int jn = col_of(s + 1);
+      const T* ev = p.e + (size_t)min(j, jn) * Mp;  // coupling between the two columns
+      const T* rn = (!kOut && p.rhs) ? p.rhs + (size_t)jn * Mp * Bpad : nullptr;
 #pragma unroll
       for (int a = 0; a < TR; ++a) {
         const int i = i0 + a;
@@ -302,16 +314,24 @@ static cudaError_t launch_tiled(const SweepParams<T>& p, int KC, cudaStream_t st
   if (blocks == 0) return cudaSuccess;
   if ((long long)blocks * p.Bp > p.Bpad) return cudaErrorInvalidValue;
   const size_t smem = sweep_smem_bytes<T>(p.Mp, p.Bp, KC, TR);
-  cudaError_t err = cudaFuncSetAttribute(sweep_kernel<T, TR, TC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+  cudaError_t err = cudaFuncSetAttribute(sweep_kernel<T, TR, TC, false>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (err == cudaSuccess)
+    err = cudaFuncSetAttribute(sweep_kernel<T, TR, TC, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
-  sweep_kernel<T, TR, TC><<<blocks, threads, smem, st>>>(p, KC);
+  const bool left = p.meet > 0, right = p.meet < p.N - 1;
+  const bool right_in = right && p.rhs;  // an input vector enters at column 0 only
+  if (left || right_in) {
+    sweep_kernel<T, TR, TC, false><<<dim3(blocks, left && right_in ? 2 : 1), threads, smem, st>>>(p, KC, left ? 0 : 1);
+    if ((err = cudaGetLastError()) != cudaSuccess) return err;
+  }
+  sweep_kernel<T, TR, TC, true><<<dim3(blocks, right && !(p.rhs && p.first_only) ? 2 : 1), threads, smem, st>>>(p, KC, 0);
   return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t launch_sweep(const SweepParams<T>& p, cudaStream_t st) {
-  if (p.Mp <= 0 || p.Bp <= 0) return cudaErrorInvalidValue;
+  if (p.Mp <= 0 || p.Bp <= 0 || p.meet < 0 || p.meet >= p.N || (!p.V && !p.rhs)) return cudaErrorInvalidValue;
   const int KC = sweep_kc<T>(p.Mp);
   if (sweep_is_narrow<T>(p.Mp, p.Bp)) return launch_tiled<T, kNarrowTR, kNarrowTC>(p, KC, st);
   return launch_tiled<T, SweepCfg<T>::TR, SweepCfg<T>::TC>(p, KC, st);
