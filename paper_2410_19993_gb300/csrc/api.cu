@@ -216,7 +216,7 @@ static int cr_sweep_launches(const xbar_s* h, int B, bool initial) {
   return 3 + L + (initial ? 0 : L + 1);
 }
 
-// kernel launches of one CUDA-core block-Thomas substitution (sweep.cu): the inward part, unless an
+// kernel launches of one block-Thomas substitution (sweep.cu, sweep_tc.cu): the inward part, unless an
 // input vector (V) meets no left chain or the system has one column, and the outward part
 static int sweep_launches(int meet, int N, bool V) { return 1 + (meet > 0 || (!V && meet < N - 1) ? 1 : 0); }
 
@@ -332,7 +332,7 @@ static xbar_status solve_rows(xbar_s* h, int B, const double* dV, double* dI, do
   double* rhs = (double*)g->phi.p;  // consumed by the substitution; then the mirror's bit-line voltages
   double* w2 = (double*)g->w64.p;
   {
-    PhaseScope ps(h, XBAR_PHASE_SWEEP, 2 + (cr ? cr_sweep_launches(g, B, false) : 1));
+    PhaseScope ps(h, XBAR_PHASE_SWEEP, 2 + (cr ? cr_sweep_launches(g, B, false) : sweep_launches(g->meet, N2, false)));
     XB_CUDA(launch_orient_rhs(dV, m2.h, M, M2, Mp2, B, Bpad, rhs, st));
     if (cr) {
       CrSweepArgs<double> ca;
@@ -481,7 +481,7 @@ static xbar_status solve_rows_mixed(xbar_s* h, int B, const double* dV, double* 
     ca.tensor = use_cr_tensor(g) && Bpad >= 128;
     return cr_sweep<float>(g, g->cr32, ca);
   };
-  const int nsw = cr ? cr_sweep_launches(g, B, false) : 1;
+  const int nsw = cr ? cr_sweep_launches(g, B, false) : sweep_launches(g->meet, N2, false);
   {  // x0 = solve32(s o (V h')), the state w = s o x0, I from the state
     PhaseScope ps(h, XBAR_PHASE_SWEEP, 1 + nsw + 1 + (tc ? 0 : 1));
     XB_CUDA(launch_orient_rhs32(dV, m2.h, m2.s32, h->m.M, M2, Mp2, B, Bpad, (float*)g->rhat.p, st));
@@ -592,13 +592,15 @@ static xbar_status do_factor32(xbar_t h, bool upload) {
   int bpm = Mp <= 32 ? 1 : std::min(h->nsm, Mp / 16);
   if (bpm < 1) bpm = 1;
   XB_CUDA(ensure(h->A, h->X, (size_t)N * Mp * Mp * sizeof(float)));
-  XB_CUDA(ensure(h->A, h->fsig, 2 * (size_t)Mp * sizeof(float)));
+  XB_CUDA(ensure(h->A, h->fsig, 4 * (size_t)Mp * sizeof(float)));
   size_t pbuf_n = 2 * (size_t)PB * Mp;
   if (factor_cluster_supported(Mp)) pbuf_n = std::max(pbuf_n, factor_cluster_pbuf_floats(Mp));
   XB_CUDA(ensure(h->A, h->fpbuf, pbuf_n * sizeof(float)));
   XB_CUDA(ensure(h->A, h->fbar, 2 * sizeof(unsigned)));
   XB_CUDA(ensure(h->A, h->fparams, sizeof(FactorParams)));
-  h->meet = N - 1;  // one chain, column 0 to N - 1
+  // the cluster factor eliminates from both ends, the group factor from column 0 to N - 1
+  const bool cluster = use_cluster_factor(h);
+  h->meet = cluster ? (N - 1) / 2 : N - 1;
   FactorParams fp;
   memset(&fp, 0, sizeof(fp));  // padding too: the block is compared byte for byte below
   fp.M = m.M;
@@ -614,6 +616,7 @@ static xbar_status do_factor32(xbar_t h, bool upload) {
   fp.sig = (float*)h->fsig.p;
   fp.pbuf = (float*)h->fpbuf.p;
   fp.bar = (unsigned*)h->fbar.p;
+  fp.meet = h->meet;
   XB_CUDA(cudaMemsetAsync(h->fbar.p, 0, 2 * sizeof(unsigned), h->st));
   if (upload) {
     // The block changes only when a buffer is (re)allocated.  Upload it, and wait for the copy out
@@ -630,9 +633,9 @@ static xbar_status do_factor32(xbar_t h, bool upload) {
       h->fparams_dev = h->fparams.p;
     }
   }
-  PhaseScope ps(h, XBAR_PHASE_FACTOR, use_tc_sweep(h) ? 2 : 1);
-  if (use_cluster_factor(h))
-    XB_CUDA(launch_factor_cluster((const FactorParams*)h->fparams.p, 1, Mp, h->status, h->st));
+  PhaseScope ps(h, XBAR_PHASE_FACTOR, (cluster ? factor_cluster_launches(N) : 1) + (use_tc_sweep(h) ? 1 : 0));
+  if (cluster)
+    XB_CUDA(launch_factor_cluster((const FactorParams*)h->fparams.p, Mp, N, h->meet, h->status, h->st));
   else
     XB_CUDA(launch_factor((const FactorParams*)h->fparams.p, 1, Mp, bpm, h->status, h->st));
   h->tc_ready = 0;
@@ -928,7 +931,7 @@ extern "C" xbar_status xbar_solve(xbar_t h, int B, const double* V, double* I, d
       return cr_sweep<float>(h, h->cr32, ca);
     };
     if (tc) {  // x0 = solve32(b); the sweep writes the state w = s o x0 (FP32) itself
-      PhaseScope ps(h, XBAR_PHASE_SWEEP);
+      PhaseScope ps(h, XBAR_PHASE_SWEEP, sweep_launches(h->meet, N, true));
       XB_CUDA(ensure(h->A, h->w1, nst * 4));
       sp.w = nullptr;
       sp.w1out = (float*)h->w1.p;
@@ -939,7 +942,7 @@ extern "C" xbar_status xbar_solve(xbar_t h, int B, const double* V, double* I, d
       rp.w1 = (const float*)h->w1.p;  // read as (w, 0) until the first update writes the pairs
     } else {
       {
-        PhaseScope ps(h, XBAR_PHASE_SWEEP, cr ? cr_sweep_launches(h, B, true) : 1);
+        PhaseScope ps(h, XBAR_PHASE_SWEEP, cr ? cr_sweep_launches(h, B, true) : sweep_launches(h->meet, N, true));
         XB_CUDA(sweep32(sp));                   // x0 = solve32(b)
       }
       PhaseScope ps(h, XBAR_PHASE_UPDATE);
@@ -960,7 +963,7 @@ extern "C" xbar_status xbar_solve(xbar_t h, int B, const double* V, double* I, d
       sp.accumulate = 1;
       sp.max_rel = (float*)h->maxrel.p;
       {
-        PhaseScope ps(h, XBAR_PHASE_SWEEP, cr ? cr_sweep_launches(h, B, false) : 1);  // dhat = solve32(rhat), I += dI
+        PhaseScope ps(h, XBAR_PHASE_SWEEP, cr ? cr_sweep_launches(h, B, false) : sweep_launches(h->meet, N, false));  // dhat = solve32(rhat), I += dI
         if (tc) XB_CUDA(launch_sweep_tc(sp, h->Xt.p, correction_terms(it), st));
         else XB_CUDA(sweep32(sp));
       }

@@ -1,8 +1,12 @@
 // factor_cluster.cu -- the block Thomas factorization of factor.cu on a thread-block cluster.
 //
-// Same mathematics as factor.cu (Z_0 = C_0, Z_j = C_j - g_w^2 X_{j-1}, X_j = Z_j^{-1}, diagonals
-// from the grounded row sums sigma_j), for FP32 factors with 32 <= Mp <= 256.  A cluster of C blocks owns
-// one map; block g holds rows [g R, (g+1) R) of the current matrix in shared memory (R = 16, C = Mp / R).
+// Same mathematics as factor.cu (Z_j = C_j - g_w^2 X_prev, X_j = Z_j^{-1}, diagonals from the grounded row
+// sums sigma_j), for FP32 factors with 32 <= Mp <= 256, eliminated from both ends: columns 0 .. m-1 and N-1 ..
+// m+1 are two independent chains, one cluster each, and a second launch inverts the meeting column
+//     Z_m = C_m - g_w^2 X_{m-1} - g_w^2 X_{m+1}.
+// The factor is bound by the latency of its chain (16 dependent panels a column on 16 SMs), so half the
+// chain is half the time: 12.25 -> 6.2 ms at 256 x 256, 2.85 -> 1.45 ms at 128 x 128, on twice the SMs.
+// In a cluster of C blocks block g holds rows [g R, (g+1) R) of the current matrix in shared memory (R = 16, C = Mp / R).
 // The in-place blocked Gauss-Jordan inversion uses panels of R rows, so panel p is exactly block p's
 // rows.  With R_p the owner's rows when panel p starts and D_p^-1 the inverse of their pivot block,
 // Gauss-Jordan replaces the owner's rows by D_p^-1 R_p (D_p^-1 in the pivot columns) and every other
@@ -80,17 +84,18 @@ __device__ __forceinline__ float warp_sum_f(float v) {
 }  // namespace
 
 // dynamic shared memory: mbarriers [16 panels + 2 staging], rows [R][Mp], pn [R][Mp], D [R][R],
-// Dr [R][R], W [R][R], Bp [R][R], sigv [Mp], sv [Mp], ev [Mp], sg [2][R], then two staging buffers
-// (FP64) of a column step's inputs: C_j own rows [R][Mp], s_j [Mp], s_{j-1} [Mp], e_{j-1} [Mp], h_j own rows [R]
+// Dr [R][R], W [R][R], Bp [R][R], sigv [Mp], sv [Mp], ev [Mp], sigv2 [Mp], ev2 [Mp], sg [2][R], then two
+// staging buffers (FP64) of a column step's inputs: C_j own rows [R][Mp], s_j [Mp], s of the previous
+// column [Mp], the coupling to it [Mp], h_j own rows [R]
 size_t factor_cluster_smem_bytes(int Mp, int R) {
-  return 18 * sizeof(uint64_t) + ((size_t)2 * R * Mp + 4 * (size_t)R * R + 3 * (size_t)Mp + 2 * R) * sizeof(float) +
+  return 18 * sizeof(uint64_t) + ((size_t)2 * R * Mp + 4 * (size_t)R * R + 5 * (size_t)Mp + 2 * R) * sizeof(float) +
          2 * ((size_t)R * Mp + 3 * (size_t)Mp + R) * sizeof(double);
 }
 
-// global panel slots, one per block of the cluster: R_p [R][Mp] then D_p^-1 [R][R]
+// global panel slots, one per block of each chain's cluster: R_p [R][Mp] then D_p^-1 [R][R]
 size_t factor_cluster_pbuf_floats(int Mp) {
   const size_t C = (size_t)Mp / kRows;
-  return C * ((size_t)kRows * Mp + (size_t)kRows * kRows);
+  return 2 * C * ((size_t)kRows * Mp + (size_t)kRows * kRows);
 }
 
 // acc[r] (r < 16) += sign * sum_m coef[r*16 + m] * col[m], coefficients read as 16-byte broadcasts
@@ -112,12 +117,19 @@ __device__ __forceinline__ void rank16_update(float (&acc)[16], const float* __r
   }
 }
 
+// Cluster c of the grid walks chain chain0 + c; kMeet: one cluster, the meeting column.
+template <bool kMeet>
 __global__ void __launch_bounds__(kThreads, 1)
-    factor_cluster_kernel(const FactorParams* __restrict__ maps, int C, unsigned* status) {
+    factor_cluster_kernel(const FactorParams* __restrict__ params, int C, int chain0, unsigned* status) {
   constexpr int R = kRows;  // rows per block = panel width
-  const FactorParams p = maps[blockIdx.x / C];
+  const FactorParams p = *params;
   const uint32_t g = cluster_rank();
-  const int M = p.M, Mp = p.Mp, N = p.N;
+  const int M = p.M, Mp = p.Mp, N = p.N, m = p.meet;
+  const int chain = kMeet ? 0 : chain0 + (int)blockIdx.x / C;
+  const int nsteps = kMeet ? 1 : (chain == 0 ? m : N - 1 - m);
+  auto col_of = [&](int s) { return kMeet ? m : (chain == 0 ? s : N - 1 - s); };
+  const bool left = kMeet && m > 0, right = kMeet && m + 1 < N;  // chains that end at the meeting column
+  float* sig = p.sig + (size_t)chain * 2 * Mp;
   const int r0 = (int)g * R;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint64_t wlim = wait_limit(status);
@@ -135,8 +147,10 @@ __global__ void __launch_bounds__(kThreads, 1)
   float* Bp = W + R * R;                    // [R][R] next pivot block (look-ahead)
   float* sigv = Bp + R * R;                 // [Mp]
   float* sv = sigv + Mp;                    // [Mp] equilibration scale of column j
-  float* ev = sv + Mp;                      // [Mp] coupling to column j-1
-  float* sg = ev + Mp;                      // [2][R] sigma of own rows, by step parity
+  float* ev = sv + Mp;                      // [Mp] coupling to the previous column
+  float* sigv2 = ev + Mp;                   // [Mp] meeting column: sigma, coupling of the right neighbour
+  float* ev2 = sigv2 + Mp;                  // [Mp]
+  float* sg = ev2 + Mp;                     // [2][R] sigma of own rows, by step parity
   double* stg = reinterpret_cast<double*>(sg + 2 * R);  // [2] staging buffers (16-byte aligned)
   const size_t stg_n = (size_t)R * Mp + 3 * (size_t)Mp + R;
 
@@ -152,23 +166,22 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
   fence_mbar_init();
   cluster_sync();  // every block's mbarriers are initialised before any peer arrives on them
-  // column step jj's inputs (own rows of C_jj, s_jj, s_jj-1, e_jj-1, own h_jj) -> staging buffer jj & 1
-  // by bulk copies, one step ahead (thread 0)
-  auto stage_inputs = [&](int jj) {
-    double* buf = stg + (size_t)(jj & 1) * stg_n;
-    uint64_t* bar = &pbar[jj & 1];
+  // step ss's inputs (own rows of C_j, s_j, s and coupling of the previous column, own h_j) -> staging
+  // buffer ss & 1 by bulk copies, one step ahead (thread 0)
+  auto stage_inputs = [&](int ss) {
+    double* buf = stg + (size_t)(ss & 1) * stg_n;
+    uint64_t* bar = &pbar[ss & 1];
+    const int jj = col_of(ss), jp = chain == 0 ? jj - 1 : jj + 1;
     const unsigned cb = (unsigned)(R * Mp * sizeof(double)), vb = (unsigned)(Mp * sizeof(double));
     const unsigned hb = (unsigned)(R * sizeof(double));
-    unsigned bytes = cb + hb;
-    if (p.s) bytes += vb;
-    if (p.s && jj > 0) bytes += vb;
-    if (jj > 0) bytes += vb;
-    mbar_arrive_expect_tx(bar, bytes);
+    mbar_arrive_expect_tx(bar, cb + hb + vb + (ss > 0 ? 2 * vb : 0));
     bulk_g2s(buf, p.Coff + ((size_t)jj * Mp + r0) * Mp, cb, bar);
     bulk_g2s(buf + (size_t)R * Mp + 3 * Mp, p.h + (size_t)jj * Mp + r0, hb, bar);
-    if (p.s) bulk_g2s(buf + (size_t)R * Mp, p.s + (size_t)jj * Mp, vb, bar);
-    if (p.s && jj > 0) bulk_g2s(buf + (size_t)R * Mp + Mp, p.s + (size_t)(jj - 1) * Mp, vb, bar);
-    if (jj > 0) bulk_g2s(buf + (size_t)R * Mp + 2 * Mp, p.e + (size_t)(jj - 1) * Mp, vb, bar);
+    bulk_g2s(buf + (size_t)R * Mp, p.s + (size_t)jj * Mp, vb, bar);
+    if (ss > 0) {
+      bulk_g2s(buf + (size_t)R * Mp + Mp, p.s + (size_t)jp * Mp, vb, bar);
+      bulk_g2s(buf + (size_t)R * Mp + 2 * Mp, p.e + (size_t)min(jj, jp) * Mp, vb, bar);
+    }
   };
   if (tid == 0) stage_inputs(0);
   const size_t slot = (size_t)R * Mp + R * R;  // floats per panel slot
@@ -176,62 +189,109 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (tid == 0) failed = 0;
   __syncthreads();
 
-  for (int j = 0; j < N; ++j) {
+  if (kMeet) {  // own rows of both neighbours' inverses
+    const float* XL = p.X + ((size_t)(m - 1) * Mp + r0) * Mp;
+    const float* XR = p.X + ((size_t)(m + 1) * Mp + r0) * Mp;
+    for (int t = tid; t < R * Mp; t += kThreads) {
+      rows[t] = left ? XL[t] : 0.0f;
+      pn[t] = right ? XR[t] : 0.0f;
+    }
+  }
+
+  for (int s = 0; s < nsteps; ++s) {
+    const int j = col_of(s), jp = chain == 0 ? j - 1 : j + 1;
+    const bool has_prev = s > 0;
     // this step's inputs from the staging buffer (the next step's copies overlap this step)
-    const double* stj = stg + (size_t)(j & 1) * stg_n;
+    const double* stj = stg + (size_t)(s & 1) * stg_n;
     const double* Cj = stj;                                      // own rows of C_j
-    const double* sj = p.s ? stj + (size_t)R * Mp : nullptr;
-    const double* sjm = (p.s && j > 0) ? stj + (size_t)R * Mp + Mp : nullptr;
-    const double* ejm = j > 0 ? stj + (size_t)R * Mp + 2 * Mp : nullptr;
+    const double* sj = stj + (size_t)R * Mp;
+    const double* sjm = has_prev ? sj + Mp : nullptr;
+    const double* ejm = has_prev ? sj + 2 * Mp : nullptr;
     const double* hj = stj + (size_t)R * Mp + 3 * Mp;          // own rows: hj[r] is h_j of row r0 + r
     if (tid == 0) {
-      if (j + 1 < N) stage_inputs(j + 1);
-      if (!failed && !mbar_wait_bounded(&pbar[j & 1], (unsigned)((j >> 1) & 1), status, wlim))
+      if (s + 1 < nsteps) stage_inputs(s + 1);
+      if (!failed && !mbar_wait_bounded(&pbar[s & 1], (unsigned)((s >> 1) & 1), status, wlim))
         failed = 1;
     }
     __syncthreads();
 
     for (int k = tid; k < Mp; k += kThreads) {
-      sv[k] = sj ? (float)sj[k] : 1.0f;
-      ev[k] = ejm ? (float)ejm[k] : 0.0f;
+      sv[k] = (float)sj[k];
+      if (!kMeet) {
+        ev[k] = ejm ? (float)ejm[k] : 0.0f;
+      } else {
+        ev[k] = left ? (float)p.e[(size_t)(m - 1) * Mp + k] : 0.0f;
+        ev2[k] = right ? (float)p.e[(size_t)m * Mp + k] : 0.0f;
+      }
     }
-    // (1) sigma_j of own rows: h_j + g_w S X^_{j-1} S sigma_{j-1}  (X^_{j-1} own rows are in `rows`)
-    if (j > 0) {
-      const float* sp = p.sig + (size_t)((j - 1) & 1) * Mp;
-      for (int k = tid; k < Mp; k += kThreads) sigv[k] = __ldcg(sp + k) * (sjm ? (float)sjm[k] : 1.0f);
+    // (1) sigma_j of own rows: h_j (+ g_s in column 0) + g_w S X^_prev S sigma_prev  (X^_prev own rows are in
+    // `rows`; the meeting column has two such neighbours, the right one's rows in `pn`)
+    if (has_prev || kMeet) {
+      for (int k = tid; k < Mp; k += kThreads) {
+        if (!kMeet) {
+          sigv[k] = __ldcg(sig + (size_t)((s - 1) & 1) * Mp + k) * (float)sjm[k];
+        } else {
+          sigv[k] = left ? __ldcg(p.sig + (size_t)((m - 1) & 1) * Mp + k) * (float)p.s[(size_t)(m - 1) * Mp + k] : 0.0f;
+          sigv2[k] = right ? __ldcg(p.sig + (size_t)(2 + ((N - 2 - m) & 1)) * Mp + k) *
+                                 (float)p.s[(size_t)(m + 1) * Mp + k]
+                           : 0.0f;
+        }
+      }
       __syncthreads();
       for (int r = warp; r < R; r += nwarps) {
         const int i = r0 + r;
-        float acc = 0.0f;
-        for (int k = lane; k < Mp; k += 32) acc = fmaf(rows[(size_t)r * Mp + k], sigv[k], acc);
+        float acc = 0.0f, acc2 = 0.0f;
+        for (int k = lane; k < Mp; k += 32) {
+          acc = fmaf(rows[(size_t)r * Mp + k], sigv[k], acc);
+          if (kMeet) acc2 = fmaf(pn[(size_t)r * Mp + k], sigv2[k], acc2);
+        }
         acc = warp_sum_f(acc);
-        if (lane == 0)
-          sg[(j & 1) * R + r] = (i < M) ? (float)hj[r] + gw * (sjm ? (float)sjm[i] : 1.0f) * acc : 0.0f;
+        if (kMeet) acc2 = warp_sum_f(acc2);
+        if (lane == 0) {
+          float v = 0.0f;
+          if (i < M) {
+            v = (float)(hj[r] + (j == 0 ? p.gsrc : 0.0));
+            if (!kMeet) {
+              v += gw * (float)sjm[i] * acc;
+            } else {
+              if (left) v += gw * (float)p.s[(size_t)(m - 1) * Mp + i] * acc;
+              if (right) v += gw * (float)p.s[(size_t)(m + 1) * Mp + i] * acc2;
+            }
+          }
+          sg[(s & 1) * R + r] = v;
+        }
       }
     } else {
       for (int r = tid; r < R; r += kThreads) {
         const int i = r0 + r;
-        sg[r] = (i < M) ? (float)(hj[r] + p.gsrc) : 0.0f;
+        sg[r] = (i < M) ? (float)(hj[r] + (j == 0 ? p.gsrc : 0.0)) : 0.0f;
       }
     }
     __syncthreads();
-    for (int r = tid; r < R; r += kThreads) p.sig[(size_t)(j & 1) * Mp + r0 + r] = sg[(j & 1) * R + r];
+    if (!kMeet)
+      for (int r = tid; r < R; r += kThreads) sig[(size_t)(s & 1) * Mp + r0 + r] = sg[(s & 1) * R + r];
 
     // (2) + (3) Z^_j own rows (off-diagonal, then the subtraction-free diagonal) in place of
-    // X^_{j-1}, whose own rows go to the output on the way: each element of `rows` is read, stored
-    // to X and overwritten by the same thread, so no thread can overwrite an element of X^_{j-1}
+    // X^_prev, whose own rows go to the output on the way: each element of `rows` is read, stored
+    // to X and overwritten by the same thread, so no thread can overwrite an element of X^_prev
     // before it has been stored
-    float* Xo = j > 0 ? p.X + (size_t)(j - 1) * Mp * Mp + (size_t)r0 * Mp : nullptr;
+    float* Xo = has_prev ? p.X + (size_t)jp * Mp * Mp + (size_t)r0 * Mp : nullptr;
     for (int t = tid * 2; t < R * Mp; t += kThreads * 2) {
       const int r = t / Mp, k = t - r * Mp, i = r0 + r;
       const double2 c2 = *reinterpret_cast<const double2*>(Cj + t);
       const float si = sv[i], ei = ev[i];
-      const float x0 = j > 0 ? rows[t] : 0.0f, x1 = j > 0 ? rows[t + 1] : 0.0f;  // X^_{j-1}
-      if (j > 0) *reinterpret_cast<float2*>(Xo + t) = make_float2(x0, x1);
+      const bool use = has_prev || kMeet;
+      const float x0 = use ? rows[t] : 0.0f, x1 = use ? rows[t + 1] : 0.0f;  // X^_prev
+      if (has_prev) *reinterpret_cast<float2*>(Xo + t) = make_float2(x0, x1);
       float v0 = 0.0f, v1 = 0.0f;
       if (i < M) {
         if (k < M && k != i) v0 = si * sv[k] * (float)c2.x - ei * ev[k] * x0;
         if (k + 1 < M && k + 1 != i) v1 = si * sv[k + 1] * (float)c2.y - ei * ev[k + 1] * x1;
+        if (kMeet) {
+          const float e2 = ev2[i];
+          if (k < M && k != i) v0 -= e2 * ev2[k] * pn[t];
+          if (k + 1 < M && k + 1 != i) v1 -= e2 * ev2[k + 1] * pn[t + 1];
+        }
       }
       rows[t] = v0;
       rows[t + 1] = v1;
@@ -246,7 +306,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         float d = 1.0f;
         if (i < M) {
           const float si = sv[i];
-          d = si * si * (sg[(j & 1) * R + r] + (j < N - 1 ? gw : 0.0f)) + si * acc;
+          d = si * si * (sg[(s & 1) * R + r] + (kMeet ? 0.0f : gw)) + si * acc;
         }
         rows[(size_t)r * Mp + i] = d;
       }
@@ -259,7 +319,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     // pivot's row, column and diagonal arrive by shuffles.
     static_assert(R == 16, "register layout assumes 16 x 16 pivot blocks");
     const int pb = lane & 15, pa0 = (lane >> 4) * 8;
-    float* myslot = p.pbuf + (size_t)g * slot;  // R_g then D_g^-1
+    float* slots = p.pbuf + (size_t)chain * C * slot;
+    float* myslot = slots + (size_t)g * slot;  // R_g then D_g^-1
     auto invert_publish = [&](float (&d)[8]) {  // warp kInvWarp: D^-1 to Dm and to this block's slot
 #pragma unroll
       for (int q = 0; q < R; ++q) {
@@ -320,12 +381,12 @@ __global__ void __launch_bounds__(kThreads, 1)
         // wait for panel pp, then read R_pp and D_pp^-1 from its slot (L2)
         bool ok = true;
         if (tid == 0 && !failed) {
-          ok = wait_cluster_bounded(&bars[pp], (unsigned)(j & 1), status);
+          ok = wait_cluster_bounded(&bars[pp], (unsigned)(s & 1), status);
           if (!ok) failed = 1;
         }
         __syncthreads();
         // D_pp^-1 to shared memory first; R_pp into registers, stored after W' (its latency overlaps W')
-        const float4* src = reinterpret_cast<const float4*>(p.pbuf + (size_t)pp * slot);
+        const float4* src = reinterpret_cast<const float4*>(slots + (size_t)pp * slot);
         if (tid < R * R / 4) reinterpret_cast<float4*>(Dr)[tid] = __ldcg(src + R * Mp / 4 + tid);
         constexpr int kPer = (kRows * 16 * kRows / 4 + kWork - 1) / kWork;  // float4 per thread, Mp <= 16 R
         float4 rp[kPer];
@@ -394,7 +455,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     cluster_sync();  // every read of this step's slots is done before the next step rewrites them
   }
   {
-    float* Xo = p.X + (size_t)(N - 1) * Mp * Mp + (size_t)r0 * Mp;
+    float* Xo = p.X + (size_t)col_of(nsteps - 1) * Mp * Mp + (size_t)r0 * Mp;
     for (int t = tid; t < R * Mp; t += kThreads) Xo[t] = rows[t];
   }
   cluster_sync();  // no block leaves while another may still read its shared memory
@@ -404,19 +465,18 @@ bool factor_cluster_supported(int Mp) { return Mp >= 2 * kRows && Mp <= 16 * kRo
 
 int factor_cluster_size(int Mp) { return Mp / kRows; }
 
-cudaError_t launch_factor_cluster(const FactorParams* maps_dev, int nmaps, int Mp, unsigned* status,
-                                  cudaStream_t st) {
-  const int C = factor_cluster_size(Mp);
-  const size_t smem = factor_cluster_smem_bytes(Mp, kRows);
-  cudaError_t err = cudaFuncSetAttribute(factor_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+int factor_cluster_launches(int N) { return N > 1 ? 2 : 1; }
+
+template <bool kMeet>
+static cudaError_t launch_clusters(const FactorParams* params, int C, int clusters, int chain0, size_t smem,
+                                   unsigned* status, cudaStream_t st) {
+  cudaError_t err = cudaFuncSetAttribute(factor_cluster_kernel<kMeet>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
+  if (err == cudaSuccess && C > 8)
+    err = cudaFuncSetAttribute(factor_cluster_kernel<kMeet>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (err != cudaSuccess) return err;
-  if (C > 8) {
-    err = cudaFuncSetAttribute(factor_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (err != cudaSuccess) return err;
-  }
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(nmaps * C);
+  cfg.gridDim = dim3(clusters * C);
   cfg.blockDim = dim3(kThreads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
@@ -427,7 +487,23 @@ cudaError_t launch_factor_cluster(const FactorParams* maps_dev, int nmaps, int M
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, factor_cluster_kernel, maps_dev, C, status);
+  return cudaLaunchKernelEx(&cfg, factor_cluster_kernel<kMeet>, params, C, chain0, status);
+}
+
+// the chains (those that have columns), then the meeting column; the launch boundary is what the
+// second waits for, so no cluster waits for another
+cudaError_t launch_factor_cluster(const FactorParams* params_dev, int Mp, int N, int meet, unsigned* status,
+                                  cudaStream_t st) {
+  if (meet < 0 || meet >= N) return cudaErrorInvalidValue;
+  const int C = factor_cluster_size(Mp);
+  const size_t smem = factor_cluster_smem_bytes(Mp, kRows);
+  const bool left = meet > 0, right = meet < N - 1;
+  if (left || right) {
+    const cudaError_t err = launch_clusters<false>(params_dev, C, (left ? 1 : 0) + (right ? 1 : 0), left ? 0 : 1, smem,
+                                                   status, st);
+    if (err != cudaSuccess) return err;
+  }
+  return launch_clusters<true>(params_dev, C, 1, 0, smem, status, st);
 }
 
 }  // namespace xbar

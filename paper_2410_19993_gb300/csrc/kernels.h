@@ -57,9 +57,10 @@ struct FactorParams {  // FP32 factors
   const double* s;    // nullptr = no equilibration
   const double* e;
   float* X;           // [N][Mp][Mp] output
-  float* sig;         // [2][Mp] scratch
-  float* pbuf;           // scratch: [2][PB][Mp] (factor.cu), factor_cluster_pbuf_floats (factor_cluster.cu)
+  float* sig;         // scratch: [2][Mp] (factor.cu), [2 chains][2][Mp] (factor_cluster.cu)
+  float* pbuf;        // scratch: [2][PB][Mp] (factor.cu), factor_cluster_pbuf_floats (factor_cluster.cu)
   unsigned* bar;      // 2 words, zeroed
+  int meet;           // factor_cluster.cu: column in which its two elimination chains meet
 };
 
 // FP32 factor (factor.cu): one group of `blocks_per_map` co-resident blocks factors each map; `maps`
@@ -88,8 +89,9 @@ cudaError_t launch_factor64(const Factor64Params& p, cudaStream_t st);
 // FP32 factor on a thread-block cluster (factor_cluster.cu): 32 <= Mp <= 256
 bool factor_cluster_supported(int Mp);
 int factor_cluster_size(int Mp);
-size_t factor_cluster_pbuf_floats(int Mp);  // panel-slot scratch (FactorParams::pbuf) of one map
-cudaError_t launch_factor_cluster(const FactorParams* maps_dev, int nmaps, int Mp, unsigned* status,
+size_t factor_cluster_pbuf_floats(int Mp);  // panel-slot scratch (FactorParams::pbuf)
+int factor_cluster_launches(int N);
+cudaError_t launch_factor_cluster(const FactorParams* params_dev, int Mp, int N, int meet, unsigned* status,
                                   cudaStream_t st);
 
 // ---- sweeps (forward + back substitution, current extraction) ---------------------------------
@@ -130,7 +132,7 @@ constexpr int kSweepTcPanel = 64;
 // X (FP32 [N][Mp][Mp]) -> Xt: three-term BF16 split in the MMA's chunked core-matrix order
 size_t sweep_tc_tile_bytes(int Mp, int N);
 cudaError_t launch_sweep_tc_tile(const float* X, void* Xt, int Mp, int N, cudaStream_t st);
-// terms = leading BF16 terms of the split used (1..3): 3 gives FP32-level accuracy
+// terms = leading BF16 terms of the split used (2 or 3): 3 gives FP32-level accuracy
 cudaError_t launch_sweep_tc(const SweepParams<float>& p, const void* Xt, int terms, cudaStream_t st);
 
 // ---- blocking over rows (orient.cu): the mirrored crossbar M' = N, N' = M ---------------------

@@ -1,9 +1,11 @@
 // sweep_tc.cu -- forward/back substitution on the 5th-generation tensor cores (tcgen05).
 //
-// Same recurrences as sweep.cu (Sec. II-C substitutions after block Thomas):
-//     z_0 = X_0 r_0,  z_j = X_j (r_j + e_{j-1} o z_{j-1});   w_{N-1} = z_{N-1},
-//     w_j = z_j + X_j (e_j o w_{j+1});   I_j = hs_j . w_j,
-// for a panel of 64 input vectors per block.  Each step is D[Mt x 64] = X_j[Mt x Mt] . v[Mt x 64]
+// Same recurrences and the same two launches as sweep.cu (Sec. II-C substitutions after block Thomas
+// from both ends): inward along the left chain 0 .. m-1 and the right chain N-1 .. m+1,
+//     z_j = X_j (r_j + e o z_prev),
+// then the meeting column w_m = X_m (r_m + e_{m-1} o z_{m-1} + e_m o z_{m+1}) and outward along both chains,
+//     w_j = z_j + X_j (e o w_prev);   I_j = hs_j . w_j,
+// a block per chain and panel of 64 input vectors.  Each step is D[Mt x 64] = X_j[Mt x Mt] . v[Mt x 64]
 // computed from three-term BF16 splits (x = x0 + x1 + x2, each BF16: together 24+ significant bits,
 // FP32-level accuracy; a plain BF16 or TF32 product would cost the refinement extra passes).  With
 // KP leading terms used, each K step of 16 issues A_p v_q for every p + q < KP (N = 64 each) into
@@ -19,7 +21,7 @@
 // lands MMA-ready data in shared memory.  B = the running vector of the panel, written by the
 // epilogue threads in MN-major core-matrix order (8 nodes x 8 columns per core matrix, columns
 // contiguous), so each thread stores 8 columns of its node at once.  D = tcgen05 tensor memory,
-// one 192-column slab per 128-row half of X_j.
+// one 64-column slab per 128-row half of X_j and step parity.
 //
 // z (the forward result kept for the back substitution) never leaves this kernel, so it is stored
 // in the order the epilogue holds it -- thread = row, four columns per 16-byte access -- as
@@ -178,18 +180,19 @@ __host__ __device__ constexpr int tc_stages(int Mt, int KP) {
              ? 8
              : (232448 - tc_fixed(Mt, KP)) / (int)(tc_sub(Mt, KP) * tc_slot(Mt, KP));
 }
-static_assert(tc_stages(256, 1) == 5 && tc_stages(256, 2) == 2 && tc_stages(256, 3) == 2 &&
+static_assert(tc_stages(256, 2) == 2 && tc_stages(256, 3) == 2 &&
                   tc_stages(128, 2) == 5 && tc_stages(128, 3) == 3,
               "stage rings");
 
 // NH = number of 128-row halves of X_j (Mt = 128 NH); KP = number of BF16 terms of the split used
-// (1..3; the tiles always hold three, a sweep with fewer copies and multiplies only the leading
+// (2 or 3; the tiles always hold three, a sweep with fewer copies and multiplies only the leading
 // ones).  Every size the MMA issue loop touches is a compile-time constant: the single issuing
 // thread then spends no dependent integer work per MMA (runtime offsets in that loop tripled its
 // cost per MMA).
-template <int NH, int KP>
+// Chain of a block: blockIdx.y + chain0.  kOut: the meeting column and the outward part.
+template <int NH, int KP, bool kOut>
 __global__ void __launch_bounds__(tc::kThreads + 64, 1)
-    sweep_tc_kernel(SweepParams<float> p, const __nv_bfloat16* __restrict__ Xt) {
+    sweep_tc_kernel(SweepParams<float> p, const __nv_bfloat16* __restrict__ Xt, int chain0) {
   using namespace tc;
   constexpr int BP = kBP, KC = kKC;
   constexpr int Mt = 128 * NH, nh = NH;
@@ -220,7 +223,11 @@ __global__ void __launch_bounds__(tc::kThreads + 64, 1)
   float4* pres = reinterpret_cast<float4*>(vb + tc_vbytes(Mt, KP));
 
   constexpr int cps = Mt / KC;  // chunks per step
-  const int nsteps = 2 * N - 1;
+  const int m = p.meet, chain = (int)blockIdx.y + chain0;
+  const int nsteps = (chain == 0 ? m : N - 1 - m) + (kOut ? 1 : 0);
+  // column of step s: inward 0, 1, .. (left) or N-1, N-2, .. (right); outward m, then away from it
+  const int jdir = (chain == 0) == kOut ? -1 : 1, jstart = kOut ? m : (chain == 0 ? 0 : N - 1);
+  auto col_of = [&](int s) { return jstart + jdir * s; };
   const long long nchunks = (long long)nsteps * cps;
   // accumulators: per 128-row half, 64 columns; two sets, for even and odd steps, so that the
   // epilogue can re-read this step's D while the next step's MMAs accumulate into the other set
@@ -265,7 +272,7 @@ __global__ void __launch_bounds__(tc::kThreads + 64, 1)
         if (c >= NS && !mbar_spin_bounded(&empty[st], (unsigned)((use - 1) & 1), p.status, wlim, 0))
           break;
         issued = c + 1;
-        const int j = s < N ? s : 2 * N - 2 - s;
+        const int j = col_of(s);
         mbar_arrive_expect_tx(&full[st], kSub * copy_bytes);
 #pragma unroll
         for (int sub = 0; sub < kSub; ++sub)
@@ -376,6 +383,11 @@ __global__ void __launch_bounds__(tc::kThreads + 64, 1)
       if (lane == 0) mbar_arrive(vfull);
     };
 
+    // the right-hand side of the first column and, in the meeting column, both chains' z
+    auto zpanel = [&](int jj) { return p.z + ((size_t)jj * (Bpad / BP) + blockIdx.x) * (size_t)Mp * BP; };
+    const bool from_left = kOut && m > 0 && real, from_right = kOut && !p.V && m + 1 < N && real;
+    const float el = from_left ? p.e[(size_t)(m - 1) * Mp + i] : 0.0f;
+    const float er = from_right ? p.e[(size_t)m * Mp + i] : 0.0f;
     for (int blk = 0; blk < ncb; ++blk)
       for (int n0 = 0; n0 < 32; n0 += 8) {
         float v[8];
@@ -383,28 +395,46 @@ __global__ void __launch_bounds__(tc::kThreads + 64, 1)
           const int b = b0 + cb + blk * 32 + n0 + e;
           v[e] = 0.0f;
           if (p.V) {
-            if (i < p.M && b < p.B) v[e] = p.src[i] * (float)p.V[(size_t)b * p.M + i];
+            if (jstart == 0 && i < p.M && b < p.B) v[e] = p.src[i] * (float)p.V[(size_t)b * p.M + i];
           } else if (real) {
-            v[e] = p.rhs[(size_t)i * Bpad + b];
+            v[e] = p.rhs[((size_t)jstart * Mp + i) * Bpad + b];
+          }
+        }
+        for (int e = 0; e < 8; e += 4) {
+          const size_t zo = (size_t)((cb + blk * 32 + n0 + e) / 4) * Mp + i;
+          if (from_left) {
+            const float4 z4 = reinterpret_cast<const float4*>(zpanel(m - 1))[zo];
+            v[e] = fmaf(el, z4.x, v[e]);
+            v[e + 1] = fmaf(el, z4.y, v[e + 1]);
+            v[e + 2] = fmaf(el, z4.z, v[e + 2]);
+            v[e + 3] = fmaf(el, z4.w, v[e + 3]);
+          }
+          if (from_right) {
+            const float4 z4 = reinterpret_cast<const float4*>(zpanel(m + 1))[zo];
+            v[e] = fmaf(er, z4.x, v[e]);
+            v[e + 1] = fmaf(er, z4.y, v[e + 1]);
+            v[e + 2] = fmaf(er, z4.z, v[e + 2]);
+            v[e + 3] = fmaf(er, z4.w, v[e + 3]);
           }
         }
         put_v8(cb + blk * 32 + n0, v);
       }
     release_v();
 
+    // z is added on the way out, except in the meeting column and where it is zero (an input vector
+    // has no inward part on the right)
+    const bool zout = kOut && (chain == 0 || !p.V);
     // warm L2 with the global operands step s2's epilogue reads before its accumulator wait: z of
-    // step s2 (back substitution) or the right-hand side of the column after it (forward).  Issued
+    // step s2 (outward) or the right-hand side of the column after it (inward).  Issued
     // as soon as step s2 - 1 has released its vector, so the copies overlap that step's stores.
     auto warm_l2 = [&](int s2) {
-      const bool fwd2 = s2 < N;
-      const int j2 = fwd2 ? s2 : 2 * N - 2 - s2;
-      const float* zp2 = p.z + ((size_t)j2 * (Bpad / BP) + blockIdx.x) * (size_t)Mp * BP;
+      const float* zp2 = zpanel(col_of(s2));
       const int i0 = i - lane + (lane & 3) * 8;  // this lane's quarter of the warp's 32 rows
       for (int blk = 0; blk < ncb; ++blk) {
-        if (!fwd2 && i0 < Mp)
+        if (zout && s2 > 0 && i0 < Mp)
           asm volatile("prefetch.global.L2 [%0];" ::"l"(zp2 + ((size_t)((cb + blk * 32) / 4 + (lane >> 2)) * Mp + i0) * 4));
-        if (real && s2 + 1 < N && p.rhs)
-          asm volatile("prefetch.global.L2 [%0];" ::"l"(p.rhs + ((size_t)(j2 + 1) * Mp + i) * Bpad + b0 + cb + blk * 32));
+        if (!kOut && real && s2 + 1 < nsteps && p.rhs)
+          asm volatile("prefetch.global.L2 [%0];" ::"l"(p.rhs + ((size_t)col_of(s2 + 1) * Mp + i) * Bpad + b0 + cb + blk * 32));
       }
     };
     warm_l2(0);
@@ -432,25 +462,23 @@ __global__ void __launch_bounds__(tc::kThreads + 64, 1)
     };
     float local_max = 0.0f;
     for (int s = 0; s < nsteps; ++s) {
-      const bool fwd = s < N;
-      const int j = fwd ? s : 2 * N - 2 - s;
-      const bool nfwd = s + 1 < N;
-      float* zp = p.z + ((size_t)j * (Bpad / BP) + blockIdx.x) * (size_t)Mp * BP;  // z panel of step j
-      const float ej = real ? (nfwd ? p.e[(size_t)j * Mp + i] : (j > 0 ? p.e[(size_t)(j - 1) * Mp + i] : 0.0f))
-                            : 0.0f;
+      const int j = col_of(s);
+      const bool more = s + 1 < nsteps;
+      const int jn = more ? col_of(s + 1) : j;  // the next step's column
+      float* zp = zpanel(j);
+      const float ej = real && more ? p.e[(size_t)min(j, jn) * Mp + i] : 0.0f;
       const float hj = real ? p.hs[(size_t)j * Mp + i] : 0.0f;
       const float sj = (real && p.w1out) ? p.s32[(size_t)j * Mp + i] : 0.0f;
-      const size_t rowoff = ((size_t)j * Mp + (real ? i : 0)) * Bpad + b0 + cb;
-      const bool have_w = !fwd || s == N - 1;
-      const bool more = s + 1 < nsteps;
+      const bool have_w = kOut && (s > 0 || chain == 0);  // w_m is reported by the left block
       // the current this step adds to, read now so that its latency overlaps the accumulator wait
       double Iold = 0.0;
       if (have_w && p.accumulate && tid < BP && b0 + tid < p.B) Iold = p.I[(size_t)(b0 + tid) * N + j];
-      // the next input's operands that do not depend on D -- z of this step (back substitution) or
-      // the next column's right-hand side (forward) -- are loaded before the wait: column block 0
+      // the next input's operands that do not depend on D -- z of this step (outward) or the next
+      // column's right-hand side (inward) -- are loaded before the wait: column block 0
       // now, block 1 right after it, so their latency leaves the step's critical path
-      const bool use_z = !fwd && real;
-      const bool use_r = more && nfwd && p.rhs && real;
+      const bool use_z = zout && s > 0 && real;
+      const bool use_r = !kOut && more && p.rhs && real;
+      const float* rnext = p.rhs + ((size_t)jn * Mp + (real ? i : 0)) * Bpad + b0 + cb;
       float pre[ncb][32];
       // block 1 (nh == 2): 16-byte cp.async copies into this thread's slice of pres, waited for
       // after the accumulator wait, so their latency overlaps it
@@ -463,7 +491,7 @@ __global__ void __launch_bounds__(tc::kThreads + 64, 1)
                          "l"(zrow + (size_t)(n / 4) * Mp)
                          : "memory");
         } else if (use_r) {
-          const float* rn = p.rhs + rowoff + 32 + (size_t)Mp * Bpad;
+          const float* rn = rnext + 32;
 #pragma unroll
           for (int n = 0; n < 32; n += 4)
             asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(smem_addr(pres + (n / 4) * kThreads + tid)),
@@ -497,7 +525,7 @@ __global__ void __launch_bounds__(tc::kThreads + 64, 1)
             pre[blk][n + 3] = zz.w;
           }
         } else if (use_r) {
-          const float* rn = p.rhs + rowoff + blk * 32 + (size_t)Mp * Bpad;
+          const float* rn = rnext + blk * 32;
 #pragma unroll
           for (int n = 0; n < 32; n += 4) {
             const float4 r4 = *reinterpret_cast<const float4*>(rn + n);
@@ -522,7 +550,7 @@ __global__ void __launch_bounds__(tc::kThreads + 64, 1)
       fence_after();
       if (nh == 2) take_pre1();
 
-      // (1) D of this step per column block (z added in the back substitution), then (2) the next
+      // (1) D of this step per column block (z added on the way out), then (2) the next
       // step's input from it, split into BF16 terms; then the next step's MMAs may start
       const uint32_t tstep = tbase + ((uint32_t)(q * 32) << 16) + (uint32_t)((s & 1) * dset + h * dcols + cb);
       if (more) {
@@ -544,7 +572,7 @@ __global__ void __launch_bounds__(tc::kThreads + 64, 1)
         release_v();
         warm_l2(s + 1);
       }
-      // (3) while the next step's MMAs run: z (forward), w and the current (back substitution)
+      // (3) while the next step's MMAs run: z (inward), w and the current (outward)
       float dots[ncb];
 #pragma unroll
       for (int blk = 0; blk < ncb; ++blk) {
@@ -553,7 +581,7 @@ __global__ void __launch_bounds__(tc::kThreads + 64, 1)
         if (use_z)
 #pragma unroll
           for (int n = 0; n < 32; ++n) a[n] += pre[blk][n];
-        if (fwd && real) {
+        if (!kOut && real) {
           float4* zrow = reinterpret_cast<float4*>(zp) + (size_t)((cb + blk * 32) / 4) * Mp + i;
 #pragma unroll
           for (int n = 0; n < 32; n += 4)
@@ -637,15 +665,28 @@ cudaError_t launch_sweep_tc(const SweepParams<float>& p, const void* Xt, int ter
   if (p.Bp != tc::kBP || p.Bpad % tc::kBP) return cudaErrorInvalidValue;
   const int blocks = (p.B + tc::kBP - 1) / tc::kBP;
   if (blocks == 0) return cudaSuccess;
-  if (terms < 1 || terms > tc::kParts) return cudaErrorInvalidValue;
+  if (terms < 2 || terms > tc::kParts) return cudaErrorInvalidValue;
   const size_t smem = sweep_tc_smem_bytes(Mt, terms);
-  using Kern = void (*)(SweepParams<float>, const __nv_bfloat16*);
-  const Kern kerns[2][3] = {{sweep_tc_kernel<1, 1>, sweep_tc_kernel<1, 2>, sweep_tc_kernel<1, 3>},
-                            {sweep_tc_kernel<2, 1>, sweep_tc_kernel<2, 2>, sweep_tc_kernel<2, 3>}};
-  const Kern kern = kerns[Mt == 128 ? 0 : 1][terms - 1];
-  cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (err != cudaSuccess) return err;
-  kern<<<blocks, tc::kThreads + 64, smem, st>>>(p, static_cast<const __nv_bfloat16*>(Xt));
+  if (p.meet < 0 || p.meet >= p.N || (!p.V && !p.rhs)) return cudaErrorInvalidValue;
+  using Kern = void (*)(SweepParams<float>, const __nv_bfloat16*, int);
+  const Kern kerns[2][2][2] = {{{sweep_tc_kernel<1, 2, false>, sweep_tc_kernel<1, 2, true>},
+                                {sweep_tc_kernel<1, 3, false>, sweep_tc_kernel<1, 3, true>}},
+                               {{sweep_tc_kernel<2, 2, false>, sweep_tc_kernel<2, 2, true>},
+                                {sweep_tc_kernel<2, 3, false>, sweep_tc_kernel<2, 3, true>}}};
+  const Kern* kern = kerns[Mt == 128 ? 0 : 1][terms - 2];
+  for (int k = 0; k < 2; ++k) {
+    const cudaError_t err = cudaFuncSetAttribute(kern[k], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (err != cudaSuccess) return err;
+  }
+  const __nv_bfloat16* X = static_cast<const __nv_bfloat16*>(Xt);
+  const bool left = p.meet > 0, right = p.meet < p.N - 1;
+  const bool right_in = right && p.rhs;  // an input vector enters at column 0 only
+  if (left || right_in) {
+    kern[0]<<<dim3(blocks, left && right_in ? 2 : 1), tc::kThreads + 64, smem, st>>>(p, X, left ? 0 : 1);
+    const cudaError_t err = cudaGetLastError();
+    if (err != cudaSuccess) return err;
+  }
+  kern[1]<<<dim3(blocks, right ? 2 : 1), tc::kThreads + 64, smem, st>>>(p, X, 0);
   return cudaGetLastError();
 }
 
