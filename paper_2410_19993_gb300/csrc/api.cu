@@ -207,13 +207,13 @@ extern "C" xbar_status xbar_assemble(int M, int N, const double* G, double R_s, 
   return XBAR_OK;
 }
 
-// kernel launches of one cyclic-reduction substitution (for the per-phase launch counts)
-static int cr_sweep_launches(const xbar_s* h, int B, bool initial) {
-  (void)B;
+// kernel launches of one cyclic-reduction substitution (for the per-phase launch counts); first_only:
+// up to the solution of column 0
+static int cr_sweep_launches(const xbar_s* h, bool initial, bool first_only) {
   const int L = (int)(h->prec == XBAR_FP64 ? h->cr64.lv.size() : h->cr32.lv.size());
   // right-hand side (or pad clear), last block, back levels, currents; forward levels in
   // correction mode (level 0: two launches)
-  return 3 + L + (initial ? 0 : L + 1);
+  return 2 + (first_only ? 0 : L + 1) + (initial ? 0 : L + 1);
 }
 
 // kernel launches of one block-Thomas substitution (sweep.cu, sweep_tc.cu): the inward part, unless an
@@ -319,7 +319,7 @@ static xbar_status solve_rows(xbar_s* h, int B, const double* dV, double* dI, do
   const int M = h->m.M, N = h->m.N, M2 = m2.M, Mp2 = m2.Mp, N2 = m2.N;
   cudaStream_t st = h->st;
   const bool cr = g->cr_active != 0;
-  const int Bp = cr ? kCrPanel : sweep_panel_width<double>(Mp2, B, g->nsm);
+  const int Bp = cr ? cr_panel(B) : sweep_panel_width<double>(Mp2, B, g->nsm);
   const int Bpad = ((B + Bp - 1) / Bp) * Bp;
   const size_t nst = (size_t)N2 * Mp2 * Bpad;
   auto need = [&](Buf& b, size_t bytes) -> bool {
@@ -332,7 +332,8 @@ static xbar_status solve_rows(xbar_s* h, int B, const double* dV, double* dI, do
   double* rhs = (double*)g->phi.p;  // consumed by the substitution; then the mirror's bit-line voltages
   double* w2 = (double*)g->w64.p;
   {
-    PhaseScope ps(h, XBAR_PHASE_SWEEP, 2 + (cr ? cr_sweep_launches(g, B, false) : sweep_launches(g->meet, N2, false)));
+    PhaseScope ps(h, XBAR_PHASE_SWEEP, 2 + (cr ? cr_sweep_launches(g, false, !dvWL && !dvBL)
+                                                       : sweep_launches(g->meet, N2, false)));
     XB_CUDA(launch_orient_rhs(dV, m2.h, M, M2, Mp2, B, Bpad, rhs, st));
     if (cr) {
       CrSweepArgs<double> ca;
@@ -346,6 +347,7 @@ static xbar_status solve_rows(xbar_s* h, int B, const double* dV, double* dI, do
       ca.e = m2.e_pl;
       ca.hs = m2.h;
       ca.I = (double*)g->sI.p;
+      ca.first_only = !dvWL && !dvBL;  // the currents are read from the first block
       XB_CUDA(cr_sweep<double>(g, g->cr64, ca));
     } else {
       SweepParams<double> sp;
@@ -371,7 +373,7 @@ static xbar_status solve_rows(xbar_s* h, int B, const double* dV, double* dI, do
       sp.status = g->status;
       XB_CUDA(launch_sweep<double>(sp, st));
     }
-    XB_CUDA(launch_orient_currents(w2, N, Bpad, B, m2.gs, dI, st));
+    XB_CUDA(launch_orient_currents(w2, N, Bpad, B, m2.gs, dI, h->status, st));
   }
   if (dvWL || dvBL) {
     PhaseScope ps(h, XBAR_PHASE_OUTPUT, 1 + (dvWL ? 1 : 0) + (dvBL ? 1 : 0));
@@ -399,7 +401,7 @@ static xbar_status solve_rows_mixed(xbar_s* h, int B, const double* dV, double* 
   cudaStream_t st = h->st;
   const bool cr = g->cr_active != 0;
   const bool tc = g->tc_ready && !cr;
-  const int Bp = cr ? kCrPanel : tc ? kSweepTcPanel : sweep_panel_width<float>(Mp2, B, g->nsm);
+  const int Bp = cr ? cr_panel(B) : tc ? kSweepTcPanel : sweep_panel_width<float>(Mp2, B, g->nsm);
   const int Bpad = ((B + Bp - 1) / Bp) * Bp;
   const size_t nst = (size_t)N2 * Mp2 * Bpad;
   XB_CUDA(ensure(g->A, g->z, nst * 4));
@@ -481,7 +483,7 @@ static xbar_status solve_rows_mixed(xbar_s* h, int B, const double* dV, double* 
     ca.tensor = use_cr_tensor(g) && Bpad >= 128;
     return cr_sweep<float>(g, g->cr32, ca);
   };
-  const int nsw = cr ? cr_sweep_launches(g, B, false) : sweep_launches(g->meet, N2, false);
+  const int nsw = cr ? cr_sweep_launches(g, false, false) : sweep_launches(g->meet, N2, false);
   {  // x0 = solve32(s o (V h')), the state w = s o x0, I from the state
     PhaseScope ps(h, XBAR_PHASE_SWEEP, 1 + nsw + 1 + (tc ? 0 : 1));
     XB_CUDA(launch_orient_rhs32(dV, m2.h, m2.s32, h->m.M, M2, Mp2, B, Bpad, (float*)g->rhat.p, st));
@@ -796,7 +798,7 @@ extern "C" xbar_status xbar_solve(xbar_t h, int B, const double* V, double* I, d
 
   const bool cr = h->cr_active != 0;
   const bool tc = mixed && h->tc_ready && !cr;
-  const int Bp = cr ? kCrPanel
+  const int Bp = cr ? cr_panel(B)
                     : tc ? kSweepTcPanel
                          : (mixed ? sweep_panel_width<float>(Mp, B, h->nsm) : sweep_panel_width<double>(Mp, B, h->nsm));
   const int nblk = (B + Bp - 1) / Bp;
@@ -851,7 +853,7 @@ extern "C" xbar_status xbar_solve(xbar_t h, int B, const double* V, double* I, d
     sp.max_rel = nullptr;
     sp.status = h->status;
     if (cr) {
-      PhaseScope ps(h, XBAR_PHASE_SWEEP, cr_sweep_launches(h, B, true));
+      PhaseScope ps(h, XBAR_PHASE_SWEEP, cr_sweep_launches(h, true, false));
       CrSweepArgs<double> ca;
       memset(&ca, 0, sizeof(ca));
       ca.B = B;
@@ -942,7 +944,7 @@ extern "C" xbar_status xbar_solve(xbar_t h, int B, const double* V, double* I, d
       rp.w1 = (const float*)h->w1.p;  // read as (w, 0) until the first update writes the pairs
     } else {
       {
-        PhaseScope ps(h, XBAR_PHASE_SWEEP, cr ? cr_sweep_launches(h, B, true) : sweep_launches(h->meet, N, true));
+        PhaseScope ps(h, XBAR_PHASE_SWEEP, cr ? cr_sweep_launches(h, true, false) : sweep_launches(h->meet, N, true));
         XB_CUDA(sweep32(sp));                   // x0 = solve32(b)
       }
       PhaseScope ps(h, XBAR_PHASE_UPDATE);
@@ -963,7 +965,7 @@ extern "C" xbar_status xbar_solve(xbar_t h, int B, const double* V, double* I, d
       sp.accumulate = 1;
       sp.max_rel = (float*)h->maxrel.p;
       {
-        PhaseScope ps(h, XBAR_PHASE_SWEEP, cr ? cr_sweep_launches(h, B, false) : sweep_launches(h->meet, N, false));  // dhat = solve32(rhat), I += dI
+        PhaseScope ps(h, XBAR_PHASE_SWEEP, cr ? cr_sweep_launches(h, false, false) : sweep_launches(h->meet, N, false));  // dhat = solve32(rhat), I += dI
         if (tc) XB_CUDA(launch_sweep_tc(sp, h->Xt.p, correction_terms(it), st));
         else XB_CUDA(sweep32(sp));
       }

@@ -183,6 +183,7 @@ __global__ void __launch_bounds__(kGthThreads) cr_gth_kernel(int Mp, const CrGth
 #pragma unroll
       for (int u = 0; u < 16; ++u) {  // fully unrolled: the loads are independent (Mp <= 256: q <= 16)
         const int m = m0 + u;
+        if (sizeof(T) == 8 && u >= q) break;  // uniform; FP64 issue costs more than the loads' overlap gains
         if (u < q && m < Mp) {
           if (hl) sa = fma(Qk[(size_t)m * Mp + i], gl[m], sa);
           if (hr) sb = fma(Pk[(size_t)m * Mp + i], gr[m], sb);
@@ -200,10 +201,16 @@ __global__ void __launch_bounds__(kGthThreads) cr_gth_kernel(int Mp, const CrGth
   const bool hn = x.pn >= 0;
   const T* wn = om + (size_t)(hn ? x.pn : 0) * Mp;
   const int half = warp & 1;
+  // rows past the block, and a half warp pair's empty half (Mp <= 128), are skipped whole: in FP64 every
+  // operation costs its issue slots whether a lane uses it or not
   for (int il = warp >> 1; il < kGthRows; il += kGthThreads / 64) {
     const int i = i0 + il;
     T off = (T)0, rc = (T)0;
-    if (i < Mp) {
+    if (i >= Mp || half * 128 >= Mp) {
+      if (lane == 0) opart[half][il] = rpart[half][il] = (T)0;
+      continue;
+    }
+    {
       const T* Drow = D + ((size_t)x.p * Mp + i) * Mp;
       const T* Urow = U + ((size_t)x.p * Mp + i) * Mp;
       T dv[4], uv[4];
@@ -211,8 +218,11 @@ __global__ void __launch_bounds__(kGthThreads) cr_gth_kernel(int Mp, const CrGth
       for (int u = 0; u < 4; ++u) {
         const int m = half * 128 + lane + 32 * u;
         const bool in = m < Mp;
-        dv[u] = (in && m != i) ? fabs(Drow[m]) * wp[m] : (T)0;
-        uv[u] = (in && hn) ? Urow[m] * wn[m] : (T)0;
+        dv[u] = uv[u] = (T)0;
+        if (half * 128 + 32 * u < Mp) {  // uniform in the warp
+          dv[u] = (in && m != i) ? fabs(Drow[m]) * wp[m] : (T)0;
+          uv[u] = (in && hn) ? Urow[m] * wn[m] : (T)0;
+        }
       }
       off = (dv[0] + dv[1]) + (dv[2] + dv[3]);
       rc = (uv[0] + uv[1]) + (uv[2] + uv[3]);
@@ -316,10 +326,12 @@ __global__ void cr_zero_pad_kernel(int M, int Mp, int Bpad, T* r) {
 // level 0, even p: r_p += e_{p-1} o y_{p-1} + e_p o y_{p+1}  (y_k = D_k^-1 r_k, held in x)
 template <typename T>
 __global__ void cr_l0_fwd_kernel(int Mp, int N, int Bpad, const T* __restrict__ e, const T* __restrict__ y, T* r) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x, i = blockIdx.y, p = 2 * blockIdx.z;
-  if (b >= Bpad) return;
+  // threads over the rows and vectors of a block together: one vector fills them as well as many
+  const int t = blockIdx.x * blockDim.x + threadIdx.x, p = 2 * blockIdx.y;
+  if (t >= Mp * Bpad) return;
+  const int i = t / Bpad;
   const size_t col = (size_t)Mp * Bpad;
-  const size_t o = ((size_t)p * Mp + i) * Bpad + b;
+  const size_t o = (size_t)p * col + t;
   T v = r[o];
   if (p > 0) v += e[(size_t)(p - 1) * Mp + i] * y[o - col];
   if (p + 1 < N) v += e[(size_t)p * Mp + i] * y[o + col];
@@ -355,9 +367,56 @@ __global__ void cr_currents_kernel(int M, int Mp, int N, int B, int Bpad, const 
   }
 }
 
+// The same for at most 16 vectors: a block per column, its threads over the column's rows and vectors
+// together (Bpad divides 128, so a thread stays with one vector).  One thread per vector walked the
+// M rows of a column one after another: 40 us for one vector of 256 x 256.
+template <typename T>
+__global__ void __launch_bounds__(128) cr_currents_few_kernel(int M, int Mp, int N, int B, int Bpad,
+                                                              const T* __restrict__ hs, const T* __restrict__ x,
+                                                              double* I, int accumulate, float* max_rel,
+                                                              unsigned* status) {
+  __shared__ T part[128];
+  const int tid = threadIdx.x, j = blockIdx.x;
+  const T* hj = hs + (size_t)j * Mp;
+  const T* xj = x + (size_t)j * Mp * Bpad;
+  T acc = (T)0;
+  for (int t = tid; t < M * Bpad; t += 128) acc = fma(hj[t / Bpad], xj[t], acc);
+  part[tid] = acc;
+  for (int o = 64; o >= Bpad; o >>= 1) {
+    __syncthreads();
+    if (tid < o) part[tid] += part[tid + o];
+  }
+  __syncthreads();
+  if (tid < B) {
+    const double dI = (double)part[tid];
+    if (!isfinite(dI)) set_status(status, XBAR_DEV_NONFINITE);
+    double* Ip = I + (size_t)tid * N + j;
+    if (accumulate) {
+      const double In = *Ip + dI;
+      *Ip = In;
+      const float rel = (float)(fabs(dI) / fmax(fabs(In), 1e-300));
+      if (max_rel && rel > 0.0f) atomic_max_nonneg(max_rel, rel);
+    } else {
+      *Ip = dI;
+    }
+  }
+}
+
 // ---------------------------------------------------------------------------------------------------
 // Host side: the level plan (built once per handle and precision), the factor and the substitution
 // ---------------------------------------------------------------------------------------------------
+// vectors per panel of a batch: 16, or for fewer than 16 the power of two that holds them (the job
+// lists depend on the panel width, so it takes few values)
+int cr_panel(int B) {
+  if (B >= kCrPanel) return kCrPanel;
+  int p = 1;
+  while (p < B) p *= 2;
+  return p;
+}
+// substitution plans kept per factorization: initial and correction form of the five narrow widths
+// and of one wide one
+constexpr size_t kCrSolvePlans = 12;
+
 namespace {
 
 template <typename T>
@@ -600,7 +659,7 @@ static cudaError_t cr_run_gemm(xbar_s* hd, const CrPlan<T>& pl, const GemmJob<T>
   if (o.aux && sizeof(T) == 4)
     return launch_gemm_jobs_tc(reinterpret_cast<const GemmJob<float>*>(jobs) + o.off, o.cnt, o.m, o.n, o.aux,
                                hd->nsm, hd->status, hd->st);
-  return launch_gemm_jobs<T>(jobs + o.off, o.cnt, o.m, o.n, hd->status, hd->st);
+  return launch_gemm_jobs<T>(jobs + o.off, o.cnt, o.m, o.n, hd->nsm, hd->st);
 }
 
 template <typename T>
@@ -771,6 +830,7 @@ static cudaError_t cr_solve_plan(xbar_s* hd, CrPlan<T>& pl, T* r, T* x, int Bpad
     const int jo = (int)jobs.size();
     seg(job(x + pl.root * MB, nullptr), Dinv + pl.root * MM, 0, r + pl.root * MB);
     gemm_op(jo);
+    sp.root_ops = sp.ops.size();
   }
   for (int l = L - 1; l >= 0; --l) {  // back substitution
     const CrLevel& lv = pl.lv[l];
@@ -787,7 +847,7 @@ static cudaError_t cr_solve_plan(xbar_s* hd, CrPlan<T>& pl, T* r, T* x, int Bpad
   }
   cudaError_t e = upload(hd->A, sp.jobs, jobs, hd->st);
   if (e != cudaSuccess) return e;
-  if (pl.solve_cache.size() >= 4) {  // oldest plan out, with its job list
+  if (pl.solve_cache.size() >= kCrSolvePlans) {  // oldest plan out, with its job list
     if (pl.solve_cache.front().jobs.p) hd->A.release(pl.solve_cache.front().jobs.p);
     pl.solve_cache.erase(pl.solve_cache.begin());
   }
@@ -813,14 +873,22 @@ cudaError_t cr_sweep(xbar_s* hd, CrPlan<T>& pl, const CrSweepArgs<T>& a) {
   }
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   const GemmJob<T>* jobs = (const GemmJob<T>*)sp->jobs.p;
-  for (const CrOp& o : sp->ops) {
+  const size_t nops = a.first_only ? sp->root_ops : sp->ops.size();
+  for (size_t k = 0; k < nops; ++k) {
+    const CrOp& o = sp->ops[k];
     if (o.kind == CR_OP_GEMM) {
-      e = cr_run_gemm<T>(hd, pl, jobs, o);
+      e = Bpad <= 16 ? launch_gemv_jobs<T>(jobs + o.off, o.cnt, o.m, Bpad, st) : cr_run_gemm<T>(hd, pl, jobs, o);
     } else if (o.kind == CR_OP_L0FWD) {
-      cr_l0_fwd_kernel<T><<<dim3((Bpad + 127) / 128, Mp, o.cnt), 128, 0, st>>>(Mp, N, Bpad, e_cpl, a.x, a.r);
+      cr_l0_fwd_kernel<T><<<dim3((Mp * Bpad + 127) / 128, o.cnt), 128, 0, st>>>(Mp, N, Bpad, e_cpl, a.x, a.r);
       e = cudaGetLastError();
     }
     if (e != cudaSuccess) return e;
+  }
+  if (a.first_only) return cudaSuccess;
+  if (Bpad <= 16) {
+    cr_currents_few_kernel<T><<<N, 128, 0, st>>>(M, Mp, N, a.B, Bpad, a.hs, a.x, a.I, a.accumulate, a.max_rel,
+                                                 hd->status);
+    return cudaGetLastError();
   }
   cr_currents_kernel<T><<<dim3((a.B + 127) / 128, N), 128, 0, st>>>(M, Mp, N, a.B, Bpad, a.hs, a.x, a.I,
                                                                      a.accumulate, a.max_rel, hd->status);

@@ -47,6 +47,7 @@ struct CrSolvePlan {
   bool initial = false, tensor = false;
   Buf jobs;
   std::vector<CrOp> ops;
+  size_t root_ops = 0;  // operations up to the last block's solution (column 0)
 };
 
 struct CrPlanBase {
@@ -82,6 +83,7 @@ struct CrSweepArgs {
   int accumulate;    // 0: I = dI, 1: I += dI
   float* max_rel;    // max |dI|/|I| (accumulate mode) or nullptr
   bool tensor;       // products on the tensor cores (FP32)
+  bool first_only;   // only column 0 of x is wanted: no back substitution, no currents
 };
 
 // build the level plan, its job lists and buffers if the shape or product engine changed

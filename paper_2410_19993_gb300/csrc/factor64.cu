@@ -78,20 +78,6 @@ __device__ __forceinline__ bool wait_count(const unsigned* f, unsigned target, u
   return true;
 }
 
-// Reciprocal of a pivot.  Normal-sized pivots take the hardware's approximate reciprocal (~2^-20) and
-// one cubic step, 1/pv = r (1 + e + e^2), e = 1 - pv r: three dependent operations against seven of
-// a division; the rest divide.
-__device__ __forceinline__ double pivot_rcp(double pv) {
-  const unsigned ex = ((unsigned)__double2hiint(pv) >> 20) & 0x7ffu;
-  if (ex - 64u < 1920u) {
-    double r;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(pv));
-    const double e = fma(-pv, r, 1.0);
-    return fma(r, fma(e, e, e), r);
-  }
-  return 1.0 / pv;
-}
-
 // named barriers of the inversion: warps 0 .. 4
 template <int ID>
 __device__ __forceinline__ void bar5_sync() { asm volatile("bar.sync %0, 160;" ::"n"(ID) : "memory"); }

@@ -13,49 +13,48 @@
 namespace xbar {
 
 // ---------------------------------------------------------------------------------------------
-// Job-list GEMM, 64 x TN output tiles (TN = 64, or 16 for narrow right-hand sides such as a few
-// input vectors), 256 threads: thread (ty, tx) computes rows ty + 16 r (r < 4) and columns
-// tx + 16 c (c < TN / 16); K is staged through shared memory in slabs of 16.
+// Job-list GEMM, TS x TS output tiles, 256 threads: thread (ty, tx) computes rows ty + 16 r and columns
+// tx + 16 c (r, c < TS / 16); K is staged through shared memory in slabs of 16.
 // ---------------------------------------------------------------------------------------------
-constexpr int kGT = 64, kGK = 16;
+constexpr int kGK = 16;
 
-template <typename T, int TN>
+template <typename T, int TS>
 __global__ void __launch_bounds__(256) gemm_jobs_kernel(const GemmJob<T>* __restrict__ jobs, int m, int n,
                                                         int tiles_n) {
-  constexpr int CW = TN / 16;
-  __shared__ T As[kGK][kGT + 1];
-  __shared__ T Bs[kGK][TN + 4];
+  constexpr int CW = TS / 16;
+  __shared__ T As[kGK][TS + 1];
+  __shared__ T Bs[kGK][TS + 4];
   const GemmJob<T>& jb = jobs[blockIdx.y];
-  const int i0 = (blockIdx.x / tiles_n) * kGT, j0 = (blockIdx.x % tiles_n) * TN;
+  const int i0 = (blockIdx.x / tiles_n) * TS, j0 = (blockIdx.x % tiles_n) * TS;
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  T acc[4][CW];
+  T acc[CW][CW];
 #pragma unroll
-  for (int r = 0; r < 4; ++r)
+  for (int r = 0; r < CW; ++r)
 #pragma unroll
     for (int c = 0; c < CW; ++c) acc[r][c] = (T)0;
 
   // the K slabs of all segments in order; the next slab's values are loaded into registers while
   // the current one is multiplied
-  T ra[4], rb[CW];
+  T ra[CW], rb[CW];
   auto load = [&](int s, int k0) {
     const T* A = jb.A[s];
     const T* B = jb.B[s];
     const int lda = jb.lda[s], ldb = jb.ldb[s], K = jb.k[s], ta = jb.ta[s], tb = jb.tb[s];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {  // A slab: rows i0..i0+63, k k0..k0+15
+    for (int u = 0; u < CW; ++u) {  // A slab: rows i0..i0+TS-1, k k0..k0+15
       const int t = tid + 256 * u;
       int i, kk;
-      if (ta) { kk = t >> 6; i = t & 63; }   // A[kk][i]: consecutive threads along i
+      if (ta) { kk = t / TS; i = t % TS; }   // A[kk][i]: consecutive threads along i
       else { i = t >> 4; kk = t & 15; }      // A[i][kk]: consecutive threads along kk
       const int gi = i0 + i, gk = k0 + kk;
       ra[u] = (gi < m && gk < K) ? (ta ? A[(size_t)gk * lda + gi] : A[(size_t)gi * lda + gk]) : (T)0;
     }
 #pragma unroll
-    for (int u = 0; u < CW; ++u) {  // B slab: k k0..k0+15, columns j0..j0+TN-1
+    for (int u = 0; u < CW; ++u) {  // B slab: k k0..k0+15, columns j0..j0+TS-1
       const int t = tid + 256 * u;
       int j, kk;
       if (tb) { j = t >> 4; kk = t & 15; }       // B[j][kk]
-      else { kk = t / TN; j = t % TN; }          // B[kk][j]
+      else { kk = t / TS; j = t % TS; }          // B[kk][j]
       const int gj = j0 + j, gk = k0 + kk;
       rb[u] = (gj < n && gk < K) ? (tb ? B[(size_t)gj * ldb + gk] : B[(size_t)gk * ldb + gj]) : (T)0;
     }
@@ -63,16 +62,16 @@ __global__ void __launch_bounds__(256) gemm_jobs_kernel(const GemmJob<T>* __rest
   auto store = [&](int s) {
     const int ta = jb.ta[s], tb = jb.tb[s];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
+    for (int u = 0; u < CW; ++u) {
       const int t = tid + 256 * u;
-      if (ta) As[t >> 6][t & 63] = ra[u];
+      if (ta) As[t / TS][t % TS] = ra[u];
       else As[t & 15][t >> 4] = ra[u];
     }
 #pragma unroll
     for (int u = 0; u < CW; ++u) {
       const int t = tid + 256 * u;
       if (tb) Bs[t & 15][t >> 4] = rb[u];
-      else Bs[t / TN][t % TN] = rb[u];
+      else Bs[t / TS][t % TS] = rb[u];
     }
   };
   const int nseg = jb.nseg;
@@ -90,13 +89,13 @@ __global__ void __launch_bounds__(256) gemm_jobs_kernel(const GemmJob<T>* __rest
     if (s < nseg) load(s, k0);
 #pragma unroll
     for (int kk = 0; kk < kGK; ++kk) {
-      T a[4], b[CW];
+      T a[CW], b[CW];
 #pragma unroll
-      for (int r = 0; r < 4; ++r) a[r] = As[kk][ty + 16 * r];
+      for (int r = 0; r < CW; ++r) a[r] = As[kk][ty + 16 * r];
 #pragma unroll
       for (int c = 0; c < CW; ++c) b[c] = Bs[kk][tx + 16 * c];
 #pragma unroll
-      for (int r = 0; r < 4; ++r)
+      for (int r = 0; r < CW; ++r)
 #pragma unroll
         for (int c = 0; c < CW; ++c) acc[r][c] = fma(a[r], b[c], acc[r][c]);
     }
@@ -104,7 +103,7 @@ __global__ void __launch_bounds__(256) gemm_jobs_kernel(const GemmJob<T>* __rest
   }
   const T alpha = jb.alpha;
 #pragma unroll
-  for (int r = 0; r < 4; ++r) {
+  for (int r = 0; r < CW; ++r) {
     const int gi = i0 + ty + 16 * r;
     if (gi >= m) continue;
 #pragma unroll
@@ -118,18 +117,162 @@ __global__ void __launch_bounds__(256) gemm_jobs_kernel(const GemmJob<T>* __rest
   }
 }
 
+// Tile size: the largest of 64, 32 and 16 that neither pads the matrix by more than the next smaller one
+// would nor leaves fewer than two blocks per SM.  A block's time is its multiply-adds per thread times
+// the K depth (an FP64 multiply-add of the block's eight warps takes 152 cycles), so a level of few small
+// jobs wants many blocks: the 32 x 32 FP64 blocks of a 256 x 32 map took 54 us a launch in one 64 x 64
+// tile each and take 9 us in 16 x 16 tiles; a level with hundreds of tiles loses nothing.
 template <typename T>
-cudaError_t launch_gemm_jobs(const GemmJob<T>* jobs_dev, int njobs, int m, int n, unsigned* status,
-                             cudaStream_t st) {
-  (void)status;
+cudaError_t launch_gemm_jobs(const GemmJob<T>* jobs_dev, int njobs, int m, int n, int nsm, cudaStream_t st) {
   if (njobs <= 0 || m <= 0 || n <= 0) return cudaSuccess;
   if (njobs > 65535) return cudaErrorInvalidValue;
-  const int tm = (m + kGT - 1) / kGT;
-  if (n <= 16) {
-    gemm_jobs_kernel<T, 16><<<dim3(tm, njobs), 256, 0, st>>>(jobs_dev, m, n, 1);
-  } else {
-    const int tn = (n + kGT - 1) / kGT;
-    gemm_jobs_kernel<T, 64><<<dim3(tm * tn, njobs), 256, 0, st>>>(jobs_dev, m, n, tn);
+  auto tiles = [](int x, int ts) { return (x + ts - 1) / ts; };
+  int ts = 64;
+  while (ts > 16) {
+    const int h = ts / 2;
+    const bool pads = tiles(m, ts) * ts > tiles(m, h) * h || tiles(n, ts) * ts > tiles(n, h) * h;
+    if (!pads && (long long)njobs * tiles(m, ts) * tiles(n, ts) >= 2 * nsm) break;
+    ts = h;
+  }
+  const int tm = tiles(m, ts), tn = tiles(n, ts);
+  const dim3 grid(tm * tn, njobs);
+  if (ts == 16) gemm_jobs_kernel<T, 16><<<grid, 256, 0, st>>>(jobs_dev, m, n, tn);
+  else if (ts == 32) gemm_jobs_kernel<T, 32><<<grid, 256, 0, st>>>(jobs_dev, m, n, tn);
+  else gemm_jobs_kernel<T, 64><<<grid, 256, 0, st>>>(jobs_dev, m, n, tn);
+  return cudaGetLastError();
+}
+
+// ---------------------------------------------------------------------------------------------
+// Job-list matrix-vector products: NV (1, 2, 4, 8 or 16) columns, tb = 0, ldb = ldc = ldcin = NV.  Bound
+// by reading each block of the factor once, so a block of 256 threads takes 16 rows of a product and
+// keeps many loads in flight: a warp reads two rows along K (ta = 0; the lanes' partial sums meet at the
+// end) or, transposed, two values of K for 16 columns.  The vectors go through shared memory.
+// One vector of a 256 x 256 map: 77 us a launch as a product padded to 16 columns in 64-row tiles.
+// ---------------------------------------------------------------------------------------------
+constexpr int kVR = 16;    // rows of the result per block
+constexpr int kVK = 128;   // K values per staged chunk
+
+// sums of NS values over the 32 lanes; afterwards lane l holds, in v[0], the sum of value l / (32 / NS')
+// with NS' = NS rounded up to a power of two (NS <= 32)
+template <typename T, int NS>
+__device__ __forceinline__ void lane_sums(T (&v)[NS], int lane) {
+  int n = NS;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    if (n > 1) {
+      const bool up = (lane & o) != 0;
+#pragma unroll
+      for (int k = 0; k < NS / 2; ++k)
+        if (k < n / 2) {
+          const T send = up ? v[k] : v[k + n / 2], keep = up ? v[k + n / 2] : v[k];
+          v[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+      n >>= 1;
+    } else {
+      v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+    }
+  }
+}
+
+template <typename T, int NV>
+__global__ void __launch_bounds__(256) gemv_jobs_kernel(const GemmJob<T>* __restrict__ jobs, int m) {
+  __shared__ T bs[kVK][NV];
+  __shared__ T red0[kVR][NV];
+  __shared__ T red1[8][kVR][NV];
+  const GemmJob<T>& jb = jobs[blockIdx.y];
+  const int i0 = blockIdx.x * kVR;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int ia = i0 + 2 * warp;                           // ta = 0: this warp's two rows
+  const int it = i0 + (lane & 15), kt = 2 * warp + (lane >> 4);  // ta = 1: column, first K value
+  T acc0[2 * NV], acc1[NV];
+#pragma unroll
+  for (int v = 0; v < 2 * NV; ++v) acc0[v] = (T)0;
+#pragma unroll
+  for (int v = 0; v < NV; ++v) acc1[v] = (T)0;
+  const int nseg = jb.nseg;
+  for (int s = 0; s < nseg; ++s) {
+    const T* A = jb.A[s];
+    const T* B = jb.B[s];
+    const int lda = jb.lda[s], K = jb.k[s], ta = jb.ta[s];
+    for (int k0 = 0; k0 < K; k0 += kVK) {
+      const int kc = min(kVK, K - k0);
+      __syncthreads();
+      for (int t = tid; t < kVK * NV; t += 256)
+        (&bs[0][0])[t] = t < kc * NV ? B[(size_t)k0 * NV + t] : (T)0;
+      // this chunk's part of A, loaded before the barrier
+      T a[8];
+      if (!ta) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int k = lane + 32 * u;
+          a[u] = (ia < m && k < kc) ? A[(size_t)ia * lda + k0 + k] : (T)0;
+          a[4 + u] = (ia + 1 < m && k < kc) ? A[(size_t)(ia + 1) * lda + k0 + k] : (T)0;
+        }
+      } else {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const int k = kt + 16 * u;
+          a[u] = (it < m && k < kc) ? A[(size_t)(k0 + k) * lda + it] : (T)0;
+        }
+      }
+      __syncthreads();
+      if (!ta) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          if (32 * u >= kc) break;  // uniform
+#pragma unroll
+          for (int v = 0; v < NV; ++v) {
+            const T b = bs[lane + 32 * u][v];
+            acc0[v] = fma(a[u], b, acc0[v]);
+            acc0[NV + v] = fma(a[4 + u], b, acc0[NV + v]);
+          }
+        }
+      } else {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          if (16 * u >= kc) break;  // uniform
+#pragma unroll
+          for (int v = 0; v < NV; ++v) acc1[v] = fma(a[u], bs[kt + 16 * u][v], acc1[v]);
+        }
+      }
+    }
+  }
+  lane_sums<T, 2 * NV>(acc0, lane);
+  {
+    constexpr int rep = 32 / (2 * NV);
+    const int k = lane / rep;
+    if (lane % rep == 0) red0[2 * warp + k / NV][k % NV] = acc0[0];
+  }
+#pragma unroll
+  for (int v = 0; v < NV; ++v) acc1[v] += __shfl_xor_sync(0xffffffffu, acc1[v], 16);
+  if (lane < 16)
+#pragma unroll
+    for (int v = 0; v < NV; ++v) red1[warp][lane][v] = acc1[v];
+  __syncthreads();
+  for (int t = tid; t < kVR * NV; t += 256) {
+    const int r = t / NV, v = t % NV, i = i0 + r;
+    if (i >= m) continue;
+    T x = red0[r][v];
+#pragma unroll
+    for (int w = 0; w < 8; ++w) x += red1[w][r][v];
+    x *= jb.alpha;
+    if (jb.Cin) x += jb.Cin[(size_t)i * NV + v];
+    jb.C[(size_t)i * NV + v] = x;
+  }
+}
+
+template <typename T>
+cudaError_t launch_gemv_jobs(const GemmJob<T>* jobs_dev, int njobs, int m, int nv, cudaStream_t st) {
+  if (njobs <= 0 || m <= 0) return cudaSuccess;
+  if (njobs > 65535) return cudaErrorInvalidValue;
+  const dim3 grid((m + kVR - 1) / kVR, njobs);
+  switch (nv) {
+    case 1: gemv_jobs_kernel<T, 1><<<grid, 256, 0, st>>>(jobs_dev, m); break;
+    case 2: gemv_jobs_kernel<T, 2><<<grid, 256, 0, st>>>(jobs_dev, m); break;
+    case 4: gemv_jobs_kernel<T, 4><<<grid, 256, 0, st>>>(jobs_dev, m); break;
+    case 8: gemv_jobs_kernel<T, 8><<<grid, 256, 0, st>>>(jobs_dev, m); break;
+    case 16: gemv_jobs_kernel<T, 16><<<grid, 256, 0, st>>>(jobs_dev, m); break;
+    default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
 }
@@ -291,26 +434,28 @@ __global__ void __launch_bounds__(NT / RPT * 32) gj_kernel(const GjJob<T>* __res
   }
 }
 
-// Single-pivot variant for FP64 (its register budget does not allow the panel form at 128 rows; the
-// FP64 inversion is bound by the FP64 FMA rate either way).  Thread (ty, tx) owns rows
-// ty + (NT/8) r (r < 8) and columns tx + 32 c (c < NT/32); each step applies one sweep operator
-// (a_qq <- 1/a_qq, a_qm <- a_qm/a_qq, a_iq <- -a_iq/a_qq, a_im <- a_im - a_iq a_qm/a_qq) with the
-// pivot row and column published through double-buffered shared memory (one barrier per step).
-template <typename T, int NT>
-__global__ void __launch_bounds__(NT * 4) gj1_kernel(const GjJob<T>* __restrict__ jobs, int n) {
+// Single-pivot variant for FP64 (its register budget does not allow the panel form at 128 rows).  Thread
+// (ty, tx) owns rows ty + (NT/8) r (r < 8) and columns tx + 32 c (c < NT/32); each step applies one
+// sweep operator (a_qq <- 1/a_qq, a_qm <- a_qm/a_qq, a_iq <- -a_iq/a_qq, a_im <- a_im - a_iq a_qm/a_qq) with
+// the pivot row and column published through double-buffered shared memory (one barrier per step).
+// Bound by FP64 issue (64 cycles an instruction and sub-partition), so a step issues as few as it can:
+// the short reciprocal, one product per column (the pivot column takes the reciprocal itself and a
+// zero to add to, so that it needs none of its own) and one multiply-add per element.
+template <int NT>
+__global__ void __launch_bounds__(NT * 4) gj1_kernel(const GjJob<double>* __restrict__ jobs, int n) {
   constexpr int RG = NT / 8;   // row groups = warps
   constexpr int CB = NT / 32;  // columns per lane
-  __shared__ T prow[2][NT], pcol[2][NT];
-  const GjJob<T> jb = jobs[blockIdx.x];
+  __shared__ double prow[2][NT], pcol[2][NT];
+  const GjJob<double> jb = jobs[blockIdx.x];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  T a[8][CB];
+  double a[8][CB];
 #pragma unroll
   for (int r = 0; r < 8; ++r) {
     const int i = ty + RG * r;
 #pragma unroll
     for (int c = 0; c < CB; ++c) {
       const int mm = tx + 32 * c;
-      a[r][c] = (i < n && mm < n) ? jb.src[(size_t)i * jb.lds + mm] : (i == mm ? (T)1 : (T)0);
+      a[r][c] = (i < n && mm < n) ? jb.src[(size_t)i * jb.lds + mm] : (i == mm ? 1.0 : 0.0);
     }
   }
 #pragma unroll
@@ -326,7 +471,7 @@ __global__ void __launch_bounds__(NT * 4) gj1_kernel(const GjJob<T>* __restrict_
       if (tx == cq) {
 #pragma unroll
         for (int r = 0; r < 8; ++r) {
-          T v = a[r][0];
+          double v = a[r][0];
 #pragma unroll
           for (int c = 1; c < CB; ++c)
             if (c == bq) v = a[r][c];
@@ -334,26 +479,19 @@ __global__ void __launch_bounds__(NT * 4) gj1_kernel(const GjJob<T>* __restrict_
         }
       }
       __syncthreads();
-      const T inv = (T)1 / prow[buf][q];
-      T rs[CB], cs[8];
+      const double inv = pivot_rcp(prow[buf][q]);
+      double f[CB], cs[8];
 #pragma unroll
-      for (int c = 0; c < CB; ++c) rs[c] = prow[buf][tx + 32 * c] * inv;
+      for (int c = 0; c < CB; ++c) f[c] = tx == cq && c == bq ? inv : prow[buf][tx + 32 * c] * inv;
 #pragma unroll
       for (int r = 0; r < 8; ++r) cs[r] = pcol[buf][ty + RG * r];
 #pragma unroll
       for (int r = 0; r < 8; ++r)
 #pragma unroll
-        for (int c = 0; c < CB; ++c) a[r][c] = fma(-cs[r], rs[c], a[r][c]);
+        for (int c = 0; c < CB; ++c) a[r][c] = fma(-cs[r], f[c], tx == cq && c == bq ? 0.0 : a[r][c]);
       if (ty == rq) {  // pivot row
 #pragma unroll
-        for (int c = 0; c < CB; ++c) a[aq][c] = rs[c];
-      }
-      if (tx == cq) {  // pivot column (and the pivot itself)
-#pragma unroll
-        for (int r = 0; r < 8; ++r)
-#pragma unroll
-          for (int c = 0; c < CB; ++c)
-            if (c == bq) a[r][c] = (ty == rq && r == aq) ? inv : -cs[r] * inv;
+        for (int c = 0; c < CB; ++c) a[aq][c] = f[c];
       }
     }
   }
@@ -374,9 +512,9 @@ cudaError_t launch_gj_inverse(const GjJob<T>* jobs_dev, int njobs, int n, unsign
   (void)status;
   if (njobs <= 0 || n <= 0) return cudaSuccess;
   if constexpr (sizeof(T) == 8) {  // FP64: single-pivot steps
-    if (n <= 32) gj1_kernel<T, 32><<<njobs, 128, 0, st>>>(jobs_dev, n);
-    else if (n <= 64) gj1_kernel<T, 64><<<njobs, 256, 0, st>>>(jobs_dev, n);
-    else if (n <= 128) gj1_kernel<T, 128><<<njobs, 512, 0, st>>>(jobs_dev, n);
+    if (n <= 32) gj1_kernel<32><<<njobs, 128, 0, st>>>(jobs_dev, n);
+    else if (n <= 64) gj1_kernel<64><<<njobs, 256, 0, st>>>(jobs_dev, n);
+    else if (n <= 128) gj1_kernel<128><<<njobs, 512, 0, st>>>(jobs_dev, n);
     else return cudaErrorInvalidValue;
   } else {
     if (n <= 32) gj_kernel<T, 32, 8><<<njobs, 128, 0, st>>>(jobs_dev, n);
@@ -387,8 +525,10 @@ cudaError_t launch_gj_inverse(const GjJob<T>* jobs_dev, int njobs, int n, unsign
   return cudaGetLastError();
 }
 
-template cudaError_t launch_gemm_jobs<float>(const GemmJob<float>*, int, int, int, unsigned*, cudaStream_t);
-template cudaError_t launch_gemm_jobs<double>(const GemmJob<double>*, int, int, int, unsigned*, cudaStream_t);
+template cudaError_t launch_gemm_jobs<float>(const GemmJob<float>*, int, int, int, int, cudaStream_t);
+template cudaError_t launch_gemm_jobs<double>(const GemmJob<double>*, int, int, int, int, cudaStream_t);
+template cudaError_t launch_gemv_jobs<float>(const GemmJob<float>*, int, int, int, cudaStream_t);
+template cudaError_t launch_gemv_jobs<double>(const GemmJob<double>*, int, int, int, cudaStream_t);
 template cudaError_t launch_gj_inverse<float>(const GjJob<float>*, int, int, unsigned*, cudaStream_t);
 template cudaError_t launch_gj_inverse<double>(const GjJob<double>*, int, int, unsigned*, cudaStream_t);
 

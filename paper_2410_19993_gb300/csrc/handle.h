@@ -186,6 +186,7 @@ bool use_cluster_factor(const xbar_s* h);
 bool use_cr(const xbar_s* h);
 // input vectors per panel of the cyclic-reduction substitution (Bpad = B rounded up to it)
 constexpr int kCrPanel = 16;
+int cr_panel(int B);  // kCrPanel, or 1, 2, 4 or 8 for a smaller batch
 
 // factor a handle (FP64 or equilibrated FP32); upload_params = false reuses the parameter block
 // already on the device (graph capture)

@@ -143,7 +143,7 @@ cudaError_t launch_orient_rhs(const double* V, const double* h2, int M, int M2, 
                               double* rhs, cudaStream_t st);
 // I[b][j] = gs2 w2[0][N-1-j][b]
 cudaError_t launch_orient_currents(const double* w2, int N, int Bpad, int B, double gs2, double* I,
-                                   cudaStream_t st);
+                                   unsigned* status, cudaStream_t st);
 // the mirror's bit-line voltages u ([M][Mp2][Bpad]) from its word-line voltages w2 and the sources
 cudaError_t launch_orient_blvolt(const MapDev& m2, const double* w2, const double* V, int M, int B, int Bpad,
                                  double* u, cudaStream_t st);
@@ -228,9 +228,12 @@ struct GemmJob {
   int lda[3], ldb[3], k[3];
   int ta[3], tb[3];
 };
-// CUDA cores (FP32 or FP64), 64 x 64 output tiles
+// CUDA cores (FP32 or FP64), output tiles of 64, 32 or 16 rows and columns
 template <typename T>
-cudaError_t launch_gemm_jobs(const GemmJob<T>* jobs_dev, int njobs, int m, int n, unsigned* status, cudaStream_t st);
+cudaError_t launch_gemm_jobs(const GemmJob<T>* jobs_dev, int njobs, int m, int n, int nsm, cudaStream_t st);
+// nv = 1, 2, 4, 8 or 16 columns, jobs with tb = 0 and ldb = ldc = ldcin = nv
+template <typename T>
+cudaError_t launch_gemv_jobs(const GemmJob<T>* jobs_dev, int njobs, int m, int nv, cudaStream_t st);
 // tensor cores (tcgen05, FP32 operands split into three BF16 terms, six products per K step, FP32
 // accumulation in tensor memory), 128 x TN output tiles with TN = 128 or 256, persistent over the
 // SMs.  k_s must be multiples of 16.

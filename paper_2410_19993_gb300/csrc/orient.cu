@@ -38,24 +38,27 @@ __global__ void mirror_gc_kernel(const double* __restrict__ Gc, int M, int Mp, i
   Gc2[(size_t)j2 * Mp2 + i2] = i2 < N ? Gc[(size_t)(N - 1 - i2) * Mp + (M - 1 - j2)] : 0.0;
 }
 
-// rhs[j'][i'][b] = V[b][M-1-j'] h'[j'][i'] for real rows and vectors, zero elsewhere
+// rhs[j'][i'][b] = V[b][M-1-j'] h'[j'][i'] for real rows and vectors, zero elsewhere.  Threads run over
+// the rows and vectors of a block together, so that one vector fills them as well as many.
 __global__ void orient_rhs_kernel(const double* __restrict__ V, const double* __restrict__ h2, int M, int M2,
                                   int Mp2, int B, int Bpad, double* __restrict__ rhs) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  const int i2 = blockIdx.y, j2 = blockIdx.z;
-  if (b >= Bpad) return;
+  const int t = blockIdx.x * blockDim.x + threadIdx.x, j2 = blockIdx.y;
+  if (t >= Mp2 * Bpad) return;
+  const int i2 = t / Bpad, b = t - i2 * Bpad;
   double v = 0.0;
   if (b < B && i2 < M2) v = V[(size_t)b * M + (M - 1 - j2)] * h2[(size_t)j2 * Mp2 + i2];
-  rhs[((size_t)j2 * Mp2 + i2) * Bpad + b] = v;
+  rhs[(size_t)j2 * Mp2 * Bpad + t] = v;
 }
 
 // I[b][j] = g_s' w'[0][N-1-j][b]
 __global__ void orient_currents_kernel(const double* __restrict__ w2, int N, int Bpad, int B, double gs2,
-                                       double* __restrict__ I) {
+                                       double* __restrict__ I, unsigned* status) {
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   const int j = blockIdx.y;
   if (b >= B) return;
-  I[(size_t)b * N + j] = gs2 * w2[(size_t)(N - 1 - j) * Bpad + b];
+  const double v = gs2 * w2[(size_t)(N - 1 - j) * Bpad + b];
+  if (!isfinite(v)) set_status(status, XBAR_DEV_NONFINITE);
+  I[(size_t)b * N + j] = v;
 }
 
 // The mirror's bit-line voltages with the source at the bottom of each chain:
@@ -183,14 +186,15 @@ cudaError_t launch_mirror_gc(const double* Gc, int M, int Mp, int N, double* Gc2
 
 cudaError_t launch_orient_rhs(const double* V, const double* h2, int M, int M2, int Mp2, int B, int Bpad,
                               double* rhs, cudaStream_t st) {
-  orient_rhs_kernel<<<dim3((Bpad + 127) / 128, Mp2, M), 128, 0, st>>>(V, h2, M, M2, Mp2, B, Bpad, rhs);
+  if ((long long)Mp2 * Bpad > 0x7fffff00ll) return cudaErrorInvalidValue;
+  orient_rhs_kernel<<<dim3((Mp2 * Bpad + 127) / 128, M), 128, 0, st>>>(V, h2, M, M2, Mp2, B, Bpad, rhs);
   return cudaGetLastError();
 }
 
 cudaError_t launch_orient_currents(const double* w2, int N, int Bpad, int B, double gs2, double* I,
-                                   cudaStream_t st) {
+                                   unsigned* status, cudaStream_t st) {
   if (B == 0) return cudaSuccess;
-  orient_currents_kernel<<<dim3((B + 127) / 128, N), 128, 0, st>>>(w2, N, Bpad, B, gs2, I);
+  orient_currents_kernel<<<dim3((B + 127) / 128, N), 128, 0, st>>>(w2, N, Bpad, B, gs2, I, status);
   return cudaGetLastError();
 }
 
