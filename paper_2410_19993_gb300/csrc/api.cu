@@ -218,7 +218,38 @@ static int cr_sweep_launches(const xbar_s* h, bool initial, bool first_only) {
 
 // kernel launches of one block-Thomas substitution (sweep.cu, sweep_tc.cu): the inward part, unless an
 // input vector (V) meets no left chain or the system has one column, and the outward part
-static int sweep_launches(int meet, int N, bool V) { return 1 + (meet > 0 || (!V && meet < N - 1) ? 1 : 0); }
+static int sweep_launches(int meet, int N, bool V, bool few = false) {
+  return 1 + (meet > 0 || (!V && meet < N - 1) ? 1 : 0) + (few ? 1 : 0);  // few: and the currents
+}
+
+// The substitution kernel of a block-Thomas factor for a batch: clusters for a few vectors
+// (sweep_few.cu), otherwise the tensor cores (mixed precision, sweep_tc.cu) or the CUDA cores.  An
+// explicit choice of the FP32 kernel (XBAR_OPT_SWEEP_KERNEL, XBAR_SWEEP) is kept.
+struct SweepKind {
+  FewPlan few;
+  bool tc = false;
+  int Bp = 0;  // vectors per panel
+};
+static SweepKind sweep_kind(const xbar_s* h, int B, bool mixed) {
+  SweepKind k;
+  const char* e = getenv("XBAR_SWEEP");
+  const bool chosen = mixed && (h->opt.sweep >= 0 || (e && (strcmp(e, "simt") == 0 || strcmp(e, "tc") == 0)));
+  if (!chosen) k.few = sweep_few_plan(h->m.Mp, B, h->nsm);
+  k.tc = mixed && h->tc_ready && !k.few.nv;
+  k.Bp = k.few.nv ? k.few.nv
+         : k.tc   ? kSweepTcPanel
+         : mixed  ? sweep_panel_width<float>(h->m.Mp, B, h->nsm)
+                  : sweep_panel_width<double>(h->m.Mp, B, h->nsm);
+  return k;
+}
+template <typename T>
+static cudaError_t run_sweep(const SweepParams<T>& sp, const SweepKind& k, const void* Xt, int terms, cudaStream_t st) {
+  if (k.few.nv) return launch_sweep_few<T>(sp, k.few, st);
+  if constexpr (sizeof(T) == 4) {
+    if (k.tc) return launch_sweep_tc(sp, Xt, terms, st);
+  }
+  return launch_sweep<T>(sp, st);
+}
 
 // BF16 terms of the tensor-core sweep for refinement correction `it` (0-based).  A correction
 // only needs accuracy relative to its own size, so the first two are solved with two terms
@@ -319,7 +350,8 @@ static xbar_status solve_rows(xbar_s* h, int B, const double* dV, double* dI, do
   const int M = h->m.M, N = h->m.N, M2 = m2.M, Mp2 = m2.Mp, N2 = m2.N;
   cudaStream_t st = h->st;
   const bool cr = g->cr_active != 0;
-  const int Bp = cr ? cr_panel(B) : sweep_panel_width<double>(Mp2, B, g->nsm);
+  const SweepKind kind = cr ? SweepKind() : sweep_kind(g, B, false);
+  const int Bp = cr ? cr_panel(B) : kind.Bp;
   const int Bpad = ((B + Bp - 1) / Bp) * Bp;
   const size_t nst = (size_t)N2 * Mp2 * Bpad;
   auto need = [&](Buf& b, size_t bytes) -> bool {
@@ -371,7 +403,7 @@ static xbar_status solve_rows(xbar_s* h, int B, const double* dV, double* dI, do
       sp.accumulate = 0;
       sp.max_rel = nullptr;
       sp.status = g->status;
-      XB_CUDA(launch_sweep<double>(sp, st));
+      XB_CUDA(run_sweep<double>(sp, kind, nullptr, 0, st));
     }
     XB_CUDA(launch_orient_currents(w2, N, Bpad, B, m2.gs, dI, h->status, st));
   }
@@ -797,10 +829,9 @@ extern "C" xbar_status xbar_solve(xbar_t h, int B, const double* V, double* I, d
   }
 
   const bool cr = h->cr_active != 0;
-  const bool tc = mixed && h->tc_ready && !cr;
-  const int Bp = cr ? cr_panel(B)
-                    : tc ? kSweepTcPanel
-                         : (mixed ? sweep_panel_width<float>(Mp, B, h->nsm) : sweep_panel_width<double>(Mp, B, h->nsm));
+  const SweepKind kind = cr ? SweepKind() : sweep_kind(h, B, mixed);
+  const bool few = kind.few.nv > 0;
+  const int Bp = cr ? cr_panel(B) : kind.Bp;
   const int nblk = (B + Bp - 1) / Bp;
   const int Bpad = nblk * Bp;
   const size_t nst = (size_t)N * Mp * Bpad;
@@ -867,8 +898,8 @@ extern "C" xbar_status xbar_solve(xbar_t h, int B, const double* V, double* I, d
       ca.I = dI;
       XB_CUDA(cr_sweep<double>(h, h->cr64, ca));
     } else {
-      PhaseScope ps(h, XBAR_PHASE_SWEEP, sweep_launches(h->meet, N, true));
-      XB_CUDA(launch_sweep<double>(sp, st));
+      PhaseScope ps(h, XBAR_PHASE_SWEEP, sweep_launches(h->meet, N, true, few));
+      XB_CUDA(run_sweep<double>(sp, kind, nullptr, 0, st));
     }
     rp.w = (double*)h->w64.p;
     rp.phi = (double*)h->phi.p;
@@ -912,10 +943,10 @@ extern "C" xbar_status xbar_solve(xbar_t h, int B, const double* V, double* I, d
     sp.accumulate = 0;
     sp.max_rel = nullptr;
     sp.status = h->status;
-    // FP32 substitution of the factor's algorithm (CUDA-core block-Thomas sweep, or cyclic
-    // reduction with the right-hand side in z (initial) or rhat (corrections), both overwritten)
-    auto sweep32 = [&](const SweepParams<float>& q) -> cudaError_t {
-      if (!cr) return launch_sweep<float>(q, st);
+    // FP32 substitution of the factor's algorithm (block-Thomas sweep, or cyclic reduction with the
+    // right-hand side in z (initial) or rhat (corrections), both overwritten)
+    auto sweep32 = [&](const SweepParams<float>& q, int terms) -> cudaError_t {
+      if (!cr) return run_sweep<float>(q, kind, h->Xt.p, terms, st);
       CrSweepArgs<float> ca;
       memset(&ca, 0, sizeof(ca));
       ca.B = B;
@@ -932,20 +963,20 @@ extern "C" xbar_status xbar_solve(xbar_t h, int B, const double* V, double* I, d
       ca.tensor = use_cr_tensor(h) && Bpad >= 128;  // wide batches: products on the tensor cores
       return cr_sweep<float>(h, h->cr32, ca);
     };
-    if (tc) {  // x0 = solve32(b); the sweep writes the state w = s o x0 (FP32) itself
-      PhaseScope ps(h, XBAR_PHASE_SWEEP, sweep_launches(h->meet, N, true));
+    if (kind.tc || few) {  // x0 = solve32(b); the sweep writes the state w = s o x0 (FP32) itself
+      PhaseScope ps(h, XBAR_PHASE_SWEEP, sweep_launches(h->meet, N, true, few));
       XB_CUDA(ensure(h->A, h->w1, nst * 4));
       sp.w = nullptr;
       sp.w1out = (float*)h->w1.p;
       sp.s32 = m.s32;
-      XB_CUDA(launch_sweep_tc(sp, h->Xt.p, kInitialTerms, st));
+      XB_CUDA(sweep32(sp, kInitialTerms));
       sp.w = (float*)h->dhat.p;
       sp.w1out = nullptr;
       rp.w1 = (const float*)h->w1.p;  // read as (w, 0) until the first update writes the pairs
     } else {
       {
         PhaseScope ps(h, XBAR_PHASE_SWEEP, cr ? cr_sweep_launches(h, true, false) : sweep_launches(h->meet, N, true));
-        XB_CUDA(sweep32(sp));                   // x0 = solve32(b)
+        XB_CUDA(sweep32(sp, kInitialTerms));    // x0 = solve32(b)
       }
       PhaseScope ps(h, XBAR_PHASE_UPDATE);
       XB_CUDA(launch_update(rp, 1, st));        // w = s o dhat, I = h . w
@@ -965,9 +996,8 @@ extern "C" xbar_status xbar_solve(xbar_t h, int B, const double* V, double* I, d
       sp.accumulate = 1;
       sp.max_rel = (float*)h->maxrel.p;
       {
-        PhaseScope ps(h, XBAR_PHASE_SWEEP, cr ? cr_sweep_launches(h, false, false) : sweep_launches(h->meet, N, false));  // dhat = solve32(rhat), I += dI
-        if (tc) XB_CUDA(launch_sweep_tc(sp, h->Xt.p, correction_terms(it), st));
-        else XB_CUDA(sweep32(sp));
+        PhaseScope ps(h, XBAR_PHASE_SWEEP, cr ? cr_sweep_launches(h, false, false) : sweep_launches(h->meet, N, false, few));
+        XB_CUDA(sweep32(sp, correction_terms(it)));  // dhat = solve32(rhat), I += dI
       }
       w_current = false;
       ++iters;
@@ -1052,9 +1082,8 @@ xbar_status xbar::solve_device_driven(xbar_s* h, int B, const double* dV, double
   if (h->cr_active)
     return fail(XBAR_ESTATE, "device-driven solves (tile batches) need a block-Thomas factorization");
   const bool mixed = h->prec == XBAR_FP32_IR;
-  const bool tc = mixed && h->tc_ready;
-  const int Bp = tc ? kSweepTcPanel
-                    : (mixed ? sweep_panel_width<float>(Mp, B, h->nsm) : sweep_panel_width<double>(Mp, B, h->nsm));
+  const SweepKind kind = sweep_kind(h, B, mixed);
+  const int Bp = kind.Bp;
   const int Bpad = ((B + Bp - 1) / Bp) * Bp;
   const size_t nst = (size_t)N * Mp * Bpad;
   auto need = [&](Buf& b, size_t bytes) -> bool {
@@ -1071,7 +1100,7 @@ xbar_status xbar::solve_device_driven(xbar_s* h, int B, const double* dV, double
     sp.V = dV; sp.rhs = nullptr; sp.meet = h->meet; sp.first_only = false; sp.z = (double*)h->z.p; sp.w = nullptr; sp.I = dI;
     sp.accumulate = 0; sp.max_rel = nullptr; sp.status = h->status;
     XB_CUDA(launch_ir_init(state, st));
-    XB_CUDA(launch_sweep<double>(sp, st));
+    XB_CUDA(run_sweep<double>(sp, kind, nullptr, 0, st));
     return XBAR_OK;
   }
   if (!need(h->z, nst * 4) || !need(h->dhat, nst * 4) || !need(h->rhat, nst * 4) || !need(h->w64, nst * 8) ||
@@ -1091,11 +1120,9 @@ xbar_status xbar::solve_device_driven(xbar_s* h, int B, const double* dV, double
   sp.X = (const float*)h->X.p; sp.e = m.e32; sp.hs = m.hs32; sp.src = m.src32;
   sp.V = dV; sp.rhs = nullptr; sp.meet = h->meet; sp.first_only = false; sp.z = (float*)h->z.p; sp.w = (float*)h->dhat.p; sp.I = dI;
   sp.accumulate = 0; sp.max_rel = nullptr; sp.status = h->status;
-  auto sweep = [&](int terms) -> cudaError_t {
-    return tc ? launch_sweep_tc(sp, h->Xt.p, terms, st) : launch_sweep<float>(sp, st);
-  };
+  auto sweep = [&](int terms) -> cudaError_t { return run_sweep<float>(sp, kind, h->Xt.p, terms, st); };
   XB_CUDA(launch_ir_init(state, st));
-  if (tc) {  // x0 = solve32(b); the sweep writes the state w = s o x0 (FP32) itself
+  if (kind.tc || kind.few.nv) {  // x0 = solve32(b); the sweep writes the state w = s o x0 (FP32) itself
     if (!need(h->w1, nst * 4)) return fail(XBAR_ENOMEM, "workspace not prepared for this batch size");
     sp.w = nullptr;
     sp.w1out = (float*)h->w1.p;
@@ -1328,6 +1355,11 @@ extern "C" xbar_status xbar_solve_noalloc(xbar_t h, int B, const double* V, doub
                 "xbar_solve_noalloc: N*Mp*Bpad*8 = %zu bytes of scratch exceeds the fixed %llu bytes "
                 "(N=%d, Mp=%d, Bpad=%d); use xbar_solve or a smaller batch",
                 need, (unsigned long long)XBAR_NOALLOC_SCRATCH_BYTES, m.N, m.Mp, Bpad);
+  // a few vectors: the cluster kernel, where its panels fit the array too
+  SweepKind kind = sweep_kind(h, B, false);
+  const int Bpad_few = kind.few.nv ? ((B + kind.Bp - 1) / kind.Bp) * kind.Bp : 0;
+  const bool few = Bpad_few && (size_t)m.N * m.Mp * Bpad_few * sizeof(double) <= XBAR_NOALLOC_SCRATCH_BYTES;
+  if (!few) kind = SweepKind();
   void* scratch = nullptr;
   {
     cudaError_t e = noalloc_scratch(h->dev, &scratch);
@@ -1338,8 +1370,8 @@ extern "C" xbar_status xbar_solve_noalloc(xbar_t h, int B, const double* V, doub
   sp.Mp = m.Mp;
   sp.N = m.N;
   sp.B = B;
-  sp.Bp = Bp;
-  sp.Bpad = Bpad;
+  sp.Bp = few ? kind.Bp : Bp;
+  sp.Bpad = few ? Bpad_few : Bpad;
   sp.X = (const double*)h->X.p;
   sp.e = m.e_pl;
   sp.hs = m.h;
@@ -1354,6 +1386,6 @@ extern "C" xbar_status xbar_solve_noalloc(xbar_t h, int B, const double* V, doub
   sp.accumulate = 0;
   sp.max_rel = nullptr;
   sp.status = h->status;
-  XB_CUDA(launch_sweep<double>(sp, h->st));
+  XB_CUDA(run_sweep<double>(sp, kind, nullptr, 0, h->st));
   return XBAR_OK;
 }

@@ -125,6 +125,14 @@ cudaError_t launch_sweep(const SweepParams<T>& p, cudaStream_t st);
 template <typename T>
 int sweep_panel_width(int Mp, int B, int nsm);
 
+// ---- sweeps of a few vectors (sweep_few.cu): a cluster of Mp / rr blocks per chain and panel of nv ----
+struct FewPlan {
+  int nv = 0, rr = 0;  // nv = 0: not for this size
+};
+FewPlan sweep_few_plan(int Mp, int B, int nsm);
+template <typename T>
+cudaError_t launch_sweep_few(const SweepParams<T>& p, FewPlan f, cudaStream_t st);
+
 // ---- tensor-core (tcgen05, three-term BF16) FP32 sweeps: panels of 64 vectors, Mp <= 256 -----
 bool sweep_tc_supported(int Mp);
 int sweep_tc_rows(int Mp);  // rows of the tiled factor (128 or 256)

@@ -307,6 +307,8 @@ __global__ void __launch_bounds__(128, 8) resid_kernel(ResidParams p) {
   const bool has_l = j > 0, has_r = j + 1 < p.N;
   const long col = (long)p.Mp * (long)rs;
   float* rh = p.rhat + o0;
+  // the substitution multiplies the padding rows too (by zeros): they must be numbers
+  for (int i = M; i < p.Mp; ++i) rh[(long)i * (long)rs] = 0.0f;
   fp2 u{0.0f, 0.0f};
   float rmax = 0.0f;  // |r| tracked in FP32: only its magnitude is reported
   if (has_l && has_r) back_walk<kW1, 3>(p, c, W, col, rh, ph2, S, j, b, u, rmax);
