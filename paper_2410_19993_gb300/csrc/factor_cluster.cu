@@ -315,28 +315,41 @@ __global__ void __launch_bounds__(kThreads, 1)
 
     // (4) blocked Gauss-Jordan inversion; panel p = rows of block p.
     // Pivot blocks are inverted in one warp's registers (Gauss-Jordan, no pivoting: the block is
-    // symmetric positive definite).  Lane l holds column l % 16 of rows 8 (l / 16) .. + 7; each
-    // pivot's row, column and diagonal arrive by shuffles.
+    // symmetric positive definite), two pivots at a time: one reciprocal (of the 2 x 2 determinant) and
+    // one round of shuffles for both, on the chain from panel to panel.  Off-diagonal entries of a part
+    // have one sign, so the products of P^-1 [r0; r1] add without cancellation; the determinant cancels
+    // exactly as the second pivot would.  Lane l holds column l % 16 of rows 8 (l / 16) .. + 7.
     static_assert(R == 16, "register layout assumes 16 x 16 pivot blocks");
     const int pb = lane & 15, pa0 = (lane >> 4) * 8;
     float* slots = p.pbuf + (size_t)chain * C * slot;
     float* myslot = slots + (size_t)g * slot;  // R_g then D_g^-1
     auto invert_publish = [&](float (&d)[8]) {  // warp kInvWarp: D^-1 to Dm and to this block's slot
 #pragma unroll
-      for (int q = 0; q < R; ++q) {
-        const int qe = q & 7, qlane = (q >> 3) << 4;
-        const float piv = __shfl_sync(0xffffffffu, d[qe], qlane | q);   // D[q][q]
-        const float rowq = __shfl_sync(0xffffffffu, d[qe], qlane | pb);  // D[q][b]
-        float colq[8];                                                   // D[a0 + e][q]
+      for (int q = 0; q < R; q += 2) {
+        const int qe = q & 7, qlane = (q >> 3) << 4;  // rows q, q+1: elements qe, qe+1 of one half-warp
+        const float p00 = __shfl_sync(0xffffffffu, d[qe], qlane | q), p01 = __shfl_sync(0xffffffffu, d[qe], qlane | (q + 1));
+        const float p10 = __shfl_sync(0xffffffffu, d[qe + 1], qlane | q);
+        const float p11 = __shfl_sync(0xffffffffu, d[qe + 1], qlane | (q + 1));
+        float r0 = __shfl_sync(0xffffffffu, d[qe], qlane | pb), r1 = __shfl_sync(0xffffffffu, d[qe + 1], qlane | pb);
+        float c0[8], c1[8];  // D[a0 + e][q], D[a0 + e][q + 1]
 #pragma unroll
-        for (int e = 0; e < 8; ++e) colq[e] = __shfl_sync(0xffffffffu, d[e], (lane & 16) | q);
-        const float ri = __fdividef(1.0f, piv);
-        // column q: -D[a][q] / piv; elsewhere D[a][b] - D[a][q] D[q][b] / piv; row q: D[q][b] / piv
-        const bool incol = pb == q;
-        const float f = incol ? ri : rowq * ri;
+        for (int e = 0; e < 8; ++e) {
+          c0[e] = __shfl_sync(0xffffffffu, d[e], (lane & 16) | q);
+          c1[e] = __shfl_sync(0xffffffffu, d[e], (lane & 16) | (q + 1));
+        }
+        const float rd = __fdividef(1.0f, fmaf(p00, p11, -p01 * p10));
+        // rows q, q+1 become P^-1 [r0; r1] (P^-1 itself in the pivot columns); all other rows lose their
+        // pivot-column entries times those
+        const bool in0 = pb == q, in1 = pb == q + 1;
+        r0 = in0 ? 1.0f : in1 ? 0.0f : r0;
+        r1 = in1 ? 1.0f : in0 ? 0.0f : r1;
+        const float f0 = fmaf(p11, r0, -p01 * r1) * rd, f1 = fmaf(p00, r1, -p10 * r0) * rd;
 #pragma unroll
-        for (int e = 0; e < 8; ++e) d[e] = fmaf(-colq[e], f, incol ? 0.0f : d[e]);
-        if ((lane & 16) == qlane) d[qe] = f;  // the half-warp holding row q
+        for (int e = 0; e < 8; ++e) d[e] = fmaf(-c1[e], f1, fmaf(-c0[e], f0, in0 || in1 ? 0.0f : d[e]));
+        if ((lane & 16) == qlane) {
+          d[qe] = f0;
+          d[qe + 1] = f1;
+        }
       }
 #pragma unroll
       for (int e = 0; e < 8; ++e) {

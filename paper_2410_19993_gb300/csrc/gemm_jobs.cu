@@ -348,7 +348,7 @@ __global__ void __launch_bounds__(NT / RPT * 32) gj_kernel(const GjJob<T>* __res
       }
     }
     __syncthreads();
-    // (2) one warp: R' = D^-1 R (8 sweep steps on the panel rows, in registers; lane l holds
+    // (2) one warp: R' = D^-1 R (8 sweep steps on the panel rows, two at a time, in registers; lane l holds
     // columns l + 32 c of the 8 rows, the pivot column's values come by shuffle from its lane)
     if (ty == 0) {
       T pr[PW][CB];
@@ -358,27 +358,31 @@ __global__ void __launch_bounds__(NT / RPT * 32) gj_kernel(const GjJob<T>* __res
         for (int c = 0; c < CB; ++c) pr[k][c] = PR[b][k][tx + 32 * c];
       const int ck = P0 / 32, src = P0 & 31;
 #pragma unroll
-      for (int k = 0; k < PW; ++k) {
-        T f[PW];  // column P0 + k of the 8 rows (lane src + k, slot ck)
+      for (int k = 0; k < PW; k += 2) {  // two pivots at a time: one reciprocal and one round of shuffles
+        T f0[PW], f1[PW];  // columns P0 + k, P0 + k + 1 of the 8 rows (lanes src + k, + 1, slot ck)
 #pragma unroll
         for (int l = 0; l < PW; ++l) {
           T v = pr[l][0];
 #pragma unroll
           for (int c = 1; c < CB; ++c)
             if (c == ck) v = pr[l][c];
-          f[l] = __shfl_sync(0xffffffffu, v, src + k);
+          f0[l] = __shfl_sync(0xffffffffu, v, src + k);
+          f1[l] = __shfl_sync(0xffffffffu, v, src + k + 1);
         }
-        const T inv = (T)1 / f[k];
+        const T p00 = f0[k], p01 = f1[k], p10 = f0[k + 1], p11 = f1[k + 1];
+        const T rd = (T)1 / fma(p00, p11, -p01 * p10);
 #pragma unroll
         for (int c = 0; c < CB; ++c) {
-          const bool piv = (tx == src + k) && (c == ck);
-          const T rk = piv ? inv : pr[k][c] * inv;
+          const bool in0 = (tx == src + k) && (c == ck), in1 = (tx == src + k + 1) && (c == ck);
+          const T r0 = in0 ? (T)1 : in1 ? (T)0 : pr[k][c], r1 = in1 ? (T)1 : in0 ? (T)0 : pr[k + 1][c];
+          const T g0 = fma(p11, r0, -p01 * r1) * rd, g1 = fma(p00, r1, -p10 * r0) * rd;
 #pragma unroll
           for (int l = 0; l < PW; ++l) {
-            if (l == k) continue;
-            pr[l][c] = piv ? -f[l] * inv : fma(-f[l], rk, pr[l][c]);
+            if (l == k || l == k + 1) continue;
+            pr[l][c] = fma(-f1[l], g1, fma(-f0[l], g0, in0 || in1 ? (T)0 : pr[l][c]));
           }
-          pr[k][c] = rk;
+          pr[k][c] = g0;
+          pr[k + 1][c] = g1;
         }
       }
 #pragma unroll

@@ -703,10 +703,18 @@ __global__ void feature_kernel(const double* Gt, const float* St, const double* 
 }
 
 // Layer 3, loss and back-propagation to dZ2; one warp per row, lane l owns hidden units 8l..8l+7.
-// Accumulates dW3, db3 and the two loss sums.
-__global__ void head_kernel(const __nv_bfloat16* H2, const float* W3, const float* b3, const float* y, long rows,
-                            long valid, float inv_rows, __nv_bfloat16* dZ2, float* dW3, float* db3, double* loss) {
-  const int lane = threadIdx.x & 31;
+// Accumulates dW3, db3 and the two loss sums: each warp over its rows in registers, the block's eight
+// warps in shared memory, then one atomic per block and sum.  (With one row a warp and its atomics
+// straight to memory, 4096 rows made 2 M atomics on 512 addresses: 310 us against 8.)
+constexpr int kHeadWarps = 8;
+__global__ void __launch_bounds__(32 * kHeadWarps) head_kernel(const __nv_bfloat16* H2, const float* W3, const float* b3,
+                                                               const float* y, long rows, long valid, float inv_rows,
+                                                               __nv_bfloat16* dZ2, float* dW3, float* db3,
+                                                               double* loss) {
+  __shared__ __align__(16) float gsum[kHeadWarps][2 * kH];
+  __shared__ float bsum[kHeadWarps][2];
+  __shared__ double lsum[kHeadWarps][2];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const long warp0 = ((long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const long nwarps = ((long)gridDim.x * blockDim.x) >> 5;
   float w0[8], w1[8], g0[8] = {0}, g1[8] = {0}, gb0 = 0.0f, gb1 = 0.0f;
@@ -753,25 +761,46 @@ __global__ void head_kernel(const __nv_bfloat16* H2, const float* W3, const floa
     gb1 += d1;
   }
 #pragma unroll
-  for (int q = 0; q < 8; ++q) {
-    atomicAdd(&dW3[lane * 8 + q], g0[q]);
-    atomicAdd(&dW3[kH + lane * 8 + q], g1[q]);
+  for (int q = 0; q < 8; q += 4) {
+    *reinterpret_cast<float4*>(&gsum[warp][lane * 8 + q]) = make_float4(g0[q], g0[q + 1], g0[q + 2], g0[q + 3]);
+    *reinterpret_cast<float4*>(&gsum[warp][kH + lane * 8 + q]) = make_float4(g1[q], g1[q + 1], g1[q + 2], g1[q + 3]);
   }
   if (lane == 0) {
-    atomicAdd(&db3[0], gb0);
-    atomicAdd(&db3[1], gb1);
-    atomicAdd(&loss[0], l0);
-    atomicAdd(&loss[1], l1);
+    bsum[warp][0] = gb0;
+    bsum[warp][1] = gb1;
+    lsum[warp][0] = l0;
+    lsum[warp][1] = l1;
+  }
+  __syncthreads();
+  for (int k = threadIdx.x; k < 2 * kH; k += blockDim.x) {
+    float t = 0.0f;
+#pragma unroll
+    for (int w = 0; w < kHeadWarps; ++w) t += gsum[w][k];
+    atomicAdd(&dW3[k], t);
+  }
+  if (threadIdx.x < 2) {
+    float t = 0.0f;
+    double l = 0.0;
+    for (int w = 0; w < kHeadWarps; ++w) {
+      t += bsum[w][threadIdx.x];
+      l += lsum[w][threadIdx.x];
+    }
+    atomicAdd(&db3[threadIdx.x], t);
+    atomicAdd(&loss[threadIdx.x], l);
   }
 }
 
-// out[k] += sum over rows of D[r][k] (bias gradients); block = 256 threads = one column each
-__global__ void colsum_kernel(const __nv_bfloat16* D, long rows, long chunk, float* out) {
+// out[k] += sum over rows of D[r][k] (bias gradients) for two matrices at once (blockIdx.y); block = 256
+// threads = one column each, `chunk` rows
+__global__ void colsum_kernel(const __nv_bfloat16* D0, const __nv_bfloat16* D1, long rows, long chunk, float* out0,
+                              float* out1) {
+  const __nv_bfloat16* D = blockIdx.y ? D1 : D0;
   const int k = threadIdx.x;
   const long r0 = blockIdx.x * chunk, r1 = min(rows, r0 + chunk);
   float s = 0.0f;
+#pragma unroll 8
   for (long r = r0; r < r1; ++r) s += __bfloat162float(D[r * kH + k]);
-  atomicAdd(&out[k], s);
+  atomicAdd((blockIdx.y ? out1 : out0) + k, s);
 }
 
 // Adam on the flat FP32 parameters
@@ -845,6 +874,7 @@ struct xbar_surrogate_s {
   // workspace (rows capacity)
   long cap = 0;
   Buf X, H1, H2, dZ2, dZ1, y, out, Iid, Iln, flag, idx, gV, gI;
+  Buf gX, gy;  // xbar_surrogate_grad's copies of its arguments
   // per-map line model and feature columns: [N][M]
   int passes = 1;
   Buf Gt, Gf, tau, St, Tl, wl, bl, xg, field;
@@ -997,13 +1027,15 @@ static xbar_status fwd_bwd(xbar_surrogate_t s, const __nv_bfloat16* X, long rows
   g.B = s->W2b; g.sBn = kH;
   g.bias = s->P + s->ob2; g.out = (__nv_bfloat16*)s->H2.p;
   XB_CUDA(launch_gemm_bf16(g, 1, s->st));
-  const int hb = (int)std::min<long>(4096, (rows + 7) / 8);
+  const int hb = (int)std::min<long>(2 * s->nsm, (rows + kHeadWarps - 1) / kHeadWarps);
   XB_CUDA(cudaMemsetAsync(s->Gr, 0, s->np * 4, s->st));
-  head_kernel<<<hb, 256, 0, s->st>>>((const __nv_bfloat16*)s->H2.p, s->P + s->oW3, s->P + s->ob3, y, rows, valid,
+  head_kernel<<<hb, 32 * kHeadWarps, 0, s->st>>>((const __nv_bfloat16*)s->H2.p, s->P + s->oW3, s->P + s->ob3, y, rows, valid,
                                      1.0f / (float)valid, (__nv_bfloat16*)s->dZ2.p, s->Gr + s->oW3, s->Gr + s->ob3,
                                      s->loss);
   XB_CUDA(cudaGetLastError());
-  const int ks = (int)std::max<long>(1, std::min<long>(64, rows / 1024));
+  // weight gradients contract over the rows: split so that the few output tiles (4 and 2 Fp / 128)
+  // fill the SMs
+  const int ks = (int)std::max<long>(1, std::min<long>(64, rows / 256));
   // dW2 = dZ2^T H1
   memset(&g, 0, sizeof(g));
   g.status = s->status;
@@ -1030,10 +1062,10 @@ static xbar_status fwd_bwd(xbar_surrogate_t s, const __nv_bfloat16* X, long rows
   g.mode = GEMM_EPI_STORE; g.C = s->Gr + s->oW1; g.ldc = Fp; g.atomic = 1;
   XB_CUDA(launch_gemm_bf16(g, ks, s->st));
   // bias gradients
-  const long chunk = 512;
+  const long chunk = std::max<long>(32, (rows + s->nsm - 1) / s->nsm);
   const int nb = (int)((rows + chunk - 1) / chunk);
-  colsum_kernel<<<nb, kH, 0, s->st>>>((const __nv_bfloat16*)s->dZ2.p, rows, chunk, s->Gr + s->ob2);
-  colsum_kernel<<<nb, kH, 0, s->st>>>((const __nv_bfloat16*)s->dZ1.p, rows, chunk, s->Gr + s->ob1);
+  colsum_kernel<<<dim3(nb, 2), kH, 0, s->st>>>((const __nv_bfloat16*)s->dZ2.p, (const __nv_bfloat16*)s->dZ1.p, rows,
+                                              chunk, s->Gr + s->ob2, s->Gr + s->ob1);
   XB_CUDA(cudaGetLastError());
   return XBAR_OK;
 }
@@ -1044,9 +1076,9 @@ extern "C" xbar_status xbar_surrogate_grad(xbar_surrogate_t s, int R, const floa
   XB_CUDA(cudaSetDevice(s->dev));
   const long rows = round_up_l(R, 128);
   if (ensure_rows(s, rows) != XBAR_OK) return XBAR_ENOMEM;
-  float *dXf = nullptr, *dy = nullptr;
-  XB_CUDA(cudaMalloc(&dXf, (size_t)R * s->F * 4));
-  XB_CUDA(cudaMalloc(&dy, (size_t)rows * 4));
+  XB_CUDA(ensure(s->A, s->gX, (size_t)R * s->F * 4));  // kept: an allocation and a free per call cost more
+  XB_CUDA(ensure(s->A, s->gy, (size_t)rows * 4));      // than the kernels of a small minibatch
+  float *dXf = (float*)s->gX.p, *dy = (float*)s->gy.p;
   XB_CUDA(cudaMemcpyAsync(dXf, X, (size_t)R * s->F * 4, cudaMemcpyDefault, s->st));
   XB_CUDA(cudaMemsetAsync(dy, 0, (size_t)rows * 4, s->st));
   XB_CUDA(cudaMemcpyAsync(dy, y, (size_t)R * 4, cudaMemcpyDefault, s->st));
@@ -1069,8 +1101,6 @@ extern "C" xbar_status xbar_surrogate_grad(xbar_surrogate_t s, int R, const floa
       loss[1] = l[1] / R;
     }
   }
-  cudaFree(dXf);
-  cudaFree(dy);
   if (st == XBAR_OK && dst)
     return set_error(dst & XBAR_DEV_TIMEOUT ? XBAR_ETIMEOUT : XBAR_ECUDA, "device status 0x%x", dst);
   return st;

@@ -45,16 +45,12 @@ __device__ __forceinline__ uint32_t few_peer(uint32_t local, uint32_t rank) {
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(local), "r"(rank));
   return r;
 }
-// asynchronous store to a block of the cluster, counted in bytes on that block's mbarrier
-__device__ __forceinline__ void st_async(uint32_t addr, double v, uint32_t bar) {
-  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(addr),
-               "l"(__double_as_longlong(v)), "r"(bar)
-               : "memory");
-}
-__device__ __forceinline__ void st_async(uint32_t addr, float v, uint32_t bar) {
-  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(addr),
-               "r"(__float_as_uint(v)), "r"(bar)
-               : "memory");
+// asynchronous 16-byte store to a block of the cluster, counted in bytes on that block's mbarrier
+__device__ __forceinline__ void st_async16(uint32_t addr, uint4 v, uint32_t bar) {
+  asm volatile(
+      "st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(addr),
+      "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "r"(bar)
+      : "memory");
 }
 
 // bounded wait for phase `parity`, acquire at cluster scope
@@ -135,7 +131,9 @@ __global__ void __launch_bounds__(kFewThreads) sweep_few_kernel(SweepParams<T> p
   T* ring = reinterpret_cast<T*>(smem_raw);           // [depth][RR][Mp]
   T* vin = ring + (size_t)depth * RR * Mp;            // [2][Mp][NV]
   __shared__ __align__(8) uint64_t full[kFewRing], vbar[2];
-  __shared__ T ybuf[NE], vout[NE], cbuf[2][NE];
+  __shared__ __align__(16) T vout[NE];
+  __shared__ T ybuf[NE], cbuf[2][NE];
+  static_assert(NE * sizeof(T) % 16 == 0, "whole 16-byte pieces");
   __shared__ unsigned fail;
 
   if (p.skip && *p.skip) return;  // the same for every block
@@ -247,9 +245,11 @@ __global__ void __launch_bounds__(kFewThreads) sweep_few_kernel(SweepParams<T> p
     }
     if (more) {
       const uint32_t dst = smem_addr(vin + ((size_t)((s + 1) & 1) * Mp + row0) * NV), bar = smem_addr(&vbar[(s + 1) & 1]);
-      for (int t = tid; t < NE * C; t += kFewThreads) {
-        const int peer = t / NE, k = t - peer * NE;
-        st_async(few_peer(dst + (uint32_t)(k * sizeof(T)), (uint32_t)peer), vout[k], few_peer(bar, (uint32_t)peer));
+      constexpr int NP = NE * (int)sizeof(T) / 16;  // 16-byte pieces of the block's elements
+      for (int t = tid; t < NP * C; t += kFewThreads) {
+        const int peer = t / NP, k = t - peer * NP;
+        st_async16(few_peer(dst + 16u * k, (uint32_t)peer), reinterpret_cast<const uint4*>(vout)[k],
+                   few_peer(bar, (uint32_t)peer));
       }
       load_operands(s + 1);
     }
