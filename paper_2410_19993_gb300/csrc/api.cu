@@ -606,7 +606,7 @@ static xbar_status do_factor64(xbar_t h) {
   fp.meet = h->meet;
   fp.gsrc = m.gs;
   fp.gw = m.gw;
-  fp.Coff = m.Coff;
+  fp.Coff = (const double*)m.Coff;
   fp.h = m.h;
   fp.X = (double*)h->X.p;
   fp.buf = (double*)h->fpbuf.p;
@@ -642,7 +642,7 @@ static xbar_status do_factor32(xbar_t h, bool upload) {
   fp.N = N;
   fp.gsrc = m.gs;
   fp.gw = m.gw;
-  fp.Coff = m.Coff;
+  fp.Coff = (const float*)m.Coff;
   fp.h = m.h;
   fp.s = m.s_eq;
   fp.e = m.e_eq;
@@ -651,6 +651,8 @@ static xbar_status do_factor32(xbar_t h, bool upload) {
   fp.pbuf = (float*)h->fpbuf.p;
   fp.bar = (unsigned*)h->fbar.p;
   fp.meet = h->meet;
+  fp.s32 = m.s32;
+  fp.e32 = m.e32;
   XB_CUDA(cudaMemsetAsync(h->fbar.p, 0, 2 * sizeof(unsigned), h->st));
   if (upload) {
     // The block changes only when a buffer is (re)allocated.  Upload it, and wait for the copy out
@@ -689,9 +691,9 @@ xbar_status xbar::factor_handle(xbar_s* h, xbar_precision p, bool upload_params)
     PhaseScope ps(h, XBAR_PHASE_FACTOR, 1);
     xbar_status s = factor_mirror(h, p);
     if (s != XBAR_OK) return s;
-    // map remap + assembly (3) + the factor (one launch, or the cyclic reduction's operations)
+    // map remap + assembly (2) + the factor (one launch, or the cyclic reduction's operations)
     const xbar_s* g = h->mirror;
-    ps.nlaunch = 4 + (g->cr_active ? (int)(p == XBAR_FP64 ? g->cr64.ops.size() : g->cr32.ops.size())
+    ps.nlaunch = 3 + (g->cr_active ? (int)(p == XBAR_FP64 ? g->cr64.ops.size() : g->cr32.ops.size())
                                    : 1 + g->tc_ready);
     h->orient_active = 1;
     h->cr_active = 0;
@@ -700,10 +702,10 @@ xbar_status xbar::factor_handle(xbar_s* h, xbar_precision p, bool upload_params)
     h->factored = 1;
     return XBAR_OK;
   }
-  if (!h->assembled) {  // the elimination data of the current conductances
-    PhaseScope ps(h, XBAR_PHASE_ASSEMBLE, 3);
-    XB_CUDA(launch_assemble(h->m, h->st));
-    h->assembled = 1;
+  if (h->assembled != assembled_for(p)) {  // the elimination data of the current conductances
+    PhaseScope ps(h, XBAR_PHASE_ASSEMBLE, 2);
+    XB_CUDA(launch_assemble(h->m, p != XBAR_FP64, h->st));
+    h->assembled = assembled_for(p);
   }
   const bool cr = use_cr(h);
   h->tc_ready = 0;
@@ -1224,11 +1226,12 @@ extern "C" xbar_status xbar_set_conductances(xbar_t h, const double* G) {
     // a device map is validated by the transposing kernel itself (status word, reported by the
     // next call that reads it), so the host does not wait for the stream here
     const bool eager = h->opt.eager_asm == 1;
-    PhaseScope ps(h, XBAR_PHASE_ASSEMBLE, eager ? 4 : 1);
+    PhaseScope ps(h, XBAR_PHASE_ASSEMBLE, eager ? 3 : 1);
     XB_CUDA(launch_store_g(m, Gd, gdev ? h->status : nullptr, h->st));
     if (eager) {  // the elimination data at once, so that a factor queued behind this call starts
-      XB_CUDA(launch_assemble(m, h->st));
-      h->assembled = 1;
+      // (the column blocks in the precision last factored; another one forms them again)
+      XB_CUDA(launch_assemble(m, h->prec != XBAR_FP64, h->st));
+      h->assembled = assembled_for(h->prec);
     }
   }
   return XBAR_OK;

@@ -65,7 +65,7 @@ template <typename T>
 struct CrInitParams {
   int M, Mp, N;
   double gs;
-  const double* Coff;  // [N][Mp][Mp] off-diagonal of the column blocks (unscaled)
+  const T* Coff;       // [N][Mp][Mp] off-diagonal of the column blocks (unscaled)
   const double* h;     // [N][Mp]
   const T* s;          // [N][Mp] equilibration in the factor's precision, or nullptr
   const T* e;          // [N][Mp] coupling column j -> j+1 (equilibrated if s is set)
@@ -86,14 +86,14 @@ __global__ void cr_init_kernel(CrInitParams<T> p) {
   const T* s = p.s;  // nullptr: unscaled
   const T si = (real && s) ? s[vo + i] : (T)1;
   T* Drow = p.D + (vo + i) * Mp;
-  const double* Crow = p.Coff + (vo + i) * Mp;
+  const T* Crow = p.Coff + (vo + i) * Mp;
   T off = (T)0;
   for (int m = lane; m < Mp; m += 32) {
     if (m == i) continue;
     T v = (T)0;
     if (real && m < M) {
       const T sm = s ? s[vo + m] : (T)1;
-      v = (T)Crow[m] * (si * sm);
+      v = Crow[m] * (si * sm);
       off += s ? fabs(v) / sm : fabs(v);
     }
     Drow[m] = v;
@@ -695,7 +695,7 @@ cudaError_t cr_factor(xbar_s* hd, CrPlan<T>& pl, bool tensor, bool equilibrate) 
         ip.Mp = Mp;
         ip.N = N;
         ip.gs = m.gs;
-        ip.Coff = m.Coff;
+        ip.Coff = (const T*)m.Coff;
         ip.h = m.h;
         ip.s = equilibrate ? (const T*)(const void*)m.s32 : nullptr;  // FP32 factors only
         ip.e = e;

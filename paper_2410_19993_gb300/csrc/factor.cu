@@ -75,7 +75,7 @@ __global__ void __launch_bounds__(kFactorThreads)
   const int npanel = Mp / PB;
 
   for (int j = 0; j < N; ++j) {
-    const double* Cj = p.Coff + (size_t)j * Mp * Mp;
+    const float* Cj = p.Coff + (size_t)j * Mp * Mp;
     const double* sj = p.s ? p.s + (size_t)j * Mp : nullptr;
     const double* sjm = (p.s && j > 0) ? p.s + (size_t)(j - 1) * Mp : nullptr;
     const double* ejm = j > 0 ? p.e + (size_t)(j - 1) * Mp : nullptr;
@@ -117,7 +117,7 @@ __global__ void __launch_bounds__(kFactorThreads)
       float v = 0;
       if (i < M && k < M && k != i) {
         const float si = sj ? (float)sj[i] : 1.0f, sk = sj ? (float)sj[k] : 1.0f;
-        v = si * sk * (float)Cj[(size_t)i * Mp + k];
+        v = si * sk * Cj[(size_t)i * Mp + k];
         if (j > 0) v -= (float)ejm[i] * (float)ejm[k] * rows[t];
       }
       rows[t] = v;

@@ -6,18 +6,28 @@
 //     Z_m = C_m - g_w^2 X_{m-1} - g_w^2 X_{m+1}.
 // The factor is bound by the latency of its chain (16 dependent panels a column on 16 SMs), so half the
 // chain is half the time: 12.25 -> 6.2 ms at 256 x 256, 2.85 -> 1.45 ms at 128 x 128, on twice the SMs.
-// In a cluster of C blocks block g holds rows [g R, (g+1) R) of the current matrix in shared memory (R = 16, C = Mp / R).
+// In a cluster of C blocks block g holds rows [g R, (g+1) R) of the current matrix in registers, one
+// thread per column (R = 16, C = Mp / R).
 // The in-place blocked Gauss-Jordan inversion uses panels of R rows, so panel p is exactly block p's
 // rows.  With R_p the owner's rows when panel p starts and D_p^-1 the inverse of their pivot block,
 // Gauss-Jordan replaces the owner's rows by D_p^-1 R_p (D_p^-1 in the pivot columns) and every other
 // block's rows by  row - W' R_p  (-W' in the pivot columns), W' = row[P] D_p^-1.  So the other blocks
-// need only R_p and D_p^-1, not the owner's formed rows: the owner publishes both to its own slot of
-// a global (L2-resident) buffer as soon as they exist and signals each peer's mbarrier (arrive with
-// release at cluster scope; the peer waits with acquire).  The next owner computes its updated pivot
-// block first and inverts it in one warp while its other warps apply the panel (look-ahead), so the
-// chain from panel to panel is signal, L2 read, W', max(update, inversion).  (Pulling panels from the
-// owner's shared memory instead makes all peers drain one SM's shared-memory port at once and is
-// several times slower.)  Every wait is bounded; a block whose wait expires records
+// need only R_p and D_p^-1, not the owner's formed rows.  What they need travels in three parts, each as
+// early as it exists, because every hand-over costs more than the arithmetic it feeds:
+//   * the owner's rows go to its slot of a global (L2-resident) buffer already before panel p-1 is applied
+//     to them; each peer's mbarrier is signalled (arrive with release at cluster scope) and its threads
+//     load their own column straight into registers.  (Pulling panels from the owner's shared memory
+//     instead makes all peers drain one SM's port at once and is several times slower.)
+//   * the owner's W' for panel p-1 (1 KB) follows when D_{p-1}^-1 is known, by asynchronous stores to every
+//     peer's shared memory that complete on the peer's mbarrier (transaction bytes); with it each thread
+//     applies panel p-1, whose column it still holds, to its column of the owner's rows: R_p.  That doubles
+//     the multiply-adds and takes the rows' update, store, signal and load (5k cycles together) off
+//     the chain;
+//   * D_p^-1 (1 KB) goes from the inverting warp the same way, to the next owner first.
+// The next owner forms W' and its updated pivot block first and one warp inverts it while the others
+// apply the panel (look-ahead).  The chain from panel to panel is then  D^-1 arrives, W', pivot block,
+// inversion.  Updates run one thread per column on pairs of rows (packed FP32 multiply-adds, coefficients
+// broadcast from shared memory).  Every wait is bounded; a block whose wait expires records
 // XBAR_DEV_TIMEOUT and stops waiting but keeps the cluster barrier sequence (one per column step).
 #include <math.h>
 
@@ -48,10 +58,23 @@ __device__ __forceinline__ uint32_t peer_addr(const void* local, uint32_t rank) 
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_addr(local)), "r"(rank));
   return r;
 }
+__device__ __forceinline__ uint32_t peer_addr32(uint32_t local, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(local), "r"(rank));
+  return r;
+}
 // arrive on a peer block's mbarrier; release at cluster scope orders this block's earlier writes
 __device__ __forceinline__ void arrive_peer(uint32_t bar_cluster_addr) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster_addr) : "memory");
 }
+// asynchronous 16-byte store to a block of the cluster, counted in bytes on that block's mbarrier
+__device__ __forceinline__ void st_async16(uint32_t addr, uint4 v, uint32_t bar) {
+  asm volatile(
+      "st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(addr),
+      "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "r"(bar)
+      : "memory");
+}
+__device__ __forceinline__ void work_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }  // the row-work warps
 // bounded wait for phase `parity` of a local mbarrier, acquire at cluster scope
 __device__ __forceinline__ bool wait_cluster_bounded(uint64_t* bar, unsigned parity, unsigned* status) {
   auto done = [&]() {
@@ -75,45 +98,71 @@ __device__ __forceinline__ bool wait_cluster_bounded(uint64_t* bar, unsigned par
   }
   return true;
 }
-__device__ __forceinline__ float warp_sum_f(float v) {
+// sums of NS values (a power of two <= 32) over the 32 lanes; lane l then holds sum l / (32 / NS) in v[0]
+template <int NS>
+__device__ __forceinline__ void warp_sums_f(float (&v)[NS], int lane) {
+  int n = NS;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
+  for (int o = 16; o > 0; o >>= 1) {
+    if (n > 1) {
+      const bool up = (lane & o) != 0;
+#pragma unroll
+      for (int q = 0; q < NS / 2; ++q)
+        if (q < n / 2) {
+          const float send = up ? v[q] : v[q + n / 2], keep = up ? v[q + n / 2] : v[q];
+          v[q] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+      n >>= 1;
+    } else {
+      v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+    }
+  }
 }
 
 }  // namespace
 
-// dynamic shared memory: mbarriers [16 panels + 2 staging], rows [R][Mp], pn [R][Mp], D [R][R],
-// Dr [R][R], W [R][R], Bp [R][R], sigv [Mp], sv [Mp], ev [Mp], sigv2 [Mp], ev2 [Mp], sg [2][R], then two
-// staging buffers (FP64) of a column step's inputs: C_j own rows [R][Mp], s_j [Mp], s of the previous
-// column [Mp], the coupling to it [Mp], h_j own rows [R]
-size_t factor_cluster_smem_bytes(int Mp, int R) {
-  return 18 * sizeof(uint64_t) + ((size_t)2 * R * Mp + 4 * (size_t)R * R + 5 * (size_t)Mp + 2 * R) * sizeof(float) +
-         2 * ((size_t)R * Mp + 3 * (size_t)Mp + R) * sizeof(double);
+// dynamic shared memory: mbarriers [16 rows + 16 inverses + 16 W' + 2 staging]; floats: W = -W'^T [R][R] of the
+// panel being applied, Bp [R][R] next pivot block, DmT [R][R] transpose of this block's inverse, Dall
+// [16][R][R] inverse pivot blocks by panel (own and received), Wall [16][R][R] the owners' -W'^T by panel, rw
+// [2][2][R] the inversion's pivot rows, pa, pb, xs [R][R+1] own rows in the columns of this panel and of the
+// next, R_p in those of the next, reductions [8][32] and [8][16], row sums [2][R], scale and coupling of the
+// right neighbour (meeting column) [2][Mp]; then two staging buffers of a column step's inputs: h_j own
+// rows [R] in FP64, C_j own rows [R][Mp], s_j, s of the previous column and the coupling to it [Mp] each
+constexpr int kPitch = kRows + 1;
+constexpr int kBars = 50;
+constexpr int kSmFloats = 3 * kRows * kPitch + (3 + 32) * kRows * kRows + 4 * kRows + 8 * 32 + 8 * 16 + 2 * kRows;
+static_assert(kSmFloats % 4 == 0, "16-byte aligned vectors after the fixed part");
+__host__ __device__ constexpr size_t stage_bytes(int Mp) {
+  return kRows * sizeof(double) + ((size_t)kRows * Mp + 3 * (size_t)Mp) * sizeof(float);
+}
+size_t factor_cluster_smem_bytes(int Mp) {
+  return kBars * sizeof(uint64_t) + ((size_t)kSmFloats + 2 * (size_t)Mp) * sizeof(float) + 2 * stage_bytes(Mp);
 }
 
-// global panel slots, one per block of each chain's cluster: R_p [R][Mp] then D_p^-1 [R][R]
+// global panel slots, one per block of each chain's cluster: R_p [R][Mp]
 size_t factor_cluster_pbuf_floats(int Mp) {
   const size_t C = (size_t)Mp / kRows;
-  return 2 * C * ((size_t)kRows * Mp + (size_t)kRows * kRows);
+  return 2 * C * (size_t)kRows * Mp;
 }
 
-// acc[r] (r < 16) += sign * sum_m coef[r*16 + m] * col[m], coefficients read as 16-byte broadcasts
-__device__ __forceinline__ void rank16_update(float (&acc)[16], const float* __restrict__ coef,
-                                              const float (&col)[16], float sign) {
+// acc[r] += sum_m coefT[m*16 + r] * x[m] (r, m < 16): two rows per packed multiply-add, coefficients read as
+// 16-byte broadcasts
+__device__ __forceinline__ void fma2(float& a0, float& a1, float w0, float w1, float x) {
+  asm("{\n\t.reg .b64 A, W, X;\n\tmov.b64 A, {%0, %1};\n\tmov.b64 W, {%2, %3};\n\tmov.b64 X, {%4, %4};\n\t"
+      "fma.rn.f32x2 A, W, X, A;\n\tmov.b64 {%0, %1}, A;\n\t}"
+      : "+f"(a0), "+f"(a1)
+      : "f"(w0), "f"(w1), "f"(x));
+}
+__device__ __forceinline__ void rank16_update(float (&acc)[16], const float* __restrict__ coefT, const float (&x)[16]) {
 #pragma unroll
-  for (int r = 0; r < 16; ++r) {
-    const float4* c4 = reinterpret_cast<const float4*>(coef + r * 16);
-    float a = acc[r];
+  for (int m = 0; m < 16; ++m) {
+    const float4* c4 = reinterpret_cast<const float4*>(coefT + m * 16);
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const float4 c = c4[q];
-      a = fmaf(sign * c.x, col[4 * q], a);
-      a = fmaf(sign * c.y, col[4 * q + 1], a);
-      a = fmaf(sign * c.z, col[4 * q + 2], a);
-      a = fmaf(sign * c.w, col[4 * q + 3], a);
+      fma2(acc[4 * q], acc[4 * q + 1], c.x, c.y, x[m]);
+      fma2(acc[4 * q + 2], acc[4 * q + 3], c.z, c.w, x[m]);
     }
-    acc[r] = a;
   }
 }
 
@@ -133,345 +182,390 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int r0 = (int)g * R;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint64_t wlim = wait_limit(status);
-  constexpr int nwarps = kThreads / 32;
 
   extern __shared__ __align__(16) unsigned char smraw[];
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smraw);  // [16]: panel p of this column step is ready
-  uint64_t* pbar = bars + 16;                            // [2]: staging buffer b has landed
-  float* sm = reinterpret_cast<float*>(smraw + 18 * sizeof(uint64_t));
-  float* rows = sm;                         // [R][Mp]
-  float* pn = rows + (size_t)R * Mp;        // [R][Mp] the current panel's R_p
-  float* Dm = pn + (size_t)R * Mp;          // [R][R] inverse of this block's pivot block
-  float* Dr = Dm + R * R;                   // [R][R] the current panel's D_p^-1
-  float* W = Dr + R * R;                    // [R][R] W' = own rows[P] D_p^-1
-  float* Bp = W + R * R;                    // [R][R] next pivot block (look-ahead)
-  float* sigv = Bp + R * R;                 // [Mp]
-  float* sv = sigv + Mp;                    // [Mp] equilibration scale of column j
-  float* ev = sv + Mp;                      // [Mp] coupling to the previous column
-  float* sigv2 = ev + Mp;                   // [Mp] meeting column: sigma, coupling of the right neighbour
-  float* ev2 = sigv2 + Mp;                  // [Mp]
-  float* sg = ev2 + Mp;                     // [2][R] sigma of own rows, by step parity
-  double* stg = reinterpret_cast<double*>(sg + 2 * R);  // [2] staging buffers (16-byte aligned)
-  const size_t stg_n = (size_t)R * Mp + 3 * (size_t)Mp + R;
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smraw);  // [16]: the rows of panel p are in its slot
+  uint64_t* dbars = bars + 16;                           // [16]: D_p^-1 is in Dall
+  uint64_t* wbars = bars + 32;                           // [16]: the owner's W' for panel p-1 is in Wall
+  uint64_t* pbar = bars + 48;                            // [2]: staging buffer b has landed
+  float* W = reinterpret_cast<float*>(smraw + kBars * sizeof(uint64_t));  // (vectors read by float4 first)
+  float* Bp = W + R * R;
+  float* DmT = Bp + R * R;
+  float* Dall = DmT + R * R;
+  float* Wall = Dall + 16 * R * R;
+  float* rw = Wall + 16 * R * R;
+  float* pa = rw + 4 * R;
+  float* pb = pa + R * kPitch;
+  float* xs = pb + R * kPitch;
+  float* red = xs + R * kPitch;
+  float* Dm = Dall + (size_t)g * R * R;  // this block's own
+  float* red2 = red + 8 * 32;
+  float* sgs = red2 + 8 * 16;
+  float* abss = sgs + R;
+  float* s2v = abss + R;
+  float* e2v = s2v + Mp;
+  unsigned char* stg = reinterpret_cast<unsigned char*>(e2v + Mp);
 
   if (Mp != C * R || C > 16 || (int)blockDim.x != kThreads) {
     if (tid == 0) set_status(status, XBAR_DEV_BADLAUNCH);
     return;  // uniform across the cluster: every block sees the same arguments
   }
   const float gw = (float)p.gw;
-  if (tid < C) mbar_init(&bars[tid], 1);
+  if (tid < C) {
+    mbar_init(&bars[tid], 1);
+    mbar_init(&dbars[tid], 1);
+    mbar_init(&wbars[tid], 1);
+  }
   if (tid == 0) {
     mbar_init(&pbar[0], 1);
     mbar_init(&pbar[1], 1);
   }
   fence_mbar_init();
   cluster_sync();  // every block's mbarriers are initialised before any peer arrives on them
-  // step ss's inputs (own rows of C_j, s_j, s and coupling of the previous column, own h_j) -> staging
-  // buffer ss & 1 by bulk copies, one step ahead (thread 0)
+  // step ss's inputs -> staging buffer ss & 1 by bulk copies, one step ahead (thread 0)
   auto stage_inputs = [&](int ss) {
-    double* buf = stg + (size_t)(ss & 1) * stg_n;
+    unsigned char* buf = stg + (size_t)(ss & 1) * stage_bytes(Mp);
+    float* bc = reinterpret_cast<float*>(buf + R * sizeof(double));
+    float* bf = bc + (size_t)R * Mp;
     uint64_t* bar = &pbar[ss & 1];
     const int jj = col_of(ss), jp = chain == 0 ? jj - 1 : jj + 1;
-    const unsigned cb = (unsigned)(R * Mp * sizeof(double)), vb = (unsigned)(Mp * sizeof(double));
+    const unsigned cb = (unsigned)(R * Mp * sizeof(float)), vb = (unsigned)(Mp * sizeof(float));
     const unsigned hb = (unsigned)(R * sizeof(double));
     mbar_arrive_expect_tx(bar, cb + hb + vb + (ss > 0 ? 2 * vb : 0));
-    bulk_g2s(buf, p.Coff + ((size_t)jj * Mp + r0) * Mp, cb, bar);
-    bulk_g2s(buf + (size_t)R * Mp + 3 * Mp, p.h + (size_t)jj * Mp + r0, hb, bar);
-    bulk_g2s(buf + (size_t)R * Mp, p.s + (size_t)jj * Mp, vb, bar);
+    bulk_g2s(bc, p.Coff + ((size_t)jj * Mp + r0) * Mp, cb, bar);
+    bulk_g2s(buf, p.h + (size_t)jj * Mp + r0, hb, bar);
+    bulk_g2s(bf, p.s32 + (size_t)jj * Mp, vb, bar);
     if (ss > 0) {
-      bulk_g2s(buf + (size_t)R * Mp + Mp, p.s + (size_t)jp * Mp, vb, bar);
-      bulk_g2s(buf + (size_t)R * Mp + 2 * Mp, p.e + (size_t)min(jj, jp) * Mp, vb, bar);
+      bulk_g2s(bf + Mp, p.s32 + (size_t)jp * Mp, vb, bar);
+      bulk_g2s(bf + 2 * Mp, p.e32 + (size_t)min(jj, jp) * Mp, vb, bar);
     }
   };
   if (tid == 0) stage_inputs(0);
-  const size_t slot = (size_t)R * Mp + R * R;  // floats per panel slot
+  const size_t slot = (size_t)R * Mp;  // floats per panel slot
   __shared__ unsigned failed;                  // a wait of this block expired: stop waiting
   if (tid == 0) failed = 0;
   __syncthreads();
 
+  const int k = tid;            // this thread's column
+  const bool colt = tid < Mp;   // (Mp <= kWork: never the inversion warp)
+  float a[R], x2[kMeet ? R : 1];
+#pragma unroll
+  for (int r = 0; r < R; ++r) a[r] = 0.0f;
   if (kMeet) {  // own rows of both neighbours' inverses
-    const float* XL = p.X + ((size_t)(m - 1) * Mp + r0) * Mp;
-    const float* XR = p.X + ((size_t)(m + 1) * Mp + r0) * Mp;
-    for (int t = tid; t < R * Mp; t += kThreads) {
-      rows[t] = left ? XL[t] : 0.0f;
-      pn[t] = right ? XR[t] : 0.0f;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      a[r] = left && colt ? p.X[((size_t)(m - 1) * Mp + r0 + r) * Mp + k] : 0.0f;
+      x2[r] = right && colt ? p.X[((size_t)(m + 1) * Mp + r0 + r) * Mp + k] : 0.0f;
     }
   }
 
+  float sg_prev = 0.0f;  // sigma of this thread's column, previous column step
   for (int s = 0; s < nsteps; ++s) {
     const int j = col_of(s), jp = chain == 0 ? j - 1 : j + 1;
     const bool has_prev = s > 0;
     // this step's inputs from the staging buffer (the next step's copies overlap this step)
-    const double* stj = stg + (size_t)(s & 1) * stg_n;
-    const double* Cj = stj;                                      // own rows of C_j
-    const double* sj = stj + (size_t)R * Mp;
-    const double* sjm = has_prev ? sj + Mp : nullptr;
-    const double* ejm = has_prev ? sj + 2 * Mp : nullptr;
-    const double* hj = stj + (size_t)R * Mp + 3 * Mp;          // own rows: hj[r] is h_j of row r0 + r
+    const double* hj = reinterpret_cast<const double*>(stg + (size_t)(s & 1) * stage_bytes(Mp));  // h_j of own rows
+    float* Cj = reinterpret_cast<float*>(stg + (size_t)(s & 1) * stage_bytes(Mp) + R * sizeof(double));  // of C_j
+    float* sj = Cj + (size_t)R * Mp;                                                    // s_j
+    float* sp = sj + Mp;                                                                // s of the previous column
+    float* ep = sp + Mp;                                                                // coupling to it
+    if (tid < C && tid != (int)g && !*(volatile unsigned*)&failed) {
+      mbar_arrive_expect_tx(&dbars[tid], R * R * sizeof(float));
+      if (tid > 0) mbar_arrive_expect_tx(&wbars[tid], R * R * sizeof(float));  // panel 0 has none before it
+    }
     if (tid == 0) {
       if (s + 1 < nsteps) stage_inputs(s + 1);
       if (!failed && !mbar_wait_bounded(&pbar[s & 1], (unsigned)((s >> 1) & 1), status, wlim))
         failed = 1;
     }
-    __syncthreads();
-
-    for (int k = tid; k < Mp; k += kThreads) {
-      sv[k] = (float)sj[k];
-      if (!kMeet) {
-        ev[k] = ejm ? (float)ejm[k] : 0.0f;
-      } else {
-        ev[k] = left ? (float)p.e[(size_t)(m - 1) * Mp + k] : 0.0f;
-        ev2[k] = right ? (float)p.e[(size_t)m * Mp + k] : 0.0f;
+    if (kMeet) {  // both neighbours' scales and couplings
+      for (int t = tid; t < Mp; t += kThreads) {
+        sp[t] = left ? p.s32[(size_t)(m - 1) * Mp + t] : 0.0f;
+        ep[t] = left ? p.e32[(size_t)(m - 1) * Mp + t] : 0.0f;
+        s2v[t] = right ? p.s32[(size_t)(m + 1) * Mp + t] : 0.0f;
+        e2v[t] = right ? p.e32[(size_t)m * Mp + t] : 0.0f;
       }
     }
-    // (1) sigma_j of own rows: h_j (+ g_s in column 0) + g_w S X^_prev S sigma_prev  (X^_prev own rows are in
-    // `rows`; the meeting column has two such neighbours, the right one's rows in `pn`)
-    if (has_prev || kMeet) {
-      for (int k = tid; k < Mp; k += kThreads) {
+    __syncthreads();
+
+    // Z^_j of own rows: X^_prev (in the registers) goes to the output and is replaced by the off-diagonal
+    // part; per row the sums of  X^_prev S sigma_prev  and of |Z^_ik| / s_k, for
+    //   sigma_j = h_j (+ g_s in column 0) + g_w S X^_prev S sigma_prev  (from both sides in the meeting column)
+    // and the subtraction-free diagonal
+    const bool use = has_prev || kMeet;
+    if (warp < kInvWarp) {
+      float v[2 * R];
+#pragma unroll
+      for (int r = 0; r < 2 * R; ++r) v[r] = 0.0f;
+      if (colt) {
+        const float sk = sj[k], ek = use ? ep[k] : 0.0f, rsk = 1.0f / sk;
+        float sgk = 0.0f;
         if (!kMeet) {
-          sigv[k] = __ldcg(sig + (size_t)((s - 1) & 1) * Mp + k) * (float)sjm[k];
-        } else {
-          sigv[k] = left ? __ldcg(p.sig + (size_t)((m - 1) & 1) * Mp + k) * (float)p.s[(size_t)(m - 1) * Mp + k] : 0.0f;
-          sigv2[k] = right ? __ldcg(p.sig + (size_t)(2 + ((N - 2 - m) & 1)) * Mp + k) *
-                                 (float)p.s[(size_t)(m + 1) * Mp + k]
-                           : 0.0f;
+          if (has_prev) sgk = sg_prev * sp[k];
+        } else if (left) {
+          sgk = __ldcg(p.sig + (size_t)((m - 1) & 1) * Mp + k) * sp[k];
+        }
+        const float e2k = kMeet ? e2v[k] : 0.0f;
+        float* Xo = p.X + ((size_t)jp * Mp + r0) * Mp + k;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          const int i = r0 + r;
+          if (has_prev) Xo[(size_t)r * Mp] = a[r];
+          v[r] = a[r] * sgk;
+          float z = sj[i] * sk * Cj[(size_t)r * Mp + k];
+          if (use) z -= ep[i] * ek * a[r];
+          if (kMeet) z -= e2v[i] * e2k * x2[r];
+          a[r] = (i < M && k < M && k != i) ? z : 0.0f;
+          v[R + r] = fabsf(a[r]) * rsk;
         }
       }
-      __syncthreads();
-      for (int r = warp; r < R; r += nwarps) {
-        const int i = r0 + r;
-        float acc = 0.0f, acc2 = 0.0f;
-        for (int k = lane; k < Mp; k += 32) {
-          acc = fmaf(rows[(size_t)r * Mp + k], sigv[k], acc);
-          if (kMeet) acc2 = fmaf(pn[(size_t)r * Mp + k], sigv2[k], acc2);
-        }
-        acc = warp_sum_f(acc);
-        if (kMeet) acc2 = warp_sum_f(acc2);
-        if (lane == 0) {
-          float v = 0.0f;
-          if (i < M) {
-            v = (float)(hj[r] + (j == 0 ? p.gsrc : 0.0));
-            if (!kMeet) {
-              v += gw * (float)sjm[i] * acc;
-            } else {
-              if (left) v += gw * (float)p.s[(size_t)(m - 1) * Mp + i] * acc;
-              if (right) v += gw * (float)p.s[(size_t)(m + 1) * Mp + i] * acc2;
-            }
-          }
-          sg[(s & 1) * R + r] = v;
-        }
-      }
-    } else {
-      for (int r = tid; r < R; r += kThreads) {
-        const int i = r0 + r;
-        sg[r] = (i < M) ? (float)(hj[r] + (j == 0 ? p.gsrc : 0.0)) : 0.0f;
+      warp_sums_f<2 * R>(v, lane);
+      red[warp * 32 + lane] = v[0];
+      if (kMeet) {
+        const float sgk = right && colt ? __ldcg(p.sig + (size_t)(2 + ((N - 2 - m) & 1)) * Mp + k) * s2v[k] : 0.0f;
+        float v2[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) v2[r] = x2[r] * sgk;
+        warp_sums_f<R>(v2, lane);
+        if ((lane & 1) == 0) red2[warp * 16 + (lane >> 1)] = v2[0];
       }
     }
     __syncthreads();
-    if (!kMeet)
-      for (int r = tid; r < R; r += kThreads) sig[(size_t)(s & 1) * Mp + r0 + r] = sg[(s & 1) * R + r];
-
-    // (2) + (3) Z^_j own rows (off-diagonal, then the subtraction-free diagonal) in place of
-    // X^_prev, whose own rows go to the output on the way: each element of `rows` is read, stored
-    // to X and overwritten by the same thread, so no thread can overwrite an element of X^_prev
-    // before it has been stored
-    float* Xo = has_prev ? p.X + (size_t)jp * Mp * Mp + (size_t)r0 * Mp : nullptr;
-    for (int t = tid * 2; t < R * Mp; t += kThreads * 2) {
-      const int r = t / Mp, k = t - r * Mp, i = r0 + r;
-      const double2 c2 = *reinterpret_cast<const double2*>(Cj + t);
-      const float si = sv[i], ei = ev[i];
-      const bool use = has_prev || kMeet;
-      const float x0 = use ? rows[t] : 0.0f, x1 = use ? rows[t + 1] : 0.0f;  // X^_prev
-      if (has_prev) *reinterpret_cast<float2*>(Xo + t) = make_float2(x0, x1);
-      float v0 = 0.0f, v1 = 0.0f;
-      if (i < M) {
-        if (k < M && k != i) v0 = si * sv[k] * (float)c2.x - ei * ev[k] * x0;
-        if (k + 1 < M && k + 1 != i) v1 = si * sv[k + 1] * (float)c2.y - ei * ev[k + 1] * x1;
-        if (kMeet) {
-          const float e2 = ev2[i];
-          if (k < M && k != i) v0 -= e2 * ev2[k] * pn[t];
-          if (k + 1 < M && k + 1 != i) v1 -= e2 * ev2[k + 1] * pn[t + 1];
-        }
-      }
-      rows[t] = v0;
-      rows[t + 1] = v1;
-    }
-    __syncthreads();
-    for (int r = warp; r < R; r += nwarps) {
-      const int i = r0 + r;
-      float acc = 0.0f;
-      for (int k = lane; k < M; k += 32) acc += fabsf(rows[(size_t)r * Mp + k]) / sv[k];
-      acc = warp_sum_f(acc);
-      if (lane == 0) {
-        float d = 1.0f;
+    if (tid < 2 * R) {
+      float t = 0.0f;
+#pragma unroll
+      for (int w = 0; w < kInvWarp; ++w) t += red[w * 32 + tid];
+      if (tid < R) {
+        const int i = r0 + tid;
+        float sg = 0.0f;
         if (i < M) {
-          const float si = sv[i];
-          d = si * si * (sg[(s & 1) * R + r] + (kMeet ? 0.0f : gw)) + si * acc;
+          sg = (float)(hj[tid] + (j == 0 ? p.gsrc : 0.0));
+          if (use) sg += gw * sp[i] * t;
+          if (kMeet) {
+            float t2 = 0.0f;
+#pragma unroll
+            for (int w = 0; w < kInvWarp; ++w) t2 += red2[w * 16 + tid];
+            sg += gw * s2v[i] * t2;
+          }
         }
-        rows[(size_t)r * Mp + i] = d;
+        sgs[tid] = sg;
+        if (!kMeet) sig[(size_t)(s & 1) * Mp + i] = sg;
+      } else {
+        abss[tid - R] = t;
       }
     }
     __syncthreads();
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      if (k == r0 + r) {
+        const float si = sj[k];
+        a[r] = k < M ? si * si * (sgs[r] + (kMeet ? 0.0f : gw)) + si * abss[r] : 1.0f;
+      }
+    }
 
     // (4) blocked Gauss-Jordan inversion; panel p = rows of block p.
     // Pivot blocks are inverted in one warp's registers (Gauss-Jordan, no pivoting: the block is
     // symmetric positive definite), two pivots at a time: one reciprocal (of the 2 x 2 determinant) and
-    // one round of shuffles for both, on the chain from panel to panel.  Off-diagonal entries of a part
-    // have one sign, so the products of P^-1 [r0; r1] add without cancellation; the determinant cancels
-    // exactly as the second pivot would.  Lane l holds column l % 16 of rows 8 (l / 16) .. + 7.
+    // one exchange for both, on the chain from panel to panel.  Off-diagonal entries of a part have one
+    // sign, so the products of P^-1 [r0; r1] add without cancellation; the determinant cancels exactly as
+    // the second pivot would.  Lane l holds column l % 16 of rows 8 (l / 16) .. + 7.  The two pivot rows
+    // go through shared memory and stand for the pivot columns too (the swept part is antisymmetric to
+    // the rest): eight loads a step against 22 shuffles, which the one warp issues no faster than
+    // one per eight cycles (2.5k cycles a block; 1.2k this way).
     static_assert(R == 16, "register layout assumes 16 x 16 pivot blocks");
-    const int pb = lane & 15, pa0 = (lane >> 4) * 8;
+    const int ib = lane & 15, pa0 = (lane >> 4) * 8;
     float* slots = p.pbuf + (size_t)chain * C * slot;
-    float* myslot = slots + (size_t)g * slot;  // R_g then D_g^-1
-    auto invert_publish = [&](float (&d)[8]) {  // warp kInvWarp: D^-1 to Dm and to this block's slot
+    float* myslot = slots + (size_t)g * slot;  // R_g
+    // one warp: a 1 KB block of this block's shared memory to the same place in every peer's, the next
+    // owner first
+    auto send_block = [&](const float* blk, uint64_t* mbar) {
+      const uint4 v0 = reinterpret_cast<const uint4*>(blk)[lane], v1 = reinterpret_cast<const uint4*>(blk)[32 + lane];
+      const uint32_t dst = smem_addr(blk) + 16u * lane, bar = smem_addr(mbar);
+      for (int q = 1; q < C; ++q) {
+        int peer = (int)g + q;
+        if (peer >= C) peer -= C;
+        const uint32_t pd = peer_addr32(dst, (uint32_t)peer), pbr = peer_addr32(bar, (uint32_t)peer);
+        st_async16(pd, v0, pbr);
+        st_async16(pd + 512u, v1, pbr);
+      }
+    };
+    auto invert_send = [&]() {  // warp kInvWarp: Bp -> D^-1 in Dm and in every peer's Dall
+      float d[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) d[e] = Bp[(pa0 + e) * R + ib];
+      if (pa0 == 0) {
+        rw[ib] = d[0];
+        rw[R + ib] = d[1];
+      }
 #pragma unroll
       for (int q = 0; q < R; q += 2) {
-        const int qe = q & 7, qlane = (q >> 3) << 4;  // rows q, q+1: elements qe, qe+1 of one half-warp
-        const float p00 = __shfl_sync(0xffffffffu, d[qe], qlane | q), p01 = __shfl_sync(0xffffffffu, d[qe], qlane | (q + 1));
-        const float p10 = __shfl_sync(0xffffffffu, d[qe + 1], qlane | q);
-        const float p11 = __shfl_sync(0xffffffffu, d[qe + 1], qlane | (q + 1));
-        float r0 = __shfl_sync(0xffffffffu, d[qe], qlane | pb), r1 = __shfl_sync(0xffffffffu, d[qe + 1], qlane | pb);
-        float c0[8], c1[8];  // D[a0 + e][q], D[a0 + e][q + 1]
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-          c0[e] = __shfl_sync(0xffffffffu, d[e], (lane & 16) | q);
-          c1[e] = __shfl_sync(0xffffffffu, d[e], (lane & 16) | (q + 1));
-        }
+        const float* rq = rw + (q & 2) * R;  // rows q, q + 1
+        __syncwarp();
+        const float2 pt = *reinterpret_cast<const float2*>(rq + q), pu = *reinterpret_cast<const float2*>(rq + R + q);
+        const float p00 = pt.x, p01 = pt.y, p10 = pu.x, p11 = pu.y;
+        float r0 = rq[ib], r1 = rq[R + ib];
+        float c0[8], c1[8];  // D[a0 + e][q], D[a0 + e][q + 1] from the rows, by symmetry
+        *reinterpret_cast<float4*>(c0) = *reinterpret_cast<const float4*>(rq + pa0);
+        *reinterpret_cast<float4*>(c0 + 4) = *reinterpret_cast<const float4*>(rq + pa0 + 4);
+        *reinterpret_cast<float4*>(c1) = *reinterpret_cast<const float4*>(rq + R + pa0);
+        *reinterpret_cast<float4*>(c1 + 4) = *reinterpret_cast<const float4*>(rq + R + pa0 + 4);
         const float rd = __fdividef(1.0f, fmaf(p00, p11, -p01 * p10));
         // rows q, q+1 become P^-1 [r0; r1] (P^-1 itself in the pivot columns); all other rows lose their
         // pivot-column entries times those
-        const bool in0 = pb == q, in1 = pb == q + 1;
+        const bool in0 = ib == q, in1 = ib == q + 1;
         r0 = in0 ? 1.0f : in1 ? 0.0f : r0;
         r1 = in1 ? 1.0f : in0 ? 0.0f : r1;
         const float f0 = fmaf(p11, r0, -p01 * r1) * rd, f1 = fmaf(p00, r1, -p10 * r0) * rd;
 #pragma unroll
-        for (int e = 0; e < 8; ++e) d[e] = fmaf(-c1[e], f1, fmaf(-c0[e], f0, in0 || in1 ? 0.0f : d[e]));
-        if ((lane & 16) == qlane) {
-          d[qe] = f0;
-          d[qe + 1] = f1;
+        for (int e = 0; e < 8; ++e) {
+          const float sgn = pa0 + e < q ? 1.0f : -1.0f;  // rows already swept: the column is minus the row
+          const float v = fmaf(sgn * c1[e], f1, fmaf(sgn * c0[e], f0, in0 || in1 ? 0.0f : d[e]));
+          d[e] = pa0 + e == q ? f0 : pa0 + e == q + 1 ? f1 : v;
+        }
+        if (q + 2 < R && pa0 == ((q + 2) & 8)) {
+          float* nx = rw + ((q + 2) & 2) * R;
+          nx[ib] = d[(q + 2) & 7];
+          nx[R + ib] = d[(q + 3) & 7];
         }
       }
 #pragma unroll
       for (int e = 0; e < 8; ++e) {
-        Dm[(pa0 + e) * R + pb] = d[e];
-        myslot[(size_t)R * Mp + (pa0 + e) * R + pb] = d[e];
+        Dm[(pa0 + e) * R + ib] = d[e];
+        DmT[ib * R + pa0 + e] = d[e];
       }
+      __syncwarp();
+      send_block(Dm, &dbars[g]);
     };
-    auto signal_peers = [&]() {  // after a __syncthreads that follows every write of the slot
+    auto signal_rows = [&]() {  // after a work_sync that follows every write of the slot
       if (tid < C && tid != (int)g) arrive_peer(peer_addr(&bars[g], (uint32_t)tid));
     };
-    for (int pp = 0; pp < C; ++pp) {
-      const int P0 = pp * R;
-      if ((int)g == pp) {
-        if (pp == 0) {  // later owners published while applying the previous panel
-          if (warp == kInvWarp) {
-            float d[8];
+    const int ar = tid >> 4, bc = tid & 15;  // this thread's element of the 16 x 16 products
+    if (warp == kInvWarp) {
+      __syncthreads();  // Bp is written
+      invert_send();
+      __syncthreads();  // Dm is written
+    } else {
+      // wait on an mbarrier of this column step (one lane per warp; the acquire orders the warp's reads)
+      auto await = [&](uint64_t* bar) {
+        if (lane == 0 && !*(volatile unsigned*)&failed && !wait_cluster_bounded(bar, (unsigned)(s & 1), status))
+          failed = 1;
+        __syncwarp();
+      };
+      auto publish_rows = [&]() {
+        if (colt)
 #pragma unroll
-            for (int e = 0; e < 8; ++e) d[e] = rows[(size_t)(pa0 + e) * Mp + P0 + pb];
-            invert_publish(d);
-          } else {
-            for (int t = tid; t < R * Mp / 4; t += kWork)
-              reinterpret_cast<float4*>(myslot)[t] = reinterpret_cast<const float4*>(rows)[t];
+          for (int r = 0; r < R; ++r) myslot[(size_t)r * Mp + k] = a[r];
+        work_sync();
+        signal_rows();
+      };
+      if ((int)g == 0) {
+        if (colt && k < R)
+#pragma unroll
+          for (int r = 0; r < R; ++r) Bp[r * R + k] = a[r];
+        __syncthreads();  // to the inversion warp
+      }
+      if ((int)g <= 1) publish_rows();
+      float x[R];   // this thread's column of R_pp (and, on entry to a panel, of the panel before)
+      float xn[R];  // its column of the next owner's rows, loaded one panel ahead
+      auto load_rows = [&](int q) {
+        if (q >= C || q == (int)g) return;
+        await(&bars[q]);
+        const float* src = slots + (size_t)q * slot + k;
+        if (colt)
+#pragma unroll
+          for (int u = 0; u < R; ++u) xn[u] = __ldcg(src + (size_t)u * Mp);
+      };
+      load_rows(0);
+      for (int pp = 0; pp < C; ++pp) {
+        const int P0 = pp * R, P1 = P0 + R;
+        const unsigned kp = (unsigned)(k - P0);  // column within the panel
+        const bool kin = colt && kp < (unsigned)R;
+        if ((int)g == pp) {
+          load_rows(pp + 1);
+          __syncthreads();  // the inversion warp has written Dm
+          // own rows become the panel rows: D^-1 R outside the pivot columns, D^-1 inside
+          float acc[R];
+#pragma unroll
+          for (int r = 0; r < R; ++r) acc[r] = 0.0f;
+          rank16_update(acc, DmT, a);
+#pragma unroll
+          for (int r = 0; r < R; ++r) {
+            x[r] = a[r];
+            a[r] = kin ? Dm[r * R + kp] : acc[r];
           }
-          __syncthreads();
-          signal_peers();
+          continue;
         }
-        // own rows become the panel rows: D^-1 R outside the pivot columns, D^-1 inside
-        for (int k = tid; k < Mp && tid < kWork; k += kWork) {
-          float col[R], acc[R];
-          const bool kin = (k >= P0 && k < P0 + R);
+        const bool ahead = (int)g == pp + 1;  // owner of the next panel
+        if (kin)
 #pragma unroll
-          for (int m = 0; m < R; ++m) {
-            col[m] = rows[(size_t)m * Mp + k];
-            acc[m] = 0.0f;
-          }
-          rank16_update(acc, Dm, col, 1.0f);
+          for (int r = 0; r < R; ++r) pa[r * kPitch + kp] = a[r];
+        if (ahead && colt && (unsigned)(k - P1) < (unsigned)R)
 #pragma unroll
-          for (int r = 0; r < R; ++r) rows[(size_t)r * Mp + k] = kin ? Dm[r * R + (k - P0)] : acc[r];
-        }
-        __syncthreads();
-      } else {
-        // wait for panel pp, then read R_pp and D_pp^-1 from its slot (L2)
-        bool ok = true;
-        if (tid == 0 && !failed) {
-          ok = wait_cluster_bounded(&bars[pp], (unsigned)(s & 1), status);
-          if (!ok) failed = 1;
-        }
-        __syncthreads();
-        // D_pp^-1 to shared memory first; R_pp into registers, stored after W' (its latency overlaps W')
-        const float4* src = reinterpret_cast<const float4*>(slots + (size_t)pp * slot);
-        if (tid < R * R / 4) reinterpret_cast<float4*>(Dr)[tid] = __ldcg(src + R * Mp / 4 + tid);
-        constexpr int kPer = (kRows * 16 * kRows / 4 + kWork - 1) / kWork;  // float4 per thread, Mp <= 16 R
-        float4 rp[kPer];
+          for (int r = 0; r < R; ++r) pb[r * kPitch + (k - P1)] = a[r];
+        // R_pp: the owner's rows before panel pp-1 (in xn), then that panel applied
+        if (pp > 0) {
+          await(&wbars[pp]);
+          const float* Wp = Wall + (size_t)pp * R * R;
+          rank16_update(xn, Wp, x);
+          const unsigned km = (unsigned)(k - (P0 - R));
+          if (colt && km < (unsigned)R)  // its pivot columns hold -W'
 #pragma unroll
-        for (int u = 0; u < kPer; ++u) {
-          const int t = tid + u * kWork;
-          if (tid < kWork && t < R * Mp / 4) rp[u] = __ldcg(src + t);
+            for (int u = 0; u < R; ++u) xn[u] = Wp[km * R + u];
         }
-        __syncthreads();
-        if (tid < kWork) {  // W' = own rows[P] D_pp^-1, one element per thread
-          const int a = tid >> 4, bcol = tid & 15;
+#pragma unroll
+        for (int u = 0; u < R; ++u) x[u] = xn[u];
+        if (ahead && colt && (unsigned)(k - P1) < (unsigned)R)
+#pragma unroll
+          for (int u = 0; u < R; ++u) xs[u * kPitch + (k - P1)] = x[u];
+        work_sync();  // pa, pb, xs
+        await(&dbars[pp]);
+        float* Wt = ahead ? Wall + (size_t)g * R * R : W;
+        {  // -W' = -own rows[P] D_pp^-1, one element per thread, stored transposed
+          const float* Dp = Dall + (size_t)pp * R * R;
           float w = 0.0f;
 #pragma unroll
-          for (int m = 0; m < R; ++m) w = fmaf(rows[(size_t)a * Mp + P0 + m], Dr[m * R + bcol], w);
-          W[tid] = w;
-#pragma unroll
-          for (int u = 0; u < kPer; ++u) {
-            const int t = tid + u * kWork;
-            if (t < R * Mp / 4) reinterpret_cast<float4*>(pn)[t] = rp[u];
-          }
+          for (int u = 0; u < R; ++u) w = fmaf(pa[ar * kPitch + u], Dp[u * R + bc], w);
+          Wt[bc * R + ar] = -w;
         }
-        __syncthreads();
-        const bool ahead = (int)g == pp + 1;  // owner of the next panel
-        const int P1 = P0 + R;
+        work_sync();
         if (ahead) {  // its pivot block after this panel, same operation order as the update below
-          if (tid < kWork) {
-            const int a = tid >> 4, bcol = tid & 15;
-            float v = rows[(size_t)a * Mp + P1 + bcol];
+          float v = pb[ar * kPitch + bc];
 #pragma unroll
-            for (int m = 0; m < R; ++m) v = fmaf(-1.0f * W[a * R + m], pn[(size_t)m * Mp + P1 + bcol], v);
-            Bp[tid] = v;
-          }
-          __syncthreads();
+          for (int u = 0; u < R; ++u) v = fmaf(Wt[u * R + ar], xs[u * kPitch + bc], v);
+          Bp[tid] = v;
+          __syncthreads();  // to the inversion warp
+          if (warp == kInvWarp - 1) send_block(Wt, &wbars[g]);
         }
-        if (ahead && warp == kInvWarp) {
-          float d[8];
+        load_rows(pp + 1);  // in flight during the update
+        //   row <- row - W' R_pp outside the pivot columns, -W' inside
+        rank16_update(a, Wt, x);
+        if (kin)  // R_pp holds D there, not D^-1
 #pragma unroll
-          for (int e = 0; e < 8; ++e) d[e] = Bp[(pa0 + e) * R + pb];
-          invert_publish(d);
-        } else {
-          //   row <- row - W' R_pp outside the pivot columns, -W' inside; the next owner also
-          //   publishes its updated rows as R_{pp+1}
-          for (int k = tid; k < Mp && tid < kWork; k += kWork) {
-            float col[R], acc[R];
-            const bool kin = (k >= P0 && k < P0 + R);  // R_pp holds D there, not D^-1: the result is -W'
-#pragma unroll
-            for (int m = 0; m < R; ++m) {
-              col[m] = pn[(size_t)m * Mp + k];
-              acc[m] = rows[(size_t)m * Mp + k];
-            }
-            rank16_update(acc, W, col, -1.0f);
-#pragma unroll
-            for (int r = 0; r < R; ++r) {
-              if (kin) acc[r] = -W[r * R + (k - P0)];
-              rows[(size_t)r * Mp + k] = acc[r];
-            }
-            if (ahead)
-#pragma unroll
-              for (int r = 0; r < R; ++r) myslot[(size_t)r * Mp + k] = acc[r];
-          }
-        }
-        __syncthreads();
-        if (ahead) signal_peers();
+          for (int r = 0; r < R; ++r) a[r] = Wt[kp * R + r];
+        if ((int)g == pp + 2) publish_rows();
       }
     }
+    // every block has published its sigma before its rows, which this one has waited for
+    if (!kMeet && colt) sg_prev = __ldcg(sig + (size_t)(s & 1) * Mp + k);
     cluster_sync();  // every read of this step's slots is done before the next step rewrites them
   }
   {
-    float* Xo = p.X + (size_t)col_of(nsteps - 1) * Mp * Mp + (size_t)r0 * Mp;
-    for (int t = tid; t < R * Mp; t += kThreads) Xo[t] = rows[t];
+    float* Xo = p.X + ((size_t)col_of(nsteps - 1) * Mp + r0) * Mp + k;
+    if (colt)
+#pragma unroll
+      for (int r = 0; r < R; ++r) Xo[(size_t)r * Mp] = a[r];
   }
-  cluster_sync();  // no block leaves while another may still read its shared memory
+  // No block leaves while a peer's store may still arrive in its shared memory: a block that has waited
+  // for everything has received everything; after a wait that ran out, a pause on either side of the
+  // barrier lets land what nobody waits for.
+  auto pause = [&]() {
+    if (!*(volatile unsigned*)&failed) return;
+    const uint64_t t0 = globaltimer_ns();
+    while (globaltimer_ns() - t0 < 200000) __nanosleep(1000);
+  };
+  pause();
+  cluster_sync();
+  pause();
 }
 
 bool factor_cluster_supported(int Mp) { return Mp >= 2 * kRows && Mp <= 16 * kRows && Mp % kRows == 0; }
@@ -509,7 +603,7 @@ cudaError_t launch_factor_cluster(const FactorParams* params_dev, int Mp, int N,
                                   cudaStream_t st) {
   if (meet < 0 || meet >= N) return cudaErrorInvalidValue;
   const int C = factor_cluster_size(Mp);
-  const size_t smem = factor_cluster_smem_bytes(Mp, kRows);
+  const size_t smem = factor_cluster_smem_bytes(Mp);
   const bool left = meet > 0, right = meet < N - 1;
   if (left || right) {
     const cudaError_t err = launch_clusters<false>(params_dev, C, (left ? 1 : 0) + (right ? 1 : 0), left ? 0 : 1, smem,

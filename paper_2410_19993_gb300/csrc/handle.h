@@ -105,7 +105,9 @@ struct xbar_s {
   double R[4] = {0, 0, 0, 0};
   cudaStream_t st = nullptr;
   int dev = 0, nsm = 0;
-  int assembled = 0;  // per-column elimination data formed from Gc (lazily, by the first factor)
+  // per-column elimination data formed from Gc (lazily, by the first factor): 0 = no, else with the
+  // column blocks in the precision p of the factors, assembled_for(p)
+  int assembled = 0;
   int factored = 0;
   xbar_precision prec = XBAR_FP64;
   xbar::DevArena A;
@@ -178,6 +180,8 @@ struct PhaseScope {
 
 // error reporting shared by the C entry points
 xbar_status set_error(xbar_status s, const char* fmt, ...);
+
+inline int assembled_for(xbar_precision p) { return p == XBAR_FP64 ? 1 : 2; }
 
 // kernel-variant selection (environment XBAR_SWEEP=simt|tc, XBAR_FACTOR=group|cluster override)
 bool use_tc_sweep(const xbar_s* h);

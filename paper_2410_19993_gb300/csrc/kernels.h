@@ -23,7 +23,8 @@ struct MapDev {
   double* thc = nullptr;    // [N][Mp]  and back sweep u_i = phi_i + thc_i u_{i+1}
   double* tdiag = nullptr;  // [N][Mp]  diagonal of the inverse bit-line chain matrix
   double* rho = nullptr;    // [N][Mp]  ratio of consecutive inverse entries along a row
-  double* Coff = nullptr;   // [N][Mp][Mp] off-diagonal of the column block after bit-line elimination
+  void* Coff = nullptr;     // [N][Mp][Mp] off-diagonal of the column block after bit-line elimination (FP64
+                            // or FP32, as the factor in use reads it)
   double* s_eq = nullptr;   // [N][Mp]  diagonal equilibration scale (dW^-1/2)
   double* e_eq = nullptr;   // [N][Mp]  coupling of column j to j+1, equilibrated
   double* e_pl = nullptr;   // [N][Mp]  coupling, plain (g_w)
@@ -46,13 +47,14 @@ struct MapDev {
 // Gc <- G (transposed to [N][Mp]); the rest of the assembly reads Gc only.  status != NULL: check
 // G on the device (XBAR_DEV_BADINPUT for a negative or non-finite entry)
 cudaError_t launch_store_g(const MapDev& m, const double* G_dev, unsigned* status, cudaStream_t st);
-cudaError_t launch_assemble(const MapDev& m, cudaStream_t st);
+// f32: the column blocks Coff as FP32 (for FP32 factors) instead of FP64
+cudaError_t launch_assemble(const MapDev& m, bool f32, cudaStream_t st);
 
 // ---- factor -----------------------------------------------------------------------------------
 struct FactorParams {  // FP32 factors
   int M, Mp, N;
   double gsrc, gw;
-  const double* Coff;
+  const float* Coff;
   const double* h;
   const double* s;    // nullptr = no equilibration
   const double* e;
@@ -61,6 +63,8 @@ struct FactorParams {  // FP32 factors
   float* pbuf;        // scratch: [2][PB][Mp] (factor.cu), factor_cluster_pbuf_floats (factor_cluster.cu)
   unsigned* bar;      // 2 words, zeroed
   int meet;           // factor_cluster.cu: column in which its two elimination chains meet
+  const float* s32;   // factor_cluster.cu: s and e in FP32
+  const float* e32;
 };
 
 // FP32 factor (factor.cu): one group of `blocks_per_map` co-resident blocks factors each map; `maps`
