@@ -38,17 +38,21 @@ namespace xbar {
 
 namespace {
 
-constexpr int kWork = 256;             // threads of the row work: one per pivot-block element / column
+constexpr int kWork = 128;             // threads of the row work: two columns and two pivot-block elements each
 constexpr int kInvWarp = kWork / 32;   // one more warp inverts pivot blocks meanwhile
 constexpr int kThreads = kWork + 32;
 constexpr int kRows = 16;
-static_assert(kWork == kRows * kRows, "one thread per element of a pivot block");
+static_assert(2 * kWork == kRows * kRows, "two elements of a pivot block per thread");
 
 __device__ __forceinline__ uint32_t cluster_rank() {
   uint32_t r;
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
   return r;
 }
+__device__ __forceinline__ void cluster_arrive_relaxed() {
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
@@ -74,7 +78,7 @@ __device__ __forceinline__ void st_async16(uint32_t addr, uint4 v, uint32_t bar)
       "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "r"(bar)
       : "memory");
 }
-__device__ __forceinline__ void work_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }  // the row-work warps
+__device__ __forceinline__ void work_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }  // the row-work warps
 // bounded wait for phase `parity` of a local mbarrier, acquire at cluster scope
 __device__ __forceinline__ bool wait_cluster_bounded(uint64_t* bar, unsigned parity, unsigned* status) {
   auto done = [&]() {
@@ -125,12 +129,12 @@ __device__ __forceinline__ void warp_sums_f(float (&v)[NS], int lane) {
 // panel being applied, Bp [R][R] next pivot block, DmT [R][R] transpose of this block's inverse, Dall
 // [16][R][R] inverse pivot blocks by panel (own and received), Wall [16][R][R] the owners' -W'^T by panel, rw
 // [2][2][R] the inversion's pivot rows, pa, pb, xs [R][R+1] own rows in the columns of this panel and of the
-// next, R_p in those of the next, reductions [8][32] and [8][16], row sums [2][R], scale and coupling of the
+// next, R_p in those of the next, reductions [4][32] and [4][16], row sums [2][R], scale and coupling of the
 // right neighbour (meeting column) [2][Mp]; then two staging buffers of a column step's inputs: h_j own
 // rows [R] in FP64, C_j own rows [R][Mp], s_j, s of the previous column and the coupling to it [Mp] each
 constexpr int kPitch = kRows + 1;
 constexpr int kBars = 50;
-constexpr int kSmFloats = 3 * kRows * kPitch + (3 + 32) * kRows * kRows + 4 * kRows + 8 * 32 + 8 * 16 + 2 * kRows;
+constexpr int kSmFloats = 3 * kRows * kPitch + (3 + 32) * kRows * kRows + 4 * kRows + 4 * 32 + 4 * 16 + 2 * kRows;
 static_assert(kSmFloats % 4 == 0, "16-byte aligned vectors after the fixed part");
 __host__ __device__ constexpr size_t stage_bytes(int Mp) {
   return kRows * sizeof(double) + ((size_t)kRows * Mp + 3 * (size_t)Mp) * sizeof(float);
@@ -145,23 +149,27 @@ size_t factor_cluster_pbuf_floats(int Mp) {
   return 2 * C * (size_t)kRows * Mp;
 }
 
-// acc[r] += sum_m coefT[m*16 + r] * x[m] (r, m < 16): two rows per packed multiply-add, coefficients read as
-// 16-byte broadcasts
+// acc[c][r] += sum_m coefT[m*16 + r] * x[c][m] (r, m < 16, two columns c): two rows per packed multiply-add,
+// coefficients read as 16-byte broadcasts
 __device__ __forceinline__ void fma2(float& a0, float& a1, float w0, float w1, float x) {
   asm("{\n\t.reg .b64 A, W, X;\n\tmov.b64 A, {%0, %1};\n\tmov.b64 W, {%2, %3};\n\tmov.b64 X, {%4, %4};\n\t"
       "fma.rn.f32x2 A, W, X, A;\n\tmov.b64 {%0, %1}, A;\n\t}"
       : "+f"(a0), "+f"(a1)
       : "f"(w0), "f"(w1), "f"(x));
 }
-__device__ __forceinline__ void rank16_update(float (&acc)[16], const float* __restrict__ coefT, const float (&x)[16]) {
+__device__ __forceinline__ void rank16_update(float (&acc)[2][16], const float* __restrict__ coefT,
+                                              const float (&x)[2][16]) {
 #pragma unroll
   for (int m = 0; m < 16; ++m) {
     const float4* c4 = reinterpret_cast<const float4*>(coefT + m * 16);
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      const float4 c = c4[q];
-      fma2(acc[4 * q], acc[4 * q + 1], c.x, c.y, x[m]);
-      fma2(acc[4 * q + 2], acc[4 * q + 3], c.z, c.w, x[m]);
+      const float4 w = c4[q];
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        fma2(acc[c][4 * q], acc[c][4 * q + 1], w.x, w.y, x[c][m]);
+        fma2(acc[c][4 * q + 2], acc[c][4 * q + 3], w.z, w.w, x[c][m]);
+      }
     }
   }
 }
@@ -199,8 +207,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   float* xs = pb + R * kPitch;
   float* red = xs + R * kPitch;
   float* Dm = Dall + (size_t)g * R * R;  // this block's own
-  float* red2 = red + 8 * 32;
-  float* sgs = red2 + 8 * 16;
+  float* red2 = red + 4 * 32;
+  float* sgs = red2 + 4 * 16;
   float* abss = sgs + R;
   float* s2v = abss + R;
   float* e2v = s2v + Mp;
@@ -246,20 +254,26 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (tid == 0) failed = 0;
   __syncthreads();
 
-  const int k = tid;            // this thread's column
-  const bool colt = tid < Mp;   // (Mp <= kWork: never the inversion warp)
-  float a[R], x2[kMeet ? R : 1];
+  // Two neighbouring columns per thread: the coefficients of an update reach every lane through shared
+  // memory's 128 bytes a cycle (a 16-byte broadcast fills 512), which bounds it, and serve both.
+  const bool colt = tid < Mp / 2;  // threads with columns
+  const int kc[2] = {2 * tid, 2 * tid + 1};
+  float a[2][R], x2[2][kMeet ? R : 1];
 #pragma unroll
-  for (int r = 0; r < R; ++r) a[r] = 0.0f;
+  for (int c = 0; c < 2; ++c)
+#pragma unroll
+    for (int r = 0; r < R; ++r) a[c][r] = 0.0f;
   if (kMeet) {  // own rows of both neighbours' inverses
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-      a[r] = left && colt ? p.X[((size_t)(m - 1) * Mp + r0 + r) * Mp + k] : 0.0f;
-      x2[r] = right && colt ? p.X[((size_t)(m + 1) * Mp + r0 + r) * Mp + k] : 0.0f;
-    }
+    for (int c = 0; c < 2; ++c)
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        a[c][r] = left && colt ? p.X[((size_t)(m - 1) * Mp + r0 + r) * Mp + kc[c]] : 0.0f;
+        x2[c][r] = right && colt ? p.X[((size_t)(m + 1) * Mp + r0 + r) * Mp + kc[c]] : 0.0f;
+      }
   }
 
-  float sg_prev = 0.0f;  // sigma of this thread's column, previous column step
+  float sg_prev[2] = {0.0f, 0.0f};  // sigma of this thread's columns, previous column step
   for (int s = 0; s < nsteps; ++s) {
     const int j = col_of(s), jp = chain == 0 ? j - 1 : j + 1;
     const bool has_prev = s > 0;
@@ -274,7 +288,6 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (tid > 0) mbar_arrive_expect_tx(&wbars[tid], R * R * sizeof(float));  // panel 0 has none before it
     }
     if (tid == 0) {
-      if (s + 1 < nsteps) stage_inputs(s + 1);
       if (!failed && !mbar_wait_bounded(&pbar[s & 1], (unsigned)((s >> 1) & 1), status, wlim))
         failed = 1;
     }
@@ -293,39 +306,61 @@ __global__ void __launch_bounds__(kThreads, 1)
     //   sigma_j = h_j (+ g_s in column 0) + g_w S X^_prev S sigma_prev  (from both sides in the meeting column)
     // and the subtraction-free diagonal
     const bool use = has_prev || kMeet;
+    // (the buffer's last readers passed this step's first barrier)
+    if (tid == 32 * kInvWarp && s + 1 < nsteps) stage_inputs(s + 1);
     if (warp < kInvWarp) {
-      float v[2 * R];
+      float v[2 * R], v2[kMeet ? R : 1];
 #pragma unroll
       for (int r = 0; r < 2 * R; ++r) v[r] = 0.0f;
+      if (kMeet)
+#pragma unroll
+        for (int r = 0; r < R; ++r) v2[r] = 0.0f;
       if (colt) {
-        const float sk = sj[k], ek = use ? ep[k] : 0.0f, rsk = 1.0f / sk;
-        float sgk = 0.0f;
-        if (!kMeet) {
-          if (has_prev) sgk = sg_prev * sp[k];
-        } else if (left) {
-          sgk = __ldcg(p.sig + (size_t)((m - 1) & 1) * Mp + k) * sp[k];
+        const int k = kc[0];  // and k + 1
+        const float2 sk = *reinterpret_cast<const float2*>(sj + k);
+        float2 ek = make_float2(0.0f, 0.0f), spk = ek, sg2 = ek, e2k = ek;
+        if (use) {
+          ek = *reinterpret_cast<const float2*>(ep + k);
+          spk = *reinterpret_cast<const float2*>(sp + k);
         }
-        const float e2k = kMeet ? e2v[k] : 0.0f;
+        if (kMeet) {
+          sg_prev[0] = left ? __ldcg(p.sig + (size_t)((m - 1) & 1) * Mp + k) : 0.0f;
+          sg_prev[1] = left ? __ldcg(p.sig + (size_t)((m - 1) & 1) * Mp + k + 1) : 0.0f;
+          const float* sr = p.sig + (size_t)(2 + ((N - 2 - m) & 1)) * Mp + k;
+          sg2 = right ? make_float2(__ldcg(sr) * s2v[k], __ldcg(sr + 1) * s2v[k + 1]) : sg2;
+          e2k = *reinterpret_cast<const float2*>(e2v + k);
+        }
+        const float g0 = sg_prev[0] * spk.x, g1 = sg_prev[1] * spk.y;
+        const float rs0 = 1.0f / sk.x, rs1 = 1.0f / sk.y;
         float* Xo = p.X + ((size_t)jp * Mp + r0) * Mp + k;
 #pragma unroll
         for (int r = 0; r < R; ++r) {
           const int i = r0 + r;
-          if (has_prev) Xo[(size_t)r * Mp] = a[r];
-          v[r] = a[r] * sgk;
-          float z = sj[i] * sk * Cj[(size_t)r * Mp + k];
-          if (use) z -= ep[i] * ek * a[r];
-          if (kMeet) z -= e2v[i] * e2k * x2[r];
-          a[r] = (i < M && k < M && k != i) ? z : 0.0f;
-          v[R + r] = fabsf(a[r]) * rsk;
+          const float x0 = a[0][r], x1 = a[1][r];
+          if (has_prev) *reinterpret_cast<float2*>(Xo + (size_t)r * Mp) = make_float2(x0, x1);
+          v[r] = fmaf(x1, g1, x0 * g0);
+          const float2 c2 = *reinterpret_cast<const float2*>(Cj + (size_t)r * Mp + k);
+          const float si = sj[i];
+          float z0 = si * sk.x * c2.x, z1 = si * sk.y * c2.y;
+          if (use) {
+            const float ei = ep[i];
+            z0 -= ei * ek.x * x0;
+            z1 -= ei * ek.y * x1;
+          }
+          if (kMeet) {
+            const float e2 = e2v[i];
+            z0 -= e2 * e2k.x * x2[0][r];
+            z1 -= e2 * e2k.y * x2[1][r];
+            v2[r] = fmaf(x2[1][r], sg2.y, x2[0][r] * sg2.x);
+          }
+          a[0][r] = (i < M && k < M && k != i) ? z0 : 0.0f;
+          a[1][r] = (i < M && k + 1 < M && k + 1 != i) ? z1 : 0.0f;
+          v[R + r] = fmaf(fabsf(a[1][r]), rs1, fabsf(a[0][r]) * rs0);
         }
       }
       warp_sums_f<2 * R>(v, lane);
       red[warp * 32 + lane] = v[0];
-      if (kMeet) {
-        const float sgk = right && colt ? __ldcg(p.sig + (size_t)(2 + ((N - 2 - m) & 1)) * Mp + k) * s2v[k] : 0.0f;
-        float v2[R];
-#pragma unroll
-        for (int r = 0; r < R; ++r) v2[r] = x2[r] * sgk;
+      if constexpr (kMeet) {
         warp_sums_f<R>(v2, lane);
         if ((lane & 1) == 0) red2[warp * 16 + (lane >> 1)] = v2[0];
       }
@@ -355,13 +390,17 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
     }
     __syncthreads();
+    if (colt)
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-      if (k == r0 + r) {
-        const float si = sj[k];
-        a[r] = k < M ? si * si * (sgs[r] + (kMeet ? 0.0f : gw)) + si * abss[r] : 1.0f;
-      }
-    }
+      for (int c = 0; c < 2; ++c)
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+          if (kc[c] == r0 + r) {
+            const float si = sj[kc[c]];
+            a[c][r] = kc[c] < M ? si * si * (sgs[r] + (kMeet ? 0.0f : gw)) + si * abss[r] : 1.0f;
+          }
+
+    if (has_prev) cluster_wait();  // the previous step's arrivals
 
     // (4) blocked Gauss-Jordan inversion; panel p = rows of block p.
     // Pivot blocks are inverted in one warp's registers (Gauss-Jordan, no pivoting: the block is
@@ -439,7 +478,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     auto signal_rows = [&]() {  // after a work_sync that follows every write of the slot
       if (tid < C && tid != (int)g) arrive_peer(peer_addr(&bars[g], (uint32_t)tid));
     };
-    const int ar = tid >> 4, bc = tid & 15;  // this thread's element of the 16 x 16 products
+    const int ar = tid >> 4, bc = tid & 15;  // this thread's elements of the 16 x 16 products: rows ar, ar + 8
     if (warp == kInvWarp) {
       __syncthreads();  // Bp is written
       invert_send();
@@ -454,107 +493,145 @@ __global__ void __launch_bounds__(kThreads, 1)
       auto publish_rows = [&]() {
         if (colt)
 #pragma unroll
-          for (int r = 0; r < R; ++r) myslot[(size_t)r * Mp + k] = a[r];
+          for (int r = 0; r < R; ++r)
+            *reinterpret_cast<float2*>(myslot + (size_t)r * Mp + kc[0]) = make_float2(a[0][r], a[1][r]);
         work_sync();
         signal_rows();
       };
-      if ((int)g == 0) {
-        if (colt && k < R)
+      // this thread's entries of `v` in the columns [c0, c0 + R) to dst (row pitch dp)
+      auto put_cols = [&](float* dst, int dp, const float (&v)[2][R], int c0) {
+        if (colt)
 #pragma unroll
-          for (int r = 0; r < R; ++r) Bp[r * R + k] = a[r];
+          for (int c = 0; c < 2; ++c) {
+            const unsigned kk = (unsigned)(kc[c] - c0);
+            if (kk < (unsigned)R)
+#pragma unroll
+              for (int r = 0; r < R; ++r) dst[r * dp + kk] = v[c][r];
+          }
+      };
+      // the pivot columns [c0, c0 + R) of v become wt's rows (wt[kk][r])
+      auto set_cols = [&](float (&v)[2][R], const float* wt, int c0) {
+        if (colt)
+#pragma unroll
+          for (int c = 0; c < 2; ++c) {
+            const unsigned kk = (unsigned)(kc[c] - c0);
+            if (kk < (unsigned)R)
+#pragma unroll
+              for (int r = 0; r < R; ++r) v[c][r] = wt[kk * R + r];
+          }
+      };
+      if ((int)g == 0) {
+        put_cols(Bp, R, a, 0);
         __syncthreads();  // to the inversion warp
       }
       if ((int)g <= 1) publish_rows();
-      float x[R];   // this thread's column of R_pp (and, on entry to a panel, of the panel before)
-      float xn[R];  // its column of the next owner's rows, loaded one panel ahead
+      float x[2][R];   // this thread's columns of R_pp (and, on entry to a panel, of the panel before)
+      float xn[2][R];  // its columns of the next owner's rows, loaded one panel ahead
       auto load_rows = [&](int q) {
         if (q >= C || q == (int)g) return;
         await(&bars[q]);
-        const float* src = slots + (size_t)q * slot + k;
+        const float* src = slots + (size_t)q * slot + kc[0];
         if (colt)
 #pragma unroll
-          for (int u = 0; u < R; ++u) xn[u] = __ldcg(src + (size_t)u * Mp);
+          for (int u = 0; u < R; ++u) {
+            const float2 t = __ldcg(reinterpret_cast<const float2*>(src + (size_t)u * Mp));
+            xn[0][u] = t.x;
+            xn[1][u] = t.y;
+          }
       };
       load_rows(0);
       for (int pp = 0; pp < C; ++pp) {
         const int P0 = pp * R, P1 = P0 + R;
-        const unsigned kp = (unsigned)(k - P0);  // column within the panel
-        const bool kin = colt && kp < (unsigned)R;
         if ((int)g == pp) {
           load_rows(pp + 1);
           __syncthreads();  // the inversion warp has written Dm
           // own rows become the panel rows: D^-1 R outside the pivot columns, D^-1 inside
-          float acc[R];
+          if (colt) {
+            float acc[2][R];
 #pragma unroll
-          for (int r = 0; r < R; ++r) acc[r] = 0.0f;
-          rank16_update(acc, DmT, a);
+            for (int c = 0; c < 2; ++c)
 #pragma unroll
-          for (int r = 0; r < R; ++r) {
-            x[r] = a[r];
-            a[r] = kin ? Dm[r * R + kp] : acc[r];
+              for (int r = 0; r < R; ++r) acc[c][r] = 0.0f;
+            rank16_update(acc, DmT, a);
+#pragma unroll
+            for (int c = 0; c < 2; ++c)
+#pragma unroll
+              for (int r = 0; r < R; ++r) {
+                x[c][r] = a[c][r];
+                a[c][r] = acc[c][r];
+              }
           }
+          set_cols(a, DmT, P0);  // (DmT[kk][r] = D^-1[r][kk])
           continue;
         }
         const bool ahead = (int)g == pp + 1;  // owner of the next panel
-        if (kin)
-#pragma unroll
-          for (int r = 0; r < R; ++r) pa[r * kPitch + kp] = a[r];
-        if (ahead && colt && (unsigned)(k - P1) < (unsigned)R)
-#pragma unroll
-          for (int r = 0; r < R; ++r) pb[r * kPitch + (k - P1)] = a[r];
+        put_cols(pa, kPitch, a, P0);
+        if (ahead) put_cols(pb, kPitch, a, P1);
         // R_pp: the owner's rows before panel pp-1 (in xn), then that panel applied
         if (pp > 0) {
           await(&wbars[pp]);
           const float* Wp = Wall + (size_t)pp * R * R;
-          rank16_update(xn, Wp, x);
-          const unsigned km = (unsigned)(k - (P0 - R));
-          if (colt && km < (unsigned)R)  // its pivot columns hold -W'
-#pragma unroll
-            for (int u = 0; u < R; ++u) xn[u] = Wp[km * R + u];
+          if (colt) rank16_update(xn, Wp, x);
+          set_cols(xn, Wp, P0 - R);  // its pivot columns hold -W'
         }
 #pragma unroll
-        for (int u = 0; u < R; ++u) x[u] = xn[u];
-        if (ahead && colt && (unsigned)(k - P1) < (unsigned)R)
+        for (int c = 0; c < 2; ++c)
 #pragma unroll
-          for (int u = 0; u < R; ++u) xs[u * kPitch + (k - P1)] = x[u];
+          for (int u = 0; u < R; ++u) x[c][u] = xn[c][u];
+        if (ahead) put_cols(xs, kPitch, x, P1);
         work_sync();  // pa, pb, xs
         await(&dbars[pp]);
         float* Wt = ahead ? Wall + (size_t)g * R * R : W;
-        {  // -W' = -own rows[P] D_pp^-1, one element per thread, stored transposed
+        {  // -W' = -own rows[P] D_pp^-1, two elements per thread, stored transposed
           const float* Dp = Dall + (size_t)pp * R * R;
-          float w = 0.0f;
+          float w0 = 0.0f, w1 = 0.0f;
 #pragma unroll
-          for (int u = 0; u < R; ++u) w = fmaf(pa[ar * kPitch + u], Dp[u * R + bc], w);
-          Wt[bc * R + ar] = -w;
+          for (int u = 0; u < R; ++u) {
+            const float d = Dp[u * R + bc];
+            w0 = fmaf(pa[ar * kPitch + u], d, w0);
+            w1 = fmaf(pa[(ar + 8) * kPitch + u], d, w1);
+          }
+          Wt[bc * R + ar] = -w0;
+          Wt[bc * R + ar + 8] = -w1;
         }
         work_sync();
         if (ahead) {  // its pivot block after this panel, same operation order as the update below
-          float v = pb[ar * kPitch + bc];
+          float v0 = pb[ar * kPitch + bc], v1 = pb[(ar + 8) * kPitch + bc];
 #pragma unroll
-          for (int u = 0; u < R; ++u) v = fmaf(Wt[u * R + ar], xs[u * kPitch + bc], v);
-          Bp[tid] = v;
+          for (int u = 0; u < R; ++u) {
+            const float d = xs[u * kPitch + bc];
+            v0 = fmaf(Wt[u * R + ar], d, v0);
+            v1 = fmaf(Wt[u * R + ar + 8], d, v1);
+          }
+          Bp[ar * R + bc] = v0;
+          Bp[(ar + 8) * R + bc] = v1;
           __syncthreads();  // to the inversion warp
           if (warp == kInvWarp - 1) send_block(Wt, &wbars[g]);
         }
         load_rows(pp + 1);  // in flight during the update
         //   row <- row - W' R_pp outside the pivot columns, -W' inside
-        rank16_update(a, Wt, x);
-        if (kin)  // R_pp holds D there, not D^-1
-#pragma unroll
-          for (int r = 0; r < R; ++r) a[r] = Wt[kp * R + r];
+        if (colt) rank16_update(a, Wt, x);
+        set_cols(a, Wt, P0);  // R_pp holds D there, not D^-1
         if ((int)g == pp + 2) publish_rows();
       }
     }
     // every block has published its sigma before its rows, which this one has waited for
-    if (!kMeet && colt) sg_prev = __ldcg(sig + (size_t)(s & 1) * Mp + k);
-    cluster_sync();  // every read of this step's slots is done before the next step rewrites them
+    if (!kMeet && colt)
+#pragma unroll
+      for (int c = 0; c < 2; ++c) sg_prev[c] = __ldcg(sig + (size_t)(s & 1) * Mp + kc[c]);
+    // every block's reads of this step's slots and blocks are done (their values are used) before the next
+    // step's first hand-over: arrive here, wait there, with the next column's formation in between; nothing
+    // this block wrote is published by it, so the arrival need not wait for its stores
+    cluster_arrive_relaxed();
   }
   {
-    float* Xo = p.X + ((size_t)col_of(nsteps - 1) * Mp + r0) * Mp + k;
     if (colt)
 #pragma unroll
-      for (int r = 0; r < R; ++r) Xo[(size_t)r * Mp] = a[r];
+      for (int r = 0; r < R; ++r)
+        *reinterpret_cast<float2*>(p.X + ((size_t)col_of(nsteps - 1) * Mp + r0 + r) * Mp + kc[0]) =
+            make_float2(a[0][r], a[1][r]);
   }
+  cluster_wait();
   // No block leaves while a peer's store may still arrive in its shared memory: a block that has waited
   // for everything has received everything; after a wait that ran out, a pause on either side of the
   // barrier lets land what nobody waits for.
