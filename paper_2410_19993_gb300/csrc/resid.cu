@@ -360,7 +360,187 @@ __global__ void blvolt_kernel(ResidParams p, double* u_out) {
   }
 }
 
+// ---- few chains: several threads per bit line ------------------------------------------------------
+// With few vectors the kernels above are a thread per chain walking M rows of dependent steps and memory
+// latencies (0.45 us a row: 120 us for one vector of 256 x 256 as for 50).  Here a chain is cut into S row
+// segments, a thread each: every step of the chain is an affine map phi -> thc_i phi + tha_i w_i with
+// non-negative coefficients, so a segment is one too; its factor prod thc and its value from zero go
+// through shared memory, each thread folds the segments before its own (at most 31 short steps) and
+// walks its rows from the true entry value.  The back substitution u_i = phi_i + thc_i u_{i+1} has the same
+// factors.  A block holds NB vectors of one column (NB = 1 .. 32, consecutive lanes) and 256 / NB
+// segments, at most 32.
+constexpr int kFewThreads = 256, kFewSegs = 32;
+// chains (vectors x columns) up to which these run: beyond, the card is full of chains and the extra passes
+// (about 1.6x the operations) cost more than the latency they hide
+constexpr long long kFewChains = 32768;
+
+struct FewShape {
+  int nb, segs;  // vectors and segments per block
+};
+static FewShape few_shape(int Bpad) {
+  FewShape f;
+  f.nb = 1;
+  while (f.nb < 32 && f.nb < Bpad) f.nb *= 2;
+  f.segs = std::min(kFewSegs, kFewThreads / f.nb);
+  return f;
+}
+static bool few_chains(const ResidParams& p) { return (long long)p.Bpad * p.N <= kFewChains; }
+
+__device__ __forceinline__ fp2 as_fp2(float2 v) { return {v.x, v.y}; }
+
+template <bool kW1>
+__global__ void __launch_bounds__(kFewThreads) resid_few_kernel(ResidParams p, int nb, int segs) {
+  if (p.skip && *p.skip) return;
+  __shared__ float2 sA[kFewThreads], sB[kFewThreads];  // [segs][nb], factor and value
+  const int tid = threadIdx.x, lb = tid % nb, seg = tid / nb, at = seg * nb + lb;
+  const int b = blockIdx.x * nb + lb, j = blockIdx.y, M = p.M;
+  const int L = (M + segs - 1) / segs, i0 = min(seg * L, M), i1 = min(i0 + L, M);
+  const bool live = b < p.Bpad;
+  const size_t base = (size_t)j * p.Mp, rs = p.Bpad, o0 = base * rs + (live ? b : 0);
+  const StateCol<kW1> W{kW1 ? p.w1 + o0 : nullptr, kW1 ? nullptr : p.w2 + o0, rs};
+  float2* ph2 = p.phi2 + o0;
+  // g_o V / d_last enters the chain's last row when the sources are on the bit lines
+  fp2 src{0.0f, 0.0f};
+  if (p.Vbl && b < p.B && i1 == M && i0 < M) {
+    const float2 c = p.thc2[base + M - 1];
+    src = pmul(split(p.go * ((double)c.x + (double)c.y) / p.gb), split(p.Vbl[(size_t)b * p.N + (p.N - 1 - j)]));
+  }
+  auto fwd = [&](int i, fp2 f) {
+    f = phi_step(p.thc2[base + i], p.tha2[base + i], f, W.at(i));
+    return p.Vbl && i == M - 1 ? padd(f, src) : f;
+  };
+  fp2 A{1.0f, 0.0f}, f{0.0f, 0.0f};
+  if (live)
+#pragma unroll 4
+    for (int i = i0; i < i1; ++i) {
+      f = fwd(i, f);
+      A = pmul_u(A, as_fp2(p.thc2[base + i]));
+    }
+  sA[at] = make_float2(A.hi, A.lo);
+  sB[at] = make_float2(f.hi, f.lo);
+  __syncthreads();
+  f = fp2{0.0f, 0.0f};
+  for (int q = 0; q < seg; ++q) f = padd_u(pmul_u(as_fp2(sA[q * nb + lb]), f), as_fp2(sB[q * nb + lb]));
+  __syncthreads();
+  fp2 u{0.0f, 0.0f};
+  if (live) {
+#pragma unroll 4
+    for (int i = i0; i < i1; ++i) {
+      f = fwd(i, f);
+      st2(ph2, (size_t)i * rs, f);
+    }
+#pragma unroll 4
+    for (int i = i1 - 1; i >= i0; --i) u = padd_u(ld2(ph2, (size_t)i * rs), pmul_u(as_fp2(p.thc2[base + i]), u));
+  }
+  sB[at] = make_float2(u.hi, u.lo);
+  __syncthreads();
+  u = fp2{0.0f, 0.0f};
+  for (int q = segs - 1; q > seg; --q) u = padd_u(pmul_u(as_fp2(sA[q * nb + lb]), u), as_fp2(sB[q * nb + lb]));
+  if (!live) return;
+  const bool has_l = j > 0, has_r = j + 1 < p.N;
+  const long col = (long)p.Mp * (long)rs;
+  const fp2 gw = split(p.gw), gs = split(p.gs);
+  float* rh = p.rhat + o0;
+  float rmax = 0.0f;
+#pragma unroll 4
+  for (int i = i1 - 1; i >= i0; --i) {
+    const fp2 w = W.at(i);
+    u = padd_u(ld2(ph2, (size_t)i * rs), pmul_u(as_fp2(p.thc2[base + i]), u));
+    fp2 e{0.0f, 0.0f};
+    if (has_l && has_r) e = pmul_u(gw, pdiff2_u(W.at(i, -col), W.at(i, col), w));
+    else if (has_l) e = pmul_u(gw, psub_u(W.at(i, -col), w));
+    else if (has_r) e = pmul_u(gw, psub_u(W.at(i, col), w));
+    if (j == 0 && b < p.B) e = padd(e, pmul(gs, psub(p.Vbl ? fp2{0.0f, 0.0f} : split(p.V[(size_t)b * p.M + i]), w)));
+    const float rf = psum_f(pmul_u(as_fp2(p.Gc2[base + i]), psub_u(u, w)), e);
+    rmax = fmaxf(rmax, fabsf(rf));
+    rh[(size_t)i * rs] = rf * p.s32[base + i];
+  }
+  if (i1 == M && i0 < M)  // the last segment with rows also clears the padding rows
+    for (int i = M; i < p.Mp; ++i) rh[(size_t)i * rs] = 0.0f;
+  if (!(rmax <= 3.0e38f)) set_status(p.status, XBAR_DEV_NONFINITE);
+  const unsigned on = __activemask();
+  rmax = __uint_as_float(__reduce_max_sync(on, __float_as_uint(rmax)));
+  if ((tid & 31) == __ffs(on) - 1 && p.rmax) atomicMax(p.rmax, (unsigned long long)__double_as_longlong((double)rmax));
+}
+
+__global__ void __launch_bounds__(kFewThreads) update_few_kernel(ResidParams p, int first, int nb, int segs) {
+  if (p.skip && *p.skip) return;
+  __shared__ float2 sI[kFewThreads];
+  const int tid = threadIdx.x, lb = tid % nb, seg = tid / nb;
+  const int b = blockIdx.x * nb + lb, j = blockIdx.y, M = p.M;
+  const int L = (M + segs - 1) / segs, i0 = min(seg * L, M), i1 = min(i0 + L, M);
+  const bool live = b < p.Bpad;
+  const size_t base = (size_t)j * p.Mp, rs = p.Bpad, o0 = base * rs + (live ? b : 0);
+  fp2 I{0.0f, 0.0f};
+  if (live)
+#pragma unroll 8
+    for (int i = i0; i < i1; ++i) {
+      const size_t o = o0 + (size_t)i * rs;
+      const float dd = p.s32[base + i] * p.dhat[o];
+      const fp2 wn = first ? fp2{dd, 0.0f} : padd(ldw_any(p, o), fp2{dd, 0.0f});
+      st2(p.w2, o, wn);
+      I = padd(I, pmul(as_fp2(p.h2[base + i]), wn));
+    }
+  sI[seg * nb + lb] = make_float2(I.hi, I.lo);
+  __syncthreads();
+  if (seg == 0 && b < p.B) {
+    for (int q = 1; q < segs; ++q) I = padd(I, as_fp2(sI[q * nb + lb]));
+    p.I[(size_t)b * p.N + j] = (double)I.hi + (double)I.lo;
+  }
+}
+
+// the same cut of the bit-line chains in FP64 (node-voltage output): u = T^-1 (G o w)
+__global__ void __launch_bounds__(kFewThreads) blvolt_few_kernel(ResidParams p, double* __restrict__ u_out, int nb, int segs) {
+  __shared__ double sA[kFewThreads], sB[kFewThreads];
+  const int tid = threadIdx.x, lb = tid % nb, seg = tid / nb, at = seg * nb + lb;
+  const int b = blockIdx.x * nb + lb, j = blockIdx.y, M = p.M;
+  const int L = (M + segs - 1) / segs, i0 = min(seg * L, M), i1 = min(i0 + L, M);
+  const bool live = b < p.Bpad;
+  const size_t base = (size_t)j * p.Mp, rs = p.Bpad, o0 = base * rs + (live ? b : 0);
+  const double* w = p.w + o0;
+  double* uo = u_out + o0;
+  const double *tha = p.tha + base, *thc = p.thc + base;
+  double A = 1.0, f = 0.0;
+  if (live)
+#pragma unroll 8
+    for (int i = i0; i < i1; ++i) {
+      f = fma(thc[i], f, tha[i] * w[(size_t)i * rs]);
+      A *= thc[i];
+    }
+  sA[at] = A;
+  sB[at] = f;
+  __syncthreads();
+  f = 0.0;
+  for (int q = 0; q < seg; ++q) f = fma(sA[q * nb + lb], f, sB[q * nb + lb]);
+  __syncthreads();
+  double u = 0.0;
+  if (live) {
+#pragma unroll 8
+    for (int i = i0; i < i1; ++i) {
+      f = fma(thc[i], f, tha[i] * w[(size_t)i * rs]);
+      uo[(size_t)i * rs] = f;
+    }
+#pragma unroll 8
+    for (int i = i1 - 1; i >= i0; --i) u = fma(thc[i], u, uo[(size_t)i * rs]);
+  }
+  sB[at] = u;
+  __syncthreads();
+  if (!live) return;
+  u = 0.0;
+  for (int q = segs - 1; q > seg; --q) u = fma(sA[q * nb + lb], u, sB[q * nb + lb]);
+#pragma unroll 8
+  for (int i = i1 - 1; i >= i0; --i) {
+    u = fma(thc[i], u, uo[(size_t)i * rs]);
+    uo[(size_t)i * rs] = u;
+  }
+}
+
 cudaError_t launch_update(const ResidParams& p, int first, cudaStream_t st) {
+  if (few_chains(p)) {
+    const FewShape f = few_shape(p.Bpad);
+    update_few_kernel<<<dim3((p.Bpad + f.nb - 1) / f.nb, p.N), f.nb * f.segs, 0, st>>>(p, first, f.nb, f.segs);
+    return cudaGetLastError();
+  }
   dim3 grid((p.Bpad + 127) / 128, p.N);
   update_kernel<<<grid, 128, 0, st>>>(p, first);
   return cudaGetLastError();
@@ -375,6 +555,13 @@ cudaError_t launch_pair_to_double(const ResidParams& p, cudaStream_t st) {
 
 cudaError_t launch_resid(const ResidParams& p, cudaStream_t st) {
   dim3 grid((p.Bpad + 127) / 128, p.N);
+  if (few_chains(p)) {
+    const FewShape f = few_shape(p.Bpad);
+    const dim3 fg((p.Bpad + f.nb - 1) / f.nb, p.N);
+    if (p.w1) resid_few_kernel<true><<<fg, f.nb * f.segs, 0, st>>>(p, f.nb, f.segs);
+    else resid_few_kernel<false><<<fg, f.nb * f.segs, 0, st>>>(p, f.nb, f.segs);
+    return cudaGetLastError();
+  }
   const size_t smem = (size_t)p.M * 28;  // M <= 1024: within the default 48 KB
   if (p.w1) resid_kernel<true><<<grid, 128, smem, st>>>(p);
   else resid_kernel<false><<<grid, 128, smem, st>>>(p);
@@ -382,6 +569,11 @@ cudaError_t launch_resid(const ResidParams& p, cudaStream_t st) {
 }
 
 cudaError_t launch_blvolt(const ResidParams& p, double* u, cudaStream_t st) {
+  if (few_chains(p)) {
+    const FewShape f = few_shape(p.Bpad);
+    blvolt_few_kernel<<<dim3((p.Bpad + f.nb - 1) / f.nb, p.N), f.nb * f.segs, 0, st>>>(p, u, f.nb, f.segs);
+    return cudaGetLastError();
+  }
   dim3 grid((p.Bpad + 127) / 128, p.N);
   blvolt_kernel<<<grid, 128, 0, st>>>(p, u);
   return cudaGetLastError();
