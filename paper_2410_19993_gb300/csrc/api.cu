@@ -229,9 +229,12 @@ struct SweepKind {
   FewPlan few;
   bool tc = false;
   int Bp = 0;  // vectors per panel
+  int nsm = 0;
+  bool beside = false;  // other solves run beside this one
 };
 static SweepKind sweep_kind(const xbar_s* h, int B, bool mixed) {
   SweepKind k;
+  k.nsm = h->nsm;
   const char* e = getenv("XBAR_SWEEP");
   const bool chosen = mixed && (h->opt.sweep >= 0 || (e && (strcmp(e, "simt") == 0 || strcmp(e, "tc") == 0)));
   if (!chosen) k.few = sweep_few_plan(h->m.Mp, B, h->nsm);
@@ -246,7 +249,7 @@ template <typename T>
 static cudaError_t run_sweep(const SweepParams<T>& sp, const SweepKind& k, const void* Xt, int terms, cudaStream_t st) {
   if (k.few.nv) return launch_sweep_few<T>(sp, k.few, st);
   if constexpr (sizeof(T) == 4) {
-    if (k.tc) return launch_sweep_tc(sp, Xt, terms, st);
+    if (k.tc) return launch_sweep_tc(sp, Xt, terms, k.nsm, k.beside, st);
   }
   return launch_sweep<T>(sp, st);
 }
@@ -499,7 +502,7 @@ static xbar_status solve_rows_mixed(xbar_s* h, int B, const double* dV, double* 
   sp.max_rel = nullptr;
   sp.status = g->status;
   auto sweep32 = [&](int terms) -> cudaError_t {  // dhat = solve32(rhat) (rhat is overwritten by cyclic reduction)
-    if (tc) return launch_sweep_tc(sp, g->Xt.p, terms, st);
+    if (tc) return launch_sweep_tc(sp, g->Xt.p, terms, g->nsm, false, st);
     if (!cr) return launch_sweep<float>(sp, st);
     CrSweepArgs<float> ca;
     memset(&ca, 0, sizeof(ca));
@@ -1068,7 +1071,7 @@ extern "C" xbar_status xbar_solve(xbar_t h, int B, const double* V, double* I, d
 }
 
 xbar_status xbar::solve_device_driven(xbar_s* h, int B, const double* dV, double* dI, double tol, int max_iter,
-                                      bool allow_alloc) {
+                                      bool allow_alloc, bool beside) {
   MapDev& m = h->m;
   const int M = m.M, Mp = m.Mp, N = m.N;
   cudaStream_t st = h->st;
@@ -1084,7 +1087,8 @@ xbar_status xbar::solve_device_driven(xbar_s* h, int B, const double* dV, double
   if (h->cr_active)
     return fail(XBAR_ESTATE, "device-driven solves (tile batches) need a block-Thomas factorization");
   const bool mixed = h->prec == XBAR_FP32_IR;
-  const SweepKind kind = sweep_kind(h, B, mixed);
+  SweepKind kind = sweep_kind(h, B, mixed);
+  kind.beside = beside;
   const int Bp = kind.Bp;
   const int Bpad = ((B + Bp - 1) / Bp) * Bp;
   const size_t nst = (size_t)N * Mp * Bpad;

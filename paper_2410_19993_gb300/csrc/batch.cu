@@ -131,7 +131,7 @@ static xbar_status enqueue_all(xbar_batch_t b, xbar_precision p, const int* B, c
     xbar_status s = factor_handle(h, p, eager);
     if (s != XBAR_OK) return s;
     if (B[t] > 0) {
-      s = solve_device_driven(h, B[t], V[t], I[t], tol, max_iter, eager);
+      s = solve_device_driven(h, B[t], V[t], I[t], tol, max_iter, eager, b->T > 1);
       if (s != XBAR_OK) return s;
     }
     XB_CUDA(cudaEventRecord(b->joins[t], b->streams[t]));
@@ -339,7 +339,7 @@ extern "C" xbar_status xbar_batch_autotune(xbar_batch_t b, xbar_precision p, con
         h->opt.sweep = sw;
         if (sw == 1 && !use_tc_sweep(h)) continue;
         if (factor_handle(h, p, true) != XBAR_OK) continue;
-        v.sweep_ms[sw] = time_ms(h->st, [&]() { return solve_device_driven(h, k.B, dV, dI, 1e-8, 2, true); });
+        v.sweep_ms[sw] = time_ms(h->st, [&]() { return solve_device_driven(h, k.B, dV, dI, 1e-8, 2, true, b->T > 1); });
       }
       v.sweep = (v.sweep_ms[1] >= 0 && (v.sweep_ms[0] < 0 || v.sweep_ms[1] <= v.sweep_ms[0])) ? 1 : 0;
       h->opt.factor = save_f;
@@ -361,7 +361,7 @@ extern "C" xbar_status xbar_batch_autotune(xbar_batch_t b, xbar_precision p, con
         h->opt.orient = o;
         v.orient_ms[o] = time_ms(h->st, [&]() {
           xbar_status s = factor_handle(h, p, true);
-          return s != XBAR_OK ? s : solve_device_driven(h, k.B, dV, dI, 1e-8, 0, true);
+          return s != XBAR_OK ? s : solve_device_driven(h, k.B, dV, dI, 1e-8, 0, true, b->T > 1);
         });
       }
       v.orient = (v.orient_ms[1] >= 0 && (v.orient_ms[0] < 0 || v.orient_ms[1] < v.orient_ms[0])) ? 1 : 0;

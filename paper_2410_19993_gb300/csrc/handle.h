@@ -199,7 +199,8 @@ xbar_status factor_handle(xbar_s* h, xbar_precision p, bool upload_params);
 // currents-only solve with device pointers, refinement driven on the device: exactly
 // `max_iter` refinement passes are enqueued and passes after convergence skip their work; no
 // host synchronisation (capturable).  The workspace must have been sized by an earlier call.
+// beside: other tiles' solves run beside this one.
 xbar_status solve_device_driven(xbar_s* h, int B, const double* V, double* I, double tol, int max_iter,
-                                bool allow_alloc);
+                                bool allow_alloc, bool beside);
 
 }  // namespace xbar

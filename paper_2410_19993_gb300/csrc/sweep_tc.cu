@@ -167,21 +167,30 @@ __device__ __forceinline__ bool epi_sync_or(bool v) {
 // stages (2 to 8) as the shared memory beside the KP-term vector operand holds.  (Five stages of two
 // chunks for a two-term 256-row step ran no faster than two of four: the ring is not what limits
 // the K loop.)
-__host__ __device__ constexpr int tc_sub(int Mt, int KP) { return (Mt == 256 && KP == 3) ? 2 : 4; }
+// Two blocks on an SM (`two`, 128-row blocks and KP = 2): stages of one chunk, as many as half an SM holds.
+__host__ __device__ constexpr int tc_sub(int Mt, int KP, bool two) { return two ? 1 : (Mt == 256 && KP == 3) ? 2 : 4; }
 __host__ __device__ constexpr uint32_t tc_slot(int Mt, int KP) { return (uint32_t)KP * tc::kKC * Mt * 2; }
 __host__ __device__ constexpr int tc_vbytes(int Mt, int KP) { return KP * (tc::kBP / 8) * (int)tc::lbo_b(Mt); }
-// 32 floats per epilogue thread: with 256-row blocks, the second 32-column block of the next step's
-// z or right-hand side, copied in ahead of the accumulator wait; in every sweep, the staging of the
-// w tiles (4 KB per warp) between those copies
-__host__ __device__ constexpr int tc_prebytes(int Mt) { return tc::kThreads * 32 * 4; }
-__host__ __device__ constexpr int tc_fixed(int Mt, int KP) { return 2304 + tc_vbytes(Mt, KP) + tc_prebytes(Mt); }
-__host__ __device__ constexpr int tc_stages(int Mt, int KP) {
-  return (232448 - tc_fixed(Mt, KP)) / (int)(tc_sub(Mt, KP) * tc_slot(Mt, KP)) > 8
-             ? 8
-             : (232448 - tc_fixed(Mt, KP)) / (int)(tc_sub(Mt, KP) * tc_slot(Mt, KP));
+// Beside the vector operand: with 256-row blocks, 32 floats per epilogue thread for the second
+// 32-column block of the next step's z or right-hand side, copied in ahead of the accumulator wait;
+// in every sweep, the staging of the w tiles (4 KB per warp) between those copies.  With two blocks on
+// an SM the inward launch, which has no w, takes none: L1 then holds the lines its right-hand side
+// loads come back to.
+__host__ __device__ constexpr int tc_prebytes(bool two, bool out) {
+  return two && !out ? 0 : tc::kThreads * 32 * 4;
 }
-static_assert(tc_stages(256, 2) == 2 && tc_stages(256, 3) == 2 &&
-                  tc_stages(128, 2) == 5 && tc_stages(128, 3) == 3,
+__host__ __device__ constexpr int tc_fixed(int Mt, int KP, bool two, bool out) {
+  return 2304 + tc_vbytes(Mt, KP) + tc_prebytes(two, out);
+}
+// shared memory of a block: 227 KB, or half of the SM's 228 KB less the 1 KB each block reserves
+__host__ __device__ constexpr int tc_budget(bool two) { return two ? 115712 : 232448; }
+__host__ __device__ constexpr int tc_stages(int Mt, int KP, bool two, bool out) {
+  const int fit = (tc_budget(two) - tc_fixed(Mt, KP, two, out)) / (int)(tc_sub(Mt, KP, two) * tc_slot(Mt, KP));
+  return fit > (two ? 5 : 8) ? (two ? 5 : 8) : fit;
+}
+static_assert(tc_stages(256, 2, false, true) == 2 && tc_stages(256, 3, false, true) == 2 &&
+                  tc_stages(128, 2, false, true) == 5 && tc_stages(128, 3, false, true) == 3 &&
+                  tc_stages(128, 2, true, true) == 5 && tc_stages(128, 2, true, false) == 5,
               "stage rings");
 
 // NH = number of 128-row halves of X_j (Mt = 128 NH); KP = number of BF16 terms of the split used
@@ -190,13 +199,14 @@ static_assert(tc_stages(256, 2) == 2 && tc_stages(256, 3) == 2 &&
 // thread then spends no dependent integer work per MMA (runtime offsets in that loop tripled its
 // cost per MMA).
 // Chain of a block: blockIdx.y + chain0.  kOut: the meeting column and the outward part.
-template <int NH, int KP, bool kOut>
-__global__ void __launch_bounds__(tc::kThreads + 64, 1)
+template <int NH, int KP, bool kOut, bool kTwo>
+__global__ void __launch_bounds__(tc::kThreads + 64, kTwo ? 2 : 1)
     sweep_tc_kernel(SweepParams<float> p, const __nv_bfloat16* __restrict__ Xt, int chain0) {
   using namespace tc;
   constexpr int BP = kBP, KC = kKC;
   constexpr int Mt = 128 * NH, nh = NH;
-  constexpr int NS = tc_stages(Mt, KP), kSub = tc_sub(Mt, KP);
+  constexpr int NS = tc_stages(Mt, KP, kTwo, kOut), kSub = tc_sub(Mt, KP, kTwo);
+  static_assert(!kTwo || (NH == 1 && KP == 2), "two blocks on an SM");
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int b0 = blockIdx.x * BP;
   const uint64_t wlim = wait_limit(p.status);  // read once: the waits below sit on critical paths
@@ -638,9 +648,8 @@ __global__ void __launch_bounds__(tc::kThreads + 64, 1)
   if (warp == 1) tmem_dealloc(tbase, ncols);
 }
 
-size_t sweep_tc_smem_bytes(int Mt, int KP) {
-  return 256 + 8 * 64 * 4 + (size_t)tc_stages(Mt, KP) * tc_sub(Mt, KP) * tc_slot(Mt, KP) + tc_vbytes(Mt, KP) +
-         tc_prebytes(Mt);
+static size_t sweep_tc_smem_bytes(int Mt, int KP, bool two, bool out) {
+  return (size_t)tc_fixed(Mt, KP, two, out) + (size_t)tc_stages(Mt, KP, two, out) * tc_sub(Mt, KP, two) * tc_slot(Mt, KP);
 }
 
 bool sweep_tc_supported(int Mp) { return Mp <= 256; }
@@ -660,34 +669,41 @@ cudaError_t launch_sweep_tc_tile(const float* X, void* Xt, int Mp, int N, cudaSt
   return cudaGetLastError();
 }
 
-cudaError_t launch_sweep_tc(const SweepParams<float>& p, const void* Xt, int terms, cudaStream_t st) {
+cudaError_t launch_sweep_tc(const SweepParams<float>& p, const void* Xt, int terms, int nsm, bool beside,
+                            cudaStream_t st) {
   const int Mt = sweep_tc_rows(p.Mp);
   if (p.Bp != tc::kBP || p.Bpad % tc::kBP) return cudaErrorInvalidValue;
   const int blocks = (p.B + tc::kBP - 1) / tc::kBP;
   if (blocks == 0) return cudaSuccess;
   if (terms < 2 || terms > tc::kParts) return cudaErrorInvalidValue;
-  const size_t smem = sweep_tc_smem_bytes(Mt, terms);
   if (p.meet < 0 || p.meet >= p.N || (!p.V && !p.rhs)) return cudaErrorInvalidValue;
   using Kern = void (*)(SweepParams<float>, const __nv_bfloat16*, int);
-  const Kern kerns[2][2][2] = {{{sweep_tc_kernel<1, 2, false>, sweep_tc_kernel<1, 2, true>},
-                                {sweep_tc_kernel<1, 3, false>, sweep_tc_kernel<1, 3, true>}},
-                               {{sweep_tc_kernel<2, 2, false>, sweep_tc_kernel<2, 2, true>},
-                                {sweep_tc_kernel<2, 3, false>, sweep_tc_kernel<2, 3, true>}}};
-  const Kern* kern = kerns[Mt == 128 ? 0 : 1][terms - 2];
-  for (int k = 0; k < 2; ++k) {
-    const cudaError_t err = cudaFuncSetAttribute(kern[k], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const Kern kerns[2][2][2] = {{{sweep_tc_kernel<1, 2, false, false>, sweep_tc_kernel<1, 2, true, false>},
+                                {sweep_tc_kernel<1, 3, false, false>, sweep_tc_kernel<1, 3, true, false>}},
+                               {{sweep_tc_kernel<2, 2, false, false>, sweep_tc_kernel<2, 2, true, false>},
+                                {sweep_tc_kernel<2, 3, false, false>, sweep_tc_kernel<2, 3, true, false>}}};
+  const Kern pair[2] = {sweep_tc_kernel<1, 2, false, true>, sweep_tc_kernel<1, 2, true, true>};
+  auto launch = [&](bool out, int chains, int chain0) {
+    // Two blocks on an SM where there is work for both: more blocks than SMs, or other tiles' solves
+    // beside this one; then one block's epilogue overlaps the other's products (a step of a 128-row
+    // block is mostly epilogue latency).  128 x 128 in mixed precision, 16384 vectors: 7.94 -> 7.14 ms,
+    // 8192: 4.75 -> 4.35 ms; 30 tiles with 4096 vectors each: 47.3 -> 44.1 ms.  A block alone runs slower at
+    // half an SM's registers and a third of its stages: 1000 vectors 2.62 against 2.72 ms.
+    const bool two = Mt == 128 && terms == 2 && (beside || blocks * chains > nsm);
+    const Kern kern = two ? pair[out] : kerns[Mt / 128 - 1][terms - 2][out];
+    const size_t smem = sweep_tc_smem_bytes(Mt, terms, two, out);
+    const cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (err != cudaSuccess) return err;
-  }
-  const __nv_bfloat16* X = static_cast<const __nv_bfloat16*>(Xt);
+    kern<<<dim3(blocks, chains), tc::kThreads + 64, smem, st>>>(p, static_cast<const __nv_bfloat16*>(Xt), chain0);
+    return cudaGetLastError();
+  };
   const bool left = p.meet > 0, right = p.meet < p.N - 1;
   const bool right_in = right && p.rhs;  // an input vector enters at column 0 only
   if (left || right_in) {
-    kern[0]<<<dim3(blocks, left && right_in ? 2 : 1), tc::kThreads + 64, smem, st>>>(p, X, left ? 0 : 1);
-    const cudaError_t err = cudaGetLastError();
+    const cudaError_t err = launch(false, left && right_in ? 2 : 1, left ? 0 : 1);
     if (err != cudaSuccess) return err;
   }
-  kern[1]<<<dim3(blocks, right ? 2 : 1), tc::kThreads + 64, smem, st>>>(p, X, 0);
-  return cudaGetLastError();
+  return launch(true, right ? 2 : 1, 0);
 }
 
 }  // namespace xbar

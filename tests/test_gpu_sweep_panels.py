@@ -1,0 +1,47 @@
+"""Tensor-core substitutions of large batches: two blocks on an SM (blocks of up to 128 rows) with grids
+of more than one round, panels that are not full, one and two elimination chains, and tiles that share
+the device."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2410_19993_gb300 import xbar
+from tests.gpu_common import case, rel_err
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+R = (1.0, 2.5, 2.5, 10.0)
+
+
+# 1e-8 is the suite's bar for refined currents; node voltages follow the same certificate
+@pytest.mark.parametrize("M,N,B", [(33, 2, 4930), (100, 5, 4865), (128, 3, 9800), (128, 1, 9729)])
+def test_large_batches(M, N, B):
+    G, V = case(M, N, B, None, seed=M + N)
+    rows = np.unique(np.concatenate([np.arange(0, B, 97), np.arange(B - 70, B)]))
+    ref = oracle.solve(M, N, G, *R, V[rows], voltages=True)
+    xb = xbar.Crossbar.assemble(torch.from_numpy(G).cuda(), *R)
+    xb.set_option("orientation", "columns").set_option("algorithm", "thomas")
+    xb.factor("fp32_ir")
+    I = torch.zeros((B, N), dtype=torch.float64, device="cuda")
+    vW = torch.zeros((B, M, N), dtype=torch.float64, device="cuda")
+    vB = torch.zeros_like(vW)
+    xb.solve(torch.from_numpy(V).cuda(), I, vWL=vW, vBL=vB, tol=1e-9)
+    assert rel_err(I.cpu().numpy()[rows], ref["I"]) <= 1e-8
+    assert rel_err(vW.cpu().numpy()[rows], ref["vWL"]) <= 1e-8
+    assert rel_err(vB.cpu().numpy()[rows], ref["vBL"]) <= 1e-8
+    xb.destroy()
+
+
+def test_tiles_side_by_side():
+    shapes = [(128, 4, 200), (100, 3, 65), (40, 2, 64), (129, 2, 130)]
+    tiles = [case(M, N, B, None, seed=M) for M, N, B in shapes]
+    b = xbar.Batch([(torch.from_numpy(G).cuda(), *R) for G, _ in tiles])
+    Vs = [torch.from_numpy(V).cuda() for _, V in tiles]
+    Is = [torch.zeros((B, N), dtype=torch.float64, device="cuda") for _, N, B in shapes]
+    for _ in range(2):  # the first run also captures
+        for I in Is:
+            I.zero_()
+        b.run("fp32_ir", Vs, Is, tol=1e-9, max_iter=6)
+        for (M, N, B), (G, V), I in zip(shapes, tiles, Is):
+            assert rel_err(I.cpu().numpy(), oracle.solve(M, N, G, *R, V)["I"]) <= 1e-8
