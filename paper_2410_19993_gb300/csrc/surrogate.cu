@@ -859,6 +859,8 @@ struct xbar_surrogate_s {
   double gs = 1e-4, vs = 0.5;
   int dev = 0, nsm = 1;
   cudaStream_t st = nullptr;
+  cudaStream_t side = nullptr;                 // prediction: the first layer beside the line model
+  cudaEvent_t forked = nullptr, joined = nullptr;
   unsigned* status = nullptr;
   DevArena A;
   // flat FP32 parameters: W1 [kH][Fp], b1 [kH], W2 [kH][kH], b2 [kH], W3 [2][kH], b3 [2]
@@ -914,7 +916,11 @@ extern "C" xbar_status xbar_surrogate_destroy(xbar_surrogate_t s) {
   if (!s) return XBAR_OK;
   cudaSetDevice(s->dev);
   cudaStreamSynchronize(s->st);
+  if (s->side) cudaStreamSynchronize(s->side);
   s->A.free_all();
+  if (s->forked) cudaEventDestroy(s->forked);
+  if (s->joined) cudaEventDestroy(s->joined);
+  if (s->side) cudaStreamDestroy(s->side);
   delete s;
   return XBAR_OK;
 }
@@ -954,6 +960,10 @@ extern "C" xbar_status xbar_surrogate_create(int M, int N, double R_s, double R_
     xbar_surrogate_destroy(s);
     return e;
   };
+  if (cudaStreamCreateWithFlags(&s->side, cudaStreamNonBlocking) != cudaSuccess ||
+      cudaEventCreateWithFlags(&s->forked, cudaEventDisableTiming) != cudaSuccess ||
+      cudaEventCreateWithFlags(&s->joined, cudaEventDisableTiming) != cudaSuccess)
+    return bail(set_error(XBAR_ECUDA, "stream/event creation"));
   if (s->A.alloc((void**)&s->P, s->np * 4) || s->A.alloc((void**)&s->Gr, s->np * 4) ||
       s->A.alloc((void**)&s->Am, s->np * 4) || s->A.alloc((void**)&s->Av, s->np * 4) ||
       s->A.alloc((void**)&s->W1b, (size_t)kH * s->Fp * 2) || s->A.alloc((void**)&s->W2b, (size_t)kH * kH * 2) ||
@@ -1106,8 +1116,10 @@ extern "C" xbar_status xbar_surrogate_grad(xbar_surrogate_t s, int R, const floa
   return st;
 }
 
-// line model and feature columns of one map (G(i, j) = G[i*sGi + j*sGj], device): Gt, St, Tl
-static xbar_status map_prep(xbar_surrogate_t s, const double* G, long sGi, long sGj) {
+// line model and feature columns of one map (G(i, j) = G[i*sGi + j*sGj], device): Gt, St, Tl.
+// columns_ready: recorded once Gt and St are queued, before the line model proper
+static xbar_status map_prep(xbar_surrogate_t s, const double* G, long sGi, long sGj,
+                            cudaEvent_t columns_ready = nullptr) {
   const int M = s->M, N = s->N;
   const size_t mn = (size_t)M * N;
   XB_CUDA(ensure(s->A, s->Gt, mn * 8));
@@ -1137,6 +1149,7 @@ static xbar_status map_prep(xbar_surrogate_t s, const double* G, long sGi, long 
   prep_rows_kernel<<<(M + rb - 1) / rb, rb * kSegL, smr, s->st>>>(G, sGi, sGj, M, N, gs, gw, 1.0 / (N * s->gs), (double*)s->Gt.p,
                                                     (float*)s->St.p, (float*)s->Gf.p, (float*)s->wl.p,
                                                     (float*)s->tau.p);
+  if (columns_ready) XB_CUDA(cudaEventRecord(columns_ready, s->st));
   prep_cols_kernel<<<(N + cb - 1) / cb, cb * kSegL, smc, s->st>>>(Gf, M, N, gb, go, (float*)s->bl.p, (float*)s->xg.p);
   const size_t smem = 3 * (size_t)N * (M + 1) * 4;
   if (smem <= kLineSmemMax) {  // one block per unit input, everything in shared memory
@@ -1294,8 +1307,6 @@ static xbar_status predict_map(xbar_surrogate_t s, const double* G, long sGi, lo
   const int M = s->M, N = s->N, Fp = s->Fp;
   const long rows = (long)B * N;
   const long Npad = round_up_l(N, 128), Bpad = round_up_l(B, 128);
-  xbar_status st = map_prep(s, G, sGi, sGj);
-  if (st != XBAR_OK) return st;
   XB_CUDA(ensure(s->A, s->Iid, (size_t)rows * 8));
   XB_CUDA(ensure(s->A, s->Iln, (size_t)rows * 8));
   XB_CUDA(ensure(s->A, s->xgs, (size_t)Npad * Fp * 2));
@@ -1304,17 +1315,15 @@ static xbar_status predict_map(xbar_surrogate_t s, const double* G, long sGi, lo
   XB_CUDA(ensure(s->A, s->Qm, (size_t)Bpad * kH * 4));
   XB_CUDA(ensure(s->A, s->g32, (size_t)M * N * 4));
   XB_CUDA(ensure(s->A, s->t32, (size_t)M * N * 4));
-  infer_xgs_kernel<<<(unsigned)((Npad * Fp + 255) / 256), 256, 0, s->st>>>(
+  // The line model (70 us of dependent chains at 128 x 128) and the first layer (two products of few
+  // tiles, 48 us) need only the feature columns of the first kernel, so they run side by side.
+  xbar_status st = map_prep(s, G, sGi, sGj, s->forked);
+  if (st != XBAR_OK) return st;
+  XB_CUDA(cudaStreamWaitEvent(s->side, s->forked, 0));
+  infer_xv_kernel<<<(unsigned)((Bpad * Fp + 255) / 256), 256, 0, s->side>>>(V, M, B, (int)Bpad, Fp, 1.0 / s->vs,
+                                                                             (__nv_bfloat16*)s->xv.p);
+  infer_xgs_kernel<<<(unsigned)((Npad * Fp + 255) / 256), 256, 0, s->side>>>(
       (const double*)s->Gt.p, (const float*)s->St.p, M, N, (int)Npad, Fp, 1.0 / s->gs, (__nv_bfloat16*)s->xgs.p);
-  infer_xv_kernel<<<(unsigned)((Bpad * Fp + 255) / 256), 256, 0, s->st>>>(V, M, B, (int)Bpad, Fp, 1.0 / s->vs,
-                                                                           (__nv_bfloat16*)s->xv.p);
-  infer_gt32_kernel<<<(unsigned)(((long)M * N + 255) / 256), 256, 0, s->st>>>(
-      (const double*)s->Gt.p, (const double*)s->Tl.p, M, N, (float*)s->g32.p, (float*)s->t32.p);
-  const size_t ic_smem = ((size_t)kVB * M + (size_t)(kIP - 1) * 2 * kVB * 128) * sizeof(float);
-  XB_CUDA(cudaFuncSetAttribute(infer_currents_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ic_smem));
-  infer_currents_kernel<<<(B + kVB - 1) / kVB, 128 * kIP, ic_smem, s->st>>>(
-      V, (const float*)s->g32.p, (const float*)s->t32.p, M, N, B, (double*)s->Iid.p, (double*)s->Iln.p);
-  XB_CUDA(cudaGetLastError());
   GemmBf16Params g;
   memset(&g, 0, sizeof(g));
   g.status = s->status;
@@ -1327,14 +1336,28 @@ static xbar_status predict_map(xbar_surrogate_t s, const double* G, long sGi, lo
   g.sBk = 1;
   g.mode = GEMM_EPI_STORE;  // not split over K: prediction stays deterministic
   g.ldc = kH;
-  g.M = (int)Npad;
-  g.A = (const __nv_bfloat16*)s->xgs.p;
-  g.C = (float*)s->Pm.p;
-  XB_CUDA(launch_gemm_bf16(g, 1, s->st));
   g.M = (int)Bpad;
   g.A = (const __nv_bfloat16*)s->xv.p;
   g.C = (float*)s->Qm.p;
-  XB_CUDA(launch_gemm_bf16(g, 1, s->st));
+  const cudaError_t e_q = launch_gemm_bf16(g, 1, s->side);
+  g.M = (int)Npad;
+  g.A = (const __nv_bfloat16*)s->xgs.p;
+  g.C = (float*)s->Pm.p;
+  const cudaError_t e_p = launch_gemm_bf16(g, 1, s->side);
+  XB_CUDA(cudaEventRecord(s->joined, s->side));  // whatever was queued: the next call waits for it too
+  infer_gt32_kernel<<<(unsigned)(((long)M * N + 255) / 256), 256, 0, s->st>>>(
+      (const double*)s->Gt.p, (const double*)s->Tl.p, M, N, (float*)s->g32.p, (float*)s->t32.p);
+  const size_t ic_smem = ((size_t)kVB * M + (size_t)(kIP - 1) * 2 * kVB * 128) * sizeof(float);
+  const cudaError_t e_a =
+      cudaFuncSetAttribute(infer_currents_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ic_smem);
+  if (e_a == cudaSuccess)
+    infer_currents_kernel<<<(B + kVB - 1) / kVB, 128 * kIP, ic_smem, s->st>>>(
+        V, (const float*)s->g32.p, (const float*)s->t32.p, M, N, B, (double*)s->Iid.p, (double*)s->Iln.p);
+  XB_CUDA(cudaStreamWaitEvent(s->st, s->joined, 0));
+  XB_CUDA(e_q);
+  XB_CUDA(e_p);
+  XB_CUDA(e_a);
+  XB_CUDA(cudaGetLastError());
   SurInferParams q;
   memset(&q, 0, sizeof(q));
   q.rows = rows;
