@@ -171,26 +171,19 @@ __device__ __forceinline__ bool epi_sync_or(bool v) {
 __host__ __device__ constexpr int tc_sub(int Mt, int KP, bool two) { return two ? 1 : (Mt == 256 && KP == 3) ? 2 : 4; }
 __host__ __device__ constexpr uint32_t tc_slot(int Mt, int KP) { return (uint32_t)KP * tc::kKC * Mt * 2; }
 __host__ __device__ constexpr int tc_vbytes(int Mt, int KP) { return KP * (tc::kBP / 8) * (int)tc::lbo_b(Mt); }
-// Beside the vector operand: with 256-row blocks, 32 floats per epilogue thread for the second
-// 32-column block of the next step's z or right-hand side, copied in ahead of the accumulator wait;
-// in every sweep, the staging of the w tiles (4 KB per warp) between those copies.  With two blocks on
-// an SM the inward launch, which has no w, takes none: L1 then holds the lines its right-hand side
-// loads come back to.
-__host__ __device__ constexpr int tc_prebytes(bool two, bool out) {
-  return two && !out ? 0 : tc::kThreads * 32 * 4;
-}
-__host__ __device__ constexpr int tc_fixed(int Mt, int KP, bool two, bool out) {
-  return 2304 + tc_vbytes(Mt, KP) + tc_prebytes(two, out);
-}
+// Beside the vector operand, 32 floats per epilogue thread (4 KB a warp).  Inward: the warp's rows of the
+// next right-hand side.  Outward: with 256-row blocks the second 32-column block of z, copied in ahead
+// of the accumulator wait, and the staging of the w tiles between those copies.
+constexpr int kPreBytes = tc::kThreads * 32 * 4;
+__host__ __device__ constexpr int tc_fixed(int Mt, int KP) { return 2304 + tc_vbytes(Mt, KP) + kPreBytes; }
 // shared memory of a block: 227 KB, or half of the SM's 228 KB less the 1 KB each block reserves
 __host__ __device__ constexpr int tc_budget(bool two) { return two ? 115712 : 232448; }
-__host__ __device__ constexpr int tc_stages(int Mt, int KP, bool two, bool out) {
-  const int fit = (tc_budget(two) - tc_fixed(Mt, KP, two, out)) / (int)(tc_sub(Mt, KP, two) * tc_slot(Mt, KP));
-  return fit > (two ? 5 : 8) ? (two ? 5 : 8) : fit;
+__host__ __device__ constexpr int tc_stages(int Mt, int KP, bool two) {
+  const int fit = (tc_budget(two) - tc_fixed(Mt, KP)) / (int)(tc_sub(Mt, KP, two) * tc_slot(Mt, KP));
+  return fit > 8 ? 8 : fit;
 }
-static_assert(tc_stages(256, 2, false, true) == 2 && tc_stages(256, 3, false, true) == 2 &&
-                  tc_stages(128, 2, false, true) == 5 && tc_stages(128, 3, false, true) == 3 &&
-                  tc_stages(128, 2, true, true) == 5 && tc_stages(128, 2, true, false) == 5,
+static_assert(tc_stages(256, 2, false) == 2 && tc_stages(256, 3, false) == 2 && tc_stages(128, 2, false) == 5 &&
+                  tc_stages(128, 3, false) == 3 && tc_stages(128, 2, true) == 5,
               "stage rings");
 
 // NH = number of 128-row halves of X_j (Mt = 128 NH); KP = number of BF16 terms of the split used
@@ -205,7 +198,7 @@ __global__ void __launch_bounds__(tc::kThreads + 64, kTwo ? 2 : 1)
   using namespace tc;
   constexpr int BP = kBP, KC = kKC;
   constexpr int Mt = 128 * NH, nh = NH;
-  constexpr int NS = tc_stages(Mt, KP, kTwo, kOut), kSub = tc_sub(Mt, KP, kTwo);
+  constexpr int NS = tc_stages(Mt, KP, kTwo), kSub = tc_sub(Mt, KP, kTwo);
   static_assert(!kTwo || (NH == 1 && KP == 2), "two blocks on an SM");
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int b0 = blockIdx.x * BP;
@@ -470,6 +463,40 @@ __global__ void __launch_bounds__(tc::kThreads + 64, kTwo ? 2 : 1)
       }
       __syncwarp();
     };
+    // Inward: the right-hand side rows [Mp][Bpad] of the column after step s2, 32 columns of the warp's 32
+    // rows, into its slice of pres by asynchronous copies of whole 128-byte row segments, skewed like
+    // the w tiles; take_r: this lane's row of them.  (Loads of 16 bytes from 32 rows each kept the
+    // load units and L1 busy; with 8192 vectors of 256 x 256 an inward correction launch took
+    // 1.57 ms against 1.40 ms now, with 1000 of 128 x 128 171 against 137 us.)
+    auto stage_r = [&](int s2, int blk) {
+      if (!kOut && p.rhs && s2 + 1 < nsteps) {
+        const float* src = p.rhs + ((size_t)col_of(s2 + 1) * Mp + (i - lane)) * Bpad + b0 + cb + blk * 32;
+#pragma unroll
+        for (int m = 0; m < 8; ++m) {
+          const int r = 4 * m + (lane >> 3), q = lane & 7;
+          if (i - lane + r < Mp)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                             smem_addr(wst + (r & 7) * kThreads + ((r & 24) | ((r + q) & 7)))),
+                         "l"(src + (size_t)r * Bpad + 4 * q)
+                         : "memory");
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+      }
+    };
+    auto take_r = [&](float (&d)[32]) {
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+      __syncwarp();
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const float4 x = wst[(lane & 7) * kThreads + ((lane & 24) | ((lane + q) & 7))];
+        d[4 * q] = x.x;
+        d[4 * q + 1] = x.y;
+        d[4 * q + 2] = x.z;
+        d[4 * q + 3] = x.w;
+      }
+      __syncwarp();
+    };
+    stage_r(0, 0);
     float local_max = 0.0f;
     for (int s = 0; s < nsteps; ++s) {
       const int j = col_of(s);
@@ -488,9 +515,8 @@ __global__ void __launch_bounds__(tc::kThreads + 64, kTwo ? 2 : 1)
       // now, block 1 right after it, so their latency leaves the step's critical path
       const bool use_z = zout && s > 0 && real;
       const bool use_r = !kOut && more && p.rhs && real;
-      const float* rnext = p.rhs + ((size_t)jn * Mp + (real ? i : 0)) * Bpad + b0 + cb;
       float pre[ncb][32];
-      // block 1 (nh == 2): 16-byte cp.async copies into this thread's slice of pres, waited for
+      // outward, block 1 (nh == 2): 16-byte cp.async copies into this thread's slice of pres, waited for
       // after the accumulator wait, so their latency overlaps it
       auto async_pre1 = [&]() {
         if (use_z) {
@@ -500,19 +526,12 @@ __global__ void __launch_bounds__(tc::kThreads + 64, kTwo ? 2 : 1)
             asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(smem_addr(pres + (n / 4) * kThreads + tid)),
                          "l"(zrow + (size_t)(n / 4) * Mp)
                          : "memory");
-        } else if (use_r) {
-          const float* rn = rnext + 32;
-#pragma unroll
-          for (int n = 0; n < 32; n += 4)
-            asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(smem_addr(pres + (n / 4) * kThreads + tid)),
-                         "l"(rn + n)
-                         : "memory");
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
       };
       auto take_pre1 = [&]() {
         asm volatile("cp.async.wait_group 0;" ::: "memory");
-        if (use_z || use_r) {
+        if (use_z) {
 #pragma unroll
           for (int n = 0; n < 32; n += 4) {
             const float4 v4 = pres[(n / 4) * kThreads + tid];
@@ -534,20 +553,18 @@ __global__ void __launch_bounds__(tc::kThreads + 64, kTwo ? 2 : 1)
             pre[blk][n + 2] = zz.z;
             pre[blk][n + 3] = zz.w;
           }
-        } else if (use_r) {
-          const float* rn = rnext + blk * 32;
-#pragma unroll
-          for (int n = 0; n < 32; n += 4) {
-            const float4 r4 = *reinterpret_cast<const float4*>(rn + n);
-            pre[blk][n] = r4.x;
-            pre[blk][n + 1] = r4.y;
-            pre[blk][n + 2] = r4.z;
-            pre[blk][n + 3] = r4.w;
-          }
         }
       };
-      load_pre(0);
-      if (nh == 2) async_pre1();
+      if constexpr (kOut) {
+        load_pre(0);
+        if (nh == 2) async_pre1();
+      } else if (more && p.rhs) {  // block 0 has been on its way since the last step
+        take_r(pre[0]);
+        if constexpr (nh == 2) {
+          stage_r(s, 1);
+          take_r(pre[1]);
+        }
+      }
       // one thread polls the accumulator barrier; the others wait on the named hardware barrier so
       // that no shared-memory polling competes with the tensor core's operand reads
       bool okd = true;
@@ -558,7 +575,7 @@ __global__ void __launch_bounds__(tc::kThreads + 64, kTwo ? 2 : 1)
         break;
       }
       fence_after();
-      if (nh == 2) take_pre1();
+      if (kOut && nh == 2) take_pre1();
 
       // (1) D of this step per column block (z added on the way out), then (2) the next
       // step's input from it, split into BF16 terms; then the next step's MMAs may start
@@ -580,6 +597,7 @@ __global__ void __launch_bounds__(tc::kThreads + 64, kTwo ? 2 : 1)
           }
         }
         release_v();
+        stage_r(s + 1, 0);
         warm_l2(s + 1);
       }
       // (3) while the next step's MMAs run: z (inward), w and the current (outward)
@@ -648,8 +666,8 @@ __global__ void __launch_bounds__(tc::kThreads + 64, kTwo ? 2 : 1)
   if (warp == 1) tmem_dealloc(tbase, ncols);
 }
 
-static size_t sweep_tc_smem_bytes(int Mt, int KP, bool two, bool out) {
-  return (size_t)tc_fixed(Mt, KP, two, out) + (size_t)tc_stages(Mt, KP, two, out) * tc_sub(Mt, KP, two) * tc_slot(Mt, KP);
+static size_t sweep_tc_smem_bytes(int Mt, int KP, bool two) {
+  return (size_t)tc_fixed(Mt, KP) + (size_t)tc_stages(Mt, KP, two) * tc_sub(Mt, KP, two) * tc_slot(Mt, KP);
 }
 
 bool sweep_tc_supported(int Mp) { return Mp <= 256; }
@@ -691,7 +709,7 @@ cudaError_t launch_sweep_tc(const SweepParams<float>& p, const void* Xt, int ter
     // half an SM's registers and a third of its stages: 1000 vectors 2.62 against 2.72 ms.
     const bool two = Mt == 128 && terms == 2 && (beside || blocks * chains > nsm);
     const Kern kern = two ? pair[out] : kerns[Mt / 128 - 1][terms - 2][out];
-    const size_t smem = sweep_tc_smem_bytes(Mt, terms, two, out);
+    const size_t smem = sweep_tc_smem_bytes(Mt, terms, two);
     const cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (err != cudaSuccess) return err;
     kern<<<dim3(blocks, chains), tc::kThreads + 64, smem, st>>>(p, static_cast<const __nv_bfloat16*>(Xt), chain0);
