@@ -498,6 +498,34 @@ __global__ void __launch_bounds__(tc::kThreads + 64, kTwo ? 2 : 1)
     };
     stage_r(0, 0);
     float local_max = 0.0f;
+    // partial dot products of step s, 64 columns a warp (nh == 1: of which it covers cb .. cb + 31)
+    auto red_at = [&](int s, int w) { return nh == 2 ? red + w * 64 : red + (s & 1) * 256 + w * 32 - (w >> 2) * 32; };
+    // the currents of step s (column j) from the warps' partial dot products
+    auto add_currents = [&](int s, int j, double Iold) {
+      if (tid >= BP) return;
+      float sum = 0.0f;
+      if (nh == 2) {
+        for (int w = 0; w < 8; ++w) sum += red_at(s, w)[tid];
+      } else {
+        const int s0 = (tid >> 5) * 4;  // warps covering this column block
+        for (int w = s0; w < s0 + 4; ++w) sum += red_at(s, w)[tid];
+      }
+      const int b = b0 + tid;
+      if (b < p.B) {
+        double* Ip = p.I + (size_t)b * N + j;
+        const double dI = (double)sum;
+        if (!isfinite(dI)) set_status(p.status, XBAR_DEV_NONFINITE);
+        if (p.accumulate) {
+          const double In = Iold + dI;
+          *Ip = In;
+          local_max = fmaxf(local_max, (float)(fabs(dI) / fmax(fabs(In), 1e-300)));
+        } else {
+          *Ip = dI;
+        }
+      }
+    };
+    bool pend = false;  // nh == 1: the last step's currents are still to be added, to Ipend
+    double Ipend = 0.0;
     for (int s = 0; s < nsteps; ++s) {
       const int j = col_of(s);
       const bool more = s + 1 < nsteps;
@@ -600,6 +628,7 @@ __global__ void __launch_bounds__(tc::kThreads + 64, kTwo ? 2 : 1)
         stage_r(s + 1, 0);
         warm_l2(s + 1);
       }
+      if (nh == 1 && pend) add_currents(s - 1, col_of(s - 1), Ipend);
       // (3) while the next step's MMAs run: z (inward), w and the current (outward)
       float dots[ncb];
 #pragma unroll
@@ -627,32 +656,23 @@ __global__ void __launch_bounds__(tc::kThreads + 64, kTwo ? 2 : 1)
           dots[blk] = transpose_sum32(a, lane);
         }
       }
+      // 128-row blocks: a step's partial dot products stay in red, by the parity of the step, until the next
+      // accumulator wait has synchronised the warps, because there the epilogue is the longer part of a step
+      // and a barrier of its own would end it; 256-row blocks (whose red has no room for two) add them now
       if (have_w)
 #pragma unroll
-        for (int blk = 0; blk < ncb; ++blk) red[warp * 64 + cb + blk * 32 + lane] = dots[blk];
-      epi_sync();
-      if (have_w && tid < BP) {
-        float sum = 0.0f;
-        if (nh == 2) {
-          for (int w = 0; w < 8; ++w) sum += red[w * 64 + tid];
-        } else {
-          const int s0 = (tid >> 5) * 4;  // warps covering this column block
-          for (int w = s0; w < s0 + 4; ++w) sum += red[w * 64 + tid];
-        }
-        const int b = b0 + tid;
-        if (b < p.B) {
-          double* Ip = p.I + (size_t)b * N + j;
-          const double dI = (double)sum;
-          if (!isfinite(dI)) set_status(p.status, XBAR_DEV_NONFINITE);
-          if (p.accumulate) {
-            const double In = Iold + dI;
-            *Ip = In;
-            local_max = fmaxf(local_max, (float)(fabs(dI) / fmax(fabs(In), 1e-300)));
-          } else {
-            *Ip = dI;
-          }
-        }
+        for (int blk = 0; blk < ncb; ++blk) red_at(s, warp)[cb + blk * 32 + lane] = dots[blk];
+      if (nh == 2) {
+        epi_sync();
+        if (have_w) add_currents(s, j, Iold);
+      } else {
+        pend = have_w;
+        Ipend = Iold;
       }
+    }
+    if (nh == 1) {
+      epi_sync();
+      if (pend) add_currents(nsteps - 1, col_of(nsteps - 1), Ipend);
     }
     if (p.max_rel) {
       for (int o = 16; o > 0; o >>= 1) local_max = fmaxf(local_max, __shfl_xor_sync(0xffffffffu, local_max, o));
