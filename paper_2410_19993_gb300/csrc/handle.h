@@ -70,6 +70,21 @@ inline cudaError_t ensure(DevArena& A, Buf& b, size_t bytes) {
 
 inline int round_up(int a, int m) { return ((a + m - 1) / m) * m; }
 
+// several scratch buffers in one allocation: each part becomes a view of slab (256-byte aligned).  The parts'
+// contents do not survive a call that needs more than slab holds.
+inline cudaError_t ensure_group(DevArena& A, Buf& slab, std::initializer_list<std::pair<Buf*, size_t>> parts) {
+  size_t total = 0;
+  for (const auto& q : parts) total += (q.second + 255) / 256 * 256;
+  const cudaError_t e = ensure(A, slab, total);
+  size_t at = 0;
+  for (const auto& q : parts) {
+    q.first->p = e == cudaSuccess ? static_cast<char*>(slab.p) + at : nullptr;
+    q.first->bytes = e == cudaSuccess ? q.second : 0;
+    at += (q.second + 255) / 256 * 256;
+  }
+  return e;
+}
+
 }  // namespace xbar
 
 #include "cr.h"

@@ -879,9 +879,9 @@ struct xbar_surrogate_s {
   Buf gX, gy;  // xbar_surrogate_grad's copies of its arguments
   // per-map line model and feature columns: [N][M]
   int passes = 1;
-  Buf Gt, Gf, tau, St, Tl, wl, bl, xg, field;
+  Buf mapbuf, Gt, Gf, tau, St, Tl, wl, bl, xg, field;  // the eight after mapbuf are views of it
   // inference: split first layer and FP32 copies for the current contractions
-  Buf xgs, xv, Pm, Qm, g32, t32;
+  Buf inferbuf, xgs, xv, Pm, Qm, g32, t32;  // views of inferbuf
   // training set
   Buf Xall, yall;
 };
@@ -1122,14 +1122,9 @@ static xbar_status map_prep(xbar_surrogate_t s, const double* G, long sGi, long 
                             cudaEvent_t columns_ready = nullptr) {
   const int M = s->M, N = s->N;
   const size_t mn = (size_t)M * N;
-  XB_CUDA(ensure(s->A, s->Gt, mn * 8));
-  XB_CUDA(ensure(s->A, s->Gf, mn * 4));
-  XB_CUDA(ensure(s->A, s->tau, mn * 4));
-  XB_CUDA(ensure(s->A, s->St, mn * 4));
-  XB_CUDA(ensure(s->A, s->Tl, mn * 8));
-  XB_CUDA(ensure(s->A, s->wl, mn * 4));
-  XB_CUDA(ensure(s->A, s->bl, mn * 4));
-  XB_CUDA(ensure(s->A, s->xg, mn * 4));
+  // one allocation: one for each buffer made the first call on a surrogate 160 us longer
+  XB_CUDA(ensure_group(s->A, s->mapbuf, {{&s->Gt, mn * 8}, {&s->Tl, mn * 8}, {&s->Gf, mn * 4}, {&s->tau, mn * 4},
+                                         {&s->St, mn * 4}, {&s->wl, mn * 4}, {&s->bl, mn * 4}, {&s->xg, mn * 4}}));
   const float gs = (float)(1.0 / s->R[0]), gw = (float)(1.0 / s->R[1]), gb = (float)(1.0 / s->R[2]),
               go = (float)(1.0 / s->R[3]);
   const float* Gf = (const float*)s->Gf.p;
@@ -1309,12 +1304,9 @@ static xbar_status predict_map(xbar_surrogate_t s, const double* G, long sGi, lo
   const long Npad = round_up_l(N, 128), Bpad = round_up_l(B, 128);
   XB_CUDA(ensure(s->A, s->Iid, (size_t)rows * 8));
   XB_CUDA(ensure(s->A, s->Iln, (size_t)rows * 8));
-  XB_CUDA(ensure(s->A, s->xgs, (size_t)Npad * Fp * 2));
-  XB_CUDA(ensure(s->A, s->xv, (size_t)Bpad * Fp * 2));
-  XB_CUDA(ensure(s->A, s->Pm, (size_t)Npad * kH * 4));
-  XB_CUDA(ensure(s->A, s->Qm, (size_t)Bpad * kH * 4));
-  XB_CUDA(ensure(s->A, s->g32, (size_t)M * N * 4));
-  XB_CUDA(ensure(s->A, s->t32, (size_t)M * N * 4));
+  XB_CUDA(ensure_group(s->A, s->inferbuf,
+                       {{&s->xgs, (size_t)Npad * Fp * 2}, {&s->xv, (size_t)Bpad * Fp * 2}, {&s->Pm, (size_t)Npad * kH * 4},
+                        {&s->Qm, (size_t)Bpad * kH * 4}, {&s->g32, (size_t)M * N * 4}, {&s->t32, (size_t)M * N * 4}}));
   // The line model (70 us of dependent chains at 128 x 128) and the first layer (two products of few
   // tiles, 48 us) need only the feature columns of the first kernel, so they run side by side.
   xbar_status st = map_prep(s, G, sGi, sGj, s->forked);
