@@ -372,31 +372,34 @@ def run_xbar(args):
     # factor run beside them on the other stream and are hidden: the step time is the solve's)
     dom = max((ph for ph in per_step if ph not in ("assemble", "factor")), key=lambda ph: per_step[ph]["ms"])
     work, _ = algorithmic_work(dom, M, N, B)
-    ms_launch = prof[dom]["ms"] / prof[dom]["launches"]
+    # a substitution is up to two launches (inward, outward): its roofline is per substitution, one for the
+    # initial solve and one for each correction
+    per = args.steps * (info_box["iters"] + 1) if dom == "sweep" else prof[dom]["launches"]
+    ms_launch = prof[dom]["ms"] / per
     mp = measured_peaks()
     peaks = pipe_peaks(mp.get("sm_max_mhz", 2070.0))
     achieved = work / (ms_launch / 1e3) / 1e12
     if dom == "sweep" and M <= 256:
-        # tensor-core sweep (tcgen05 kind::f16 with BF16 operands: six split products per algorithmic
-        # multiply-add in the initial solve, three in the corrections); timed inside a seconds-long
-        # step, so the sustained BF16 figure
+        # tensor-core sweep (tcgen05 kind::f16 with BF16 operands, three split products per algorithmic
+        # multiply-add); timed inside a seconds-long step, so the sustained BF16 figure.  An input vector
+        # has no inward part on the right, so the initial solve has 1.5 N block products, a correction 2 N - 1
+        work *= (1.5 * N + info_box["iters"] * (2 * N - 1)) / ((info_box["iters"] + 1) * (2 * N - 1))
         bf16 = mp.get("bf16_tflops_sustained", mp.get("bf16_tflops", 1704.4))
         bound, peak, note = "tensor", bf16, ("BF16 dense, measured sustained cuBLAS figure (of measured); achieved "
-                                            "counts algorithmic flops only, averaged over the solve's sweep launches "
-                                            "(the initial one issues six BF16 products per multiply-add, the "
-                                            "corrections three)")
+                                            "counts algorithmic flops only, averaged over the solve's substitutions "
+                                            "(three BF16 products per multiply-add)")
     elif dom in ("sweep", "factor", "update"):
         bound, peak, note = "alu", peaks["fp32_tflops"], "FP32 FMA pipe, 152 SM x 128 lanes x 2 x max SM clock"
     else:
         bound, peak, note = "alu", peaks["fp64_tflops"], "FP64 FMA pipe, 152 SM x 2 DFMA x 2 x max SM clock"
     traffic, traffic_note = None, None
     if dom == "sweep" and (M, N) == (256, 256) and bound == "tensor":
-        # ncu DRAM read + write per sweep_tc_kernel launch at B = 2048 (the capture fits the size
-        # rule; the full batch does not), averaged over the solve's launches (1.667 GB initial, which
-        # writes the FP32 state, and 2.218 GB for each correction), scaled by B / 2048: the kernel's
+        # ncu DRAM read + write per substitution (two sweep_tc_kernel launches) at B = 2048 (the capture fits the size
+        # rule; the full batch does not), averaged over the solve's three (1.061 GB initial, which has no inward part on the right and
+        # writes the FP32 state, and 2.197 GB for each correction), scaled by B / 2048: the kernel's
         # streams are per vector, the factor blocks it re-reads come from L2
-        traffic = 2.034e9 * B / 2048
-        traffic_note = (f"ncu dram__bytes_read+write at B=2048 (mean of the solve's three sweep launches) "
+        traffic = 1.818e9 * B / 2048
+        traffic_note = (f"ncu dram__bytes_read+write at B=2048 (mean of the solve's three substitutions) "
                         f"x B/2048 = {B / 2048:g}")
     roofline = {"kernel": dom, "bound": bound, "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                 "frac": achieved / peak, "traffic": traffic, "traffic_note": traffic_note, "peak_note": note,
