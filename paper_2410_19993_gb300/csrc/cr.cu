@@ -180,15 +180,37 @@ __global__ void __launch_bounds__(kGthThreads) cr_gth_kernel(int Mp, const CrGth
       const T* Up = U + (size_t)(hu ? x.pp : 0) * MM;
       const T* wpp = om + (size_t)(hu ? x.pp : 0) * Mp;
       T sa = (T)0, sb = (T)0, sc = (T)0;
+      if constexpr (sizeof(T) == 8) {
 #pragma unroll
-      for (int u = 0; u < 16; ++u) {  // fully unrolled: the loads are independent (Mp <= 256: q <= 16)
-        const int m = m0 + u;
-        if (sizeof(T) == 8 && u >= q) break;  // uniform; FP64 issue costs more than the loads' overlap gains
-        if (u < q && m < Mp) {
-          if (hl) sa = fma(Qk[(size_t)m * Mp + i], gl[m], sa);
-          if (hr) sb = fma(Pk[(size_t)m * Mp + i], gr[m], sb);
-          if (hu) sc = fma(Up[(size_t)m * Mp + i], wpp[m], sc);
+        for (int u = 0; u < 16; ++u) {
+          const int m = m0 + u;
+          if (u >= q) break;  // uniform; FP64 issue costs more than the loads' overlap gains
+          if (m < Mp) {
+            if (hl) sa = fma(Qk[(size_t)m * Mp + i], gl[m], sa);
+            if (hr) sb = fma(Pk[(size_t)m * Mp + i], gr[m], sb);
+            if (hu) sc = fma(Up[(size_t)m * Mp + i], wpp[m], sc);
+          }
         }
+      } else {
+        // all loads of a sum before its multiply-adds (Mp <= 256: q <= 16): with a load behind each of
+        // them, under the three conditions, a launch was a chain of memory latencies (128 blocks of
+        // 256 rows: 110 -> 51 us)
+        auto column = [&](const T* A, const T* w) {
+          T v[16], c[16], t = (T)0;
+#pragma unroll
+          for (int u = 0; u < 16; ++u) {
+            const int m = m0 + u;
+            const bool in = u < q && m < Mp;
+            v[u] = in ? A[(size_t)m * Mp + i] : (T)0;
+            c[u] = in ? w[m] : (T)0;
+          }
+#pragma unroll
+          for (int u = 0; u < 16; ++u) t = fma(v[u], c[u], t);
+          return t;
+        };
+        if (hl) sa = column(Qk, gl);
+        if (hr) sb = column(Pk, gr);
+        if (hu) sc = column(Up, wpp);
       }
       g = sa + sb;
       lc = sc;
@@ -203,7 +225,42 @@ __global__ void __launch_bounds__(kGthThreads) cr_gth_kernel(int Mp, const CrGth
   const int half = warp & 1;
   // rows past the block, and a half warp pair's empty half (Mp <= 128), are skipped whole: in FP64 every
   // operation costs its issue slots whether a lane uses it or not
-  for (int il = warp >> 1; il < kGthRows; il += kGthThreads / 64) {
+  constexpr int kStep = kGthThreads / 64;                  // a warp pair's rows are kStep apart
+  constexpr int RB = sizeof(T) == 8 ? 1 : kGthRows / kStep;  // rows loaded at a time
+  if constexpr (RB > 1) {  // FP32: all of a warp's rows
+    T dv[RB][4], uv[RB][4];
+#pragma unroll
+    for (int r = 0; r < RB; ++r) {
+      const int i = i0 + (warp >> 1) + r * kStep;
+      const T* Drow = D + ((size_t)x.p * Mp + i) * Mp;
+      const T* Urow = U + ((size_t)x.p * Mp + i) * Mp;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int m = half * 128 + lane + 32 * u;
+        const bool in = i < Mp && m < Mp;
+        dv[r][u] = in && m != i ? fabs(Drow[m]) : (T)0;
+        uv[r][u] = in && hn ? Urow[m] : (T)0;
+      }
+    }
+    T wpm[4], wnm[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int m = half * 128 + lane + 32 * u;
+      wpm[u] = m < Mp ? wp[m] : (T)0;
+      wnm[u] = m < Mp && hn ? wn[m] : (T)0;
+    }
+#pragma unroll
+    for (int r = 0; r < RB; ++r) {
+      const int il = (warp >> 1) + r * kStep;
+      const T off = cr_warp_sum((dv[r][0] * wpm[0] + dv[r][1] * wpm[1]) + (dv[r][2] * wpm[2] + dv[r][3] * wpm[3]));
+      const T rc = cr_warp_sum((uv[r][0] * wnm[0] + uv[r][1] * wnm[1]) + (uv[r][2] * wnm[2] + uv[r][3] * wnm[3]));
+      if (lane == 0) {
+        opart[half][il] = off;
+        rpart[half][il] = rc;
+      }
+    }
+  }
+  for (int il = warp >> 1; RB == 1 && il < kGthRows; il += kStep) {
     const int i = i0 + il;
     T off = (T)0, rc = (T)0;
     if (i >= Mp || half * 128 >= Mp) {
