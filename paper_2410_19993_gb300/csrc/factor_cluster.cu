@@ -5,7 +5,8 @@
 // m+1 are two independent chains, one cluster each, and a second launch inverts the meeting column
 //     Z_m = C_m - g_w^2 X_{m-1} - g_w^2 X_{m+1}.
 // The factor is bound by the latency of its chain (16 dependent panels a column on 16 SMs), so half the
-// chain is half the time: 12.25 -> 6.2 ms at 256 x 256, 2.85 -> 1.45 ms at 128 x 128, on twice the SMs.
+// chain is half the time: 12.25 -> 6.2 ms at 256 x 256, 2.85 -> 1.45 ms at 128 x 128, on twice the SMs
+// (4.5 and 1.22 ms with the early hand-over and the shared coefficient broadcasts below).
 // In a cluster of C blocks block g holds rows [g R, (g+1) R) of the current matrix in registers, one
 // thread per column (R = 16, C = Mp / R).
 // The in-place blocked Gauss-Jordan inversion uses panels of R rows, so panel p is exactly block p's
