@@ -334,6 +334,7 @@ static xbar_status factor_mirror(xbar_s* h, xbar_precision p) {
   xbar_s* g = h->mirror;
   g->opt = h->opt;
   g->opt.orient = 0;
+  g->beside = h->beside;
   // automatic algorithm: the mirror's many small blocks (M blocks of N rows) are what cyclic
   // reduction is for, against M dependent block steps of block Thomas
   if (h->opt.algo < 0 && cr_supported(g->m.Mp, g->m.N)) g->opt.algo = 1;
@@ -615,6 +616,7 @@ static xbar_status do_factor64(xbar_t h) {
   fp.buf = (double*)h->fpbuf.p;
   fp.flags = (unsigned*)h->fbar.p;
   fp.status = h->status;
+  fp.beside = h->beside;
   PhaseScope ps(h, XBAR_PHASE_FACTOR, 1);
   XB_CUDA(launch_factor64(fp, h->st));
   h->tc_ready = 0;

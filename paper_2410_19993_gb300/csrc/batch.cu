@@ -109,6 +109,7 @@ extern "C" xbar_status xbar_batch_create(int T, const xbar_tile* desc, void* cud
     const xbar_tile& d = desc[t];
     xbar_status st = xbar_assemble(d.M, d.N, d.G, d.R_s, d.R_w, d.R_b, d.R_sense, s, &h);
     if (st != XBAR_OK) return bail(st);
+    h->beside = T > 1;
     b->tiles.push_back(h);
   }
   *out = b;

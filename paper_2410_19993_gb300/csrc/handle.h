@@ -120,6 +120,7 @@ struct xbar_s {
   double R[4] = {0, 0, 0, 0};
   cudaStream_t st = nullptr;
   int dev = 0, nsm = 0;
+  bool beside = false;  // a tile of a batch: other tiles' factors and solves run beside this one's
   // per-column elimination data formed from Gc (lazily, by the first factor): 0 = no, else with the
   // column blocks in the precision p of the factors, assembled_for(p)
   int assembled = 0;

@@ -84,6 +84,7 @@ struct Factor64Params {
   double* buf;        // factor64_buf_bytes scratch
   unsigned* flags;    // factor64_flag_bytes
   unsigned* status;
+  bool beside;        // other factors run beside this one: fewer, larger worker blocks
 };
 int factor64_meet(int Mp, int N);  // the meeting column
 size_t factor64_buf_bytes(int Mp);

@@ -45,3 +45,15 @@ def test_tiles_side_by_side():
         b.run("fp32_ir", Vs, Is, tol=1e-9, max_iter=6)
         for (M, N, B), (G, V), I in zip(shapes, tiles, Is):
             assert rel_err(I.cpu().numpy(), oracle.solve(M, N, G, *R, V)["I"]) <= 1e-8
+
+
+# tiles of a batch take the FP64 factor with eight rows a worker block; 1e-10 is the suite's FP64 bar
+def test_fp64_tiles_side_by_side():
+    shapes = [(16, 9, 3), (32, 17, 64), (33, 20, 5), (100, 51, 65), (128, 65, 20), (130, 66, 9), (256, 129, 4)]
+    tiles = [case(M, N, B, None, seed=M) for M, N, B in shapes]
+    b = xbar.Batch([(torch.from_numpy(G).cuda(), *R) for G, _ in tiles])
+    Vs = [torch.from_numpy(V).cuda() for _, V in tiles]
+    Is = [torch.zeros((B, N), dtype=torch.float64, device="cuda") for _, N, B in shapes]
+    b.run("fp64", Vs, Is)
+    for (M, N, B), (G, V), I in zip(shapes, tiles, Is):
+        assert rel_err(I.cpu().numpy(), oracle.solve(M, N, G, *R, V)["I"]) <= 1e-10
