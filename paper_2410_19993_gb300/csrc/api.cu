@@ -308,7 +308,7 @@ static bool use_cr_tensor(const xbar_s* h) {
 // XBAR_ORIENT=rows|columns; automatic (-1): rows for FP64 factors when 2N <= M, where the N x N
 // blocks make the factor ~(M/N)^2 and each substitution ~M/N times cheaper (mixed precision keeps
 // columns unless asked).  The mirror has N rows per block, so N must be within the handle limit.
-static bool use_rows(const xbar_s* h, xbar_precision p) {
+bool xbar::use_rows(const xbar_s* h, xbar_precision p) {
   if (h->m.N > 1024) return false;
   const char* e = getenv("XBAR_ORIENT");
   if (e && strcmp(e, "columns") == 0) return false;

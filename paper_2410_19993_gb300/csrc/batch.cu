@@ -160,8 +160,10 @@ extern "C" xbar_status xbar_batch_run(xbar_batch_t b, xbar_precision p, const in
   bool same = b->exec && b->sig_prec == (int)p && b->sig_iter == iters && b->sig_tol == tol;
   for (int t = 0; same && t < T; ++t)
     same = b->sigB[t] == B[t] && b->sigV[t] == (const void*)V[t] && b->sigI[t] == (const void*)I[t] &&
-           b->tiles[t]->assembled == assembled_for(p);  // new conductances (or blocks in the other precision):
-                                                        // the eager run assembles them outside the graph
+           // new conductances (or blocks in the other precision): the eager run assembles them outside
+           // the graph.  A tile blocked over rows is mirrored and assembled inside it (taking its own
+           // elimination data, which it never has, for stale ran every batch with one twice)
+           (b->tiles[t]->assembled == assembled_for(p) || (b->tiles[t]->orient_active && use_rows(b->tiles[t], p)));
   if (!same) {
     destroy_graph(b);
     // eager run: sizes every workspace and uploads the factor parameters

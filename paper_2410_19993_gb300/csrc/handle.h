@@ -211,6 +211,8 @@ int cr_panel(int B);  // kCrPanel, or 1, 2, 4 or 8 for a smaller batch
 // factor a handle (FP64 or equilibrated FP32); upload_params = false reuses the parameter block
 // already on the device (graph capture)
 xbar_status factor_handle(xbar_s* h, xbar_precision p, bool upload_params);
+// whether a factor in precision p blocks over the rows (the mirrored crossbar)
+bool use_rows(const xbar_s* h, xbar_precision p);
 
 // currents-only solve with device pointers, refinement driven on the device: exactly
 // `max_iter` refinement passes are enqueued and passes after convergence skip their work; no

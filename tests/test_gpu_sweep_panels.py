@@ -57,3 +57,20 @@ def test_fp64_tiles_side_by_side():
     b.run("fp64", Vs, Is)
     for (M, N, B), (G, V), I in zip(shapes, tiles, Is):
         assert rel_err(I.cpu().numpy(), oracle.solve(M, N, G, *R, V)["I"]) <= 1e-10
+
+
+def test_row_blocked_tile_new_conductances():
+    """A batch with a tile blocked over rows replays its graph; the graph mirrors the tile's current map."""
+    shapes = [(96, 20, 65), (40, 32, 64)]
+    b = xbar.Batch([(torch.from_numpy(case(M, N, B, None, seed=M)[0]).cuda(), *R) for M, N, B in shapes])
+    Vs = [torch.from_numpy(case(M, N, B, None, seed=M)[1]).cuda() for M, N, B in shapes]
+    Is = [torch.zeros((B, N), dtype=torch.float64, device="cuda") for _, N, B in shapes]
+    Gs = [case(M, N, B, None, seed=M)[0] for M, N, B in shapes]
+    for k in range(4):
+        if k == 2:  # the row-blocked tile only: the graph is replayed with its new map
+            Gs[0] = case(96, 20, 65, None, seed=7)[0]
+            xbar._check(xbar.load().xbar_set_conductances(b.tile_handle(0), xbar._ptr(torch.from_numpy(Gs[0]).cuda())))
+            torch.cuda.synchronize()
+        b.run("fp64", Vs, Is)
+        for (M, N, B), G, V, I in zip(shapes, Gs, Vs, Is):
+            assert rel_err(I.cpu().numpy(), oracle.solve(M, N, G, *R, V.cpu().numpy())["I"]) <= 1e-10
