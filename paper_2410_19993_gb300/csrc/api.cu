@@ -728,6 +728,7 @@ extern "C" xbar_status xbar_factor(xbar_t h, xbar_precision p) {
   if (!h) return fail(XBAR_EINVAL, "handle is NULL");
   if (p != XBAR_FP64 && p != XBAR_FP32_IR) return fail(XBAR_EINVAL, "unknown precision %d", (int)p);
   XB_CUDA(cudaSetDevice(h->dev));
+  ++h->calls;
   return factor_handle(h, p, true);
 }
 
@@ -745,6 +746,7 @@ extern "C" xbar_status xbar_set_option(xbar_t h, xbar_option opt, int value) {
     return XBAR_OK;
   }
   if (value < -1 || value > 1) return fail(XBAR_EINVAL, "option value %d outside [-1, 1]", value);
+  ++h->calls;
   switch (opt) {
     case XBAR_OPT_SWEEP_KERNEL: h->opt.sweep = value; break;
     case XBAR_OPT_FACTOR_KERNEL: h->opt.factor = value; break;

@@ -7,7 +7,9 @@
 // the device-driven solve of every tile become parallel branches of one graph (fork/join events
 // on an origin stream), refinement runs a fixed number of passes whose kernels skip their work
 // once a device-side flag says the tile has converged, and no host synchronisation happens inside.
-// Later runs with the same signature replay the instantiated graph with a single cudaGraphLaunch.
+// Later runs with the same signature replay the instantiated graph with a single cudaGraphLaunch.  A
+// tile's handle can be used between runs (xbar_batch_tile); what such a call may change under the graph
+// is part of the signature (graph_epoch).
 //
 // The autotuner times the kernel variants (tensor-core vs CUDA-core FP32 substitutions, cluster
 // vs cooperative-group FP32 factor; for FP64, blocks over columns vs over rows -- the mirrored
@@ -54,6 +56,7 @@ struct xbar_batch_s {
   cudaGraph_t graph = nullptr;
   std::vector<int> sigB;
   std::vector<const void*> sigV, sigI;
+  std::vector<unsigned long long> sig_epoch;  // graph_epoch of every tile
   int sig_prec = -1, sig_iter = -1;
   double sig_tol = -1.0;
 };
@@ -160,9 +163,11 @@ extern "C" xbar_status xbar_batch_run(xbar_batch_t b, xbar_precision p, const in
   bool same = b->exec && b->sig_prec == (int)p && b->sig_iter == iters && b->sig_tol == tol;
   for (int t = 0; same && t < T; ++t)
     same = b->sigB[t] == B[t] && b->sigV[t] == (const void*)V[t] && b->sigI[t] == (const void*)I[t] &&
+           // a direct call on the tile since the capture may have moved a buffer the graph points into
+           b->sig_epoch[t] == graph_epoch(b->tiles[t]) &&
            // new conductances (or blocks in the other precision): the eager run assembles them outside
-           // the graph.  A tile blocked over rows is mirrored and assembled inside it (taking its own
-           // elimination data, which it never has, for stale ran every batch with one twice)
+           // the graph.  A tile blocked over rows is mirrored and assembled inside it and has no
+           // elimination data of its own
            (b->tiles[t]->assembled == assembled_for(p) || (b->tiles[t]->orient_active && use_rows(b->tiles[t], p)));
   if (!same) {
     destroy_graph(b);
@@ -185,6 +190,8 @@ extern "C" xbar_status xbar_batch_run(xbar_batch_t b, xbar_precision p, const in
     b->sigB.assign(B, B + T);
     b->sigV.assign((const void* const*)V, (const void* const*)V + T);
     b->sigI.assign((const void* const*)I, (const void* const*)I + T);
+    b->sig_epoch.clear();
+    for (xbar_t h : b->tiles) b->sig_epoch.push_back(graph_epoch(h));
     b->sig_prec = (int)p;
     b->sig_iter = iters;
     b->sig_tol = tol;

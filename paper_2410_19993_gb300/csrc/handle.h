@@ -19,12 +19,16 @@ bool alloc_injected_failure();
 
 struct DevArena {
   std::vector<void*> ptrs;
+  unsigned long long changes = 0;  // allocations and releases so far: a captured graph holds these pointers
   cudaError_t alloc(void** p, size_t bytes) {
     *p = nullptr;
     if (bytes == 0) bytes = 16;
     if (alloc_injected_failure()) return cudaErrorMemoryAllocation;
     cudaError_t e = cudaMalloc(p, bytes);
-    if (e == cudaSuccess) ptrs.push_back(*p);
+    if (e == cudaSuccess) {
+      ptrs.push_back(*p);
+      ++changes;
+    }
     return e;
   }
   void release(void* p) {
@@ -32,6 +36,7 @@ struct DevArena {
       if (ptrs[k] == p) {
         cudaFree(p);
         ptrs.erase(ptrs.begin() + k);
+        ++changes;
         return;
       }
   }
@@ -130,6 +135,7 @@ struct xbar_s {
   unsigned* status = nullptr;      // device status block (xbar::DevStatus)
   unsigned long long wait_ns = 0;  // limit of the device waits, 0 = the default (host copy)
   xbar_opts opt;
+  unsigned long long calls = 0;  // xbar_factor and xbar_set_option calls: what they leave a captured graph does not know
   // factor
   xbar::Buf X, fsig, fpbuf, fbar, fparams;
   // host copy of the parameter block last uploaded to `fparams` (skip identical uploads)
@@ -196,6 +202,13 @@ struct PhaseScope {
 
 // error reporting shared by the C entry points
 xbar_status set_error(xbar_status s, const char* fmt, ...);
+
+// Changes whenever something that a graph captured over this handle relies on may have: its device buffers
+// and those of its mirror (workspaces, job lists), its kernel choices, the factor and the parameter block
+// that a direct call leaves behind.  Sums of counters that only grow, so equal means unchanged.
+inline unsigned long long graph_epoch(const xbar_s* h) {
+  return h->calls + h->A.changes + (h->mirror ? h->mirror->A.changes : 0);
+}
 
 inline int assembled_for(xbar_precision p) { return p == XBAR_FP64 ? 1 : 2; }
 
