@@ -198,6 +198,9 @@ extern "C" xbar_status xbar_batch_run(xbar_batch_t b, xbar_precision p, const in
   }
   XB_CUDA(cudaGraphLaunch(b->exec, b->origin));
   XB_CUDA(cudaStreamSynchronize(b->origin));
+  // the graph has factored every tile in the way of the capture (nothing else the host knows of a factor has
+  // changed since, see graph_epoch); xbar_set_conductances may have marked a tile unfactored
+  for (xbar_t h : b->tiles) h->factored = 1;
   // per-tile results
   bool all_conv = true;
   int first_bad = -1;

@@ -100,3 +100,22 @@ def test_other_precision_between_runs():
     s.run()
     for t in range(len(SHAPES)):
         s.solve(t, 9)
+
+
+def test_solve_on_a_tile_after_new_conductances():
+    """A run factors a tile's new map: the tile's handle can be solved with afterwards, replayed or not."""
+    s = Tiles("fp64")
+    s.run()
+    s.run()
+    for k in range(2):
+        for t, (M, N, B) in enumerate(SHAPES):
+            s.maps[t] = (case(M, N, B, None, seed=100 + 10 * k + t)[0], s.maps[t][1])
+            G = _dev(s.maps[t][0])
+            torch.cuda.synchronize()
+            xbar._check(xbar.load().xbar_set_conductances(s.tile(t), xbar._ptr(G)))
+            torch.cuda.synchronize()
+            s.run()
+            s.solve(t, 3)
+            Geff = torch.zeros((M, N), dtype=torch.float64, device="cuda")
+            xbar._check(xbar.load().xbar_transfer_matrix(s.tile(t), 1e-9, 10, xbar._ptr(Geff), None))
+            assert rel_err((s.V[t] @ Geff).cpu().numpy(), oracle.solve(M, N, s.maps[t][0], *R, s.maps[t][1])["I"]) <= 1e-10
