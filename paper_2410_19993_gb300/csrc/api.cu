@@ -729,6 +729,7 @@ extern "C" xbar_status xbar_factor(xbar_t h, xbar_precision p) {
   if (p != XBAR_FP64 && p != XBAR_FP32_IR) return fail(XBAR_EINVAL, "unknown precision %d", (int)p);
   XB_CUDA(cudaSetDevice(h->dev));
   ++h->calls;
+  ++h->queued;
   return factor_handle(h, p, true);
 }
 
@@ -778,6 +779,7 @@ extern "C" xbar_status xbar_solve(xbar_t h, int B, const double* V, double* I, d
   if (mixed && max_iter < 1) return fail(XBAR_EINVAL, "max_iter=%d < 1", max_iter);
   if (mixed && !(tol >= 0.0)) return fail(XBAR_EINVAL, "tol=%g must be >= 0", tol);
   XB_CUDA(cudaSetDevice(h->dev));
+  ++h->queued;
   MapDev& m = h->m;
   const int M = m.M, Mp = m.Mp, N = m.N;
   cudaStream_t st = h->st;
@@ -1213,6 +1215,7 @@ extern "C" xbar_status xbar_profile_read(xbar_t h, xbar_profile* out, int reset)
 extern "C" xbar_status xbar_set_conductances(xbar_t h, const double* G) {
   if (!h || !G) return fail(XBAR_EINVAL, "handle or G is NULL");
   XB_CUDA(cudaSetDevice(h->dev));
+  ++h->queued;
   MapDev& m = h->m;
   const size_t n = (size_t)m.M * m.N;
   const bool gdev = is_device_ptr(G);
@@ -1320,6 +1323,7 @@ extern "C" xbar_status xbar_solve_transfer(xbar_t h, int B, const double* V, dou
   if (B == 0) return XBAR_OK;
   if (!V || !I) return fail(XBAR_EINVAL, "V and I must not be NULL");
   XB_CUDA(cudaSetDevice(h->dev));
+  ++h->queued;
   const int M = h->m.M, N = h->m.N;
   cudaStream_t st = h->st;
   const bool vdev = is_device_ptr(V), idev = is_device_ptr(I);
@@ -1357,6 +1361,7 @@ extern "C" xbar_status xbar_solve_noalloc(xbar_t h, int B, const double* V, doub
   if (!is_device_ptr(V) || !is_device_ptr(I))
     return fail(XBAR_EINVAL, "xbar_solve_noalloc takes device pointers only (host buffers would need staging)");
   XB_CUDA(cudaSetDevice(h->dev));
+  ++h->queued;
   const MapDev& m = h->m;
   const int Bp = sweep_panel_width<double>(m.Mp, B, h->nsm);
   const int Bpad = ((B + Bp - 1) / Bp) * Bp;

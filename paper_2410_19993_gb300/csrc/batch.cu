@@ -57,6 +57,7 @@ struct xbar_batch_s {
   std::vector<int> sigB;
   std::vector<const void*> sigV, sigI;
   std::vector<unsigned long long> sig_epoch;  // graph_epoch of every tile
+  std::vector<unsigned long long> waited;     // direct calls of every tile (xbar_s::queued) that a run has waited for
   int sig_prec = -1, sig_iter = -1;
   double sig_tol = -1.0;
 };
@@ -114,6 +115,7 @@ extern "C" xbar_status xbar_batch_create(int T, const xbar_tile* desc, void* cud
     if (st != XBAR_OK) return bail(st);
     h->beside = T > 1;
     b->tiles.push_back(h);
+    b->waited.push_back(h->queued);
   }
   *out = b;
   return XBAR_OK;
@@ -169,6 +171,14 @@ extern "C" xbar_status xbar_batch_run(xbar_batch_t b, xbar_precision p, const in
            // the graph.  A tile blocked over rows is mirrored and assembled inside it and has no
            // elimination data of its own
            (b->tiles[t]->assembled == assembled_for(p) || (b->tiles[t]->orient_active && use_rows(b->tiles[t], p)));
+  // The graph runs on `origin`: it starts after the work that direct calls have queued on the tiles' own
+  // streams (asynchronous copies of new conductances, solves that use the same workspaces).
+  for (int t = 0; t < T; ++t) {
+    if (b->waited[t] == b->tiles[t]->queued) continue;
+    XB_CUDA(cudaEventRecord(b->joins[t], b->streams[t]));
+    XB_CUDA(cudaStreamWaitEvent(b->origin, b->joins[t], 0));
+    b->waited[t] = b->tiles[t]->queued;
+  }
   if (!same) {
     destroy_graph(b);
     // eager run: sizes every workspace and uploads the factor parameters

@@ -136,6 +136,7 @@ struct xbar_s {
   unsigned long long wait_ns = 0;  // limit of the device waits, 0 = the default (host copy)
   xbar_opts opt;
   unsigned long long calls = 0;  // xbar_factor and xbar_set_option calls: what they leave a captured graph does not know
+  unsigned long long queued = 0;  // direct calls that queue work on st: a graph replayed elsewhere waits for it
   // factor
   xbar::Buf X, fsig, fpbuf, fbar, fparams;
   // host copy of the parameter block last uploaded to `fparams` (skip identical uploads)

@@ -119,3 +119,23 @@ def test_solve_on_a_tile_after_new_conductances():
             Geff = torch.zeros((M, N), dtype=torch.float64, device="cuda")
             xbar._check(xbar.load().xbar_transfer_matrix(s.tile(t), 1e-9, 10, xbar._ptr(Geff), None))
             assert rel_err((s.V[t] @ Geff).cpu().numpy(), oracle.solve(M, N, s.maps[t][0], *R, s.maps[t][1])["I"]) <= 1e-10
+
+
+def test_run_follows_the_work_queued_on_a_tile():
+    """set_conductances from device memory returns before the tile's stream has stored the map; the next run,
+    a replay of the row-blocked tile's graph on another stream, uses the last map set."""
+    M, N, B = 256, 100, 4
+    s = Tiles("fp64", [(M, N, B)])
+    lib, old = xbar.load(), _dev(case(M, N, 1, None, seed=5)[0])
+    xbar._check(lib.xbar_set_option(s.tile(0), xbar.OPTIONS["eager_assembly"], 1))  # makes each call longer
+    s.run()
+    for k in range(3):
+        s.run()
+        G = case(M, N, 1, None, seed=20 + k)[0]
+        s.maps[0] = (G, s.maps[0][1])
+        new = _dev(G)
+        torch.cuda.synchronize()
+        for _ in range(150):  # a queue on the tile's stream that outlasts the run's start
+            lib.xbar_set_conductances(s.tile(0), xbar._ptr(old))
+        xbar._check(lib.xbar_set_conductances(s.tile(0), xbar._ptr(new)))
+    s.run()
