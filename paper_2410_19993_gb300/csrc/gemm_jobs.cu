@@ -358,7 +358,7 @@ __global__ void __launch_bounds__(NT / RPT * 32) gj_kernel(const GjJob<T>* __res
         for (int c = 0; c < CB; ++c) pr[k][c] = PR[b][k][tx + 32 * c];
       const int ck = P0 / 32, src = P0 & 31;
 #pragma unroll
-      for (int k = 0; k < PW; k += 2) {  // two pivots at a time: one reciprocal and one round of shuffles
+      for (int k = 0; k < PW; k += 2) {  // two pivots at a time: one round of shuffles
         T f0[PW], f1[PW];  // columns P0 + k, P0 + k + 1 of the 8 rows (lanes src + k, + 1, slot ck)
 #pragma unroll
         for (int l = 0; l < PW; ++l) {
@@ -370,12 +370,14 @@ __global__ void __launch_bounds__(NT / RPT * 32) gj_kernel(const GjJob<T>* __res
           f1[l] = __shfl_sync(0xffffffffu, v, src + k + 1);
         }
         const T p00 = f0[k], p01 = f1[k], p10 = f0[k + 1], p11 = f1[k + 1];
-        const T rd = (T)1 / fma(p00, p11, -p01 * p10);
+        // each pivot with its own reciprocal, the second one that of the Schur complement: solving for both rows
+        // by the 2 x 2 determinant rounds once more and errs by 3.9e-8 instead of 1.7e-8 (64 rows)
+        const T i0 = (T)1 / p00, t = p01 * i0, i1 = (T)1 / fma(-p10, t, p11);
 #pragma unroll
         for (int c = 0; c < CB; ++c) {
           const bool in0 = (tx == src + k) && (c == ck), in1 = (tx == src + k + 1) && (c == ck);
           const T r0 = in0 ? (T)1 : in1 ? (T)0 : pr[k][c], r1 = in1 ? (T)1 : in0 ? (T)0 : pr[k + 1][c];
-          const T g0 = fma(p11, r0, -p01 * r1) * rd, g1 = fma(p00, r1, -p10 * r0) * rd;
+          const T h0 = r0 * i0, g1 = fma(-p10, h0, r1) * i1, g0 = fma(-t, g1, h0);
 #pragma unroll
           for (int l = 0; l < PW; ++l) {
             if (l == k || l == k + 1) continue;
