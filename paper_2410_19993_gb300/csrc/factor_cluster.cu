@@ -405,10 +405,10 @@ __global__ void __launch_bounds__(kThreads, 1)
 
     // (4) blocked Gauss-Jordan inversion; panel p = rows of block p.
     // Pivot blocks are inverted in one warp's registers (Gauss-Jordan, no pivoting: the block is
-    // symmetric positive definite), two pivots at a time: one reciprocal (of the 2 x 2 determinant) and
-    // one exchange for both, on the chain from panel to panel.  Off-diagonal entries of a part have one
-    // sign, so the products of P^-1 [r0; r1] add without cancellation; the determinant cancels exactly as
-    // the second pivot would.  Lane l holds column l % 16 of rows 8 (l / 16) .. + 7.  The two pivot rows
+    // symmetric positive definite), two pivots at a time: one exchange for both, on the chain from panel to
+    // panel, and each pivot with its own reciprocal, the second one that of the Schur complement (solving
+    // for both rows by the 2 x 2 determinant needs one reciprocal, but rounds once more: 4.1e-8 instead of
+    // 1.7e-8 for the inverse of a 128-row block).  Lane l holds column l % 16 of rows 8 (l / 16) .. + 7.  The two pivot rows
     // go through shared memory and stand for the pivot columns too (the swept part is antisymmetric to
     // the rest): eight loads a step against 22 shuffles, which the one warp issues no faster than
     // one per eight cycles (2.5k cycles a block; 1.2k this way).
@@ -449,13 +449,13 @@ __global__ void __launch_bounds__(kThreads, 1)
         *reinterpret_cast<float4*>(c0 + 4) = *reinterpret_cast<const float4*>(rq + pa0 + 4);
         *reinterpret_cast<float4*>(c1) = *reinterpret_cast<const float4*>(rq + R + pa0);
         *reinterpret_cast<float4*>(c1 + 4) = *reinterpret_cast<const float4*>(rq + R + pa0 + 4);
-        const float rd = __fdividef(1.0f, fmaf(p00, p11, -p01 * p10));
+        const float i0 = __fdividef(1.0f, p00), t = p01 * i0, i1 = __fdividef(1.0f, fmaf(-p10, t, p11));
         // rows q, q+1 become P^-1 [r0; r1] (P^-1 itself in the pivot columns); all other rows lose their
         // pivot-column entries times those
         const bool in0 = ib == q, in1 = ib == q + 1;
         r0 = in0 ? 1.0f : in1 ? 0.0f : r0;
         r1 = in1 ? 1.0f : in0 ? 0.0f : r1;
-        const float f0 = fmaf(p11, r0, -p01 * r1) * rd, f1 = fmaf(p00, r1, -p10 * r0) * rd;
+        const float h0 = r0 * i0, f1 = fmaf(-p10, h0, r1) * i1, f0 = fmaf(-t, f1, h0);
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
           const float sgn = pa0 + e < q ? 1.0f : -1.0f;  // rows already swept: the column is minus the row

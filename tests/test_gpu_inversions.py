@@ -75,3 +75,50 @@ def test_panel_inversion(tmp_path):
             err += _error(dst.cpu().numpy().astype(np.float64), Z)
             ref += _error(_emulated(Z), Z)
         assert err <= BAR * ref, (n, err, ref)
+
+
+CLUSTER = """
+#include <string.h>
+#include "factor_cluster.cu"
+// a crossbar of one column: X = (off + the grounded diagonal)^-1
+extern "C" int cluster32(int n, const float* off, const double* h, const float* ones, float* X, float* work, void* par,
+                         unsigned* status) {
+  xbar::FactorParams p;
+  memset(&p, 0, sizeof(p));
+  p.M = p.Mp = n;
+  p.N = 1;
+  p.gw = 1.0;
+  p.Coff = off;
+  p.h = h;
+  p.X = X;
+  p.s32 = ones;
+  p.e32 = ones;
+  p.sig = work;
+  p.pbuf = work + 4 * n;
+  if (cudaMemcpy(par, &p, sizeof(p), cudaMemcpyHostToDevice)) return 1;
+  if (xbar::launch_factor_cluster((const xbar::FactorParams*)par, n, 1, 0, status, 0)) return 2;
+  return cudaDeviceSynchronize() ? 3 : 0;
+}
+extern "C" int cluster_work_floats(int n) { return 4 * n + (int)xbar::factor_cluster_pbuf_floats(n); }
+"""
+
+
+def test_cluster_inversion(tmp_path):
+    """The pivot blocks of the cluster factor (two to sixteen blocks a cluster)."""
+    lib = compile_probe(tmp_path, "cluster", CLUSTER)
+    for n in (32, 48, 64, 128, 144, 256):
+        err = ref = 0.0
+        for s in SEEDS:
+            off, rowsum = _block(n, np.random.default_rng(s))
+            Z = _matrix(off, rowsum)
+            X = torch.zeros((n, n), dtype=torch.float32, device="cuda")
+            work = torch.zeros(lib.cluster_work_floats(n), dtype=torch.float32, device="cuda")
+            par = torch.zeros(512, dtype=torch.uint8, device="cuda")
+            st = torch.zeros(4, dtype=torch.int32, device="cuda")
+            dev = [torch.from_numpy(a).cuda() for a in (off.astype(np.float32), rowsum, np.ones(n, dtype=np.float32))]
+            torch.cuda.synchronize()
+            assert lib.cluster32(n, *[ptr(d) for d in dev], ptr(X), ptr(work), ptr(par), ptr(st)) == 0
+            assert int(st[0]) == 0
+            err += _error(X.cpu().numpy().astype(np.float64), Z)
+            ref += _error(_emulated(Z), Z)
+        assert err <= BAR * ref, (n, err, ref)
