@@ -268,7 +268,7 @@ constexpr int kInitialTerms = 2;
 // Kernel variants.  FP32 substitutions run on the tensor cores (sweep_tc.cu) when the block fits
 // (Mp <= 256) and FP32 factors on a thread-block cluster (factor_cluster.cu) when 32 <= Mp <= 256,
 // unless the handle's options (xbar_set_option, set by the batch autotuner) or the environment
-// (XBAR_SWEEP=simt|tc, XBAR_FACTOR=group|cluster) choose otherwise.
+// (XBAR_SWEEP=simt|tc, XBAR_FACTOR=group|cluster; group: FP64 factors too) choose otherwise.
 bool xbar::use_tc_sweep(const xbar_s* h) {
   if (!sweep_tc_supported(h->m.Mp)) return false;
   const char* e = getenv("XBAR_SWEEP");
@@ -596,64 +596,40 @@ static xbar_status do_factor_cr(xbar_t h, bool equilibrate) {
   return XBAR_OK;
 }
 
-// FP64 block Thomas, eliminated from both ends (factor64.cu)
-static xbar_status do_factor64(xbar_t h) {
-  MapDev& m = h->m;
-  XB_CUDA(ensure(h->A, h->X, (size_t)m.N * m.Mp * m.Mp * sizeof(double)));
-  XB_CUDA(ensure(h->A, h->fpbuf, factor64_buf_bytes(m.Mp)));
-  XB_CUDA(ensure(h->A, h->fbar, factor64_flag_bytes()));
-  h->meet = factor64_meet(m.Mp, m.N);
-  Factor64Params fp;
-  fp.M = m.M;
-  fp.Mp = m.Mp;
-  fp.N = m.N;
-  fp.meet = h->meet;
-  fp.gsrc = m.gs;
-  fp.gw = m.gw;
-  fp.Coff = (const double*)m.Coff;
-  fp.h = m.h;
-  fp.X = (double*)h->X.p;
-  fp.buf = (double*)h->fpbuf.p;
-  fp.flags = (unsigned*)h->fbar.p;
-  fp.status = h->status;
-  fp.beside = h->beside;
-  PhaseScope ps(h, XBAR_PHASE_FACTOR, 1);
-  XB_CUDA(launch_factor64(fp, h->st));
-  h->tc_ready = 0;
-  return XBAR_OK;
-}
-
-static xbar_status do_factor32(xbar_t h, bool upload) {
+// Block Thomas by the cluster kernel (FP32 where it fits) or the group kernel, equilibrated in FP32
+template <typename T>
+static xbar_status do_factor_thomas(xbar_t h, bool upload) {
   MapDev& m = h->m;
   const int Mp = m.Mp, N = m.N;
+  constexpr bool f32 = sizeof(T) == 4;
   const int PB = factor_panel_width();
-  // latency-bound: few blocks (cheap cross-block barriers) with 16 rows each
-  int bpm = Mp <= 32 ? 1 : std::min(h->nsm, Mp / 16);
-  if (bpm < 1) bpm = 1;
-  XB_CUDA(ensure(h->A, h->X, (size_t)N * Mp * Mp * sizeof(float)));
-  XB_CUDA(ensure(h->A, h->fsig, 4 * (size_t)Mp * sizeof(float)));
+  // blocks of the group: FP64 needs many SMs (the FP64 pipe is 1/64 of FP32); FP32 is latency-bound, so fewer
+  // (cheap cross-block barriers), 16 rows each
+  const int blocks = Mp <= 32 ? 1 : std::max(1, std::min(h->nsm, Mp / (f32 ? 16 : 2)));
+  XB_CUDA(ensure(h->A, h->X, (size_t)N * Mp * Mp * sizeof(T)));
+  XB_CUDA(ensure(h->A, h->fsig, 4 * (size_t)Mp * sizeof(T)));
   size_t pbuf_n = 2 * (size_t)PB * Mp;
-  if (factor_cluster_supported(Mp)) pbuf_n = std::max(pbuf_n, factor_cluster_pbuf_floats(Mp));
-  XB_CUDA(ensure(h->A, h->fpbuf, pbuf_n * sizeof(float)));
+  if (f32 && factor_cluster_supported(Mp)) pbuf_n = std::max(pbuf_n, factor_cluster_pbuf_floats(Mp));
+  XB_CUDA(ensure(h->A, h->fpbuf, pbuf_n * sizeof(T)));
   XB_CUDA(ensure(h->A, h->fbar, 2 * sizeof(unsigned)));
-  XB_CUDA(ensure(h->A, h->fparams, sizeof(FactorParams)));
+  XB_CUDA(ensure(h->A, h->fparams, sizeof(FactorParams<T>)));
   // the cluster factor eliminates from both ends, the group factor from column 0 to N - 1
-  const bool cluster = use_cluster_factor(h);
+  const bool cluster = f32 && use_cluster_factor(h);
   h->meet = cluster ? (N - 1) / 2 : N - 1;
-  FactorParams fp;
+  FactorParams<T> fp;
   memset(&fp, 0, sizeof(fp));  // padding too: the block is compared byte for byte below
   fp.M = m.M;
   fp.Mp = Mp;
   fp.N = N;
   fp.gsrc = m.gs;
   fp.gw = m.gw;
-  fp.Coff = (const float*)m.Coff;
+  fp.Coff = (const T*)m.Coff;
   fp.h = m.h;
-  fp.s = m.s_eq;
-  fp.e = m.e_eq;
-  fp.X = (float*)h->X.p;
-  fp.sig = (float*)h->fsig.p;
-  fp.pbuf = (float*)h->fpbuf.p;
+  fp.s = f32 ? m.s_eq : nullptr;
+  fp.e = f32 ? m.e_eq : m.e_pl;
+  fp.X = (T*)h->X.p;
+  fp.sig = (T*)h->fsig.p;
+  fp.pbuf = (T*)h->fpbuf.p;
   fp.bar = (unsigned*)h->fbar.p;
   fp.meet = h->meet;
   fp.s32 = m.s32;
@@ -674,17 +650,48 @@ static xbar_status do_factor32(xbar_t h, bool upload) {
       h->fparams_dev = h->fparams.p;
     }
   }
-  PhaseScope ps(h, XBAR_PHASE_FACTOR, (cluster ? factor_cluster_launches(N) : 1) + (use_tc_sweep(h) ? 1 : 0));
+  const bool tile = f32 && use_tc_sweep(h);
+  PhaseScope ps(h, XBAR_PHASE_FACTOR, (cluster ? factor_cluster_launches(N) : 1) + (tile ? 1 : 0));
   if (cluster)
-    XB_CUDA(launch_factor_cluster((const FactorParams*)h->fparams.p, Mp, N, h->meet, h->status, h->st));
+    XB_CUDA(launch_factor_cluster((const FactorParams<float>*)h->fparams.p, Mp, N, h->meet, h->status, h->st));
   else
-    XB_CUDA(launch_factor((const FactorParams*)h->fparams.p, 1, Mp, bpm, h->status, h->st));
+    XB_CUDA(launch_factor<T>((const FactorParams<T>*)h->fparams.p, Mp, blocks, h->status, h->st));
   h->tc_ready = 0;
-  if (use_tc_sweep(h)) {
+  if (tile) {
     XB_CUDA(ensure(h->A, h->Xt, sweep_tc_tile_bytes(Mp, N)));
     XB_CUDA(launch_sweep_tc_tile((const float*)h->X.p, h->Xt.p, Mp, N, h->st));
     h->tc_ready = 1;
   }
+  return XBAR_OK;
+}
+
+// FP64 block Thomas, eliminated from both ends (factor64.cu) where its blocks fit the device at once
+static xbar_status do_factor64(xbar_t h, bool upload) {
+  MapDev& m = h->m;
+  const char* e = getenv("XBAR_FACTOR");
+  const Factor64Plan plan = factor64_plan(m.Mp, m.N, h->nsm, h->beside);
+  if (!plan.rows || (e && strcmp(e, "group") == 0)) return do_factor_thomas<double>(h, upload);
+  XB_CUDA(ensure(h->A, h->X, (size_t)m.N * m.Mp * m.Mp * sizeof(double)));
+  XB_CUDA(ensure(h->A, h->fpbuf, factor64_buf_bytes(m.Mp)));
+  XB_CUDA(ensure(h->A, h->fbar, factor64_flag_bytes()));
+  h->meet = plan.meet;
+  Factor64Params fp;
+  fp.M = m.M;
+  fp.Mp = m.Mp;
+  fp.N = m.N;
+  fp.meet = plan.meet;
+  fp.rows = plan.rows;
+  fp.gsrc = m.gs;
+  fp.gw = m.gw;
+  fp.Coff = (const double*)m.Coff;
+  fp.h = m.h;
+  fp.X = (double*)h->X.p;
+  fp.buf = (double*)h->fpbuf.p;
+  fp.flags = (unsigned*)h->fbar.p;
+  fp.status = h->status;
+  PhaseScope ps(h, XBAR_PHASE_FACTOR, 1);
+  XB_CUDA(launch_factor64(fp, h->st));
+  h->tc_ready = 0;
   return XBAR_OK;
 }
 
@@ -716,7 +723,7 @@ xbar_status xbar::factor_handle(xbar_s* h, xbar_precision p, bool upload_params)
   h->tc_ready = 0;
   xbar_status s;
   if (cr) s = (p == XBAR_FP64) ? do_factor_cr<double>(h, false) : do_factor_cr<float>(h, true);
-  else s = (p == XBAR_FP64) ? do_factor64(h) : do_factor32(h, upload_params);
+  else s = (p == XBAR_FP64) ? do_factor64(h, upload_params) : do_factor_thomas<float>(h, upload_params);
   if (s != XBAR_OK) return s;
   h->cr_active = cr ? 1 : 0;
   h->prec = p;

@@ -630,10 +630,6 @@ __global__ void __launch_bounds__(256, 1) factor64_kernel(Factor64Params p) {
   }
 }
 
-// Meeting in the middle: both chains equally long, the left one with the meeting column.  Above 512
-// rows one chain already takes 128 blocks of 8 rows, which two chains could not share the SMs with.
-int factor64_meet(int Mp, int N) { return Mp <= 512 ? (N - 1) / 2 : N - 1; }
-
 size_t factor64_buf_bytes(int Mp) {
   return (Mp == kPB ? (size_t)Mp : 2 * chain_doubles(Mp)) * sizeof(double);
 }
@@ -658,13 +654,8 @@ cudaError_t launch_factor64(const Factor64Params& p, cudaStream_t st) {
     cfg.numAttrs = chains > 1 ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, factor64_small_kernel, p);
   }
-  // rows per worker block: as many workers as two chains can keep resident, 64 a chain at 128 and at
-  // 256 rows (the FP64 work of a panel then takes no longer than its pivot chain), and 8 rows above
-  // (128 workers for the one chain of 1024 rows)
-  // The tiles of a batch share the SMs, a block fills one, and a factor starts when all its blocks fit at
-  // once: with 8 rows a worker four times as many tiles run side by side.  256 x 256, one vector, as four
-  // 128-row tiles 17.5 -> 5.1 ms, as sixteen of 64 rows 9.6 -> 3.2, as 64 of 32 rows 6.7 -> 3.7.
-  const int R = Mp > 256 || p.beside ? 8 : Mp <= 128 ? 2 : 4, KC = Mp <= 256 ? 1 : Mp <= 512 ? 2 : 4;
+  const int R = p.rows, KC = Mp <= 256 ? 1 : Mp <= 512 ? 2 : 4;
+  if (R != 8 && (Mp > 256 || (R != 4 && (R != 2 || Mp > 128)))) return cudaErrorInvalidValue;
   cfg.gridDim = dim3(chains * (Mp / R + 1));
   const int cols = (Mp + KC - 1) / KC;
   cfg.blockDim = dim3(R == 8 || cols > 192 ? 256 : 192);

@@ -178,9 +178,9 @@ __device__ __forceinline__ void rank16_update(float (&acc)[2][16], const float* 
 // Cluster c of the grid walks chain chain0 + c; kMeet: one cluster, the meeting column.
 template <bool kMeet>
 __global__ void __launch_bounds__(kThreads, 1)
-    factor_cluster_kernel(const FactorParams* __restrict__ params, int C, int chain0, unsigned* status) {
+    factor_cluster_kernel(const FactorParams<float>* __restrict__ params, int C, int chain0, unsigned* status) {
   constexpr int R = kRows;  // rows per block = panel width
-  const FactorParams p = *params;
+  const FactorParams<float> p = *params;
   const uint32_t g = cluster_rank();
   const int M = p.M, Mp = p.Mp, N = p.N, m = p.meet;
   const int chain = kMeet ? 0 : chain0 + (int)blockIdx.x / C;
@@ -648,12 +648,10 @@ __global__ void __launch_bounds__(kThreads, 1)
 
 bool factor_cluster_supported(int Mp) { return Mp >= 2 * kRows && Mp <= 16 * kRows && Mp % kRows == 0; }
 
-int factor_cluster_size(int Mp) { return Mp / kRows; }
-
 int factor_cluster_launches(int N) { return N > 1 ? 2 : 1; }
 
 template <bool kMeet>
-static cudaError_t launch_clusters(const FactorParams* params, int C, int clusters, int chain0, size_t smem,
+static cudaError_t launch_clusters(const FactorParams<float>* params, int C, int clusters, int chain0, size_t smem,
                                    unsigned* status, cudaStream_t st) {
   cudaError_t err = cudaFuncSetAttribute(factor_cluster_kernel<kMeet>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
@@ -677,10 +675,10 @@ static cudaError_t launch_clusters(const FactorParams* params, int C, int cluste
 
 // the chains (those that have columns), then the meeting column; the launch boundary is what the
 // second waits for, so no cluster waits for another
-cudaError_t launch_factor_cluster(const FactorParams* params_dev, int Mp, int N, int meet, unsigned* status,
+cudaError_t launch_factor_cluster(const FactorParams<float>* params_dev, int Mp, int N, int meet, unsigned* status,
                                   cudaStream_t st) {
   if (meet < 0 || meet >= N) return cudaErrorInvalidValue;
-  const int C = factor_cluster_size(Mp);
+  const int C = Mp / kRows;
   const size_t smem = factor_cluster_smem_bytes(Mp);
   const bool left = meet > 0, right = meet < N - 1;
   if (left || right) {

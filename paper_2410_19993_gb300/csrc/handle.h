@@ -140,7 +140,7 @@ struct xbar_s {
   // factor
   xbar::Buf X, fsig, fpbuf, fbar, fparams;
   // host copy of the parameter block last uploaded to `fparams` (skip identical uploads)
-  unsigned char fparams_host[sizeof(xbar::FactorParams)] = {};
+  unsigned char fparams_host[sizeof(xbar::FactorParams<double>)] = {};
   size_t fparams_bytes = 0;
   const void* fparams_dev = nullptr;
   xbar::Buf Xt;    // tensor-core tiled TF32 hi/lo copy of the FP32 factor

@@ -51,32 +51,56 @@ cudaError_t launch_store_g(const MapDev& m, const double* G_dev, unsigned* statu
 cudaError_t launch_assemble(const MapDev& m, bool f32, cudaStream_t st);
 
 // ---- factor -----------------------------------------------------------------------------------
-struct FactorParams {  // FP32 factors
+template <typename T>
+struct FactorParams {  // factor.cu, factor_cluster.cu
   int M, Mp, N;
   double gsrc, gw;
-  const float* Coff;
+  const T* Coff;
   const double* h;
   const double* s;    // nullptr = no equilibration
   const double* e;
-  float* X;           // [N][Mp][Mp] output
-  float* sig;         // scratch: [2][Mp] (factor.cu), [2 chains][2][Mp] (factor_cluster.cu)
-  float* pbuf;        // scratch: [2][PB][Mp] (factor.cu), factor_cluster_pbuf_floats (factor_cluster.cu)
+  T* X;               // [N][Mp][Mp] output
+  T* sig;             // scratch: [2][Mp] (factor.cu), [2 chains][2][Mp] (factor_cluster.cu)
+  T* pbuf;            // scratch: [2][PB][Mp] (factor.cu), factor_cluster_pbuf_floats (factor_cluster.cu)
   unsigned* bar;      // 2 words, zeroed
   int meet;           // factor_cluster.cu: column in which its two elimination chains meet
   const float* s32;   // factor_cluster.cu: s and e in FP32
   const float* e32;
 };
 
-// FP32 factor (factor.cu): one group of `blocks_per_map` co-resident blocks factors each map; `maps`
-// is a device array.
-cudaError_t launch_factor(const FactorParams* maps_dev, int nmaps, int Mp_max, int blocks_per_map,
-                          unsigned* status, cudaStream_t st);
+// factor.cu: a group of `blocks` co-resident blocks (any number; rows in shared memory), one chain
+template <typename T>
+cudaError_t launch_factor(const FactorParams<T>* params_dev, int Mp, int blocks, unsigned* status, cudaStream_t st);
 int factor_panel_width();
 
 // FP64 factor (factor64.cu): two chains that meet in column `meet` (left 0 .. meet - 1, right N - 1 ..
-// meet + 1); Mp <= 1024.  One cooperative launch; `flags` is cleared by it.
+// meet + 1; meet = N - 1: one chain); Mp <= 1024.  One cooperative launch; `flags` is cleared by it.
+//
+// A chain takes a pivot block and Mp / rows worker blocks (at 16 rows one block in all), and every block of the
+// launch fills an SM.  The plan for a device of nsm SMs:
+//   * rows per worker: as few as two chains can keep resident, 64 workers a chain at 128 and at 256 rows
+//     (the FP64 work of a panel then takes no longer than its pivot chain), and 8 rows above.  `beside`: the
+//     tiles of a batch share the SMs and a factor starts when all its blocks fit at once, so with 8 rows
+//     four times as many tiles run side by side.  256 x 256, one vector, as four 128-row tiles 17.5 -> 5.1 ms,
+//     as sixteen of 64 rows 9.6 -> 3.2;
+//   * both chains equally long, the left one with the meeting column.  Above 512 rows one chain already takes
+//     more than half of the SMs, and there is only that;
+//   * with fewer SMs 8 rows, then one chain, then no plan (rows = 0): the group kernel of factor.cu.
+struct Factor64Plan {
+  int rows = 0, meet = 0;
+};
+inline int factor64_blocks(int Mp, int N, Factor64Plan f) {
+  return (f.meet < N - 1 ? 2 : 1) * (Mp == 16 ? 1 : Mp / f.rows + 1);
+}
+inline Factor64Plan factor64_plan(int Mp, int N, int nsm, bool beside) {
+  const int first = Mp > 256 || beside ? 8 : Mp <= 128 ? 2 : 4, two = (N - 1) / 2;
+  const Factor64Plan plans[3] = {{first, Mp <= 512 ? two : N - 1}, {8, Mp <= 512 ? two : N - 1}, {8, N - 1}};
+  for (const Factor64Plan& f : plans)
+    if (factor64_blocks(Mp, N, f) <= nsm) return f;
+  return {};
+}
 struct Factor64Params {
-  int M, Mp, N, meet;
+  int M, Mp, N, meet, rows;
   double gsrc, gw;
   const double* Coff;
   const double* h;
@@ -84,19 +108,16 @@ struct Factor64Params {
   double* buf;        // factor64_buf_bytes scratch
   unsigned* flags;    // factor64_flag_bytes
   unsigned* status;
-  bool beside;        // other factors run beside this one: fewer, larger worker blocks
 };
-int factor64_meet(int Mp, int N);  // the meeting column
 size_t factor64_buf_bytes(int Mp);
 size_t factor64_flag_bytes();
 cudaError_t launch_factor64(const Factor64Params& p, cudaStream_t st);
 
 // FP32 factor on a thread-block cluster (factor_cluster.cu): 32 <= Mp <= 256
 bool factor_cluster_supported(int Mp);
-int factor_cluster_size(int Mp);
 size_t factor_cluster_pbuf_floats(int Mp);  // panel-slot scratch (FactorParams::pbuf)
 int factor_cluster_launches(int N);
-cudaError_t launch_factor_cluster(const FactorParams* params_dev, int Mp, int N, int meet, unsigned* status,
+cudaError_t launch_factor_cluster(const FactorParams<float>* params_dev, int Mp, int N, int meet, unsigned* status,
                                   cudaStream_t st);
 
 // ---- sweeps (forward + back substitution, current extraction) ---------------------------------

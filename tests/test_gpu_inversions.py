@@ -83,7 +83,7 @@ CLUSTER = """
 // a crossbar of one column: X = (off + the grounded diagonal)^-1
 extern "C" int cluster32(int n, const float* off, const double* h, const float* ones, float* X, float* work, void* par,
                          unsigned* status) {
-  xbar::FactorParams p;
+  xbar::FactorParams<float> p;
   memset(&p, 0, sizeof(p));
   p.M = p.Mp = n;
   p.N = 1;
@@ -96,7 +96,7 @@ extern "C" int cluster32(int n, const float* off, const double* h, const float* 
   p.sig = work;
   p.pbuf = work + 4 * n;
   if (cudaMemcpy(par, &p, sizeof(p), cudaMemcpyHostToDevice)) return 1;
-  if (xbar::launch_factor_cluster((const xbar::FactorParams*)par, n, 1, 0, status, 0)) return 2;
+  if (xbar::launch_factor_cluster((const xbar::FactorParams<float>*)par, n, 1, 0, status, 0)) return 2;
   return cudaDeviceSynchronize() ? 3 : 0;
 }
 extern "C" int cluster_work_floats(int n) { return 4 * n + (int)xbar::factor_cluster_pbuf_floats(n); }
