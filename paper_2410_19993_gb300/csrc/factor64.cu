@@ -308,6 +308,7 @@ __device__ void pivot_chain(const Factor64Params& p, int chain, int nsteps, int 
     bool ok = true;
     if (lane == 0) ok = wait_count(fS + q * kFlagStride, (unsigned)(s + 1) * owners, p.flags, p.status, limit);
     ok = __shfl_sync(0xffffffffu, ok, 0);
+    __syncwarp();  // lane 0's acquire orders the other lanes' reads (a shuffle orders no memory)
     if (!ok) {
       if (lane == 0) fail = 1;
       return;
