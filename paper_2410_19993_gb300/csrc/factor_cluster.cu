@@ -50,9 +50,7 @@ __device__ __forceinline__ uint32_t cluster_rank() {
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
   return r;
 }
-__device__ __forceinline__ void cluster_arrive_relaxed() {
-  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
-}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -620,10 +618,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (!kMeet && colt)
 #pragma unroll
       for (int c = 0; c < 2; ++c) sg_prev[c] = __ldcg(sig + (size_t)(s & 1) * Mp + kc[c]);
-    // every block's reads of this step's slots and blocks are done (their values are used) before the next
-    // step's first hand-over: arrive here, wait there, with the next column's formation in between; nothing
-    // this block wrote is published by it, so the arrival need not wait for its stores
-    cluster_arrive_relaxed();
+    // every block's reads of this step's slots and blocks come before the next step's first hand-over: arrive
+    // here (release: a relaxed arrival would not order the reads), wait there, with the next column's
+    // formation in between
+    cluster_arrive();
   }
   {
     if (colt)
