@@ -384,10 +384,10 @@ __global__ void cr_zero_pad_kernel(int M, int Mp, int Bpad, T* r) {
 template <typename T>
 __global__ void cr_l0_fwd_kernel(int Mp, int N, int Bpad, const T* __restrict__ e, const T* __restrict__ y, T* r) {
   // threads over the rows and vectors of a block together: one vector fills them as well as many
-  const int t = blockIdx.x * blockDim.x + threadIdx.x, p = 2 * blockIdx.y;
-  if (t >= Mp * Bpad) return;
-  const int i = t / Bpad;
-  const size_t col = (size_t)Mp * Bpad;
+  const size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x, col = (size_t)Mp * Bpad;  // may pass 2^31
+  const int p = 2 * blockIdx.y;
+  if (t >= col) return;
+  const int i = (int)(t / Bpad);
   const size_t o = (size_t)p * col + t;
   T v = r[o];
   if (p > 0) v += e[(size_t)(p - 1) * Mp + i] * y[o - col];
@@ -936,7 +936,7 @@ cudaError_t cr_sweep(xbar_s* hd, CrPlan<T>& pl, const CrSweepArgs<T>& a) {
     if (o.kind == CR_OP_GEMM) {
       e = Bpad <= 16 ? launch_gemv_jobs<T>(jobs + o.off, o.cnt, o.m, Bpad, st) : cr_run_gemm<T>(hd, pl, jobs, o);
     } else if (o.kind == CR_OP_L0FWD) {
-      cr_l0_fwd_kernel<T><<<dim3((Mp * Bpad + 127) / 128, o.cnt), 128, 0, st>>>(Mp, N, Bpad, e_cpl, a.x, a.r);
+      cr_l0_fwd_kernel<T><<<dim3((unsigned)(((size_t)Mp * Bpad + 127) / 128), o.cnt), 128, 0, st>>>(Mp, N, Bpad, e_cpl, a.x, a.r);
       e = cudaGetLastError();
     }
     if (e != cudaSuccess) return e;

@@ -42,12 +42,13 @@ __global__ void mirror_gc_kernel(const double* __restrict__ Gc, int M, int Mp, i
 // the rows and vectors of a block together, so that one vector fills them as well as many.
 __global__ void orient_rhs_kernel(const double* __restrict__ V, const double* __restrict__ h2, int M, int M2,
                                   int Mp2, int B, int Bpad, double* __restrict__ rhs) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x, j2 = blockIdx.y;
-  if (t >= Mp2 * Bpad) return;
-  const int i2 = t / Bpad, b = t - i2 * Bpad;
+  const size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x, blk = (size_t)Mp2 * Bpad;  // may pass 2^31
+  const int j2 = blockIdx.y;
+  if (t >= blk) return;
+  const int i2 = (int)(t / Bpad), b = (int)(t - (size_t)i2 * Bpad);
   double v = 0.0;
   if (b < B && i2 < M2) v = V[(size_t)b * M + (M - 1 - j2)] * h2[(size_t)j2 * Mp2 + i2];
-  rhs[(size_t)j2 * Mp2 * Bpad + t] = v;
+  rhs[j2 * blk + t] = v;
 }
 
 // I[b][j] = g_s' w'[0][N-1-j][b]
@@ -186,8 +187,7 @@ cudaError_t launch_mirror_gc(const double* Gc, int M, int Mp, int N, double* Gc2
 
 cudaError_t launch_orient_rhs(const double* V, const double* h2, int M, int M2, int Mp2, int B, int Bpad,
                               double* rhs, cudaStream_t st) {
-  if ((long long)Mp2 * Bpad > 0x7fffff00ll) return cudaErrorInvalidValue;
-  orient_rhs_kernel<<<dim3((Mp2 * Bpad + 127) / 128, M), 128, 0, st>>>(V, h2, M, M2, Mp2, B, Bpad, rhs);
+  orient_rhs_kernel<<<dim3((unsigned)(((size_t)Mp2 * Bpad + 127) / 128), M), 128, 0, st>>>(V, h2, M, M2, Mp2, B, Bpad, rhs);
   return cudaGetLastError();
 }
 
