@@ -334,7 +334,7 @@ static xbar_status factor_mirror(xbar_s* h, xbar_precision p) {
   xbar_s* g = h->mirror;
   g->opt = h->opt;
   g->opt.orient = 0;
-  g->beside = h->beside;
+  g->tiles = h->tiles;
   // automatic algorithm: the mirror's many small blocks (M blocks of N rows) are what cyclic
   // reduction is for, against M dependent block steps of block Thomas
   if (h->opt.algo < 0 && cr_supported(g->m.Mp, g->m.N)) g->opt.algo = 1;
@@ -669,7 +669,7 @@ static xbar_status do_factor_thomas(xbar_t h, bool upload) {
 static xbar_status do_factor64(xbar_t h, bool upload) {
   MapDev& m = h->m;
   const char* e = getenv("XBAR_FACTOR");
-  const Factor64Plan plan = factor64_plan(m.Mp, m.N, h->nsm, h->beside);
+  const Factor64Plan plan = factor64_plan(m.Mp, m.N, h->nsm, h->tiles > 1);
   if (!plan.rows || (e && strcmp(e, "group") == 0)) return do_factor_thomas<double>(h, upload);
   XB_CUDA(ensure(h->A, h->X, (size_t)m.N * m.Mp * m.Mp * sizeof(double)));
   XB_CUDA(ensure(h->A, h->fpbuf, factor64_buf_bytes(m.Mp)));
@@ -1084,7 +1084,7 @@ extern "C" xbar_status xbar_solve(xbar_t h, int B, const double* V, double* I, d
 }
 
 xbar_status xbar::solve_device_driven(xbar_s* h, int B, const double* dV, double* dI, double tol, int max_iter,
-                                      bool allow_alloc, bool beside) {
+                                      bool allow_alloc, int tiles) {
   MapDev& m = h->m;
   const int M = m.M, Mp = m.Mp, N = m.N;
   cudaStream_t st = h->st;
@@ -1101,7 +1101,7 @@ xbar_status xbar::solve_device_driven(xbar_s* h, int B, const double* dV, double
     return fail(XBAR_ESTATE, "device-driven solves (tile batches) need a block-Thomas factorization");
   const bool mixed = h->prec == XBAR_FP32_IR;
   SweepKind kind = sweep_kind(h, B, mixed);
-  kind.beside = beside;
+  kind.beside = tiles > 1;
   const int Bp = kind.Bp;
   const int Bpad = ((B + Bp - 1) / Bp) * Bp;
   const size_t nst = (size_t)N * Mp * Bpad;
@@ -1133,7 +1133,7 @@ xbar_status xbar::solve_device_driven(xbar_s* h, int B, const double* dV, double
   rp.w = (double*)h->w64.p; rp.dhat = (const float*)h->dhat.p; rp.phi = (double*)h->phi.p;
   rp.w2 = (float2*)h->w64.p; rp.phi2 = (float2*)h->phi.p;
   rp.Gc2 = m.Gc2; rp.h2 = m.h2; rp.tha2 = m.tha2; rp.thc2 = m.thc2;
-  rp.rhat = (float*)h->rhat.p; rp.rmax = &state->rmax;
+  rp.rhat = (float*)h->rhat.p; rp.rmax = &state->rmax; rp.tiles = tiles;
   SweepParams<float> sp;
   sp.M = M; sp.Mp = Mp; sp.N = N; sp.B = B; sp.Bp = Bp; sp.Bpad = Bpad;
   sp.X = (const float*)h->X.p; sp.e = m.e32; sp.hs = m.hs32; sp.src = m.src32;

@@ -113,7 +113,7 @@ extern "C" xbar_status xbar_batch_create(int T, const xbar_tile* desc, void* cud
     const xbar_tile& d = desc[t];
     xbar_status st = xbar_assemble(d.M, d.N, d.G, d.R_s, d.R_w, d.R_b, d.R_sense, s, &h);
     if (st != XBAR_OK) return bail(st);
-    h->beside = T > 1;
+    h->tiles = T;
     b->tiles.push_back(h);
     b->waited.push_back(h->queued);
   }
@@ -137,7 +137,7 @@ static xbar_status enqueue_all(xbar_batch_t b, xbar_precision p, const int* B, c
     xbar_status s = factor_handle(h, p, eager);
     if (s != XBAR_OK) return s;
     if (B[t] > 0) {
-      s = solve_device_driven(h, B[t], V[t], I[t], tol, max_iter, eager, b->T > 1);
+      s = solve_device_driven(h, B[t], V[t], I[t], tol, max_iter, eager, b->T);
       if (s != XBAR_OK) return s;
     }
     XB_CUDA(cudaEventRecord(b->joins[t], b->streams[t]));
@@ -362,7 +362,7 @@ extern "C" xbar_status xbar_batch_autotune(xbar_batch_t b, xbar_precision p, con
         h->opt.sweep = sw;
         if (sw == 1 && !use_tc_sweep(h)) continue;
         if (factor_handle(h, p, true) != XBAR_OK) continue;
-        v.sweep_ms[sw] = time_ms(h->st, [&]() { return solve_device_driven(h, k.B, dV, dI, 1e-8, 2, true, b->T > 1); });
+        v.sweep_ms[sw] = time_ms(h->st, [&]() { return solve_device_driven(h, k.B, dV, dI, 1e-8, 2, true, b->T); });
       }
       v.sweep = (v.sweep_ms[1] >= 0 && (v.sweep_ms[0] < 0 || v.sweep_ms[1] <= v.sweep_ms[0])) ? 1 : 0;
       h->opt.factor = save_f;
@@ -384,7 +384,7 @@ extern "C" xbar_status xbar_batch_autotune(xbar_batch_t b, xbar_precision p, con
         h->opt.orient = o;
         v.orient_ms[o] = time_ms(h->st, [&]() {
           xbar_status s = factor_handle(h, p, true);
-          return s != XBAR_OK ? s : solve_device_driven(h, k.B, dV, dI, 1e-8, 0, true, b->T > 1);
+          return s != XBAR_OK ? s : solve_device_driven(h, k.B, dV, dI, 1e-8, 0, true, b->T);
         });
       }
       v.orient = (v.orient_ms[1] >= 0 && (v.orient_ms[0] < 0 || v.orient_ms[1] < v.orient_ms[0])) ? 1 : 0;

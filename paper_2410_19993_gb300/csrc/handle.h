@@ -125,7 +125,7 @@ struct xbar_s {
   double R[4] = {0, 0, 0, 0};
   cudaStream_t st = nullptr;
   int dev = 0, nsm = 0;
-  bool beside = false;  // a tile of a batch: other tiles' factors and solves run beside this one's
+  int tiles = 1;  // tiles of the batch this handle is one of: their factors and solves run beside this one's
   // per-column elimination data formed from Gc (lazily, by the first factor): 0 = no, else with the
   // column blocks in the precision p of the factors, assembled_for(p)
   int assembled = 0;
@@ -231,8 +231,8 @@ bool use_rows(const xbar_s* h, xbar_precision p);
 // currents-only solve with device pointers, refinement driven on the device: exactly
 // `max_iter` refinement passes are enqueued and passes after convergence skip their work; no
 // host synchronisation (capturable).  The workspace must have been sized by an earlier call.
-// beside: other tiles' solves run beside this one.
+// tiles: solves of this size that run side by side (those of a batch), this one among them.
 xbar_status solve_device_driven(xbar_s* h, int B, const double* V, double* I, double tol, int max_iter,
-                                bool allow_alloc, bool beside);
+                                bool allow_alloc, int tiles);
 
 }  // namespace xbar

@@ -293,6 +293,7 @@ bool cr_supported(int Mp, int N);
 // ---- FP64 refinement kernels and node voltages ------------------------------------------------
 struct ResidParams {
   int M, Mp, N, B, Bpad;
+  int tiles;            // solves of about this size that run side by side (0 or 1: this one alone)
   double gs, gw;
   double gb, go;        // bit-line segment and sense conductances (bit-line sources only)
   const double* Gc;
