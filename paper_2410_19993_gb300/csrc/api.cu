@@ -225,6 +225,9 @@ static int sweep_launches(int meet, int N, bool V, bool few = false) {
 // The substitution kernel of a block-Thomas factor for a batch: clusters for a few vectors
 // (sweep_few.cu), otherwise the tensor cores (mixed precision, sweep_tc.cu) or the CUDA cores.  An
 // explicit choice of the FP32 kernel (XBAR_OPT_SWEEP_KERNEL, XBAR_SWEEP) is kept.
+// tiles: solves of about this size side by side.  Their clusters have small blocks, several of which share an
+// SM, so they may take four times the SMs between them: 64 tiles of 32 x 32 in mixed precision with one vector
+// each 2.51 ms a run (2.70 on the tensor cores), with 64 vectors 4.40 against 2.70 ms, which is beyond it.
 struct SweepKind {
   FewPlan few;
   bool tc = false;
@@ -232,12 +235,12 @@ struct SweepKind {
   int nsm = 0;
   bool beside = false;  // other solves run beside this one
 };
-static SweepKind sweep_kind(const xbar_s* h, int B, bool mixed) {
+static SweepKind sweep_kind(const xbar_s* h, int B, bool mixed, int tiles = 1) {
   SweepKind k;
   k.nsm = h->nsm;
   const char* e = getenv("XBAR_SWEEP");
   const bool chosen = mixed && (h->opt.sweep >= 0 || (e && (strcmp(e, "simt") == 0 || strcmp(e, "tc") == 0)));
-  if (!chosen) k.few = sweep_few_plan(h->m.Mp, B, h->nsm);
+  if (!chosen) k.few = sweep_few_plan(h->m.Mp, B, std::min(h->nsm, 4 * h->nsm / std::max(1, tiles)));
   k.tc = mixed && h->tc_ready && !k.few.nv;
   k.Bp = k.few.nv ? k.few.nv
          : k.tc   ? kSweepTcPanel
@@ -1100,7 +1103,7 @@ xbar_status xbar::solve_device_driven(xbar_s* h, int B, const double* dV, double
   if (h->cr_active)
     return fail(XBAR_ESTATE, "device-driven solves (tile batches) need a block-Thomas factorization");
   const bool mixed = h->prec == XBAR_FP32_IR;
-  SweepKind kind = sweep_kind(h, B, mixed);
+  SweepKind kind = sweep_kind(h, B, mixed, tiles);
   kind.beside = tiles > 1;
   const int Bp = kind.Bp;
   const int Bpad = ((B + Bp - 1) / Bp) * Bp;
