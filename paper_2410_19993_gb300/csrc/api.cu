@@ -233,11 +233,12 @@ struct SweepKind {
   bool tc = false;
   int Bp = 0;  // vectors per panel
   int nsm = 0;
-  bool beside = false;  // other solves run beside this one
+  int tiles = 1;  // solves side by side
 };
 static SweepKind sweep_kind(const xbar_s* h, int B, bool mixed, int tiles = 1) {
   SweepKind k;
   k.nsm = h->nsm;
+  k.tiles = tiles;
   const char* e = getenv("XBAR_SWEEP");
   const bool chosen = mixed && (h->opt.sweep >= 0 || (e && (strcmp(e, "simt") == 0 || strcmp(e, "tc") == 0)));
   if (!chosen) k.few = sweep_few_plan(h->m.Mp, B, std::min(h->nsm, 4 * h->nsm / std::max(1, tiles)));
@@ -252,7 +253,7 @@ template <typename T>
 static cudaError_t run_sweep(const SweepParams<T>& sp, const SweepKind& k, const void* Xt, int terms, cudaStream_t st) {
   if (k.few.nv) return launch_sweep_few<T>(sp, k.few, st);
   if constexpr (sizeof(T) == 4) {
-    if (k.tc) return launch_sweep_tc(sp, Xt, terms, k.nsm, k.beside, st);
+    if (k.tc) return launch_sweep_tc(sp, Xt, terms, k.nsm, k.tiles, st);
   }
   return launch_sweep<T>(sp, st);
 }
@@ -506,7 +507,7 @@ static xbar_status solve_rows_mixed(xbar_s* h, int B, const double* dV, double* 
   sp.max_rel = nullptr;
   sp.status = g->status;
   auto sweep32 = [&](int terms) -> cudaError_t {  // dhat = solve32(rhat) (rhat is overwritten by cyclic reduction)
-    if (tc) return launch_sweep_tc(sp, g->Xt.p, terms, g->nsm, false, st);
+    if (tc) return launch_sweep_tc(sp, g->Xt.p, terms, g->nsm, 1, st);
     if (!cr) return launch_sweep<float>(sp, st);
     CrSweepArgs<float> ca;
     memset(&ca, 0, sizeof(ca));
@@ -1104,7 +1105,6 @@ xbar_status xbar::solve_device_driven(xbar_s* h, int B, const double* dV, double
     return fail(XBAR_ESTATE, "device-driven solves (tile batches) need a block-Thomas factorization");
   const bool mixed = h->prec == XBAR_FP32_IR;
   SweepKind kind = sweep_kind(h, B, mixed, tiles);
-  kind.beside = tiles > 1;
   const int Bp = kind.Bp;
   const int Bpad = ((B + Bp - 1) / Bp) * Bp;
   const size_t nst = (size_t)N * Mp * Bpad;

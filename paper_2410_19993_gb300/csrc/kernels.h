@@ -167,8 +167,8 @@ constexpr int kSweepTcPanel = 64;
 size_t sweep_tc_tile_bytes(int Mp, int N);
 cudaError_t launch_sweep_tc_tile(const float* X, void* Xt, int Mp, int N, cudaStream_t st);
 // terms = leading BF16 terms of the split used (2 or 3): 3 gives FP32-level accuracy
-// beside: other solves run beside this one (the tiles of a batch)
-cudaError_t launch_sweep_tc(const SweepParams<float>& p, const void* Xt, int terms, int nsm, bool beside,
+// tiles: solves of about this size that run side by side (the tiles of a batch)
+cudaError_t launch_sweep_tc(const SweepParams<float>& p, const void* Xt, int terms, int nsm, int tiles,
                             cudaStream_t st);
 
 // ---- blocking over rows (orient.cu): the mirrored crossbar M' = N, N' = M ---------------------

@@ -712,7 +712,7 @@ cudaError_t launch_sweep_tc_tile(const float* X, void* Xt, int Mp, int N, cudaSt
   return cudaGetLastError();
 }
 
-cudaError_t launch_sweep_tc(const SweepParams<float>& p, const void* Xt, int terms, int nsm, bool beside,
+cudaError_t launch_sweep_tc(const SweepParams<float>& p, const void* Xt, int terms, int nsm, int tiles,
                             cudaStream_t st) {
   const int Mt = sweep_tc_rows(p.Mp);
   if (p.Bp != tc::kBP || p.Bpad % tc::kBP) return cudaErrorInvalidValue;
@@ -727,12 +727,13 @@ cudaError_t launch_sweep_tc(const SweepParams<float>& p, const void* Xt, int ter
                                 {sweep_tc_kernel<2, 3, false, false>, sweep_tc_kernel<2, 3, true, false>}}};
   const Kern pair[2] = {sweep_tc_kernel<1, 2, false, true>, sweep_tc_kernel<1, 2, true, true>};
   auto launch = [&](bool out, int chains, int chain0) {
-    // Two blocks on an SM where there is work for both: more blocks than SMs, or other tiles' solves
-    // beside this one; then one block's epilogue overlaps the other's products (a step of a 128-row
-    // block is mostly epilogue latency).  128 x 128 in mixed precision, 16384 vectors: 7.94 -> 7.14 ms,
-    // 8192: 4.75 -> 4.35 ms; 30 tiles with 4096 vectors each: 47.3 -> 44.1 ms.  A block alone runs slower at
-    // half an SM's registers and a third of its stages: 1000 vectors 2.62 against 2.72 ms.
-    const bool two = Mt == 128 && terms == 2 && (beside || blocks * chains > nsm);
+    // Two blocks on an SM where there is work for both: more blocks than SMs, of all tiles of a batch twice as
+    // many (they do not start together); then one block's epilogue overlaps the other's products (a step of
+    // a 128-row block is mostly epilogue latency).  128 x 128 in mixed precision, 16384 vectors: 7.94 -> 7.14 ms,
+    // 8192: 4.75 -> 4.35 ms; 30 tiles with 4096 vectors each: 47.3 -> 44.1 ms.  A block alone runs slower at half
+    // an SM's registers and a third of its stages: 1000 vectors 2.62 against 2.72 ms, four 128 x 128 tiles with
+    // 512 each 2.82 against 3.36 ms.
+    const bool two = Mt == 128 && terms == 2 && (long long)blocks * chains * tiles > (tiles > 1 ? 2 : 1) * nsm;
     const Kern kern = two ? pair[out] : kerns[Mt / 128 - 1][terms - 2][out];
     const size_t smem = sweep_tc_smem_bytes(Mt, terms, two);
     const cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
