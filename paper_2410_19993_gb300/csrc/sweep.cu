@@ -109,8 +109,10 @@ __device__ __forceinline__ void load_vec(T (&r)[n], const T* p) {
   }
 }
 
-// chain of a block: blockIdx.y + chain0.  kOut: the meeting column and the outward part.
-template <typename T, int TR, int TC, bool kOut>
+// Chain of a block: blockIdx.y + chain0.  The inward part, the meeting column and the outward part, or with a
+// single chain (m = N - 1) both, one after the other: a block's z is then its own threads'.
+enum { kIn, kOutward, kBoth };
+template <typename T, int TR, int TC, int kPart>
 __global__ void __launch_bounds__(sweep_max_threads<TR, TC>()) sweep_kernel(SweepParams<T> p, int KC, int chain0) {
   const int Mp = p.Mp, N = p.N, Bp = p.Bp, Bpad = p.Bpad;
   const int nrg = Mp / TR, ncg = Bp / TC;
@@ -135,28 +137,34 @@ __global__ void __launch_bounds__(sweep_max_threads<TR, TC>()) sweep_kernel(Swee
   const int chunks_per_step = Mp / KC;
   const int m = p.meet, chain = (int)blockIdx.y + chain0;
   const int len = chain == 0 ? m : N - 1 - m;  // columns of the chain
-  const int nsteps = len + (kOut ? 1 : 0);
-  // column of step s: inward 0, 1, .. (left) or N-1, N-2, .. (right); outward m, then away from it
-  const int jdir = (chain == 0) == kOut ? -1 : 1, jstart = kOut ? m : (chain == 0 ? 0 : N - 1);
-  auto col_of = [&](int s) { return jstart + jdir * s; };
-  const long long nchunks = (long long)nsteps * chunks_per_step;
   const unsigned chunk_bytes = (unsigned)(KC * Mp * sizeof(T));
-  auto chunk_src = [&](long long c) -> const T* {
-    const int s = (int)(c / chunks_per_step);
-    const int k0 = (int)(c - (long long)s * chunks_per_step) * KC;
-    const int j = col_of(s);
-    return p.X + ((size_t)j * Mp + k0) * Mp;
-  };
-
   if (tid == 0) {
     mbar_init(&mbar[0], 1);
     mbar_init(&mbar[1], 1);
     fence_mbar_init();
   }
   __syncthreads();
+  long long c = 0;  // chunks used so far: buffer and phase
+  float local_max = 0.0f;
+  for (int part = kPart == kBoth && len > 0 ? kIn : kPart == kIn ? kIn : kOutward; part <= (kPart == kIn ? kIn : kOutward);
+       ++part) {
+  const bool kOut = kPart == kBoth ? part == kOutward : kPart == kOutward;
+  const int nsteps = len + (kOut ? 1 : 0);
+  // column of step s: inward 0, 1, .. (left) or N-1, N-2, .. (right); outward m, then away from it
+  const int jdir = (chain == 0) == kOut ? -1 : 1, jstart = kOut ? m : (chain == 0 ? 0 : N - 1);
+  auto col_of = [&](int s) { return jstart + jdir * s; };
+  const long long cend = c + (long long)nsteps * chunks_per_step, cbase = c;
+  auto chunk_src = [&](long long q) -> const T* {
+    q -= cbase;
+    const int s = (int)(q / chunks_per_step);
+    const int k0 = (int)(q - (long long)s * chunks_per_step) * KC;
+    const int j = col_of(s);
+    return p.X + ((size_t)j * Mp + k0) * Mp;
+  };
   if (tid == 0) {
-    mbar_arrive_expect_tx(&mbar[0], chunk_bytes);
-    bulk_g2s(xs, chunk_src(0), chunk_bytes, &mbar[0]);
+    if (c > 0) fence_proxy_async_smem();
+    mbar_arrive_expect_tx(&mbar[c & 1], chunk_bytes);
+    bulk_g2s(xs + (size_t)(c & 1) * KC * Mp, chunk_src(c), chunk_bytes, &mbar[c & 1]);
   }
 
   // input of step 0: the right-hand side of its column and, in the meeting column, both chains' z
@@ -178,8 +186,6 @@ __global__ void __launch_bounds__(sweep_max_threads<TR, TC>()) sweep_kernel(Swee
   __syncthreads();
 
   T acc[TR][TC];
-  long long c = 0;
-  float local_max = 0.0f;
   for (int s = 0; s < nsteps; ++s) {
     const int j = col_of(s);
 #pragma unroll
@@ -188,7 +194,7 @@ __global__ void __launch_bounds__(sweep_max_threads<TR, TC>()) sweep_kernel(Swee
       for (int b = 0; b < TC; ++b) acc[a][b] = (T)0;
 
     for (int kc = 0; kc < chunks_per_step; ++kc, ++c) {
-      if (tid == 0 && c + 1 < nchunks) {
+      if (tid == 0 && c + 1 < cend) {
         const int nb = (int)((c + 1) & 1);
         fence_proxy_async_smem();
         mbar_arrive_expect_tx(&mbar[nb], chunk_bytes);
@@ -299,6 +305,7 @@ __global__ void __launch_bounds__(sweep_max_threads<TR, TC>()) sweep_kernel(Swee
     }
     __syncthreads();
   }
+  }
   if (p.max_rel) {
     for (int o = 16; o > 0; o >>= 1) local_max = fmaxf(local_max, __shfl_xor_sync(0xffffffffu, local_max, o));
     if ((tid & 31) == 0 && local_max > 0.0f) atomic_max_nonneg(p.max_rel, local_max);
@@ -314,19 +321,22 @@ static cudaError_t launch_tiled(const SweepParams<T>& p, int KC, cudaStream_t st
   if (blocks == 0) return cudaSuccess;
   if ((long long)blocks * p.Bp > p.Bpad) return cudaErrorInvalidValue;
   const size_t smem = sweep_smem_bytes<T>(p.Mp, p.Bp, KC, TR);
-  cudaError_t err = cudaFuncSetAttribute(sweep_kernel<T, TR, TC, false>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (err == cudaSuccess)
-    err = cudaFuncSetAttribute(sweep_kernel<T, TR, TC, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (err != cudaSuccess) return err;
+  auto launch = [&](void (*kern)(SweepParams<T>, int, int), int chains, int chain0) {
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    kern<<<dim3(blocks, chains), threads, smem, st>>>(p, KC, chain0);
+    return cudaGetLastError();
+  };
   const bool left = p.meet > 0, right = p.meet < p.N - 1;
+  // one chain and narrow tiles: one launch (no block reads another's z)
+  if constexpr (TR == kNarrowTR)
+    if (!right) return launch(sweep_kernel<T, TR, TC, kBoth>, 1, 0);
   const bool right_in = right && p.rhs;  // an input vector enters at column 0 only
   if (left || right_in) {
-    sweep_kernel<T, TR, TC, false><<<dim3(blocks, left && right_in ? 2 : 1), threads, smem, st>>>(p, KC, left ? 0 : 1);
-    if ((err = cudaGetLastError()) != cudaSuccess) return err;
+    const cudaError_t err = launch(sweep_kernel<T, TR, TC, kIn>, left && right_in ? 2 : 1, left ? 0 : 1);
+    if (err != cudaSuccess) return err;
   }
-  sweep_kernel<T, TR, TC, true><<<dim3(blocks, right && !(p.rhs && p.first_only) ? 2 : 1), threads, smem, st>>>(p, KC, 0);
-  return cudaGetLastError();
+  return launch(sweep_kernel<T, TR, TC, kOutward>, right && !(p.rhs && p.first_only) ? 2 : 1, 0);
 }
 
 template <typename T>

@@ -196,8 +196,10 @@ static_assert(tc_stages(256, 2, false) == 2 && tc_stages(256, 3, false) == 2 && 
 // ones).  Every size the MMA issue loop touches is a compile-time constant: the single issuing
 // thread then spends no dependent integer work per MMA (runtime offsets in that loop tripled its
 // cost per MMA).
-// Chain of a block: blockIdx.y + chain0.  kOut: the meeting column and the outward part.
-template <int NH, int KP, bool kOut, bool kTwo>
+// Chain of a block: blockIdx.y + chain0.  The inward part, the meeting column and the outward part, or (blocks of
+// up to 128 rows, a single chain: m = N - 1) both in one walk of 2N - 1 steps, which a block's z does not leave.
+enum { kIn, kOutward, kBoth };
+template <int NH, int KP, int kPart, bool kTwo>
 __global__ void __launch_bounds__(tc::kThreads + 64, kTwo ? 2 : 1)
     sweep_tc_kernel(SweepParams<float> p, const __nv_bfloat16* __restrict__ Xt, int chain0) {
   using namespace tc;
@@ -205,6 +207,8 @@ __global__ void __launch_bounds__(tc::kThreads + 64, kTwo ? 2 : 1)
   constexpr int Mt = 128 * NH, nh = NH;
   constexpr int NS = tc_stages(Mt, KP, kTwo), kSub = tc_sub(Mt, KP, kTwo);
   static_assert(!kTwo || (NH == 1 && KP == 2), "two blocks on an SM");
+  static_assert(kPart != kBoth || NH == 1, "both parts: blocks of up to 128 rows");
+  constexpr bool kOut = kPart == kOutward;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int b0 = blockIdx.x * BP;
   const uint64_t wlim = wait_limit(p.status);  // read once: the waits below sit on critical paths
@@ -232,10 +236,10 @@ __global__ void __launch_bounds__(tc::kThreads + 64, kTwo ? 2 : 1)
 
   constexpr int cps = Mt / KC;  // chunks per step
   const int m = p.meet, chain = (int)blockIdx.y + chain0;
-  const int nsteps = (chain == 0 ? m : N - 1 - m) + (kOut ? 1 : 0);
+  const int nsteps = kPart == kBoth ? 2 * m + 1 : (chain == 0 ? m : N - 1 - m) + (kOut ? 1 : 0);
   // column of step s: inward 0, 1, .. (left) or N-1, N-2, .. (right); outward m, then away from it
   const int jdir = (chain == 0) == kOut ? -1 : 1, jstart = kOut ? m : (chain == 0 ? 0 : N - 1);
-  auto col_of = [&](int s) { return jstart + jdir * s; };
+  auto col_of = [&](int s) { return kPart == kBoth ? (s <= m ? s : 2 * m - s) : jstart + jdir * s; };
   const long long nchunks = (long long)nsteps * cps;
   // accumulators: per 128-row half, 64 columns; two sets, for even and odd steps, so that the
   // epilogue can re-read this step's D while the next step's MMAs accumulate into the other set
@@ -439,9 +443,9 @@ __global__ void __launch_bounds__(tc::kThreads + 64, kTwo ? 2 : 1)
       const float* zp2 = zpanel(col_of(s2));
       const int i0 = i - lane + (lane & 3) * 8;  // this lane's quarter of the warp's 32 rows
       for (int blk = 0; blk < ncb; ++blk) {
-        if (zout && s2 > 0 && i0 < Mp)
+        if ((kPart == kBoth ? s2 > m : zout && s2 > 0) && i0 < Mp)
           asm volatile("prefetch.global.L2 [%0];" ::"l"(zp2 + ((size_t)((cb + blk * 32) / 4 + (lane >> 2)) * Mp + i0) * 4));
-        if (!kOut && real && s2 + 1 < nsteps && p.rhs)
+        if (!kOut && real && (kPart == kBoth ? s2 < m : s2 + 1 < nsteps) && p.rhs)
           asm volatile("prefetch.global.L2 [%0];" ::"l"(p.rhs + ((size_t)col_of(s2 + 1) * Mp + i) * Bpad + b0 + cb + blk * 32));
       }
     };
@@ -474,7 +478,7 @@ __global__ void __launch_bounds__(tc::kThreads + 64, kTwo ? 2 : 1)
     // load units and L1 busy; with 8192 vectors of 256 x 256 an inward correction launch took
     // 1.57 ms against 1.40 ms now, with 1000 of 128 x 128 171 against 137 us.)
     auto stage_r = [&](int s2, int blk) {
-      if (!kOut && p.rhs && s2 + 1 < nsteps) {
+      if (!kOut && p.rhs && (kPart == kBoth ? s2 < m : s2 + 1 < nsteps)) {
         const float* src = p.rhs + ((size_t)col_of(s2 + 1) * Mp + (i - lane)) * Bpad + b0 + cb + blk * 32;
 #pragma unroll
         for (int m = 0; m < 8; ++m) {
@@ -539,15 +543,17 @@ __global__ void __launch_bounds__(tc::kThreads + 64, kTwo ? 2 : 1)
       const float ej = real && more ? p.e[(size_t)min(j, jn) * Mp + i] : 0.0f;
       const float hj = real ? p.hs[(size_t)j * Mp + i] : 0.0f;
       const float sj = (real && p.w1out) ? p.s32[(size_t)j * Mp + i] : 0.0f;
-      const bool have_w = kOut && (s > 0 || chain == 0);  // w_m is reported by the left block
+      const bool out = kPart == kBoth ? s >= m : kOut;                          // not an inward step
+      const bool have_w = kPart == kBoth ? out : kOut && (s > 0 || chain == 0);  // w_m is reported by the left block
       // the current this step adds to, read now so that its latency overlaps the accumulator wait
       double Iold = 0.0;
       if (have_w && p.accumulate && tid < BP && b0 + tid < p.B) Iold = p.I[(size_t)(b0 + tid) * N + j];
       // the next input's operands that do not depend on D -- z of this step (outward) or the next
       // column's right-hand side (inward) -- are loaded before the wait: column block 0
       // now, block 1 right after it, so their latency leaves the step's critical path
-      const bool use_z = zout && s > 0 && real;
-      const bool use_r = !kOut && more && p.rhs && real;
+      const bool use_z = (kPart == kBoth ? s > m : zout && s > 0) && real;
+      const bool next_r = !kOut && (kPart == kBoth ? s < m : more) && p.rhs;
+      const bool use_r = next_r && real;
       float pre[ncb][32];
       // outward, block 1 (nh == 2): 16-byte cp.async copies into this thread's slice of pres, waited for
       // after the accumulator wait, so their latency overlaps it
@@ -591,7 +597,9 @@ __global__ void __launch_bounds__(tc::kThreads + 64, kTwo ? 2 : 1)
       if constexpr (kOut) {
         load_pre(0);
         if (nh == 2) async_pre1();
-      } else if (more && p.rhs) {  // block 0 has been on its way since the last step
+      } else if (kPart == kBoth && out) {
+        load_pre(0);
+      } else if (next_r) {  // block 0 has been on its way since the last step
         take_r(pre[0]);
         if constexpr (nh == 2) {
           stage_r(s, 1);
@@ -643,7 +651,7 @@ __global__ void __launch_bounds__(tc::kThreads + 64, kTwo ? 2 : 1)
         if (use_z)
 #pragma unroll
           for (int n = 0; n < 32; ++n) a[n] += pre[blk][n];
-        if (!kOut && real) {
+        if (!out && real) {
           float4* zrow = reinterpret_cast<float4*>(zp) + (size_t)((cb + blk * 32) / 4) * Mp + i;
 #pragma unroll
           for (int n = 0; n < 32; n += 4)
@@ -721,12 +729,14 @@ cudaError_t launch_sweep_tc(const SweepParams<float>& p, const void* Xt, int ter
   if (terms < 2 || terms > tc::kParts) return cudaErrorInvalidValue;
   if (p.meet < 0 || p.meet >= p.N || (!p.V && !p.rhs)) return cudaErrorInvalidValue;
   using Kern = void (*)(SweepParams<float>, const __nv_bfloat16*, int);
-  const Kern kerns[2][2][2] = {{{sweep_tc_kernel<1, 2, false, false>, sweep_tc_kernel<1, 2, true, false>},
-                                {sweep_tc_kernel<1, 3, false, false>, sweep_tc_kernel<1, 3, true, false>}},
-                               {{sweep_tc_kernel<2, 2, false, false>, sweep_tc_kernel<2, 2, true, false>},
-                                {sweep_tc_kernel<2, 3, false, false>, sweep_tc_kernel<2, 3, true, false>}}};
-  const Kern pair[2] = {sweep_tc_kernel<1, 2, false, true>, sweep_tc_kernel<1, 2, true, true>};
-  auto launch = [&](bool out, int chains, int chain0) {
+  const Kern kerns[2][2][3] = {
+      {{sweep_tc_kernel<1, 2, kIn, false>, sweep_tc_kernel<1, 2, kOutward, false>, sweep_tc_kernel<1, 2, kBoth, false>},
+       {sweep_tc_kernel<1, 3, kIn, false>, sweep_tc_kernel<1, 3, kOutward, false>, sweep_tc_kernel<1, 3, kBoth, false>}},
+      {{sweep_tc_kernel<2, 2, kIn, false>, sweep_tc_kernel<2, 2, kOutward, false>, nullptr},
+       {sweep_tc_kernel<2, 3, kIn, false>, sweep_tc_kernel<2, 3, kOutward, false>, nullptr}}};
+  const Kern pair[3] = {sweep_tc_kernel<1, 2, kIn, true>, sweep_tc_kernel<1, 2, kOutward, true>,
+                        sweep_tc_kernel<1, 2, kBoth, true>};
+  auto launch = [&](int part, int chains, int chain0) {
     // Two blocks on an SM where there is work for both: more blocks than SMs, of all tiles of a batch twice as
     // many (they do not start together); then one block's epilogue overlaps the other's products (a step of
     // a 128-row block is mostly epilogue latency).  128 x 128 in mixed precision, 16384 vectors: 7.94 -> 7.14 ms,
@@ -734,7 +744,7 @@ cudaError_t launch_sweep_tc(const SweepParams<float>& p, const void* Xt, int ter
     // an SM's registers and a third of its stages: 1000 vectors 2.62 against 2.72 ms, four 128 x 128 tiles with
     // 512 each 2.82 against 3.36 ms.
     const bool two = Mt == 128 && terms == 2 && (long long)blocks * chains * tiles > (tiles > 1 ? 2 : 1) * nsm;
-    const Kern kern = two ? pair[out] : kerns[Mt / 128 - 1][terms - 2][out];
+    const Kern kern = two ? pair[part] : kerns[Mt / 128 - 1][terms - 2][part];
     const size_t smem = sweep_tc_smem_bytes(Mt, terms, two);
     const cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (err != cudaSuccess) return err;
@@ -742,12 +752,13 @@ cudaError_t launch_sweep_tc(const SweepParams<float>& p, const void* Xt, int ter
     return cudaGetLastError();
   };
   const bool left = p.meet > 0, right = p.meet < p.N - 1;
+  if (Mt == 128 && left && !right) return launch(kBoth, 1, 0);
   const bool right_in = right && p.rhs;  // an input vector enters at column 0 only
   if (left || right_in) {
-    const cudaError_t err = launch(false, left && right_in ? 2 : 1, left ? 0 : 1);
+    const cudaError_t err = launch(kIn, left && right_in ? 2 : 1, left ? 0 : 1);
     if (err != cudaSuccess) return err;
   }
-  return launch(true, right ? 2 : 1, 0);
+  return launch(kOutward, right ? 2 : 1, 0);
 }
 
 }  // namespace xbar
