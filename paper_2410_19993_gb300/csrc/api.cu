@@ -241,8 +241,12 @@ static SweepKind sweep_kind(const xbar_s* h, int B, bool mixed, int tiles = 1) {
   k.tiles = tiles;
   const char* e = getenv("XBAR_SWEEP");
   const bool chosen = mixed && (h->opt.sweep >= 0 || (e && (strcmp(e, "simt") == 0 || strcmp(e, "tc") == 0)));
-  if (!chosen) k.few = sweep_few_plan(h->m.Mp, B, std::min(h->nsm, 4 * h->nsm / std::max(1, tiles)));
-  k.tc = mixed && h->tc_ready && !k.few.nv;
+  // a batch's 16-row FP32 factors (one chain): both parts of a substitution in one launch, on the CUDA cores for
+  // up to half a tensor-core panel; the run's time is that of its many graph nodes (256 tiles, one vector each:
+  // 8.04 ms, clusters 8.65, tensor cores 8.25)
+  const bool one = mixed && tiles > 1 && h->meet == h->m.N - 1 && h->m.Mp == 16;
+  if (!chosen && !one) k.few = sweep_few_plan(h->m.Mp, B, std::min(h->nsm, 4 * h->nsm / std::max(1, tiles)));
+  k.tc = mixed && h->tc_ready && !k.few.nv && !(!chosen && one && B <= 32);
   k.Bp = k.few.nv ? k.few.nv
          : k.tc   ? kSweepTcPanel
          : mixed  ? sweep_panel_width<float>(h->m.Mp, B, h->nsm)
