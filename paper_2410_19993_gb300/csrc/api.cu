@@ -343,6 +343,7 @@ static xbar_status factor_mirror(xbar_s* h, xbar_precision p) {
   g->opt = h->opt;
   g->opt.orient = 0;
   g->tiles = h->tiles;
+  g->tile_vectors = h->tile_vectors;
   // automatic algorithm: the mirror's many small blocks (M blocks of N rows) are what cyclic
   // reduction is for, against M dependent block steps of block Thomas
   if (h->opt.algo < 0 && cr_supported(g->m.Mp, g->m.N)) g->opt.algo = 1;
@@ -678,7 +679,12 @@ static xbar_status do_factor64(xbar_t h, bool upload) {
   MapDev& m = h->m;
   const char* e = getenv("XBAR_FACTOR");
   const Factor64Plan plan = factor64_plan(m.Mp, m.N, h->nsm, h->tiles > 1);
-  if (!plan.rows || (e && strcmp(e, "group") == 0)) return do_factor_thomas<double>(h, upload);
+  // many 32-row tiles with few vectors each (the substitutions, which one chain makes longer, are short): one
+  // block a tile, where ten of factor64.cu would wait for SMs; 64 tiles of 32 x 32, one vector, 3.01 ms a run
+  // against 3.63, with 512 vectors 7.00 against 6.37
+  const bool crowd = plan.rows && m.Mp == 32 && h->tile_vectors <= 64 &&
+                     (long long)h->tiles * factor64_blocks(m.Mp, m.N, plan) > 3 * h->nsm;
+  if (!plan.rows || crowd || (e && strcmp(e, "group") == 0)) return do_factor_thomas<double>(h, upload);
   XB_CUDA(ensure(h->A, h->X, (size_t)m.N * m.Mp * m.Mp * sizeof(double)));
   XB_CUDA(ensure(h->A, h->fpbuf, factor64_buf_bytes(m.Mp)));
   XB_CUDA(ensure(h->A, h->fbar, factor64_flag_bytes()));

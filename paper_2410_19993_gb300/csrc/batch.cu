@@ -134,6 +134,7 @@ static xbar_status enqueue_all(xbar_batch_t b, xbar_precision p, const int* B, c
   for (int t = 0; t < b->T; ++t) {
     xbar_t h = b->tiles[t];
     XB_CUDA(cudaStreamWaitEvent(b->streams[t], b->fork, 0));
+    h->tile_vectors = B[t];
     xbar_status s = factor_handle(h, p, eager);
     if (s != XBAR_OK) return s;
     if (B[t] > 0) {

@@ -126,6 +126,7 @@ struct xbar_s {
   cudaStream_t st = nullptr;
   int dev = 0, nsm = 0;
   int tiles = 1;  // tiles of the batch this handle is one of: their factors and solves run beside this one's
+  int tile_vectors = 0;  // and its vectors in the batch's run
   // per-column elimination data formed from Gc (lazily, by the first factor): 0 = no, else with the
   // column blocks in the precision p of the factors, assembled_for(p)
   int assembled = 0;
