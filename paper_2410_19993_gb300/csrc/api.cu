@@ -605,6 +605,16 @@ static xbar_status do_factor_cr(xbar_t h, bool equilibrate) {
   return XBAR_OK;
 }
 
+// Two chains halve the dependent steps of a factor and of its substitutions, but double their blocks and
+// launches, which a chain of one or two columns does not earn back, nor one of a few more among tiles that
+// fill the device anyway.  64 tiles of 32 x 8 with 4096 vectors: 6.24 ms a run from both ends, 5.54 from one;
+// 16 tiles of 64 x 3: 1.27 against 1.04; one 256 x 3 map with 16384: 1.11 against 1.02 (with one 0.32 against 0.37).
+static bool one_chain(const xbar_s* h) {
+  const int N = h->m.N;
+  const long long blocks = 2ll * (h->m.Mp / 16) * h->tiles, sweeps = 2ll * ((h->tile_vectors + 63) / 64) * h->tiles;
+  return N <= 4 || (h->tiles > 1 && ((N <= 16 && blocks > h->nsm) || (N <= 8 && sweeps > 4 * h->nsm)));
+}
+
 // Block Thomas by the cluster kernel (FP32 where it fits) or the group kernel, equilibrated in FP32
 template <typename T>
 static xbar_status do_factor_thomas(xbar_t h, bool upload) {
@@ -624,7 +634,7 @@ static xbar_status do_factor_thomas(xbar_t h, bool upload) {
   XB_CUDA(ensure(h->A, h->fparams, sizeof(FactorParams<T>)));
   // the cluster factor eliminates from both ends, the group factor from column 0 to N - 1
   const bool cluster = f32 && use_cluster_factor(h);
-  h->meet = cluster ? (N - 1) / 2 : N - 1;
+  h->meet = cluster && !one_chain(h) ? (N - 1) / 2 : N - 1;
   FactorParams<T> fp;
   memset(&fp, 0, sizeof(fp));  // padding too: the block is compared byte for byte below
   fp.M = m.M;

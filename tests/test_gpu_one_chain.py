@@ -1,6 +1,6 @@
 """Substitutions of a factor with a single elimination chain, both parts in one launch (tensor-core panels of
 blocks of up to 128 rows, narrow CUDA-core panels): two to many columns, ragged rows, full and ragged
-panels, currents alone and with node voltages."""
+panels, currents alone and with node voltages; and factors of maps with few columns, which take one chain."""
 import numpy as np
 import pytest
 
@@ -41,3 +41,26 @@ def test_group_factor(M, N, sweep, monkeypatch):
     monkeypatch.setenv("XBAR_FACTOR", "group")
     monkeypatch.setenv("XBAR_SWEEP", sweep)
     _check(M, N, [1, 5, 64, 65, 300])
+
+
+@pytest.mark.parametrize("M,N", [(32, 2), (100, 3), (129, 4), (256, 3)])
+def test_few_columns(M, N):
+    _check(M, N, [1, 40, 700])
+
+
+def test_crowded_tiles():
+    """Tiles that fill the device: one chain, no clusters for few vectors, FP64 factors of 32 rows by one block."""
+    for precision, bar in (("fp32_ir", 1e-8), ("fp64", 1e-10)):
+        for M, N, B in [(32, 12, 3), (32, 8, 65), (16, 5, 2), (16, 5, 40)]:
+            T = 56
+            maps = [case(M, N, B, None, seed=t) for t in range(T)]
+            b = xbar.Batch([(torch.from_numpy(G).cuda(), *R) for G, _ in maps])
+            for t in range(T):
+                xbar._check(xbar.load().xbar_set_option(b.tile_handle(t), xbar.OPTIONS["orientation"], 0))
+            Vs = [torch.from_numpy(V).cuda() for _, V in maps]
+            Is = [torch.zeros((B, N), dtype=torch.float64, device="cuda") for _ in maps]
+            for _ in range(2):
+                b.run(precision, Vs, Is, tol=1e-9, max_iter=6)
+            for (G, V), I in zip(maps, Is):
+                assert rel_err(I.cpu().numpy(), oracle.solve(M, N, G, *R, V)["I"]) <= bar
+            b.destroy()
