@@ -319,8 +319,8 @@ xbar_status xbar_batch_run(xbar_batch_t b, xbar_precision p, const int* B, const
 
 /*
  * xbar_batch_autotune -- for every distinct (M, N, B[t]) time the kernel variants (tensor-core
- * vs CUDA-core FP32 substitutions, cluster vs cooperative-group FP32 factor) on one tile, keep
- * the fastest for all tiles of that shape.  cache_path (may be NULL) is a JSON file of earlier
+ * vs CUDA-core FP32 substitutions and, for few vectors, the automatic choice; cluster vs
+ * cooperative-group FP32 factor) on one tile, keep the fastest for all tiles of that shape.  cache_path (may be NULL) is a JSON file of earlier
  * choices, read first and rewritten with new ones.  Only XBAR_FP32_IR has variants.
  */
 xbar_status xbar_batch_autotune(xbar_batch_t b, xbar_precision p, const int* B, const char* cache_path);

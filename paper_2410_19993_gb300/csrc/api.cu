@@ -253,6 +253,9 @@ static SweepKind sweep_kind(const xbar_s* h, int B, bool mixed, int tiles = 1) {
                   : sweep_panel_width<double>(h->m.Mp, B, h->nsm);
   return k;
 }
+bool xbar::chooses_few(const xbar_s* h, int B, int tiles) {
+  return sweep_kind(h, B, h->prec == XBAR_FP32_IR, tiles).few.nv > 0;
+}
 template <typename T>
 static cudaError_t run_sweep(const SweepParams<T>& sp, const SweepKind& k, const void* Xt, int terms, cudaStream_t st) {
   if (k.few.nv) return launch_sweep_few<T>(sp, k.few, st);

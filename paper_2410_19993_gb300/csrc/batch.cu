@@ -11,8 +11,8 @@
 // tile's handle can be used between runs (xbar_batch_tile); what such a call may change under the graph
 // is part of the signature (graph_epoch).
 //
-// The autotuner times the kernel variants (tensor-core vs CUDA-core FP32 substitutions, cluster
-// vs cooperative-group FP32 factor; for FP64, blocks over columns vs over rows -- the mirrored
+// The autotuner times the kernel variants (tensor-core vs CUDA-core FP32 substitutions vs the clusters for
+// few vectors, cluster vs cooperative-group FP32 factor; for FP64, blocks over columns vs over rows -- the mirrored
 // crossbar of orient.cu) on one tile of every distinct (M, N, B), keeps the fastest, and can
 // persist its choices in a small JSON file keyed by shape.
 #include <math.h>
@@ -262,7 +262,9 @@ struct TuneKey {
 };
 struct TuneVal {
   int sweep = -1, factor = -1, orient = -1;
+  int few = -1;  // FP32 substitutions left to the automatic choice, the clusters for few vectors (-1: not known)
   float sweep_ms[2] = {-1, -1}, factor_ms[2] = {-1, -1};
+  float few_ms = -1;
   float orient_ms[2] = {-1, -1};  // FP64: factor + solve, blocks over columns / rows
 };
 
@@ -281,8 +283,9 @@ static std::map<TuneKey, TuneVal> load_cache(const char* path) {
   while (fgets(line, sizeof(line), f)) {
     TuneKey k;
     TuneVal v;
-    const int n = sscanf(line, " \"M=%d,N=%d,B=%d,prec=%d\": {\"sweep\": %d, \"factor\": %d, \"orient\": %d", &k.M,
-                         &k.N, &k.B, &k.p, &v.sweep, &v.factor, &v.orient);
+    const int n = sscanf(line,
+                         " \"M=%d,N=%d,B=%d,prec=%d\": {\"sweep\": %d, \"factor\": %d, \"orient\": %d, \"few\": %d", &k.M,
+                         &k.N, &k.B, &k.p, &v.sweep, &v.factor, &v.orient, &v.few);
     if (n >= 6) c[k] = v;  // files written before the orientation field: automatic orientation
   }
   fclose(f);
@@ -298,10 +301,10 @@ static void save_cache(const char* path, const std::map<TuneKey, TuneVal>& c) {
   for (const auto& kv : c) {
     const TuneVal& v = kv.second;
     fprintf(f,
-            "  \"%s\": {\"sweep\": %d, \"factor\": %d, \"orient\": %d, \"sweep_ms\": [%.4f, %.4f], "
-            "\"factor_ms\": [%.4f, %.4f], \"orient_ms\": [%.4f, %.4f]}%s\n",
-            key_str(kv.first).c_str(), v.sweep, v.factor, v.orient, v.sweep_ms[0], v.sweep_ms[1], v.factor_ms[0],
-            v.factor_ms[1], v.orient_ms[0], v.orient_ms[1], ++n < c.size() ? "," : "");
+            "  \"%s\": {\"sweep\": %d, \"factor\": %d, \"orient\": %d, \"few\": %d, \"sweep_ms\": [%.4f, %.4f], "
+            "\"few_ms\": %.4f, \"factor_ms\": [%.4f, %.4f], \"orient_ms\": [%.4f, %.4f]}%s\n",
+            key_str(kv.first).c_str(), v.sweep, v.factor, v.orient, v.few, v.sweep_ms[0], v.sweep_ms[1], v.few_ms,
+            v.factor_ms[0], v.factor_ms[1], v.orient_ms[0], v.orient_ms[1], ++n < c.size() ? "," : "");
   }
   fprintf(f, "}\n");
   fclose(f);
@@ -342,7 +345,8 @@ extern "C" xbar_status xbar_batch_autotune(xbar_batch_t b, xbar_precision p, con
     xbar_t h = b->tiles[kv.second];
     TuneVal v;
     auto it = cache.find(k);
-    if (it != cache.end()) {
+    // a choice of an earlier file that does not say whether the clusters were timed is made again
+    if (it != cache.end() && (p != XBAR_FP32_IR || it->second.few >= 0)) {
       v = it->second;
     } else if (p == XBAR_FP32_IR && k.B > 0) {
       // scratch inputs for timing: V = 0.25 V everywhere (values do not affect the kernels' speed)
@@ -366,6 +370,12 @@ extern "C" xbar_status xbar_batch_autotune(xbar_batch_t b, xbar_precision p, con
         v.sweep_ms[sw] = time_ms(h->st, [&]() { return solve_device_driven(h, k.B, dV, dI, 1e-8, 2, true, b->T); });
       }
       v.sweep = (v.sweep_ms[1] >= 0 && (v.sweep_ms[0] < 0 || v.sweep_ms[1] <= v.sweep_ms[0])) ? 1 : 0;
+      h->opt.sweep = -1;
+      v.few = 0;
+      if (factor_handle(h, p, true) == XBAR_OK && chooses_few(h, k.B, b->T)) {
+        v.few_ms = time_ms(h->st, [&]() { return solve_device_driven(h, k.B, dV, dI, 1e-8, 2, true, b->T); });
+        v.few = v.few_ms >= 0 && (v.sweep_ms[v.sweep] < 0 || v.few_ms <= v.sweep_ms[v.sweep]) ? 1 : 0;
+      }
       h->opt.factor = save_f;
       h->opt.sweep = save_s;
       cudaFree(dV);
@@ -399,7 +409,7 @@ extern "C" xbar_status xbar_batch_autotune(xbar_batch_t b, xbar_precision p, con
     for (int t = 0; t < b->T; ++t) {
       xbar_t ht = b->tiles[t];
       if (ht->m.M == k.M && ht->m.N == k.N && B[t] == k.B) {
-        ht->opt.sweep = v.sweep;
+        ht->opt.sweep = v.few == 1 ? -1 : v.sweep;
         ht->opt.factor = v.factor;
         if (p == XBAR_FP64) ht->opt.orient = v.orient;
       }

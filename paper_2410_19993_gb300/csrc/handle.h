@@ -217,6 +217,8 @@ inline int assembled_for(xbar_precision p) { return p == XBAR_FP64 ? 1 : 2; }
 // kernel-variant selection (environment XBAR_SWEEP=simt|tc, XBAR_FACTOR=group|cluster override)
 bool use_tc_sweep(const xbar_s* h);
 bool use_cluster_factor(const xbar_s* h);
+// whether a solve of B vectors, one of `tiles` side by side, takes the clusters for few vectors when left to choose
+bool chooses_few(const xbar_s* h, int B, int tiles);
 // block cyclic reduction (handle option XBAR_OPT_ALGORITHM, environment XBAR_ALGO=cr|thomas)
 bool use_cr(const xbar_s* h);
 // input vectors per panel of the cyclic-reduction substitution (Bpad = B rounded up to it)
