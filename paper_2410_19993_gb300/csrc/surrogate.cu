@@ -790,17 +790,21 @@ __global__ void __launch_bounds__(32 * kHeadWarps) head_kernel(const __nv_bfloat
   }
 }
 
-// out[k] += sum over rows of D[r][k] (bias gradients) for two matrices at once (blockIdx.y); block = 256
-// threads = one column each, `chunk` rows
-__global__ void colsum_kernel(const __nv_bfloat16* D0, const __nv_bfloat16* D1, long rows, long chunk, float* out0,
-                              float* out1) {
+// out[k] += sum over rows of D[r][k] (bias gradients) for two matrices at once (blockIdx.y); a block takes `chunk`
+// rows, four threads a column
+constexpr int kColParts = 4;
+__global__ void __launch_bounds__(kColParts* kH) colsum_kernel(const __nv_bfloat16* D0, const __nv_bfloat16* D1,
+                                                               long rows, long chunk, float* out0, float* out1) {
+  __shared__ float part[kColParts][kH];
   const __nv_bfloat16* D = blockIdx.y ? D1 : D0;
-  const int k = threadIdx.x;
+  const int k = threadIdx.x % kH, q = threadIdx.x / kH;
   const long r0 = blockIdx.x * chunk, r1 = min(rows, r0 + chunk);
   float s = 0.0f;
 #pragma unroll 8
-  for (long r = r0; r < r1; ++r) s += __bfloat162float(D[r * kH + k]);
-  atomicAdd((blockIdx.y ? out1 : out0) + k, s);
+  for (long r = r0 + q; r < r1; r += kColParts) s += __bfloat162float(D[r * kH + k]);
+  part[q][k] = s;
+  __syncthreads();
+  if (q == 0) atomicAdd((blockIdx.y ? out1 : out0) + k, (part[0][k] + part[1][k]) + (part[2][k] + part[3][k]));
 }
 
 // Adam on the flat FP32 parameters
@@ -1043,9 +1047,10 @@ static xbar_status fwd_bwd(xbar_surrogate_t s, const __nv_bfloat16* X, long rows
                                      1.0f / (float)valid, (__nv_bfloat16*)s->dZ2.p, s->Gr + s->oW3, s->Gr + s->ob3,
                                      s->loss);
   XB_CUDA(cudaGetLastError());
-  // weight gradients contract over the rows: split so that the few output tiles (4 and 2 Fp / 128)
-  // fill the SMs
-  const int ks = (int)std::max<long>(1, std::min<long>(64, rows / 256));
+  // Weight gradients contract over the rows: split so that the few output tiles (4 and 2 Fp / 128) fill the SMs.
+  // The parts meet in atomic additions to zero, whose order does not matter for two: below 3072 rows (up to
+  // 1024 for the bias gradients) there are no more, and a minibatch gives the same bits every time.
+  const int ks = (int)std::max<long>(1, std::min<long>(rows < 3072 ? 2 : 64, rows / 256));
   // dW2 = dZ2^T H1
   memset(&g, 0, sizeof(g));
   g.status = s->status;
@@ -1072,9 +1077,9 @@ static xbar_status fwd_bwd(xbar_surrogate_t s, const __nv_bfloat16* X, long rows
   g.mode = GEMM_EPI_STORE; g.C = s->Gr + s->oW1; g.ldc = Fp; g.atomic = 1;
   XB_CUDA(launch_gemm_bf16(g, ks, s->st));
   // bias gradients
-  const long chunk = std::max<long>(32, (rows + s->nsm - 1) / s->nsm);
+  const long chunk = rows <= 1024 ? rows / 2 : std::max<long>(32, (rows + s->nsm - 1) / s->nsm);
   const int nb = (int)((rows + chunk - 1) / chunk);
-  colsum_kernel<<<dim3(nb, 2), kH, 0, s->st>>>((const __nv_bfloat16*)s->dZ2.p, (const __nv_bfloat16*)s->dZ1.p, rows,
+  colsum_kernel<<<dim3(nb, 2), kColParts * kH, 0, s->st>>>((const __nv_bfloat16*)s->dZ2.p, (const __nv_bfloat16*)s->dZ1.p, rows,
                                               chunk, s->Gr + s->ob2, s->Gr + s->ob1);
   XB_CUDA(cudaGetLastError());
   return XBAR_OK;
