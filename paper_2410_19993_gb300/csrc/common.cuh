@@ -185,9 +185,14 @@ __device__ __forceinline__ void atomic_max_nonneg(float* addr, float v) {
   atomicMax(reinterpret_cast<int*>(addr), __float_as_int(v));
 }
 
-// Reciprocal of an FP64 pivot.  Normal-sized pivots take the hardware's approximate reciprocal (~2^-20) and
-// one cubic step, 1/pv = r (1 + e + e^2), e = 1 - pv r: three dependent operations against seven of
-// a division; the rest divide.
+// Reciprocal of an FP64 pivot.  Pivots of normal size take the hardware's approximate reciprocal r and one step
+// of the third-order Chebyshev (Householder) iteration for 1/pv, the start of the series
+//     1/pv = r / (1 - e) = r (1 + e + e^2 + ...),   e = 1 - pv r;
+// the rest divide.  Error: r carries about 20 bits, so e (exact to 2^-73: r has few bits, one fused operation)
+// is at most about 2^-20 and the terms left out are e^3 ~ 2^-60 of the result, 2^-7 of its last place; with
+// the final rounding the result is within 0.51 units in the last place, where a division is within 0.5.
+// The chains of pivots are made of this operation: FP64 factor and solve of one vector, 256 x 256 17.9 ms against
+// 18.3 with a division, 256 x 32 (cyclic reduction) 576 against 596 us.
 __device__ __forceinline__ double pivot_rcp(double pv) {
   const unsigned ex = ((unsigned)__double2hiint(pv) >> 20) & 0x7ffu;
   if (ex - 64u < 1920u) {
