@@ -43,6 +43,7 @@ constexpr int kWork = 128;             // threads of the row work: two columns a
 constexpr int kInvWarp = kWork / 32;   // one more warp inverts pivot blocks meanwhile
 constexpr int kThreads = kWork + 32;
 constexpr int kRows = 16;
+static_assert(kThreads == 160, "named barriers");
 static_assert(2 * kWork == kRows * kRows, "two elements of a pivot block per thread");
 
 __device__ __forceinline__ uint32_t cluster_rank() {
@@ -50,7 +51,19 @@ __device__ __forceinline__ uint32_t cluster_rank() {
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
   return r;
 }
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+// Arrival of a block on the cluster barrier that orders the block's reads before it.  A release by every warp costs
+// each of them a fence (256 x 256: 55 us a factor); here the work warps arrive on a block barrier, which
+// orders their reads before the inversion warp's part of it, and relaxed on the cluster barrier, and the
+// inversion warp, which has nothing else to do then, releases for all.
+__device__ __forceinline__ void cluster_arrive(bool work) {
+  if (work) {
+    asm volatile("bar.arrive 2, 160;" ::: "memory");
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+  } else {
+    asm volatile("bar.sync 2, 160;" ::: "memory");
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  }
+}
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -619,9 +632,8 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
       for (int c = 0; c < 2; ++c) sg_prev[c] = __ldcg(sig + (size_t)(s & 1) * Mp + kc[c]);
     // every block's reads of this step's slots and blocks come before the next step's first hand-over: arrive
-    // here (release: a relaxed arrival would not order the reads), wait there, with the next column's
-    // formation in between
-    cluster_arrive();
+    // here, wait there, with the next column's formation in between
+    cluster_arrive(warp < kInvWarp);
   }
   {
     if (colt)
