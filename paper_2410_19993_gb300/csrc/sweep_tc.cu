@@ -752,7 +752,10 @@ cudaError_t launch_sweep_tc(const SweepParams<float>& p, const void* Xt, int ter
     return cudaGetLastError();
   };
   const bool left = p.meet > 0, right = p.meet < p.N - 1;
-  if (Mt == 128 && left && !right) return launch(kBoth, 1, 0);
+  // One chain: both parts in one launch where a launch is long against the chain (256 tiles of 16 x 16 with 512
+  // vectors each 11.47 -> 10.81 ms a run); the 16 x 128 tiles among 30 with 4096 vectors: 43.65 ms in two launches,
+  // 43.9 in one.
+  if (Mt == 128 && left && !right && p.N <= 64) return launch(kBoth, 1, 0);
   const bool right_in = right && p.rhs;  // an input vector enters at column 0 only
   if (left || right_in) {
     const cudaError_t err = launch(kIn, left && right_in ? 2 : 1, left ? 0 : 1);
