@@ -109,62 +109,44 @@ __device__ __forceinline__ void load_vec(T (&r)[n], const T* p) {
   }
 }
 
-// Chain of a block: blockIdx.y + chain0.  The inward part, the meeting column and the outward part, or with a
-// single chain (m = N - 1) both, one after the other: a block's z is then its own threads'.
-enum { kIn, kOutward, kBoth };
-template <typename T, int TR, int TC, int kPart>
-__global__ void __launch_bounds__(sweep_max_threads<TR, TC>()) sweep_kernel(SweepParams<T> p, int KC, int chain0) {
+// One part of a chain's walk: the inward part, or (kOut) the meeting column and the outward part.  `used`: chunks the
+// block has copied before.  False when a wait ran out.
+template <typename T, int TR, int TC, bool kOut>
+__device__ __forceinline__ bool sweep_part(const SweepParams<T>& p, int KC, int chain, unsigned char* smem_raw,
+                                           uint64_t wlim, long long used, float& local_max) {
   const int Mp = p.Mp, N = p.N, Bp = p.Bp, Bpad = p.Bpad;
   const int nrg = Mp / TR, ncg = Bp / TC;
   const int tid = threadIdx.x;
-  const uint64_t wlim = wait_limit(p.status);  // read once: the waits below sit on critical paths
   const int rg = tid / ncg, cg = tid - rg * ncg;
   const int i0 = rg * TR, c0 = cg * TC;
   const int b0 = blockIdx.x * Bp;
 
-  extern __shared__ __align__(128) unsigned char smem_raw[];
   uint64_t* mbar = reinterpret_cast<uint64_t*>(smem_raw);                  // 2 mbarriers
   T* xs = reinterpret_cast<T*>(smem_raw + 64);                             // [2][KC][Mp]
   T* vin = xs + 2 * (size_t)KC * Mp;                                       // [Mp][Bp]
   T* red = vin + (size_t)Mp * Bp;                                          // [nrg][Bp]
 
-  if (p.skip && *p.skip) return;
-  if (nrg * ncg != (int)blockDim.x || b0 + Bp > Bpad) {
-    if (tid == 0) set_status(p.status, XBAR_DEV_BADLAUNCH);
-    return;
-  }
-
   const int chunks_per_step = Mp / KC;
-  const int m = p.meet, chain = (int)blockIdx.y + chain0;
+  const int m = p.meet;
   const int len = chain == 0 ? m : N - 1 - m;  // columns of the chain
-  const unsigned chunk_bytes = (unsigned)(KC * Mp * sizeof(T));
-  if (tid == 0) {
-    mbar_init(&mbar[0], 1);
-    mbar_init(&mbar[1], 1);
-    fence_mbar_init();
-  }
-  __syncthreads();
-  long long c = 0;  // chunks used so far: buffer and phase
-  float local_max = 0.0f;
-  for (int part = kPart == kBoth && len > 0 ? kIn : kPart == kIn ? kIn : kOutward; part <= (kPart == kIn ? kIn : kOutward);
-       ++part) {
-  const bool kOut = kPart == kBoth ? part == kOutward : kPart == kOutward;
   const int nsteps = len + (kOut ? 1 : 0);
   // column of step s: inward 0, 1, .. (left) or N-1, N-2, .. (right); outward m, then away from it
   const int jdir = (chain == 0) == kOut ? -1 : 1, jstart = kOut ? m : (chain == 0 ? 0 : N - 1);
   auto col_of = [&](int s) { return jstart + jdir * s; };
-  const long long cend = c + (long long)nsteps * chunks_per_step, cbase = c;
-  auto chunk_src = [&](long long q) -> const T* {
-    q -= cbase;
-    const int s = (int)(q / chunks_per_step);
-    const int k0 = (int)(q - (long long)s * chunks_per_step) * KC;
+  const long long nchunks = (long long)nsteps * chunks_per_step;
+  const unsigned chunk_bytes = (unsigned)(KC * Mp * sizeof(T));
+  auto chunk_src = [&](long long c) -> const T* {
+    const int s = (int)(c / chunks_per_step);
+    const int k0 = (int)(c - (long long)s * chunks_per_step) * KC;
     const int j = col_of(s);
     return p.X + ((size_t)j * Mp + k0) * Mp;
   };
+
   if (tid == 0) {
-    if (c > 0) fence_proxy_async_smem();
-    mbar_arrive_expect_tx(&mbar[c & 1], chunk_bytes);
-    bulk_g2s(xs + (size_t)(c & 1) * KC * Mp, chunk_src(c), chunk_bytes, &mbar[c & 1]);
+    const int nb = (int)(used & 1);
+    if (used) fence_proxy_async_smem();
+    mbar_arrive_expect_tx(&mbar[nb], chunk_bytes);
+    bulk_g2s(xs + (size_t)nb * KC * Mp, chunk_src(0), chunk_bytes, &mbar[nb]);
   }
 
   // input of step 0: the right-hand side of its column and, in the meeting column, both chains' z
@@ -186,6 +168,7 @@ __global__ void __launch_bounds__(sweep_max_threads<TR, TC>()) sweep_kernel(Swee
   __syncthreads();
 
   T acc[TR][TC];
+  long long c = 0;
   for (int s = 0; s < nsteps; ++s) {
     const int j = col_of(s);
 #pragma unroll
@@ -194,16 +177,16 @@ __global__ void __launch_bounds__(sweep_max_threads<TR, TC>()) sweep_kernel(Swee
       for (int b = 0; b < TC; ++b) acc[a][b] = (T)0;
 
     for (int kc = 0; kc < chunks_per_step; ++kc, ++c) {
-      if (tid == 0 && c + 1 < cend) {
-        const int nb = (int)((c + 1) & 1);
+      if (tid == 0 && c + 1 < nchunks) {
+        const int nb = (int)((used + c + 1) & 1);
         fence_proxy_async_smem();
         mbar_arrive_expect_tx(&mbar[nb], chunk_bytes);
         bulk_g2s(xs + (size_t)nb * KC * Mp, chunk_src(c + 1), chunk_bytes, &mbar[nb]);
       }
-      const bool ok = mbar_wait_bounded(&mbar[c & 1], (unsigned)((c >> 1) & 1), p.status,
+      const bool ok = mbar_wait_bounded(&mbar[(used + c) & 1], (unsigned)(((used + c) >> 1) & 1), p.status,
                                         wlim);
-      if (__syncthreads_or(!ok)) return;
-      const T* xb = xs + (size_t)(c & 1) * KC * Mp;
+      if (__syncthreads_or(!ok)) return false;
+      const T* xb = xs + (size_t)((used + c) & 1) * KC * Mp;
       const T* vb = vin + (size_t)kc * KC * Bp;
 #pragma unroll 4
       for (int k = 0; k < KC; ++k) {
@@ -305,6 +288,37 @@ __global__ void __launch_bounds__(sweep_max_threads<TR, TC>()) sweep_kernel(Swee
     }
     __syncthreads();
   }
+  return true;
+}
+
+// Chain of a block: blockIdx.y + chain0.  The inward part, the outward part, or with a single chain (m = N - 1) both,
+// one after the other: a block's z is then its own threads'.
+enum { kIn, kOutward, kBoth };
+template <typename T, int TR, int TC, int kPart>
+__global__ void __launch_bounds__(sweep_max_threads<TR, TC>()) sweep_kernel(SweepParams<T> p, int KC, int chain0) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  const int tid = threadIdx.x, chain = (int)blockIdx.y + chain0;
+  const uint64_t wlim = wait_limit(p.status);  // read once: the waits sit on critical paths
+  uint64_t* mbar = reinterpret_cast<uint64_t*>(smem_raw);
+  if (p.skip && *p.skip) return;
+  if ((p.Mp / TR) * (p.Bp / TC) != (int)blockDim.x || (int)(blockIdx.x * p.Bp) + p.Bp > p.Bpad) {
+    if (tid == 0) set_status(p.status, XBAR_DEV_BADLAUNCH);
+    return;
+  }
+
+  if (tid == 0) {
+    mbar_init(&mbar[0], 1);
+    mbar_init(&mbar[1], 1);
+    fence_mbar_init();
+  }
+  __syncthreads();
+  float local_max = 0.0f;
+  if constexpr (kPart == kBoth) {
+    if (!sweep_part<T, TR, TC, false>(p, KC, chain, smem_raw, wlim, 0, local_max)) return;
+    const long long used = (long long)p.meet * (p.Mp / KC);
+    if (!sweep_part<T, TR, TC, true>(p, KC, chain, smem_raw, wlim, used, local_max)) return;
+  } else {
+    if (!sweep_part<T, TR, TC, kPart == kOutward>(p, KC, chain, smem_raw, wlim, 0, local_max)) return;
   }
   if (p.max_rel) {
     for (int o = 16; o > 0; o >>= 1) local_max = fmaxf(local_max, __shfl_xor_sync(0xffffffffu, local_max, o));
@@ -328,9 +342,11 @@ static cudaError_t launch_tiled(const SweepParams<T>& p, int KC, cudaStream_t st
     return cudaGetLastError();
   };
   const bool left = p.meet > 0, right = p.meet < p.N - 1;
-  // one chain and narrow tiles: one launch (no block reads another's z)
+  // one chain of small blocks on narrow tiles: one launch (no block reads another's z).  Taller blocks have more
+  // to lose than a launch: 300 x 40 in FP32, one vector 3.10 ms a solve against 3.21 in two, 1000 vectors 12.8
+  // against 10.3
   if constexpr (TR == kNarrowTR)
-    if (!right) return launch(sweep_kernel<T, TR, TC, kBoth>, 1, 0);
+    if (left && !right && p.Mp <= 32) return launch(sweep_kernel<T, TR, TC, kBoth>, 1, 0);
   const bool right_in = right && p.rhs;  // an input vector enters at column 0 only
   if (left || right_in) {
     const cudaError_t err = launch(sweep_kernel<T, TR, TC, kIn>, left && right_in ? 2 : 1, left ? 0 : 1);
