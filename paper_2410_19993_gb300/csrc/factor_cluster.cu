@@ -6,7 +6,8 @@
 //     Z_m = C_m - g_w^2 X_{m-1} - g_w^2 X_{m+1}.
 // The factor is bound by the latency of its chain (16 dependent panels a column on 16 SMs), so half the
 // chain is half the time: 12.25 -> 6.2 ms at 256 x 256, 2.85 -> 1.45 ms at 128 x 128, on twice the SMs
-// (4.5 and 1.22 ms with the early hand-over and the shared coefficient broadcasts below).
+// (4.87 and 1.31 ms with the early hand-over and the shared coefficient broadcasts below).  Few columns, and
+// the tiles of a crowded batch, are eliminated from one end (one_chain in api.cu).
 // In a cluster of C blocks block g holds rows [g R, (g+1) R) of the current matrix in registers, one
 // thread per column (R = 16, C = Mp / R).
 // The in-place blocked Gauss-Jordan inversion uses panels of R rows, so panel p is exactly block p's
@@ -419,10 +420,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     // symmetric positive definite), two pivots at a time: one exchange for both, on the chain from panel to
     // panel, and each pivot with its own reciprocal, the second one that of the Schur complement (solving
     // for both rows by the 2 x 2 determinant needs one reciprocal, but rounds once more: 4.1e-8 instead of
-    // 1.7e-8 for the inverse of a 128-row block).  Lane l holds column l % 16 of rows 8 (l / 16) .. + 7.  The two pivot rows
-    // go through shared memory and stand for the pivot columns too (the swept part is antisymmetric to
-    // the rest): eight loads a step against 22 shuffles, which the one warp issues no faster than
-    // one per eight cycles (2.5k cycles a block; 1.2k this way).
+    // 1.7e-8 for the inverse of a 128-row block).  Lane l holds column l % 16 of rows 8 (l / 16) .. + 7.  The two
+    // pivot rows go through shared memory and stand for the pivot columns too (the swept part is antisymmetric
+    // to the rest): eight loads a step against 22 shuffles, which the one warp issues no faster than one per
+    // eight cycles.
     static_assert(R == 16, "register layout assumes 16 x 16 pivot blocks");
     const int ib = lane & 15, pa0 = (lane >> 4) * 8;
     float* slots = p.pbuf + (size_t)chain * C * slot;

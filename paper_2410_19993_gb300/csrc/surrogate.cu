@@ -1127,7 +1127,7 @@ static xbar_status map_prep(xbar_surrogate_t s, const double* G, long sGi, long 
                             cudaEvent_t columns_ready = nullptr) {
   const int M = s->M, N = s->N;
   const size_t mn = (size_t)M * N;
-  // one allocation: one for each buffer made the first call on a surrogate 160 us longer
+  // one allocation for the eight buffers, which a surrogate's first call waits for
   XB_CUDA(ensure_group(s->A, s->mapbuf, {{&s->Gt, mn * 8}, {&s->Tl, mn * 8}, {&s->Gf, mn * 4}, {&s->tau, mn * 4},
                                          {&s->St, mn * 4}, {&s->wl, mn * 4}, {&s->bl, mn * 4}, {&s->xg, mn * 4}}));
   const float gs = (float)(1.0 / s->R[0]), gw = (float)(1.0 / s->R[1]), gb = (float)(1.0 / s->R[2]),

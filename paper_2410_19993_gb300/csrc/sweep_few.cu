@@ -312,8 +312,10 @@ __global__ void few_currents_kernel(SweepParams<T> p, int C, int RR) {
 // Widths.  Both chains' clusters of every panel run at once (2 panels C <= SMs), with as few vectors a
 // panel as that allows: a step's products take NV Mp RR / 1.7 cycles in FP64 (16 rows of 256: 2.4k a
 // vector) beside about 1.2k of exchange.  Eight rows a block up to 128 rows, where the cluster still
-// fits, else sixteen.  Wider batches go to the panels of sweep.cu / sweep_tc.cu: beyond eight vectors
-// a panel the FP64 pipe is as busy there, and a tensor-core step no longer costs more than four of these.
+// fits, else sixteen.  Wider batches go to the panels of sweep.cu / sweep_tc.cu.  At the border, a solve with eight
+// vectors a panel against one on panels: 256 rows, 32 vectors: FP64 4.10 ms (33 vectors on panels 7.10), mixed
+// 2.05 (3.88); 128 rows, 72 vectors: FP64 1.15 (1.80), mixed 0.84 (0.98); 64 rows, 152 vectors: 0.41 (0.50) and
+// 0.44 (0.53); 16 rows, 608 vectors: mixed 0.27 (0.32).
 FewPlan sweep_few_plan(int Mp, int B, int nsm) {
   FewPlan f;
   if (Mp > 256 || B < 1) return f;
