@@ -216,12 +216,6 @@ static int cr_sweep_launches(const xbar_s* h, bool initial, bool first_only) {
   return 2 + (first_only ? 0 : L + 1) + (initial ? 0 : L + 1);
 }
 
-// kernel launches of one block-Thomas substitution (sweep.cu, sweep_tc.cu): the inward part, unless an
-// input vector (V) meets no left chain or the system has one column, and the outward part
-static int sweep_launches(int meet, int N, bool V, bool few = false) {
-  return 1 + (meet > 0 || (!V && meet < N - 1) ? 1 : 0) + (few ? 1 : 0);  // few: and the currents
-}
-
 // The substitution kernel of a block-Thomas factor for a batch: clusters for a few vectors
 // (sweep_few.cu), otherwise the tensor cores (mixed precision, sweep_tc.cu) or the CUDA cores.  An
 // explicit choice of the FP32 kernel (XBAR_OPT_SWEEP_KERNEL, XBAR_SWEEP) is kept.
@@ -253,6 +247,18 @@ static SweepKind sweep_kind(const xbar_s* h, int B, bool mixed, int tiles = 1) {
                   : sweep_panel_width<double>(h->m.Mp, B, h->nsm);
   return k;
 }
+// kernel launches of one block-Thomas substitution (sweep.cu, sweep_tc.cu, sweep_few.cu): the inward part, unless an
+// input vector (V) meets no left chain or the system has one column, the outward part (one launch of both for some
+// single chains), and with few vectors the currents, unless only the first block is wanted
+static int sweep_launches(const xbar_s* h, const SweepKind& k, bool mixed, bool V, bool first_only = false) {
+  const int Mp = h->m.Mp, N = h->m.N, meet = h->meet;
+  if (!k.few.nv && (k.tc    ? sweep_tc_one_launch(Mp, N, meet)
+                    : mixed ? sweep_one_launch<float>(Mp, k.Bp, N, meet)
+                            : sweep_one_launch<double>(Mp, k.Bp, N, meet)))
+    return 1;
+  return 1 + (meet > 0 || (!V && meet < N - 1) ? 1 : 0) + (k.few.nv && !first_only ? 1 : 0);
+}
+
 bool xbar::chooses_few(const xbar_s* h, int B, int tiles) {
   return sweep_kind(h, B, h->prec == XBAR_FP32_IR, tiles).few.nv > 0;
 }
@@ -381,7 +387,7 @@ static xbar_status solve_rows(xbar_s* h, int B, const double* dV, double* dI, do
   double* w2 = (double*)g->w64.p;
   {
     PhaseScope ps(h, XBAR_PHASE_SWEEP, 2 + (cr ? cr_sweep_launches(g, false, !dvWL && !dvBL)
-                                                       : sweep_launches(g->meet, N2, false)));
+                                               : sweep_launches(g, kind, false, false, !dvWL && !dvBL)));
     XB_CUDA(launch_orient_rhs(dV, m2.h, M, M2, Mp2, B, Bpad, rhs, st));
     if (cr) {
       CrSweepArgs<double> ca;
@@ -531,7 +537,10 @@ static xbar_status solve_rows_mixed(xbar_s* h, int B, const double* dV, double* 
     ca.tensor = use_cr_tensor(g) && Bpad >= 128;
     return cr_sweep<float>(g, g->cr32, ca);
   };
-  const int nsw = cr ? cr_sweep_launches(g, false, false) : sweep_launches(g->meet, N2, false);
+  SweepKind kind;  // panels (no clusters)
+  kind.tc = tc;
+  kind.Bp = Bp;
+  const int nsw = cr ? cr_sweep_launches(g, false, false) : sweep_launches(g, kind, true, false);
   {  // x0 = solve32(s o (V h')), the state w = s o x0, I from the state
     PhaseScope ps(h, XBAR_PHASE_SWEEP, 1 + nsw + 1 + (tc ? 0 : 1));
     XB_CUDA(launch_orient_rhs32(dV, m2.h, m2.s32, h->m.M, M2, Mp2, B, Bpad, (float*)g->rhat.p, st));
@@ -730,10 +739,11 @@ xbar_status xbar::factor_handle(xbar_s* h, xbar_precision p, bool upload_params)
     PhaseScope ps(h, XBAR_PHASE_FACTOR, 1);
     xbar_status s = factor_mirror(h, p);
     if (s != XBAR_OK) return s;
-    // map remap + assembly (2) + the factor (one launch, or the cyclic reduction's operations)
+    // map remap + assembly (2) + the factor (block Thomas, or the cyclic reduction's operations)
     const xbar_s* g = h->mirror;
+    const int thomas = p == XBAR_FP64 || !use_cluster_factor(g) ? 1 : factor_cluster_launches(g->m.N);
     ps.nlaunch = 3 + (g->cr_active ? (int)(p == XBAR_FP64 ? g->cr64.ops.size() : g->cr32.ops.size())
-                                   : 1 + g->tc_ready);
+                                   : thomas + g->tc_ready);
     h->orient_active = 1;
     h->cr_active = 0;
     h->tc_ready = 0;
@@ -943,7 +953,7 @@ extern "C" xbar_status xbar_solve(xbar_t h, int B, const double* V, double* I, d
       ca.I = dI;
       XB_CUDA(cr_sweep<double>(h, h->cr64, ca));
     } else {
-      PhaseScope ps(h, XBAR_PHASE_SWEEP, sweep_launches(h->meet, N, true, few));
+      PhaseScope ps(h, XBAR_PHASE_SWEEP, sweep_launches(h, kind, false, true));
       XB_CUDA(run_sweep<double>(sp, kind, nullptr, 0, st));
     }
     rp.w = (double*)h->w64.p;
@@ -1009,7 +1019,7 @@ extern "C" xbar_status xbar_solve(xbar_t h, int B, const double* V, double* I, d
       return cr_sweep<float>(h, h->cr32, ca);
     };
     if (kind.tc || few) {  // x0 = solve32(b); the sweep writes the state w = s o x0 (FP32) itself
-      PhaseScope ps(h, XBAR_PHASE_SWEEP, sweep_launches(h->meet, N, true, few));
+      PhaseScope ps(h, XBAR_PHASE_SWEEP, sweep_launches(h, kind, true, true));
       XB_CUDA(ensure(h->A, h->w1, nst * 4));
       sp.w = nullptr;
       sp.w1out = (float*)h->w1.p;
@@ -1020,7 +1030,7 @@ extern "C" xbar_status xbar_solve(xbar_t h, int B, const double* V, double* I, d
       rp.w1 = (const float*)h->w1.p;  // read as (w, 0) until the first update writes the pairs
     } else {
       {
-        PhaseScope ps(h, XBAR_PHASE_SWEEP, cr ? cr_sweep_launches(h, true, false) : sweep_launches(h->meet, N, true));
+        PhaseScope ps(h, XBAR_PHASE_SWEEP, cr ? cr_sweep_launches(h, true, false) : sweep_launches(h, kind, true, true));
         XB_CUDA(sweep32(sp, kInitialTerms));    // x0 = solve32(b)
       }
       PhaseScope ps(h, XBAR_PHASE_UPDATE);
@@ -1041,7 +1051,7 @@ extern "C" xbar_status xbar_solve(xbar_t h, int B, const double* V, double* I, d
       sp.accumulate = 1;
       sp.max_rel = (float*)h->maxrel.p;
       {
-        PhaseScope ps(h, XBAR_PHASE_SWEEP, cr ? cr_sweep_launches(h, false, false) : sweep_launches(h->meet, N, false, few));
+        PhaseScope ps(h, XBAR_PHASE_SWEEP, cr ? cr_sweep_launches(h, false, false) : sweep_launches(h, kind, true, false));
         XB_CUDA(sweep32(sp, correction_terms(it)));  // dhat = solve32(rhat), I += dI
       }
       w_current = false;

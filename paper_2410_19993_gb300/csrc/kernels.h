@@ -150,6 +150,10 @@ template <typename T>
 cudaError_t launch_sweep(const SweepParams<T>& p, cudaStream_t st);
 template <typename T>
 int sweep_panel_width(int Mp, int B, int nsm);
+// whether a single chain's inward and outward part are one launch (sweep.cu, sweep_tc.cu)
+template <typename T>
+bool sweep_one_launch(int Mp, int Bp, int N, int meet);
+bool sweep_tc_one_launch(int Mp, int N, int meet);
 
 // ---- sweeps of a few vectors (sweep_few.cu): a cluster of Mp / rr blocks per chain and panel of nv ----
 struct FewPlan {

@@ -16,7 +16,8 @@
 // has no inward part; refinement passes give a full r).  Every step is a dense (Mp x Mp) x (Mp x Bp)
 // product over a panel of Bp input vectors.  The inward and the outward parts are two launches; in each
 // a block owns one panel and one chain, so the chains of a panel run side by side and a solve is N
-// dependent steps deep instead of 2N - 1, with 1.5 N products for an input vector instead of 2N - 1.
+// dependent steps deep instead of 2N - 1, with 1.5 N products for an input vector instead of 2N - 1.  (A
+// single chain's two parts are one launch for small blocks, see sweep_one_launch.)
 // (Both blocks of a panel form w_m, one product of N.)  z_j goes to global memory in between.
 //
 // Data movement: X_j is streamed through shared memory in chunks of KC rows by the bulk-copy
@@ -326,6 +327,13 @@ __global__ void __launch_bounds__(sweep_max_threads<TR, TC>()) sweep_kernel(Swee
   }
 }
 
+// One chain of small blocks on narrow tiles (no block reads another's z).  Taller blocks have more to lose than a
+// launch: 300 x 40 in FP32, one vector 3.10 ms a solve against 3.21 in two, 1000 vectors 12.8 against 10.3.
+template <typename T>
+bool sweep_one_launch(int Mp, int Bp, int N, int meet) {
+  return meet > 0 && meet == N - 1 && Mp <= 32 && sweep_is_narrow<T>(Mp, Bp);
+}
+
 template <typename T, int TR, int TC>
 static cudaError_t launch_tiled(const SweepParams<T>& p, int KC, cudaStream_t st) {
   if (p.Mp % TR || p.Bp % TC || p.Mp % KC) return cudaErrorInvalidValue;
@@ -342,11 +350,8 @@ static cudaError_t launch_tiled(const SweepParams<T>& p, int KC, cudaStream_t st
     return cudaGetLastError();
   };
   const bool left = p.meet > 0, right = p.meet < p.N - 1;
-  // one chain of small blocks on narrow tiles: one launch (no block reads another's z).  Taller blocks have more
-  // to lose than a launch: 300 x 40 in FP32, one vector 3.10 ms a solve against 3.21 in two, 1000 vectors 12.8
-  // against 10.3
   if constexpr (TR == kNarrowTR)
-    if (left && !right && p.Mp <= 32) return launch(sweep_kernel<T, TR, TC, kBoth>, 1, 0);
+    if (sweep_one_launch<T>(p.Mp, p.Bp, p.N, p.meet)) return launch(sweep_kernel<T, TR, TC, kBoth>, 1, 0);
   const bool right_in = right && p.rhs;  // an input vector enters at column 0 only
   if (left || right_in) {
     const cudaError_t err = launch(sweep_kernel<T, TR, TC, kIn>, left && right_in ? 2 : 1, left ? 0 : 1);
@@ -363,6 +368,8 @@ cudaError_t launch_sweep(const SweepParams<T>& p, cudaStream_t st) {
   return launch_tiled<T, SweepCfg<T>::TR, SweepCfg<T>::TC>(p, KC, st);
 }
 
+template bool sweep_one_launch<float>(int, int, int, int);
+template bool sweep_one_launch<double>(int, int, int, int);
 template int sweep_panel_width<float>(int, int, int);
 template int sweep_panel_width<double>(int, int, int);
 template cudaError_t launch_sweep<float>(const SweepParams<float>&, cudaStream_t);

@@ -5,7 +5,8 @@
 //     z_j = X_j (r_j + e o z_prev),
 // then the meeting column w_m = X_m (r_m + e_{m-1} o z_{m-1} + e_m o z_{m+1}) and outward along both chains,
 //     w_j = z_j + X_j (e o w_prev);   I_j = hs_j . w_j,
-// a block per chain and panel of 64 input vectors.  Each step is D[Mt x 64] = X_j[Mt x Mt] . v[Mt x 64]
+// a block per chain and panel of 64 input vectors (a short single chain: both parts in one launch).
+// Each step is D[Mt x 64] = X_j[Mt x Mt] . v[Mt x 64]
 // computed from three-term BF16 splits (x = x0 + x1 + x2, each BF16: together 24+ significant bits,
 // FP32-level accuracy; a plain BF16 or TF32 product would cost the refinement extra passes).  With
 // KP leading terms used, each K step of 16 issues A_p v_q for every p + q < KP (N = 64 each) into
@@ -705,6 +706,11 @@ static size_t sweep_tc_smem_bytes(int Mt, int KP, bool two) {
 
 bool sweep_tc_supported(int Mp) { return Mp <= 256; }
 
+// One chain: both parts in one launch where a launch is long against the chain (256 tiles of 16 x 16 with 512
+// vectors each 11.47 -> 10.81 ms a run); the 16 x 128 tiles among 30 with 4096 vectors: 43.65 ms in two launches,
+// 43.9 in one.
+bool sweep_tc_one_launch(int Mp, int N, int meet) { return Mp <= 128 && meet > 0 && meet == N - 1 && N <= 64; }
+
 int sweep_tc_rows(int Mp) { return Mp <= 128 ? 128 : 256; }
 
 size_t sweep_tc_tile_bytes(int Mp, int N) {
@@ -752,10 +758,7 @@ cudaError_t launch_sweep_tc(const SweepParams<float>& p, const void* Xt, int ter
     return cudaGetLastError();
   };
   const bool left = p.meet > 0, right = p.meet < p.N - 1;
-  // One chain: both parts in one launch where a launch is long against the chain (256 tiles of 16 x 16 with 512
-  // vectors each 11.47 -> 10.81 ms a run); the 16 x 128 tiles among 30 with 4096 vectors: 43.65 ms in two launches,
-  // 43.9 in one.
-  if (Mt == 128 && left && !right && p.N <= 64) return launch(kBoth, 1, 0);
+  if (sweep_tc_one_launch(p.Mp, p.N, p.meet)) return launch(kBoth, 1, 0);
   const bool right_in = right && p.rhs;  // an input vector enters at column 0 only
   if (left || right_in) {
     const cudaError_t err = launch(kIn, left && right_in ? 2 : 1, left ? 0 : 1);
