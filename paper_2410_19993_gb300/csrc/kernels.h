@@ -81,8 +81,8 @@ int factor_panel_width();
 //   * rows per worker: as few as two chains can keep resident, 64 workers a chain at 128 and at 256 rows
 //     (the FP64 work of a panel then takes no longer than its pivot chain), and 8 rows above.  `beside`: the
 //     tiles of a batch share the SMs and a factor starts when all its blocks fit at once, so with 8 rows
-//     four times as many tiles run side by side.  256 x 256, one vector, as four 128-row tiles 17.5 -> 5.1 ms,
-//     as sixteen of 64 rows 9.6 -> 3.2;
+//     four times as many tiles run side by side.  256 x 256, one vector, as four 128-row tiles 5.1 ms (17.5 with
+//     2 rows a worker), as sixteen of 64 rows 3.2 (9.6);
 //   * both chains equally long, the left one with the meeting column.  Above 512 rows one chain already takes
 //     more than half of the SMs, and there is only that;
 //   * with fewer SMs 8 rows, then one chain, then no plan (rows = 0): the group kernel of factor.cu.
